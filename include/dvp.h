@@ -166,9 +166,8 @@ typedef struct {
  *                 a second, the launch ends by itself with undefined outputs and
  *                 dvp_row_wait_status reports code 1 or 2
  *
- * Rows whose start is 32-byte aligned in all three matrices take the
- * vectorised kernels; any other layout takes a scalar kernel, same results.
- * Needs no workspace.  Errors: DVP_ERR_INVALID_ARG for NULL required
+ * Any row stride and any base that is aligned to its element type is taken at full
+ * width: rows are cut at their own 32-byte boundaries.  Needs no workspace.  Errors: DVP_ERR_INVALID_ARG for NULL required
  * pointers, T < 0, V < 1, ld < V, rho outside [0,1] or NaN, upstream without
  * grad_train or the reverse, a malformed launch_hint; DVP_ERR_UNSUPPORTED
  * for unknown dtypes or V >= 2^31 - 256.  Rows too long for the on-chip row

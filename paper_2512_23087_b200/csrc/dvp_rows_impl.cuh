@@ -438,12 +438,51 @@ __device__ __forceinline__ SumCount cluster_reduce_sumcount(SumCount v, float *s
   return r;
 }
 
+// A row as the sweeps see it.  Granules are cut at the row's own 32-byte boundaries, so that a row may
+// start at any element (an odd vocabulary with its rows back to back): `head` elements lie in front of
+// the first boundary and, as those behind the last whole granule, are taken one per thread outside the
+// sweeps (at most 2 * kElems - 2 of them, fewer than a block has threads).
+// Measured against element-wise loads for such rows: float16, T = 1111 x V = 50,021, with the gradient,
+// 96 against 338 us; rows on 32-byte boundaries keep their time.
+template <typename TIn>
+struct RowView {
+  const TIn *row;   // element 0
+  const TIn *base;  // first element of this block's granules, 32-byte aligned
+  int V;
+  int head;      // elements in front of the row's first 32-byte boundary
+  int n_all;     // whole granules of the row
+  int g_first;   // first granule of this block (a cluster's blocks share the granules)
+  int n_full;    // whole granules of this block
+  bool extras;   // this block takes the elements outside the granules
+
+  __device__ __forceinline__ void set(const TIn *r, int V_, int rank, int n_ranks) {
+    constexpr int kElems = Granule<TIn>::kElems;
+    row = r;
+    V = V_;
+    const int mis = (int)(((uintptr_t)r & 31u) / sizeof(TIn));
+    head = min(V, mis ? kElems - mis : 0);
+    n_all = (V - head) / kElems;
+    const int per = (n_all + n_ranks - 1) / n_ranks;
+    g_first = min(rank * per, n_all);
+    n_full = min(per, n_all - g_first);
+    base = r + head + (size_t)g_first * kElems;
+    extras = rank == 0;
+  }
+  // element of the row that this thread takes outside the granules; none when it is >= V
+  __device__ __forceinline__ int extra() const {
+    const int tid = (int)threadIdx.x;
+    return !extras ? V : tid < head ? tid : tid + n_all * Granule<TIn>::kElems;
+  }
+  // element k of the row counted from `base`
+  __device__ __forceinline__ int rel(int k) const { return k - head - g_first * Granule<TIn>::kElems; }
+};
+
 // Sweep 1 over (a part of) a row: block-wide log-sum-exp state; granule bounds
 // are left in shared memory.
 template <typename TIn, int kStage>
-__device__ __forceinline__ LogSum row_sweep1(const TIn *row, int V, uint16_t *bound, float *scratch) {
-  constexpr int kElems = Granule<TIn>::kElems;
-  const int n_full = V / kElems;  // the sweeps take whole granules; see row_tail
+__device__ __forceinline__ LogSum row_sweep1(const RowView<TIn> &v, uint16_t *bound, float *scratch) {
+  const TIn *row = v.base;
+  const int n_full = v.n_full;
   const int per_step = kStage * (int)blockDim.x;
   const int n_steps = (n_full + per_step - 1) / per_step;
   LogSum acc = {kNegInf, kNegInf, 0.f};
@@ -459,10 +498,10 @@ __device__ __forceinline__ LogSum row_sweep1(const TIn *row, int V, uint16_t *bo
     }
     if (step < n_steps) absorb_stage<TIn, kStage>(s0, step, acc, bound);
   }
-  // the elements behind the last whole granule, one per thread
-  const int k_tail = n_full * kElems + (int)threadIdx.x;
-  if (k_tail < V) {
-    const float x = Storage<TIn>::widen(row[k_tail]);
+  // the elements outside the granules, one per thread
+  const int k_extra = v.extra();
+  if (k_extra < v.V) {
+    const float x = Storage<TIn>::widen(v.row[k_extra]);
     if (x > kNegInf) {
       if (x > acc.m) {
         const float cn = x * kLog2e;
@@ -476,25 +515,25 @@ __device__ __forceinline__ LogSum row_sweep1(const TIn *row, int V, uint16_t *bo
   return block_reduce_logsum(acc, scratch);
 }
 
-// Sweep 2 over (a part of) a row: masked sum without the sampled token and count,
-// block-wide.  `a` is relative to `row` (outside [0, V): not in this part).
+// Sweep 2 over (a part of) a row: masked sum without the sampled token `a_row` and count, block-wide.
 template <typename TIn, int kStage>
-__device__ __forceinline__ SumCount row_sweep2(const TIn *row, int V, int a, float tau, float m,
+__device__ __forceinline__ SumCount row_sweep2(const RowView<TIn> &v, int a_row, float tau, float m,
                                                const uint16_t *bound, float *scratch,
                                                uint16_t *hot_smem, HotList &hot) {
-  constexpr int kElems = Granule<TIn>::kElems;
-  const int n_full = V / kElems;
+  const TIn *row = v.base;
+  const int n_full = v.n_full;
+  const int a = a_row >= 0 ? v.rel(a_row) : -1;
   const int per_step = kStage * (int)blockDim.x;
   const int n_slots = ((n_full + per_step - 1) / per_step) * kStage;  // whole granules per thread
   const int tid = threadIdx.x;
   SumCount sc = {0.f, 0};
-  {  // the elements behind the last whole granule, one per thread
-    const int k_tail = n_full * kElems + tid;
-    if (k_tail < V) {
-      const float x = Storage<TIn>::widen(row[k_tail]);
+  {  // the elements outside the granules, one per thread
+    const int k_extra = v.extra();
+    if (k_extra < v.V) {
+      const float x = Storage<TIn>::widen(v.row[k_extra]);
       if (x >= tau && x > kNegInf) {
         ++sc.n;
-        if (k_tail != a) sc.s += ex2((x - m) * kLog2e);
+        if (k_extra != a_row) sc.s += ex2((x - m) * kLog2e);
       }
     }
   }
@@ -533,14 +572,25 @@ __device__ __forceinline__ SumCount row_sweep2(const TIn *row, int V, int a, flo
   return block_reduce_sumcount(sc, scratch);
 }
 
-// Statistics of one side of one row.  `row` is the whole row (V elements); this
-// block sweeps the part [off, off + v_part) of it.
+// Statistics of one side of one row (this block sweeps its part of it).
 template <typename TIn, int kStage, int kCluster>
-__device__ __forceinline__ SideStats row_stats(const TIn *row, int V, int off, int v_part, int a,
-                                               double log_rho, int mode, float mask_value,
-                                               uint16_t *bound, float *scratch, float *cl_slots,
-                                               uint16_t *hot_smem, HotList &hot) {
-  const LogSum part = row_sweep1<TIn, kStage>(row + off, v_part, bound, scratch);
+__device__ __forceinline__ SideStats row_stats(const RowView<TIn> &v, int a, double log_rho, int mode,
+                                               float mask_value, uint16_t *bound, float *scratch,
+                                               float *cl_slots, uint16_t *hot_smem, HotList &hot) {
+  const TIn *row = v.row;
+  const int V = v.V;
+#ifdef DVP_DEBUG_BOUNDS
+  {  // extents of this block's part of the row and of its tables
+    const int per_step = kStage * (int)blockDim.x;
+    __syncthreads();
+    DVP_BOUNDS_SET(n_gran, v.n_full);
+    DVP_BOUNDS_SET(V, (long long)v.n_full * Granule<TIn>::kElems);
+    DVP_BOUNDS_SET(n_bound, (long long)((v.n_full + per_step - 1) / per_step) * per_step);
+    DVP_BOUNDS_SET(n_hot, kHotCap);  // entries of one warp's hot list
+    DVP_BOUNDS_SYNC();
+  }
+#endif
+  const LogSum part = row_sweep1<TIn, kStage>(v, bound, scratch);
   const LogSum all = cluster_reduce_logsum<kCluster>(part, cl_slots);
 
   SideStats st;
@@ -554,9 +604,8 @@ __device__ __forceinline__ SideStats row_stats(const TIn *row, int V, int off, i
   st.member = has_a && st.z_a >= st.tau;
   st.e_a = st.member ? ex2((st.z_a - st.m) * kLog2e) : 0.f;
 
-  const int a_part = (has_a && a >= off && a < off + v_part) ? a - off : -1;
-  const SumCount sc = row_sweep2<TIn, kStage>(row + off, v_part, a_part, st.tau, st.m, bound,
-                                              scratch, hot_smem, hot);
+  const SumCount sc =
+      row_sweep2<TIn, kStage>(v, has_a ? a : -1, st.tau, st.m, bound, scratch, hot_smem, hot);
   const SumCount tot = cluster_reduce_sumcount<kCluster>(sc, cl_slots + 4);
   st.s_x = tot.s;
   st.n = tot.n;
@@ -580,14 +629,59 @@ __device__ __forceinline__ void write_mask_row(const TIn *row, int V, float tau,
   }
 }
 
+// Gradient rows may be stored in granules when each of them starts, with its logits granule, on a
+// boundary of the granule's store (32 bytes, or 16 for float32 logits with a 2-byte gradient): elements.
+template <typename TIn, typename TGrad>
+__host__ __device__ constexpr int grad_align() {
+  return Granule<TIn>::kElems < 32 / (int)sizeof(TGrad) ? Granule<TIn>::kElems : 32 / (int)sizeof(TGrad);
+}
+
+// Sweep 3 when the gradient row lies differently than its logits row (another row stride or base):
+// zeros first, in the gradient row's own 32-byte pieces, then the safe tokens one by one.
+template <typename TIn, typename TGrad, int kStage>
+__device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *grow, int a, float tau, float tau_b,
+                                               float m, float coef, float g_a, const uint16_t *bound) {
+  constexpr int kElems = Granule<TIn>::kElems, kOut = 32 / (int)sizeof(TGrad);
+  const int tid = threadIdx.x, n_thr = (int)blockDim.x;
+  const int k0 = v.head + v.g_first * kElems, k1 = k0 + v.n_full * kElems;  // this block's granules, as elements
+  TGrad *dst = grow + k0;
+  const int n = k1 - k0;
+  const int mis = (int)(((uintptr_t)dst & 31u) / sizeof(TGrad));
+  const int head = min(n, mis ? kOut - mis : 0), n_vec = (n - head) / kOut;
+  const uint32_t z[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  if (tid < head) dst[tid] = Storage<TGrad>::narrow(0.f);
+  for (int i = tid; i < n_vec; i += n_thr) st_stream32(dst + head + (size_t)i * kOut, z);
+  const int k_rest = head + n_vec * kOut + tid;
+  if (k_rest < n) dst[k_rest] = Storage<TGrad>::narrow(0.f);
+  __syncthreads();  // the zeros of this block's part are in place before single elements replace them
+  const int n_slots = ((v.n_full + kStage * n_thr - 1) / (kStage * n_thr)) * kStage;
+  for (int i = 0; i < n_slots; ++i) {
+    const int g = i * n_thr + tid;
+    if (g >= v.n_full || !DVP_IN(bound_index<kStage>(i, tid), n_bound, DVP_OOB_BOUND)) break;
+    if (!(bf16_bits_to_float(bound[bound_index<kStage>(i, tid)]) >= tau_b)) continue;
+    Granule<TIn> gr;
+    gr.load_whole(v.base, v.n_full, g);
+    float x[kElems];
+    gr.get(x);
+    const int ja = a - g * kElems;
+#pragma unroll
+    for (int j = 0; j < kElems; ++j)
+      if (x[j] >= tau)
+        dst[(size_t)g * kElems + j] =
+            Storage<TGrad>::narrow(j == ja ? g_a : coef * ex2((x[j] - m) * kLog2e));
+  }
+}
+
 // Sweep 3: gradient of g * ln pi^mp(a) over the row.  Granules without a safe
 // token are written as zeros without being read.
-template <typename TIn, typename TGrad, int kStage>
-__device__ __forceinline__ void row_grad(const TIn *row, TGrad *grow, int V, int a,
+template <typename TIn, typename TGrad, int kStage, bool kLoose>
+__device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all, int a_row,
                                          const SideStats &st, float g, const uint16_t *bound,
                                          const HotList &hot) {
   constexpr int kElems = Granule<TIn>::kElems;
-  const int n_full = V / kElems;
+  const TIn *row = v.base;
+  const int n_full = v.n_full;
+  TGrad *grow = grow_all + (v.base - v.row);
   const int per_step = kStage * (int)blockDim.x;
   const int n_slots = ((n_full + per_step - 1) / per_step) * kStage;
   const int tid = threadIdx.x;
@@ -597,19 +691,24 @@ __device__ __forceinline__ void row_grad(const TIn *row, TGrad *grow, int V, int
   const bool live = st.live;
   const float coef = live ? -g / s_tot : 0.f;
   const float g_a = st.member ? g * ((st.s_x + st.s_mask) / s_tot) : 0.f;
-  const int a_live = (live && st.member) ? a : -1;
+  const int a_here = (live && st.member) ? a_row : -1;
+  const int a_live = a_here >= 0 ? v.rel(a_here) : -1;
   const bool listed = live && hot.fits();
   const float tau = live ? st.tau : -kNegInf;  // +inf: nothing passes
   const float tau_b = live ? bf16_round_down(st.tau) : -kNegInf;
 
-  {  // the elements behind the last whole granule, one per thread
-    const int k_tail = n_full * kElems + tid;
-    if (k_tail < V) {
-      const float x = Storage<TIn>::widen(row[k_tail]);
+  {  // the elements outside the granules, one per thread
+    const int k_extra = v.extra();
+    if (k_extra < v.V) {
+      const float x = Storage<TIn>::widen(v.row[k_extra]);
       float out = x >= tau ? coef * ex2((x - st.m) * kLog2e) : 0.f;
-      if (k_tail == a_live) out = g_a;
-      grow[k_tail] = Storage<TGrad>::narrow(out);
+      if (k_extra == a_here) out = g_a;
+      grow_all[k_extra] = Storage<TGrad>::narrow(out);
     }
+  }
+  if constexpr (kLoose) {
+    row_grad_loose<TIn, TGrad, kStage>(v, grow_all, a_live, tau, tau_b, st.m, coef, g_a, bound);
+    return;
   }
   for (int i = 0; i < n_slots; ++i) {
     const int gi = i * (int)blockDim.x + tid;
@@ -665,7 +764,10 @@ __host__ __device__ inline int smem_words_fixed(int threads) {
 // kWeighted: the upstream gradient is multiplied by the token's importance weight, which
 // needs the inference side's statistics before sweep 3 of the training row: that
 // instantiation sweeps the inference row first.
-template <typename TIn, typename TGrad, int kStage, int kThreads, int kBlocks, int kCluster, bool kWeighted>
+// kLoose: the gradient row lies differently than its logits row (an instantiation of its own: its code
+// between the sweeps costs the others up to 1 %).
+template <typename TIn, typename TGrad, int kStage, int kThreads, int kBlocks, int kCluster, bool kWeighted,
+          bool kLoose>
 __global__ void __launch_bounds__(kThreads, kBlocks) dvp_row_kernel(const RowParams p) {
   extern __shared__ __align__(16) float smem[];
   float *scratch = smem;        // 96 floats for the block reductions
@@ -681,22 +783,6 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_row_kernel(const RowPar
   const bool has_id = id >= 0, bad_id = id >= p.V;
   const int a = (has_id && !bad_id) ? (int)id : -1;
   const int V = (int)p.V;
-  // this block's part of the row, in whole granules
-  const int n_gran = (V + kElems - 1) / kElems;
-  const int per_rank = (n_gran + kCluster - 1) / kCluster;
-  const int off = min(rank * per_rank, n_gran) * kElems;
-  const int v_part = max(0, min(V - off, per_rank * kElems));
-#ifdef DVP_DEBUG_BOUNDS
-  {  // extents of this block's part of the row and of its tables
-    const int part_gran = (v_part + kElems - 1) / kElems, per_step = kStage * (int)blockDim.x;
-    DVP_BOUNDS_SET(n_gran, part_gran);
-    DVP_BOUNDS_SET(V, v_part);
-    DVP_BOUNDS_SET(n_bound, (long long)((part_gran + per_step - 1) / per_step) * per_step);
-    DVP_BOUNDS_SET(n_hot, kHotCap);  // entries of one warp's hot list
-    DVP_BOUNDS_SYNC();
-  }
-#endif
-
   const TIn *trow = reinterpret_cast<const TIn *>(p.train) + t * p.ld_train;
   uint32_t *mask_t = p.out_t.mask ? p.out_t.mask + t * ((p.V + 31) / 32) : nullptr;
   HotList hot;
@@ -704,12 +790,16 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_row_kernel(const RowPar
   if (kWeighted && p.infer) {  // otherwise an earlier launch left the inference side's results
     const TIn *irow = reinterpret_cast<const TIn *>(p.infer) + t * p.ld_infer;
     HotList hot_i;
-    si = row_stats<TIn, kStage, kCluster>(irow, V, off, v_part, a, p.log_rho, p.mode, p.mask_value, bound,
-                                          scratch, cl_slots + 8, hot_smem, hot_i);
+    RowView<TIn> vi;
+    vi.set(irow, V, rank, kCluster);
+    si = row_stats<TIn, kStage, kCluster>(vi, a, p.log_rho, p.mode, p.mask_value, bound, scratch, cl_slots + 8,
+                                          hot_smem, hot_i);
     __syncthreads();  // the bounds and the hot lists are reused for the second matrix
   }
-  st = row_stats<TIn, kStage, kCluster>(trow, V, off, v_part, a, p.log_rho, p.mode, p.mask_value, bound,
-                                        scratch, cl_slots, hot_smem, hot);
+  RowView<TIn> vt;
+  vt.set(trow, V, rank, kCluster);
+  st = row_stats<TIn, kStage, kCluster>(vt, a, p.log_rho, p.mode, p.mask_value, bound, scratch, cl_slots, hot_smem,
+                                        hot);
 
   if (p.grad) {
     float g = p.upstream[t];
@@ -718,9 +808,8 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_row_kernel(const RowPar
       if (w == w) g *= w;
       if (p.weight_out && threadIdx.x == 0 && rank == 0) p.weight_out[t] = w;
     }
-    const int a_part = (a >= off && a < off + v_part) ? a - off : -1;
-    row_grad<TIn, TGrad, kStage>(trow + off, reinterpret_cast<TGrad *>(p.grad) + t * p.ld_grad + off,
-                                 v_part, a_part, st, g, bound, hot);
+    row_grad<TIn, TGrad, kStage, kLoose>(vt, reinterpret_cast<TGrad *>(p.grad) + t * p.ld_grad, a, st, g, bound,
+                                         hot);
   }
 
   if constexpr (!kWeighted) {
@@ -728,8 +817,10 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_row_kernel(const RowPar
       __syncthreads();  // the bounds and the hot lists are reused for the second matrix
       const TIn *irow = reinterpret_cast<const TIn *>(p.infer) + t * p.ld_infer;
       HotList hot_i;
-      si = row_stats<TIn, kStage, kCluster>(irow, V, off, v_part, a, p.log_rho, p.mode, p.mask_value,
-                                            bound, scratch, cl_slots + 8, hot_smem, hot_i);
+      RowView<TIn> vi;
+      vi.set(irow, V, rank, kCluster);
+      si = row_stats<TIn, kStage, kCluster>(vi, a, p.log_rho, p.mode, p.mask_value, bound, scratch, cl_slots + 8,
+                                            hot_smem, hot_i);
     }
   }
 
@@ -747,7 +838,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_row_kernel(const RowPar
     }
     if (p.flags) p.flags[t] = flags;
   }
-  if (off == 0) {  // the first block of a row's cluster writes the row's masks
+  if (rank == 0) {  // the first block of a row's cluster writes the row's masks
     if (mask_t) write_mask_row<TIn>(trow, V, st.tau, mask_t);
     if (p.infer && p.out_i.mask)
       write_mask_row<TIn>(reinterpret_cast<const TIn *>(p.infer) + t * p.ld_infer, V, si.tau,
@@ -757,9 +848,9 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_row_kernel(const RowPar
   if constexpr (kCluster > 1) cluster_sync_all();
 }
 
-// ---- scalar kernel: any alignment, any row length ---------------------------
-// Three plain sweeps per matrix with element-wise loads; used when a row does
-// not start on a 32-byte boundary or is too long for the granule bounds.
+// ---- scalar kernel: any row length --------------------------------------------
+// Three plain sweeps per matrix with element-wise loads; used when a row is too long
+// for the granule bounds.
 
 template <typename TIn>
 __device__ __forceinline__ SideStats row_stats_scalar(const TIn *row, long long V, long long a,
@@ -929,9 +1020,10 @@ static inline bool aligned32(const void *base, long long ld, size_t elem) {
   return base == nullptr || (((uintptr_t)base % 32 == 0) && ((ld * (long long)elem) % 32 == 0));
 }
 
-template <typename TIn, typename TGrad, int kStage, int kThreads, int kBlocks, int kCluster, bool kWeighted = false>
+template <typename TIn, typename TGrad, int kStage, int kThreads, int kBlocks, int kCluster, bool kWeighted = false,
+          bool kLoose = false>
 static cudaError_t launch_rows_vec(const RowParams &p, int threads, size_t smem, cudaStream_t s) {
-  auto k = dvp_row_kernel<TIn, TGrad, kStage, kThreads, kBlocks, kCluster, kWeighted>;
+  auto k = dvp_row_kernel<TIn, TGrad, kStage, kThreads, kBlocks, kCluster, kWeighted, kLoose>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -1009,10 +1101,17 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
   const bool vec_ok = aligned32(p.train, p.ld_train, sizeof(TIn)) &&
                       aligned32(p.infer, p.ld_infer, sizeof(TIn)) &&
                       aligned32(p.grad, p.ld_grad, sizeof(TGrad));
+  bool loose = false;
+  if (p.grad) {  // do the gradient's granules start on store boundaries wherever the logits' do?
+    constexpr long long kA = grad_align<TIn, TGrad>();
+    const long long shift = (long long)((uintptr_t)p.grad / sizeof(TGrad) % kA) -
+                            (long long)((uintptr_t)p.train / sizeof(TIn) % kA);
+    loose = shift % kA != 0 || (p.T > 1 && (p.ld_grad - p.ld_train) % kA != 0);
+  }
   const long long n_gran_row = (p.V + kElems - 1) / kElems;
   if (cluster == 0) cluster = 1;
   const bool weighted = p.weight_kind != DVP_WEIGHT_NONE;  // one block per row only
-  if (weighted) cluster = 1;
+  if (weighted || loose) cluster = 1;
   if (cluster > 1 && (n_gran_row < 4096 || p.T * cluster > 0x7fffffffLL)) cluster = 1;
   const long long n_gran = (n_gran_row + cluster - 1) / cluster;  // granules per block
   // shrink the block for short rows so that threads are not idle
@@ -1039,11 +1138,18 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
       if (e != cudaErrorNotSupported) return e;
     }
   }
-  if (vec_ok && hot_ok && smem <= 200 * 1024) {
+  if (hot_ok && smem <= 200 * 1024) {
     if (cluster == 4 && threads <= 256 && stage == 2)
       return launch_rows_vec<TIn, TGrad, 2, 256, 4, 4>(p, threads, smem, s);
     if (cluster == 2 && threads <= 256 && stage == 2)
       return launch_rows_vec<TIn, TGrad, 2, 256, 4, 2>(p, threads, smem, s);
+    if (loose) {
+      if (weighted)
+        return threads > 256 ? launch_rows_vec<TIn, TGrad, 2, 512, 2, 1, true, true>(p, threads, smem, s)
+                             : launch_rows_vec<TIn, TGrad, 2, 256, 4, 1, true, true>(p, threads, smem, s);
+      return threads > 256 ? launch_rows_vec<TIn, TGrad, 2, 512, 2, 1, false, true>(p, threads, smem, s)
+                           : launch_rows_vec<TIn, TGrad, 2, 256, 4, 1, false, true>(p, threads, smem, s);
+    }
     if (weighted) {
       if (threads > 256) return launch_rows_vec<TIn, TGrad, 2, 512, 2, 1, true>(p, threads, smem, s);
       return launch_rows_vec<TIn, TGrad, 2, 256, 4, 1, true>(p, threads, smem, s);

@@ -1,0 +1,73 @@
+"""Rows that start anywhere: odd vocabularies with their rows back to back, bases off the 32-byte grid,
+and gradient matrices that lie differently than their logits.  The row kernels cut each row at its own
+32-byte boundaries; the elements in front of the first and behind the last whole piece, and the pieces
+themselves, must all be taken exactly once, and nothing outside the rows may be written."""
+import dataclasses
+
+import pytest
+import torch
+
+from paper_2512_23087_b200 import binding, inputs
+
+import parity
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+W = inputs.WORKLOADS
+
+
+def _place(x, ld, offset):
+    """The same rows with stride `ld`, starting `offset` elements into a fresh buffer; outside them a huge logit."""
+    T, V = x.shape
+    buf = torch.full((offset + T * ld + 64,), 3.0e4, dtype=x.dtype, device=x.device)
+    view = buf[offset:offset + T * ld].view(T, ld)[:, :V]
+    view.copy_(x)
+    return view
+
+
+# V: below one piece, around one and two pieces, an odd middle size, several sweeps of a block;
+# (ld - V, offset of the logits, offset of the gradient): alike, and alike only in some or no rows
+@pytest.mark.parametrize("pad,offset,grad_pad,grad_offset", [(0, 0, 0, 0), (3, 5, 3, 5), (1, 8, 0, 3), (16, 1, 8, 0)])
+@pytest.mark.parametrize("V", [5, 31, 47, 2999, 50021])
+@pytest.mark.parametrize("dtype,grad_dtype", [("bf16", torch.bfloat16), ("f16", torch.float32), ("f32", torch.float32),
+                                              ("f32", torch.bfloat16)])
+@pytest.mark.parametrize("checks", [False, True], ids=["", "bounds"])
+def test_rows_that_start_anywhere(dtype, grad_dtype, V, pad, offset, grad_pad, grad_offset, checks):
+    T = 13
+    w = dataclasses.replace(W["c0_small_f32"], dtype=dtype, head_boost=5.0)
+    b = inputs.make_rows(w, seed=V + pad, device=DEV, T=T, V=V)
+    train, infer = _place(b.train, V + pad, offset), _place(b.infer, V + pad + 2, offset + 1)
+    b = dataclasses.replace(b, train=train, infer=infer)
+    ld = V + grad_pad
+    buf = torch.full((grad_offset + T * ld + 64,), 7.0, dtype=grad_dtype, device=DEV)
+    grad = buf[grad_offset:grad_offset + T * ld].view(T, ld)[:, :V]
+
+    def run(rho):
+        res = binding.dvp_forward(b.train, b.ids, rho, infer_logits=b.infer, upstream=b.upstream, grad_train=grad,
+                                  want_mask=True)
+        torch.cuda.synchronize()
+        return res
+
+    for rho in (1e-3, 0.0):
+        buf.fill_(7.0)
+        if checks:
+            with binding.bounds_checking_library():
+                res = run(rho)
+                assert binding.dvp_debug_bounds_status() == 0, "an index was out of range"
+        else:
+            res = run(rho)
+        parity.check_forward(res, b, rho, V, True)
+        outside = torch.ones_like(buf, dtype=torch.bool)
+        outside[grad_offset:grad_offset + T * ld].view(T, ld)[:, :V] = False
+        assert (buf[outside] == 7.0).all(), "written outside the gradient's rows"
+
+
+@pytest.mark.parametrize("cluster", [2, 4])
+@pytest.mark.parametrize("V,grad_pad", [(151935, 0), (70001, 1)])
+def test_clusters_share_rows_that_start_anywhere(V, grad_pad, cluster):
+    b = inputs.make_rows(W["c2_bf16_fwdbwd"], seed=V, device=DEV, T=5, V=V)
+    grad = torch.empty(5, V + grad_pad, dtype=torch.bfloat16, device=DEV)[:, :V]
+    res = binding.dvp_forward(b.train, b.ids, 1e-4, infer_logits=b.infer, upstream=b.upstream, grad_train=grad,
+                              want_mask=True, launch_hint=256 | (cluster << 24))
+    torch.cuda.synchronize()
+    parity.check_forward(res, b, 1e-4, V, True)
