@@ -370,7 +370,12 @@ struct RowParams {
   const float *given_logp_mp_i;
   const uint8_t *given_flags_i;
   unsigned int *bounds_status;  // the bounds-checking build's status word; unused otherwise
+  // the row kernel sweeps one row per token (`train`, `out_t`); with two launches for a call:
+  int side;  // kSide*
+  char *li;  // where ln pi^mp_infer(a) of token t passes from one to the other: two 2-byte halves at t * li_stride
+  long long li_stride;
 };
+enum { kSideAlone = 0, kSideInfer = 1, kSideTrain = 2 };
 
 __device__ __forceinline__ long long load_id(const void *ids, int is_i32, long long t) {
   return is_i32 ? (long long)reinterpret_cast<const int *>(ids)[t]
@@ -470,6 +475,23 @@ __device__ __forceinline__ float log_ratio_of(bool in_train, bool in_infer, floa
   if (!in_train) return kNegInf;
   if (!in_infer) return -kNegInf;
   return lt - li;
+}
+
+// The same with ln pi^mp_infer(a) alone: it is -inf when a is outside V'_S, unless the mask is finite.
+__device__ __forceinline__ float log_ratio_from(int mode, bool in_train, float lt, float li) {
+  return (mode & DVP_MODE_FINITE_MASK) ? lt - li : log_ratio_of(in_train, li > kNegInf, lt, li);
+}
+
+__device__ __forceinline__ float load_li(const RowParams &p, long long t) {
+  if (!p.li) return 0.f;
+  const uint16_t *h = reinterpret_cast<const uint16_t *>(p.li + t * p.li_stride);
+  return __uint_as_float((uint32_t)h[0] | ((uint32_t)h[1] << 16));
+}
+__device__ __forceinline__ void store_li(const RowParams &p, long long t, float li) {
+  if (!p.li) return;
+  uint16_t *h = reinterpret_cast<uint16_t *>(p.li + t * p.li_stride);
+  h[0] = (uint16_t)__float_as_uint(li);
+  h[1] = (uint16_t)(__float_as_uint(li) >> 16);
 }
 
 // Token-level importance weight from the log-ratio r (DVP_WEIGHT_*): the per-token

@@ -13,6 +13,11 @@
 // of the gradient; with a dense safe set the same code degrades to three
 // sweeps, still correct.
 #pragma once
+#include <float.h>
+#include <limits.h>
+
+#include <type_traits>
+
 #include "dvp_common.cuh"
 
 namespace dvp {
@@ -123,22 +128,12 @@ __device__ __forceinline__ uint16_t bf16_bits_round_up(float v) {
   // positive: bump the magnitude unless the low half is zero; negative: truncate
   return (uint16_t)(((b & 0x80000000u) ? b : b + 0xffffu) >> 16);
 }
-__device__ __forceinline__ float bf16_bits_to_float(uint16_t b) {
-  return __uint_as_float((uint32_t)b << 16);
-}
 // Largest bfloat16 that is <= v, as a float: comparing the stored upper bounds with
 // it flags a superset of the granules whose bound reaches v.
 __device__ __forceinline__ float bf16_round_down(float v) {
   const uint32_t b = __float_as_uint(v);
   return __uint_as_float(((b & 0x80000000u) ? b + 0xffffu : b) & 0xffff0000u);
 }
-// The bounds of one thread's kStage granules of a step sit side by side, so that a
-// step's pair is one 32-bit word: slot i = step * kStage + u of thread tid.
-template <int kStage>
-__device__ __forceinline__ int bound_index(int slot, int tid) {
-  return ((slot / kStage) * (int)blockDim.x + tid) * kStage + (slot % kStage);
-}
-
 template <typename TGrad, int kElems>
 __device__ __forceinline__ void store_granule(TGrad *dst, const float *out) {
   constexpr int kBytes = kElems * (int)sizeof(TGrad);
@@ -196,65 +191,17 @@ struct HotList {
   __device__ __forceinline__ bool fits() const { return count <= kHotCap; }
 };
 
-// tau_b: the threshold rounded down to bfloat16.  Each thread first gathers the
-// flags of its own slots into a register (16 steps at a time: one packed compare per
-// step), then a warp prefix sum hands out list positions: the cost of the scan does
-// not depend on how many granules are hot, and the order of the list is fixed.
-template <int kStage>
-__device__ __forceinline__ HotList build_hot_list(const uint16_t *bound, int n_steps, float tau_b,
-                                                  uint16_t *hot_smem) {
-  static_assert(kStage == 2, "the packed scan reads the two bounds of a step as one word");
-  const int lane = threadIdx.x & 31, tid = threadIdx.x;
-  HotList h;
-  h.slots = hot_smem + (tid >> 5) * kHotCap;
-  h.count = 0;
-  const uint32_t *words = reinterpret_cast<const uint32_t *>(bound);
-  const __nv_bfloat16 tb = __float2bfloat16_rz(tau_b);  // exact: tau_b is a bfloat16 value
-  const __nv_bfloat162 tau2 = __halves2bfloat162(tb, tb);
-  for (int step0 = 0; step0 < n_steps; step0 += 16) {
-    uint32_t acc = 0;  // bit s: first granule of step step0 + s, bit 16 + s: second granule
-    const int n = min(16, n_steps - step0);
-    for (int s = 0; s < n; ++s) {
-      const int wi = (step0 + s) * (int)blockDim.x + tid;
-      const uint32_t w = DVP_IN(2 * wi + 1, n_bound, DVP_OOB_BOUND) ? words[wi] : 0u;
-      const uint32_t m = __hge2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&w), tau2);
-      acc |= (m & 0x00010001u) << s;
-    }
-    const int cnt = __popc(acc);
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int up = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += up;
-    }
-    int pos = h.count + incl - cnt;
-    while (acc) {
-      const int b = __ffs(acc) - 1;
-      acc &= acc - 1;
-      const int slot = (step0 + (b & 15)) * 2 + (b >> 4);
-      if (pos < kHotCap) h.slots[pos] = (uint16_t)(slot * 32 + lane);
-      ++pos;
-    }
-    h.count += __shfl_sync(0xffffffffu, incl, 31);
-  }
-  __syncwarp();
-  return h;
-}
-
-// Contribution of one granule to the masked sum and the count (Def. 5.2).
+// Contribution of one granule to the masked sum and the count (Def. 5.2).  tau is finite: no fill passes.
 template <typename TIn>
-__device__ __forceinline__ void granule_masked_sum(const Granule<TIn> &gr, int g, int a, float tau,
-                                                   float m, SumCount &sc) {
+__device__ __forceinline__ void granule_masked_sum(const Granule<TIn> &gr, float tau, float m, SumCount &sc) {
   constexpr int kElems = Granule<TIn>::kElems;
   float x[kElems];
   gr.get(x);
-  // the sampled token is left out so that 1 - pi^mp(a) has no cancellation
-  const int ja = a - g * kElems;  // in [0, kElems) only inside the owner granule
 #pragma unroll
   for (int j = 0; j < kElems; ++j) {
-    if (x[j] >= tau && x[j] > kNegInf) {  // the fill of a ragged last granule is never a token
+    if (x[j] >= tau) {
       ++sc.n;
-      if (j != ja) sc.s += ex2((x[j] - m) * kLog2e);
+      sc.s += ex2((x[j] - m) * kLog2e);
     }
   }
 }
@@ -330,113 +277,271 @@ struct Stage {
     }
   }
   // the whole granules of the step only
-  __device__ __forceinline__ void load_whole(const TIn *row, int n_full, int step) {
-    const int g0 = step * kStage * (int)blockDim.x + threadIdx.x;
-    if ((step + 1) * kStage * (int)blockDim.x <= n_full &&
-        DVP_IN(g0 + (kStage - 1) * (int)blockDim.x, n_gran, DVP_OOB_GRANULE)) {
+  template <int kBlk>
+  __device__ __forceinline__ void load_block(const TIn *row, int n_full, int step) {
+    const int g0 = step * kStage * kBlk + (int)threadIdx.x;
+    if ((step + 1) * kStage * kBlk <= n_full && DVP_IN(g0 + (kStage - 1) * kBlk, n_gran, DVP_OOB_GRANULE)) {
+      const TIn *p = row + (size_t)g0 * Granule<TIn>::kElems;
 #pragma unroll
-      for (int u = 0; u < kStage; ++u)
-        g[u].load(row + (size_t)(g0 + u * (int)blockDim.x) * Granule<TIn>::kElems);
+      for (int u = 0; u < kStage; ++u) g[u].load(p + u * kBlk * Granule<TIn>::kElems);
     } else {
 #pragma unroll
-      for (int u = 0; u < kStage; ++u) g[u].load_whole(row, n_full, g0 + u * (int)blockDim.x);
+      for (int u = 0; u < kStage; ++u) g[u].load_whole(row, n_full, g0 + u * kBlk);
+    }
+  }
+  // granule `hole`, one of this step's, becomes -inf in the thread that holds it
+  template <int kBlk>
+  __device__ __forceinline__ void punch(int step, int hole) {
+    const int u_here = hole - step * kStage * kBlk - (int)threadIdx.x;
+#pragma unroll
+    for (int u = 0; u < kStage; ++u)
+      if (u_here == u * kBlk) g[u].load_whole(nullptr, 0, 0);
+    __syncwarp();  // keeps this a branch: predicated, its moves would be issued in every step
+  }
+};
+
+// ---- sweep 1 ---------------------------------------------------------------------
+
+// Two floats in a 64-bit register pair: one FMA, addition or product for both.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// What depends on the storage type.  The maxima of a step's two granules are one word of shared memory:
+// exact, in the storage type, for 2-byte logits; bfloat16 upper bounds for float32.
+template <typename TIn>
+struct SweepOps {  // 2-byte logits, two at a time
+  using T2 = typename Pair<TIn>::type;
+  using Max = T2;
+  static __device__ __forceinline__ uint32_t bits(T2 v) { return *reinterpret_cast<const uint32_t *>(&v); }
+  static __device__ __forceinline__ T2 pair(uint32_t v) { return *reinterpret_cast<const T2 *>(&v); }
+  static __device__ __forceinline__ Max start(float v) {
+    T2 r;
+    r.x = r.y = Storage<TIn>::narrow(v);  // exact: v was stored as TIn
+    return r;
+  }
+  static __device__ __forceinline__ T2 tree(const Granule<TIn> &g) {
+    T2 p[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) p[i] = pair(g.w[i]);
+#pragma unroll
+    for (int s = 4; s > 0; s >>= 1)
+#pragma unroll
+      for (int i = 0; i < s; ++i) p[i] = __hmax2(p[i], p[i + s]);
+    return p[0];
+  }
+  // the step's word; raises the running maximum
+  static __device__ __forceinline__ uint32_t bounds(const Stage<TIn, 2> &st, Max &mx) {
+    const uint32_t a = bits(tree(st.g[0])), b = bits(tree(st.g[1]));
+    const T2 w = __hmax2(pair(__byte_perm(a, b, 0x5410)), pair(__byte_perm(a, b, 0x7632)));
+    mx = __hmax2(mx, w);
+    return bits(w);
+  }
+  static __device__ __forceinline__ float value(Max m) {
+    return fmaxf(Storage<TIn>::widen(m.x), Storage<TIn>::widen(m.y));
+  }
+  // 0x0000ffff, 0xffff0000: the step's first, second granule may hold a value that reaches the threshold
+  using Key = uint32_t;
+  static __device__ __forceinline__ Key key(float tau) { return threshold(tau); }
+  static __device__ __forceinline__ uint32_t reach(uint32_t word, Key k) { return __hge2_mask(pair(word), pair(k)); }
+  static constexpr uint32_t kTop = std::is_same<TIn, __nv_bfloat16>::value ? 0x7f7fu : 0x7bffu;  // largest finite
+  // the threshold, rounded up to the storage type: a stored value reaches tau when it reaches that
+  using Tau = uint32_t;
+  static __device__ __forceinline__ Tau threshold(float tau) {
+    T2 t;
+    if constexpr (std::is_same<TIn, __nv_bfloat16>::value)
+      t.x = __float2bfloat16_ru(tau);
+    else
+      t.x = __float2half_ru(tau);
+    t.y = t.x;
+    return bits(t);
+  }
+  // adds e0, e1 to s where the granule's pair i reaches the threshold and counts them in n (see count())
+  static __device__ __forceinline__ void masked(const Granule<TIn> &g, int i, float, float, float e0, float e1, Tau tau,
+                                                float &s, uint32_t &n) {
+    if constexpr (std::is_same<TIn, __nv_bfloat16>::value)
+      asm("{\n\t.reg .pred p, q;\n\tsetp.ge.bf16x2 p|q, %1, %2;\n\t"
+          "@p add.f32 %0, %0, %3;\n\t@q add.f32 %0, %0, %4;\n\t}"
+          : "+f"(s)
+          : "r"(g.w[i]), "r"(tau), "f"(e0), "f"(e1));
+    else
+      asm("{\n\t.reg .pred p, q;\n\tsetp.ge.f16x2 p|q, %1, %2;\n\t"
+          "@p add.f32 %0, %0, %3;\n\t@q add.f32 %0, %0, %4;\n\t}"
+          : "+f"(s)
+          : "r"(g.w[i]), "r"(tau), "f"(e0), "f"(e1));
+    n += __hge2_mask(pair(g.w[i]), pair(tau));
+  }
+  // A mask has 0xffff in the halves that pass, so that a sum of masks is 0xffff n_lo + 0xffff0000 n_hi
+  // = -(n_lo + 2^16 (n_hi - n_lo)) modulo 2^32: exact while both are below 2^16.
+  static __device__ __forceinline__ int count(uint32_t cnt) {
+    const uint32_t v = 0u - cnt, lo = v & 0xffffu;
+    return (int)(lo + (((v >> 16) + lo) & 0xffffu));
+  }
+};
+template <>
+struct SweepOps<float> {
+  using Max = float;
+  static __device__ __forceinline__ Max start(float v) { return v; }
+  static __device__ __forceinline__ uint32_t bounds(const Stage<float, 2> &st, Max &mx) {
+    const float a = st.g[0].max(), b = st.g[1].max();
+    mx = fmaxf(mx, fmaxf(a, b));
+    return (uint32_t)bf16_bits_round_up(a) | ((uint32_t)bf16_bits_round_up(b) << 16);
+  }
+  static __device__ __forceinline__ float value(Max m) { return m; }
+  using Key = uint32_t;  // the threshold rounded down to bfloat16, twice
+  static __device__ __forceinline__ Key key(float tau) {
+    const uint32_t b = __float_as_uint(bf16_round_down(tau));
+    return b | (b >> 16);
+  }
+  static __device__ __forceinline__ uint32_t reach(uint32_t word, Key k) {
+    return __hge2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&word), *reinterpret_cast<const __nv_bfloat162 *>(&k));
+  }
+  static constexpr uint32_t kTop = 0x7f7fu;
+  using Tau = float;
+  static __device__ __forceinline__ Tau threshold(float tau) { return tau; }
+  static __device__ __forceinline__ void masked(const Granule<float> &, int, float x0, float x1, float e0, float e1,
+                                                Tau tau, float &s, uint32_t &n) {
+    if (x0 >= tau) {
+      s += e0;
+      ++n;
+    }
+    if (x1 >= tau) {
+      s += e1;
+      ++n;
+    }
+  }
+  static __device__ __forceinline__ int count(uint32_t cnt) { return (int)cnt; }
+};
+
+// What a thread carries through sweep 1, all without the sampled token: the sum of 2^{z l - c}, c = fl(guess l),
+// and the masked sum and count under the threshold of a guess of the row's maximum.
+template <typename TIn>
+struct Sweep1 {
+  using Ops = SweepOps<TIn>;
+  typename Ops::Max mx;    // the largest value seen
+  typename Ops::Tau tau;   // the guess's threshold
+  float guess, c;          // block-uniform
+  uint64_t sum;            // two partial sums
+  float safe_s;            // masked sum and count over the steps from `first` on
+  int safe_n;
+  uint32_t cnt;            // counts not yet in safe_n
+  int first;
+  bool wide;               // a value so far above the guess was met that the sums may have overflowed
+
+  // the threshold is finite: rho = 0 keeps every finite logit, and the fill of a missing granule never passes
+  __device__ __forceinline__ void set_guess(float m, double log_rho, int mode) {
+    guess = m;
+    c = m * kLog2e;
+    tau = Ops::threshold(fmaxf(threshold_of<TIn>(m, log_rho, mode), -FLT_MAX));
+    safe_s = 0.f;
+    safe_n = 0;
+    cnt = 0;
+  }
+
+  __device__ __forceinline__ void flush_count() {
+    safe_n += Ops::count(cnt);
+    cnt = 0;
+  }
+
+  __device__ __forceinline__ void absorb(const Stage<TIn, 2> &st, uint32_t *bound) {
+    *bound = Ops::bounds(st, mx);
+    constexpr int kElems = Granule<TIn>::kElems;
+    const uint64_t l2 = pack2(kLog2e, kLog2e), c2 = pack2(-c, -c);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      float x[kElems];
+      st.g[u].get(x);
+#pragma unroll
+      for (int j = 0; j < kElems; j += 2) {
+        float e0, e1;
+        unpack2(fma2(pack2(x[j], x[j + 1]), l2, c2), e0, e1);
+        e0 = ex2(e0);
+        e1 = ex2(e1);
+        sum = add2(sum, pack2(e0, e1));
+        Ops::masked(st.g[u], j / 2, x[j], x[j + 1], e0, e1, tau, safe_s, cnt);
+      }
     }
   }
 };
 
-template <typename TIn, int kStage>
-__device__ __forceinline__ void absorb_stage(const Stage<TIn, kStage> &st, int step, LogSum &acc,
-                                             uint16_t *bound) {
-  constexpr int kElems = Granule<TIn>::kElems;
-  float cm = kNegInf;
-#pragma unroll
-  for (int u = 0; u < kStage; ++u) {
-    const float gm = st.g[u].max();
-    const int bi = bound_index<kStage>(step * kStage + u, threadIdx.x);
-    if (DVP_IN(bi, n_bound, DVP_OOB_BOUND)) bound[bi] = bf16_bits_round_up(gm);
-    cm = fmaxf(cm, gm);
-  }
-  if (cm > kNegInf) {
-    if (cm > acc.m) {
-      const float cn = cm * kLog2e;
-      acc.s *= ex2(acc.c - cn);  // acc.c = -inf at the start: the factor is 0
-      acc.m = cm;
-      acc.c = cn;
-    }
-    const float neg_c = -acc.c;
-    float part = 0.f;
-#pragma unroll
-    for (int u = 0; u < kStage; ++u) {
-      float x[kElems];
-      st.g[u].get(x);
-#pragma unroll
-      for (int j = 0; j < kElems; ++j) part += ex2(fmaf(x[j], kLog2e, neg_c));
-    }
-    acc.s += part;
-  }
-}
-
-// ---- a row split over a thread-block cluster -----------------------------------
-// With kCluster > 1 the blocks of a cluster share one row: block `rank` owns a
-// contiguous part of it, partial results meet through distributed shared memory.
-// Fewer rows are then in flight (one per cluster instead of one per block), so
-// the granules that sweeps 2 and 3 revisit are still in L2.
+// ---- thread-block clusters ------------------------------------------------------
+// With few tokens a row is split over the blocks of a cluster: block `part` owns a contiguous part of it,
+// partial results meet through distributed shared memory.
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void cluster_sync_all() {
+__device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ float ld_cluster_f32(const float *local, uint32_t rank) {
+__device__ __forceinline__ uint32_t cluster_addr(const void *local, uint32_t rank) {
   uint32_t laddr = (uint32_t)__cvta_generic_to_shared(local), raddr;
-  float v;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(raddr) : "r"(laddr), "r"(rank));
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(raddr) : "memory");
+  return raddr;
+}
+__device__ __forceinline__ float ld_cluster_f32(const float *local, uint32_t rank) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr(local, rank)) : "memory");
   return v;
 }
+struct RowGroup {
+  int parts, part;
+  float *slots;  // 4 floats of shared memory, each written once per kernel
 
-// slot: 4 floats of this block's shared memory, written once per kernel.
-template <int kCluster>
-__device__ __forceinline__ LogSum cluster_reduce_logsum(LogSum v, float *slot) {
-  if constexpr (kCluster == 1) return v;
-  if (threadIdx.x == 0) {
-    slot[0] = v.m;
-    slot[1] = v.c;
-    slot[2] = v.s;
+  __device__ __forceinline__ float max(float m) const {
+    if (parts == 1) return m;
+    if (threadIdx.x == 0) slots[0] = m;
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    float hi = kNegInf;
+    for (int k = 0; k < parts; ++k) hi = fmaxf(hi, ld_cluster_f32(slots + 0, (uint32_t)k));
+    return hi;
   }
-  cluster_sync_all();
-  LogSum r = {kNegInf, kNegInf, 0.f};
-#pragma unroll
-  for (uint32_t k = 0; k < (uint32_t)kCluster; ++k) {  // rank order: same result in every block
-    LogSum o;
-    o.m = ld_cluster_f32(slot + 0, k);
-    o.c = ld_cluster_f32(slot + 1, k);
-    o.s = ld_cluster_f32(slot + 2, k);
-    r = combine(r, o);
+  __device__ __forceinline__ void sums(float &all, SumCount &safe) const {
+    if (parts == 1) return;
+    if (threadIdx.x == 0) {
+      slots[1] = all;
+      slots[2] = safe.s;
+      slots[3] = __int_as_float(safe.n);
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    all = 0.f;
+    safe = {0.f, 0};
+    for (int k = 0; k < parts; ++k) {  // in order: same result in every block
+      all += ld_cluster_f32(slots + 1, (uint32_t)k);
+      safe.s += ld_cluster_f32(slots + 2, (uint32_t)k);
+      safe.n += __float_as_int(ld_cluster_f32(slots + 3, (uint32_t)k));
+    }
   }
-  return r;
-}
-
-template <int kCluster>
-__device__ __forceinline__ SumCount cluster_reduce_sumcount(SumCount v, float *slot) {
-  if constexpr (kCluster == 1) return v;
-  if (threadIdx.x == 0) {
-    slot[0] = v.s;
-    slot[1] = __int_as_float(v.n);
-  }
-  cluster_sync_all();
-  SumCount r = {0.f, 0};
-#pragma unroll
-  for (uint32_t k = 0; k < (uint32_t)kCluster; ++k) {
-    r.s += ld_cluster_f32(slot + 0, k);
-    r.n += __float_as_int(ld_cluster_f32(slot + 1, k));
-  }
-  return r;
-}
+};
 
 // A row as the sweeps see it.  Granules are cut at the row's own 32-byte boundaries, so that a row may
 // start at any element (an odd vocabulary with its rows back to back): `head` elements lie in front of
@@ -455,14 +560,14 @@ struct RowView {
   int n_full;    // whole granules of this block
   bool extras;   // this block takes the elements outside the granules
 
-  __device__ __forceinline__ void set(const TIn *r, int V_, int rank, int n_ranks) {
+  __device__ __forceinline__ void set(const TIn *r, int V_, int rank, int log_ranks) {
     constexpr int kElems = Granule<TIn>::kElems;
     row = r;
     V = V_;
     const int mis = (int)(((uintptr_t)r & 31u) / sizeof(TIn));
     head = min(V, mis ? kElems - mis : 0);
     n_all = (V - head) / kElems;
-    const int per = (n_all + n_ranks - 1) / n_ranks;
+    const int per = (n_all + (1 << log_ranks) - 1) >> log_ranks;
     g_first = min(rank * per, n_all);
     n_full = min(per, n_all - g_first);
     base = r + head + (size_t)g_first * kElems;
@@ -473,144 +578,276 @@ struct RowView {
     const int tid = (int)threadIdx.x;
     return !extras ? V : tid < head ? tid : tid + n_all * Granule<TIn>::kElems;
   }
+  // this block's granule that holds element a, -1 when there is none
+  __device__ __forceinline__ int granule_of(int a) const {
+    const int r = a < 0 ? -1 : rel(a);
+    return r >= 0 && r < n_full * Granule<TIn>::kElems ? r / Granule<TIn>::kElems : -1;
+  }
+  // the same element when sums without the sampled token a are formed: the other elements of its granule
+  // g_a count among those outside the granules (threads 32 to 32 + kElems - 1), the token itself is nobody's
+  __device__ __forceinline__ int extra_but(int a, int g_a) const {
+    const int j = (int)threadIdx.x - 32;
+    int k = j < 0 ? extra() : V;
+    if (g_a >= 0 && j >= 0 && j < Granule<TIn>::kElems)
+      k = head + (g_first + g_a) * Granule<TIn>::kElems + j;
+    return k == a ? V : k;
+  }
   // element k of the row counted from `base`
   __device__ __forceinline__ int rel(int k) const { return k - head - g_first * Granule<TIn>::kElems; }
 };
 
-// Sweep 1 over (a part of) a row: block-wide log-sum-exp state; granule bounds
-// are left in shared memory.
-template <typename TIn, int kStage>
-__device__ __forceinline__ LogSum row_sweep1(const RowView<TIn> &v, uint16_t *bound, float *scratch) {
-  const TIn *row = v.base;
-  const int n_full = v.n_full;
-  const int per_step = kStage * (int)blockDim.x;
-  const int n_steps = (n_full + per_step - 1) / per_step;
-  LogSum acc = {kNegInf, kNegInf, 0.f};
-  if (n_steps > 0) {  // two stages in flight
-    Stage<TIn, kStage> s0, s1;
-    s0.load_whole(row, n_full, 0);
-    int step = 0;
-    for (; step + 1 < n_steps; step += 2) {
-      s1.load_whole(row, n_full, step + 1);
-      absorb_stage<TIn, kStage>(s0, step, acc, bound);
-      if (step + 2 < n_steps) s0.load_whole(row, n_full, step + 2);
-      absorb_stage<TIn, kStage>(s1, step + 1, acc, bound);
-    }
-    if (step < n_steps) absorb_stage<TIn, kStage>(s0, step, acc, bound);
+// A float as an integer of the same order, and back.
+__device__ __forceinline__ int order_key(float v) {
+  const int b = __float_as_int(v);
+  return b ^ ((b >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float key_value(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
+
+// Block reductions of the row kernel: two alternating sets of words for maxima (one barrier each), one for
+// sums (a maximum's barrier lies between two of them).  Fixed order; every thread gets the result.
+constexpr int kMaxWarps = 16, kRedWords = 5 * kMaxWarps;
+template <int kBlk>
+struct BlockReduce {
+  static constexpr int kWarps = kBlk / 32;
+  float *words;
+  int parity;
+
+  __device__ __forceinline__ float max(float v) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int *slot = reinterpret_cast<int *>(words) + parity * kMaxWarps;
+    parity ^= 1;
+    const int k = __reduce_max_sync(0xffffffffu, order_key(v));
+    if (lane == 0) slot[warp] = k;
+    __syncthreads();
+    return key_value(__reduce_max_sync(0xffffffffu, slot[lane % kWarps]));
   }
-  // the elements outside the granules, one per thread
-  const int k_extra = v.extra();
-  if (k_extra < v.V) {
-    const float x = Storage<TIn>::widen(v.row[k_extra]);
-    if (x > kNegInf) {
-      if (x > acc.m) {
-        const float cn = x * kLog2e;
-        acc.s *= ex2(acc.c - cn);
-        acc.m = x;
-        acc.c = cn;
-      }
-      acc.s += ex2(fmaf(x, kLog2e, -acc.c));
+  __device__ __forceinline__ void sums(float &all, SumCount &safe) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float *w = words + 2 * kMaxWarps;
+    uint64_t v = pack2(all, safe.s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = add2(v, __shfl_xor_sync(0xffffffffu, v, o));
+    safe.n = __reduce_add_sync(0xffffffffu, safe.n);
+    if (lane == 0) {
+      unpack2(v, all, safe.s);
+      w[warp] = all;
+      w[kMaxWarps + warp] = safe.s;
+      w[2 * kMaxWarps + warp] = __int_as_float(safe.n);
     }
+    __syncthreads();
+    v = pack2(w[lane % kWarps], w[kMaxWarps + lane % kWarps]);
+#pragma unroll
+    for (int o = kWarps / 2; o > 0; o >>= 1) v = add2(v, __shfl_xor_sync(0xffffffffu, v, o));
+    unpack2(v, all, safe.s);
+    safe.n = __reduce_add_sync(0xffffffffu, lane < kWarps ? __float_as_int(w[2 * kMaxWarps + lane]) : 0);
   }
-  return block_reduce_logsum(acc, scratch);
+};
+
+// Each thread first gathers the flags of its own granules into a register (16 steps at a time: one packed
+// compare per step), then a warp prefix sum hands out list positions: the order of the list is fixed.
+template <typename TIn, int kBlk>
+__device__ __forceinline__ HotList build_hot_list(const uint32_t *bound, int n_steps,
+                                                  typename SweepOps<TIn>::Key key, uint16_t *hot_smem) {
+  const int lane = threadIdx.x & 31, tid = threadIdx.x;
+  HotList h;
+  h.slots = hot_smem + (tid >> 5) * kHotCap;
+  h.count = 0;
+  __syncwarp();  // the warp's list of an earlier row may still be read
+  for (int step0 = 0; step0 < n_steps; step0 += 16) {
+    uint32_t acc = 0;  // bit s: first granule of step step0 + s, bit 16 + s: second granule
+    const int n = min(16, n_steps - step0);
+    for (int s = 0; s < n; ++s) {
+      const int wi = (step0 + s) * kBlk + tid;
+      const uint32_t w = DVP_IN(wi, n_bound, DVP_OOB_BOUND) ? bound[wi] : 0u;
+      acc |= (SweepOps<TIn>::reach(w, key) & 0x00010001u) << s;
+    }
+    const int cnt = __popc(acc);
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int up = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += up;
+    }
+    int pos = h.count + incl - cnt;
+    while (acc) {
+      const int b = __ffs(acc) - 1;
+      acc &= acc - 1;
+      const int slot = (step0 + (b & 15)) * 2 + (b >> 4);
+      if (pos < kHotCap) h.slots[pos] = (uint16_t)(slot * 32 + lane);
+      ++pos;
+    }
+    h.count += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  __syncwarp();
+  return h;
 }
 
-// Sweep 2 over (a part of) a row: masked sum without the sampled token `a_row` and count, block-wide.
-template <typename TIn, int kStage>
-__device__ __forceinline__ SumCount row_sweep2(const RowView<TIn> &v, int a_row, float tau, float m,
-                                               const uint16_t *bound, float *scratch,
-                                               uint16_t *hot_smem, HotList &hot) {
+// Sweep 1 over (a part of) a row.
+//
+// The first guess of the maximum is the largest of `cand` (a value of the row: the sampled token's, which is
+// the maximum in most rows) and of what the first step loaded.  The block's threads exchange their maxima
+// every kSyncSteps steps: a larger one becomes the guess, and the masked sum starts again from there
+// (`first`).  All of it happens at fixed places, so that reruns are bit-identical.  `hole`: the granule
+// that reads as -inf (the sampled token's; its bound says that it can hold anything); xe: a value outside the
+// granules.
+constexpr int kSyncSteps = 4;
+constexpr float kWide = 60.f;  // e^60 times the longest row is far from overflow
+template <typename TIn, int kBlk>
+__device__ __forceinline__ void row_sweep1(const RowView<TIn> &v, int hole, float xe, float cand, double log_rho,
+                                           int mode, uint32_t *bound, BlockReduce<kBlk> &red, Sweep1<TIn> &sw) {
   const TIn *row = v.base;
-  const int n_full = v.n_full;
-  const int a = a_row >= 0 ? v.rel(a_row) : -1;
-  const int per_step = kStage * (int)blockDim.x;
-  const int n_slots = ((n_full + per_step - 1) / per_step) * kStage;  // whole granules per thread
-  const int tid = threadIdx.x;
-  SumCount sc = {0.f, 0};
-  {  // the elements outside the granules, one per thread
-    const int k_extra = v.extra();
-    if (k_extra < v.V) {
-      const float x = Storage<TIn>::widen(v.row[k_extra]);
-      if (x >= tau && x > kNegInf) {
-        ++sc.n;
-        if (k_extra != a_row) sc.s += ex2((x - m) * kLog2e);
+  const int n_full = v.n_full, tid = (int)threadIdx.x;
+  const int per_step = 2 * kBlk;
+  const int n_steps = (n_full + per_step - 1) / per_step;
+  sw.mx = SweepOps<TIn>::start(xe);
+  sw.sum = 0;  // two zeros
+  sw.first = 0;
+  sw.wide = false;
+  sw.set_guess(cand, log_rho, mode);
+  const int hole_step = hole >= 0 ? hole / per_step : -1;
+  Stage<TIn, 2> s0, s1;
+  s0.template load_block<kBlk>(row, n_full, 0);
+  for (int step = 0; step < n_steps; step += 2) {  // two stages in flight
+    const bool second = step + 1 < n_steps;
+    if (second) s1.template load_block<kBlk>(row, n_full, step + 1);
+    if (step == hole_step) s0.template punch<kBlk>(step, hole);
+    if (step % kSyncSteps == 0) {
+      if (step == 0) (void)SweepOps<TIn>::bounds(s0, sw.mx);
+      const float m = red.max(SweepOps<TIn>::value(sw.mx));
+      if (m > sw.guess) {
+        if (step > 0 && m - sw.guess > kWide) sw.wide = true;
+        const float f = ex2(sw.c - m * kLog2e);
+        sw.sum = mul2(sw.sum, pack2(f, f));
+        sw.set_guess(m, log_rho, mode);
+        sw.first = step;
       }
     }
+    const int wi = step * kBlk + tid;
+    if (!DVP_IN(wi, n_bound, DVP_OOB_BOUND)) break;
+    sw.absorb(s0, bound + wi);
+    if (step + 2 < n_steps) s0.template load_block<kBlk>(row, n_full, step + 2);
+    if (second && DVP_IN(wi + kBlk, n_bound, DVP_OOB_BOUND)) {
+      if (step + 1 == hole_step) s1.template punch<kBlk>(step + 1, hole);
+      sw.absorb(s1, bound + wi + kBlk);
+    }
+    if ((step & 1023) == 1022) sw.flush_count();
   }
-  const float tau_b = bf16_round_down(tau);
-  hot = build_hot_list<kStage>(bound, n_slots / kStage, tau_b, hot_smem);
-  if (hot.fits()) {
+  sw.flush_count();
+  if (hole >= 0 && hole % kBlk == tid) {
+    const int wi = hole_step * kBlk + tid, sh = (hole / kBlk & 1) * 16;
+    if (DVP_IN(wi, n_bound, DVP_OOB_BOUND))
+      bound[wi] = (bound[wi] & (0xffff0000u >> sh)) | (SweepOps<TIn>::kTop << sh);
+  }
+}
+
+// Sweep 2: masked sum and count over the granules of the steps below n_steps (`list` names granules of these
+// steps and perhaps of later ones), without granule `hole`.
+template <typename TIn, int kBlk>
+__device__ __forceinline__ void row_sweep2(const RowView<TIn> &v, int hole, float tau, float m, int n_steps,
+                                           typename SweepOps<TIn>::Key key, const uint32_t *bound, const HotList &list, SumCount &sc) {
+  const TIn *row = v.base;
+  const int n_full = v.n_full;
+  const int n_slots = n_steps * 2;
+  const int tid = threadIdx.x;
+  if (list.fits()) {
     const int wbase = tid & ~31, lane = tid & 31;
-    for (int q = lane; q < hot.count; q += 64) {
+    for (int q = lane; q < list.count; q += 64) {
       if (!DVP_IN(q, n_hot, DVP_OOB_HOT)) break;
-      const uint32_t e0 = hot.slots[q];
-      const bool two = q + 32 < hot.count && DVP_IN(q + 32, n_hot, DVP_OOB_HOT);
-      const uint32_t e1 = two ? hot.slots[q + 32] : e0;
-      const int g0 = (int)(e0 >> 5) * (int)blockDim.x + wbase + (int)(e0 & 31);
-      const int g1 = (int)(e1 >> 5) * (int)blockDim.x + wbase + (int)(e1 & 31);
+      const uint32_t e0 = list.slots[q];
+      const uint32_t e1 =
+          q + 32 < list.count && DVP_IN(q + 32, n_hot, DVP_OOB_HOT) ? list.slots[q + 32] : 0xffffffffu;
+      const int g0 = (int)(e0 >> 5) * kBlk + wbase + (int)(e0 & 31);
+      const int g1 = (int)(e1 >> 5) * kBlk + wbase + (int)(e1 & 31);
+      const bool one = (int)(e0 >> 5) < n_slots && g0 != hole, two = (e1 >> 5) < (uint32_t)n_slots && g1 != hole;
       Granule<TIn> a0, a1;
-      a0.load_whole(row, n_full, g0);
+      if (one) a0.load_whole(row, n_full, g0);
       if (two) a1.load_whole(row, n_full, g1);
-      granule_masked_sum<TIn>(a0, g0, a, tau, m, sc);
-      if (two) granule_masked_sum<TIn>(a1, g1, a, tau, m, sc);
+      if (one) granule_masked_sum<TIn>(a0, tau, m, sc);
+      if (two) granule_masked_sum<TIn>(a1, tau, m, sc);
     }
   } else {
     // a dense safe set: all of the thread's granules, a step's two at a time (both loads before either is used)
-    static_assert(kStage == 2, "a step's two bounds are neighbours");
-    for (int i = 0; i < n_slots; i += 2) {
-      if (!DVP_IN(bound_index<kStage>(i + 1, tid), n_bound, DVP_OOB_BOUND)) break;
-      const bool hot0 = bf16_bits_to_float(bound[bound_index<kStage>(i, tid)]) >= tau_b;
-      const bool hot1 = bf16_bits_to_float(bound[bound_index<kStage>(i + 1, tid)]) >= tau_b;
-      const int g0 = i * (int)blockDim.x + tid, g1 = g0 + (int)blockDim.x;
+    for (int step = 0; step < n_steps; ++step) {
+      const int wi = step * kBlk + tid;
+      if (!DVP_IN(wi, n_bound, DVP_OOB_BOUND)) break;
+      const uint32_t b = SweepOps<TIn>::reach(bound[wi], key);
+      const int g0 = 2 * step * kBlk + tid, g1 = g0 + kBlk;
+      const bool hot0 = (b & 1u) && g0 != hole, hot1 = (b & 0x10000u) && g1 != hole;
       Granule<TIn> a0, a1;
       if (hot0) a0.load_whole(row, n_full, g0);
       if (hot1) a1.load_whole(row, n_full, g1);
-      if (hot0) granule_masked_sum<TIn>(a0, g0, a, tau, m, sc);
-      if (hot1) granule_masked_sum<TIn>(a1, g1, a, tau, m, sc);
+      if (hot0) granule_masked_sum<TIn>(a0, tau, m, sc);
+      if (hot1) granule_masked_sum<TIn>(a1, tau, m, sc);
     }
   }
-  return block_reduce_sumcount(sc, scratch);
 }
 
-// Statistics of one side of one row (this block sweeps its part of it).
-template <typename TIn, int kStage, int kCluster>
+// Statistics of one row (this block sweeps its part of it).  `listed`: the caller needs the hot list of the
+// whole part.
+template <typename TIn, int kBlk>
 __device__ __forceinline__ SideStats row_stats(const RowView<TIn> &v, int a, double log_rho, int mode,
-                                               float mask_value, uint16_t *bound, float *scratch,
-                                               float *cl_slots, uint16_t *hot_smem, HotList &hot) {
-  const TIn *row = v.row;
-  const int V = v.V;
+                                               float mask_value, bool listed, uint32_t *bound, BlockReduce<kBlk> &red,
+                                               const RowGroup &grp, uint16_t *hot_smem, HotList &list) {
+  const int n_steps = (v.n_full + 2 * kBlk - 1) / (2 * kBlk);
 #ifdef DVP_DEBUG_BOUNDS
   {  // extents of this block's part of the row and of its tables
-    const int per_step = kStage * (int)blockDim.x;
     __syncthreads();
     DVP_BOUNDS_SET(n_gran, v.n_full);
     DVP_BOUNDS_SET(V, (long long)v.n_full * Granule<TIn>::kElems);
-    DVP_BOUNDS_SET(n_bound, (long long)((v.n_full + per_step - 1) / per_step) * per_step);
+    DVP_BOUNDS_SET(n_bound, (long long)n_steps * kBlk);
     DVP_BOUNDS_SET(n_hot, kHotCap);  // entries of one warp's hot list
     DVP_BOUNDS_SYNC();
   }
 #endif
-  const LogSum part = row_sweep1<TIn, kStage>(v, bound, scratch);
-  const LogSum all = cluster_reduce_logsum<kCluster>(part, cl_slots);
+  const bool has_a = a >= 0 && a < v.V;
+  const float z_0 = Storage<TIn>::widen(v.row[has_a ? a : 0]);
+  const int hole = has_a ? v.granule_of(a) : -1;
+  const int k_extra = v.extra_but(has_a ? a : -1, hole);
+  const float xe = k_extra < v.V ? Storage<TIn>::widen(v.row[k_extra]) : kNegInf;
+  Sweep1<TIn> sw;
+  float cand = z_0, m;
+  for (;;) {
+    row_sweep1<TIn, kBlk>(v, hole, xe, cand, log_rho, mode, bound, red, sw);
+    m = fmaxf(red.max(SweepOps<TIn>::value(sw.mx)), sw.guess);
+    if (!sw.wide && !(m - sw.guess > kWide)) break;
+    cand = m;  // the second time it is the maximum
+  }
+  m = grp.max(m);
 
   SideStats st;
-  st.m = all.m;
-  st.lse = lse_from_logsum(all);
-  st.sum_c = (double)all.c;
-  st.sum_s = all.s;
-  st.tau = threshold_of<TIn>(all.m, log_rho, mode);
-  const bool has_a = a >= 0 && a < V;
-  st.z_a = has_a ? Storage<TIn>::widen(row[a]) : 0.f;
+  st.m = m;
+  st.tau = threshold_of<TIn>(m, log_rho, mode);
+  st.z_a = has_a ? z_0 : 0.f;
   st.member = has_a && st.z_a >= st.tau;
   st.e_a = st.member ? ex2((st.z_a - st.m) * kLog2e) : 0.f;
 
-  const SumCount sc =
-      row_sweep2<TIn, kStage>(v, has_a ? a : -1, st.tau, st.m, bound, scratch, hot_smem, hot);
-  const SumCount tot = cluster_reduce_sumcount<kCluster>(sc, cl_slots + 4);
-  st.s_x = tot.s;
-  st.n = tot.n;
-  set_mask_mass(st, V, mode, Storage<TIn>::widen(Storage<TIn>::narrow(mask_value)), has_a);
-
+  const float c = m * kLog2e;
+  float p0, p1;
+  unpack2(sw.sum, p0, p1);
+  float all = (p0 + p1) * ex2(sw.c - c) + ex2(fmaf(xe, kLog2e, -c));
+  SumCount safe = {0.f, 0};
+  const bool guessed = sw.guess == m;  // block-uniform
+  // the sum's terms are 2^{z l - c}; those of the definition (and of sweep 2) 2^{(z - m) l}
+  if (guessed) safe = {sw.safe_s * ex2(-fmaf(m, kLog2e, -c)), sw.safe_n};
+  const int n_again = guessed ? sw.first : n_steps;  // steps whose masked sum is still missing
+  const typename SweepOps<TIn>::Key key = SweepOps<TIn>::key(fmaxf(st.tau, -FLT_MAX));
+  list.slots = hot_smem;
+  list.count = 0;
+  if (n_again > 0 || listed) list = build_hot_list<TIn, kBlk>(bound, listed ? n_steps : n_again, key, hot_smem);
+  if (n_again > 0) row_sweep2<TIn, kBlk>(v, hole, fmaxf(st.tau, -FLT_MAX), m, n_again, key, bound, list, safe);
+  if (xe >= st.tau && xe > kNegInf) {
+    ++safe.n;
+    safe.s += ex2((xe - m) * kLog2e);
+  }
+  red.sums(all, safe);
+  grp.sums(all, safe);
+  if (has_a) all += ex2(fmaf(st.z_a, kLog2e, -c));
+  st.lse = 0.0;  // from sum_c and sum_s, by the thread that writes it
+  st.sum_c = (double)c;
+  st.sum_s = all;
+  st.s_x = safe.s;
+  st.n = safe.n + (st.member ? 1 : 0);
+  set_mask_mass(st, v.V, mode, Storage<TIn>::widen(Storage<TIn>::narrow(mask_value)), has_a);
   return st;
 }
 
@@ -638,11 +875,12 @@ __host__ __device__ constexpr int grad_align() {
 
 // Sweep 3 when the gradient row lies differently than its logits row (another row stride or base):
 // zeros first, in the gradient row's own 32-byte pieces, then the safe tokens one by one.
-template <typename TIn, typename TGrad, int kStage>
-__device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *grow, int a, float tau, float tau_b,
-                                               float m, float coef, float g_a, const uint16_t *bound) {
+template <typename TIn, typename TGrad, int kBlk>
+__device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *grow, int a, float tau,
+                                               typename SweepOps<TIn>::Key key, bool live, float m, float coef,
+                                               float g_a, const uint32_t *bound) {
   constexpr int kElems = Granule<TIn>::kElems, kOut = 32 / (int)sizeof(TGrad);
-  const int tid = threadIdx.x, n_thr = (int)blockDim.x;
+  const int tid = threadIdx.x, n_thr = kBlk;
   const int k0 = v.head + v.g_first * kElems, k1 = k0 + v.n_full * kElems;  // this block's granules, as elements
   TGrad *dst = grow + k0;
   const int n = k1 - k0;
@@ -654,11 +892,11 @@ __device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *gro
   const int k_rest = head + n_vec * kOut + tid;
   if (k_rest < n) dst[k_rest] = Storage<TGrad>::narrow(0.f);
   __syncthreads();  // the zeros of this block's part are in place before single elements replace them
-  const int n_slots = ((v.n_full + kStage * n_thr - 1) / (kStage * n_thr)) * kStage;
-  for (int i = 0; i < n_slots; ++i) {
-    const int g = i * n_thr + tid;
-    if (g >= v.n_full || !DVP_IN(bound_index<kStage>(i, tid), n_bound, DVP_OOB_BOUND)) break;
-    if (!(bf16_bits_to_float(bound[bound_index<kStage>(i, tid)]) >= tau_b)) continue;
+  if (!live) return;
+  for (int i = 0;; ++i) {
+    const int g = i * n_thr + tid, wi = (i >> 1) * n_thr + tid;
+    if (g >= v.n_full || !DVP_IN(wi, n_bound, DVP_OOB_BOUND)) break;
+    if (!((SweepOps<TIn>::reach(bound[wi], key) >> (16 * (i & 1))) & 1u)) continue;
     Granule<TIn> gr;
     gr.load_whole(v.base, v.n_full, g);
     float x[kElems];
@@ -674,16 +912,15 @@ __device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *gro
 
 // Sweep 3: gradient of g * ln pi^mp(a) over the row.  Granules without a safe
 // token are written as zeros without being read.
-template <typename TIn, typename TGrad, int kStage, bool kLoose>
+template <typename TIn, typename TGrad, int kBlk, bool kLoose>
 __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all, int a_row,
-                                         const SideStats &st, float g, const uint16_t *bound,
-                                         const HotList &hot) {
+                                         const SideStats &st, float g, const uint32_t *bound,
+                                         const HotList &list) {
   constexpr int kElems = Granule<TIn>::kElems;
   const TIn *row = v.base;
   const int n_full = v.n_full;
   TGrad *grow = grow_all + (v.base - v.row);
-  const int per_step = kStage * (int)blockDim.x;
-  const int n_slots = ((n_full + per_step - 1) / per_step) * kStage;
+  const int n_steps = (n_full + 2 * kBlk - 1) / (2 * kBlk);
   const int tid = threadIdx.x;
   const float s_tot = st.s_x + st.e_a + st.s_mask;
   // a missing sampled token, or a pruned one under the -inf semantics, has weight zero:
@@ -693,9 +930,9 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
   const float g_a = st.member ? g * ((st.s_x + st.s_mask) / s_tot) : 0.f;
   const int a_here = (live && st.member) ? a_row : -1;
   const int a_live = a_here >= 0 ? v.rel(a_here) : -1;
-  const bool listed = live && hot.fits();
+  const bool listed = live && list.fits();
   const float tau = live ? st.tau : -kNegInf;  // +inf: nothing passes
-  const float tau_b = live ? bf16_round_down(st.tau) : -kNegInf;
+  const typename SweepOps<TIn>::Key key = SweepOps<TIn>::key(fmaxf(st.tau, -FLT_MAX));
 
   {  // the elements outside the granules, one per thread
     const int k_extra = v.extra();
@@ -707,27 +944,28 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
     }
   }
   if constexpr (kLoose) {
-    row_grad_loose<TIn, TGrad, kStage>(v, grow_all, a_live, tau, tau_b, st.m, coef, g_a, bound);
+    row_grad_loose<TIn, TGrad, kBlk>(v, grow_all, a_live, tau, key, live, st.m, coef, g_a, bound);
     return;
   }
-  for (int i = 0; i < n_slots; ++i) {
-    const int gi = i * (int)blockDim.x + tid;
-    if (gi >= n_full) break;
-    if (!DVP_IN(bound_index<kStage>(i, tid), n_bound, DVP_OOB_BOUND)) break;
-    if (bf16_bits_to_float(bound[bound_index<kStage>(i, tid)]) >= tau_b) {
-      // a granule that can hold safe tokens: written below
-    } else if (DVP_IN((long long)gi * kElems + kElems - 1, V, DVP_OOB_GLOBAL)) {
-      store_zero_granule<TGrad, kElems>(grow + (size_t)gi * kElems);
-    }
+  for (int step = 0; step < n_steps; ++step) {
+    const int wi = step * kBlk + tid;
+    if (!DVP_IN(wi, n_bound, DVP_OOB_BOUND)) break;
+    const uint32_t b = live ? SweepOps<TIn>::reach(bound[wi], key) : 0u;
+    const int g0 = 2 * step * kBlk + tid, g1 = g0 + kBlk;
+    // granules that can hold safe tokens are written below
+    if (!(b & 1u) && g0 < n_full && DVP_IN((long long)g0 * kElems + kElems - 1, V, DVP_OOB_GLOBAL))
+      store_zero_granule<TGrad, kElems>(grow + (size_t)g0 * kElems);
+    if (!(b & 0x10000u) && g1 < n_full && DVP_IN((long long)g1 * kElems + kElems - 1, V, DVP_OOB_GLOBAL))
+      store_zero_granule<TGrad, kElems>(grow + (size_t)g1 * kElems);
   }
   if (live && !listed) {
     // a dense safe set: all of the thread's hot granules, a step's two at a time (both loads before either is used)
-    static_assert(kStage == 2, "a step's two bounds are neighbours");
-    for (int i = 0; i < n_slots; i += 2) {
-      if (!DVP_IN(bound_index<kStage>(i + 1, tid), n_bound, DVP_OOB_BOUND)) break;
-      const int g0 = i * (int)blockDim.x + tid, g1 = g0 + (int)blockDim.x;
-      const bool hot0 = g0 < n_full && bf16_bits_to_float(bound[bound_index<kStage>(i, tid)]) >= tau_b;
-      const bool hot1 = g1 < n_full && bf16_bits_to_float(bound[bound_index<kStage>(i + 1, tid)]) >= tau_b;
+    for (int step = 0; step < n_steps; ++step) {
+      const int wi = step * kBlk + tid;
+      if (!DVP_IN(wi, n_bound, DVP_OOB_BOUND)) break;
+      const uint32_t h = SweepOps<TIn>::reach(bound[wi], key);
+      const int g0 = 2 * step * kBlk + tid, g1 = g0 + kBlk;
+      const bool hot0 = h & 1u, hot1 = h & 0x10000u;
       Granule<TIn> a0, a1;
       if (hot0) a0.load_whole(row, n_full, g0);
       if (hot1) a1.load_whole(row, n_full, g1);
@@ -737,13 +975,13 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
   }
   if (listed) {
     const int wbase = tid & ~31, lane = tid & 31;
-    for (int q = lane; q < hot.count; q += 64) {
+    for (int q = lane; q < list.count; q += 64) {
       if (!DVP_IN(q, n_hot, DVP_OOB_HOT)) break;
-      const uint32_t e0 = hot.slots[q];
-      const bool two = q + 32 < hot.count && DVP_IN(q + 32, n_hot, DVP_OOB_HOT);
-      const uint32_t e1 = two ? hot.slots[q + 32] : e0;
-      const int g0 = (int)(e0 >> 5) * (int)blockDim.x + wbase + (int)(e0 & 31);
-      const int g1 = (int)(e1 >> 5) * (int)blockDim.x + wbase + (int)(e1 & 31);
+      const uint32_t e0 = list.slots[q];
+      const bool two = q + 32 < list.count && DVP_IN(q + 32, n_hot, DVP_OOB_HOT);
+      const uint32_t e1 = two ? list.slots[q + 32] : e0;
+      const int g0 = (int)(e0 >> 5) * kBlk + wbase + (int)(e0 & 31);
+      const int g1 = (int)(e1 >> 5) * kBlk + wbase + (int)(e1 & 31);
       Granule<TIn> a0, a1;
       a0.load_whole(row, n_full, g0);
       if (two) a1.load_whole(row, n_full, g1);
@@ -753,99 +991,91 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
   }
 }
 
-// Shared-memory layout of the row kernel, in 4-byte words: 96 for the block
-// reductions, 16 for the cluster exchange, then the hot lists, then the bounds.
+// Shared-memory layout of the row kernel, in 4-byte words: the block reductions, 8 for what blocks of a
+// cluster exchange, then the hot lists, then the bounds.
 __host__ __device__ inline int smem_words_fixed(int threads) {
-  return 96 + 16 + (threads / 32) * kHotCap / 2;
+  return kRedWords + 8 + (threads / 32) * kHotCap / 2;
 }
 
-// kThreads / kBlocks: the launch bounds (largest block, blocks per SM) that set
-// the register budget of this instantiation.  kCluster blocks share one row.
-// kWeighted: the upstream gradient is multiplied by the token's importance weight, which
-// needs the inference side's statistics before sweep 3 of the training row: that
-// instantiation sweeps the inference row first.
-// kLoose: the gradient row lies differently than its logits row (an instantiation of its own: its code
-// between the sweeps costs the others up to 1 %).
-template <typename TIn, typename TGrad, int kStage, int kThreads, int kBlocks, int kCluster, bool kWeighted,
-          bool kLoose>
-__global__ void __launch_bounds__(kThreads, kBlocks) dvp_row_kernel(const RowParams p) {
-  extern __shared__ __align__(16) float smem[];
-  float *scratch = smem;        // 96 floats for the block reductions
-  float *cl_slots = smem + 96;  // 4 exchanges x 4 floats, each written once
-  uint16_t *hot_smem = reinterpret_cast<uint16_t *>(smem + 112);  // kHotCap per warp
-  uint16_t *bound = reinterpret_cast<uint16_t *>(smem + smem_words_fixed(blockDim.x));
+// The gradient of a launch: none; stored in granules; or with rows that lie differently than the logits'.
+enum class Grad { kNone, kGranules, kLoose };
 
-  constexpr int kElems = Granule<TIn>::kElems;
+// One row per block, or per cluster of 2^log_parts blocks.  kBlk: threads of a block, 1024 of them on an SM;
+// a compile-time constant, because it makes the sweeps' indices immediate operands.
+//
+// A token's two rows are swept by two launches, the inference rows' first: two copies of the sweeps in one
+// kernel stall on instruction fetches, a loop over the two rows spills 460 bytes a thread (rows 12 to 17 %
+// slower), and pairs of blocks in a cluster wait for two free places at once (18 % slower with two blocks
+// per SM).  The training rows' launch may begin while the last inference rows are still swept; it waits for
+// them where it needs ln pi^mp_infer(a) and the membership, which they leave at p.li and in p.flags.
+template <typename TIn, typename TGrad, int kBlk, Grad kGrad>
+__global__ void __launch_bounds__(kBlk, 1024 / kBlk)
+dvp_row_kernel(const __grid_constant__ RowParams p, const long long t0, const int log_parts) {
+  extern __shared__ __align__(16) float smem[];
+  BlockReduce<kBlk> red{smem, 0};
+  uint16_t *hot_smem = reinterpret_cast<uint16_t *>(smem + kRedWords + 8);  // kHotCap per warp
+  uint32_t *bound = reinterpret_cast<uint32_t *>(smem + smem_words_fixed(kBlk));
+
   DVP_BOUNDS_BEGIN(p.bounds_status);
-  const long long t = blockIdx.x / kCluster;
-  const int rank = kCluster > 1 ? (int)cluster_rank() : 0;
+  if (p.side == kSideInfer) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int parts = 1 << log_parts;
+  const RowGroup grp{parts, parts > 1 ? (int)cluster_rank() : 0, smem + kRedWords};
+  const long long t = t0 + (blockIdx.x >> log_parts);
   const long long id = p.ids ? load_id(p.ids, p.id_is_i32, t) : -1;
   const bool has_id = id >= 0, bad_id = id >= p.V;
   const int a = (has_id && !bad_id) ? (int)id : -1;
-  const int V = (int)p.V;
-  const TIn *trow = reinterpret_cast<const TIn *>(p.train) + t * p.ld_train;
-  uint32_t *mask_t = p.out_t.mask ? p.out_t.mask + t * ((p.V + 31) / 32) : nullptr;
-  HotList hot;
-  SideStats st, si;
-  if (kWeighted && p.infer) {  // otherwise an earlier launch left the inference side's results
-    const TIn *irow = reinterpret_cast<const TIn *>(p.infer) + t * p.ld_infer;
-    HotList hot_i;
-    RowView<TIn> vi;
-    vi.set(irow, V, rank, kCluster);
-    si = row_stats<TIn, kStage, kCluster>(vi, a, p.log_rho, p.mode, p.mask_value, bound, scratch, cl_slots + 8,
-                                          hot_smem, hot_i);
-    __syncthreads();  // the bounds and the hot lists are reused for the second matrix
-  }
-  RowView<TIn> vt;
-  vt.set(trow, V, rank, kCluster);
-  st = row_stats<TIn, kStage, kCluster>(vt, a, p.log_rho, p.mode, p.mask_value, bound, scratch, cl_slots, hot_smem,
-                                        hot);
-
-  if (p.grad) {
+  const bool writer = threadIdx.x == 0 && grp.part == 0;
+  RowView<TIn> v;
+  v.set(reinterpret_cast<const TIn *>(p.train) + t * p.ld_train, (int)p.V, grp.part, log_parts);
+  HotList list;
+  SideStats st = row_stats<TIn, kBlk>(v, a, p.log_rho, p.mode, p.mask_value, kGrad == Grad::kGranules, bound, red,
+                                      grp, hot_smem, list);
+  if (parts > 1) cluster_arrive();  // this block has read the others' slots
+  float li = 0.f;
+  const bool weighted = p.weight_kind != DVP_WEIGHT_NONE;
+  if constexpr (kGrad != Grad::kNone) {
     float g = p.upstream[t];
-    if constexpr (kWeighted) {
-      const float w = p.infer ? row_weight(p, st, si, a >= 0) : row_weight_given(p, st, t, a >= 0);
+    if (weighted) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      li = load_li(p, t);
+      const float w = a < 0 ? __int_as_float(0x7fc00000)
+                            : token_weight(log_ratio_from(p.mode, st.member, logp_mp_of(st), li), p.weight_kind,
+                                           p.weight_lo, p.weight_hi);
       if (w == w) g *= w;
-      if (p.weight_out && threadIdx.x == 0 && rank == 0) p.weight_out[t] = w;
+      if (parts > 1) {  // every block of the row has li before the place that holds it is overwritten
+        cluster_wait();
+        cluster_arrive();
+        cluster_wait();
+      } else {
+        __syncthreads();
+      }
+      if (p.weight_out && writer) p.weight_out[t] = w;
     }
-    row_grad<TIn, TGrad, kStage, kLoose>(vt, reinterpret_cast<TGrad *>(p.grad) + t * p.ld_grad, a, st, g, bound,
-                                         hot);
+    row_grad<TIn, TGrad, kBlk, kGrad == Grad::kLoose>(v, reinterpret_cast<TGrad *>(p.grad) + t * p.ld_grad, a, st, g,
+                                                      bound, list);
   }
-
-  if constexpr (!kWeighted) {
-    if (p.infer) {
-      __syncthreads();  // the bounds and the hot lists are reused for the second matrix
-      const TIn *irow = reinterpret_cast<const TIn *>(p.infer) + t * p.ld_infer;
-      HotList hot_i;
-      RowView<TIn> vi;
-      vi.set(irow, V, rank, kCluster);
-      si = row_stats<TIn, kStage, kCluster>(vi, a, p.log_rho, p.mode, p.mask_value, bound, scratch, cl_slots + 8,
-                                            hot_smem, hot_i);
+  if (writer) {
+    if (p.side == kSideTrain && !weighted) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      li = load_li(p, t);
     }
-  }
-
-  if (threadIdx.x == 0 && rank == 0) {
+    st.lse = lse_from_logsum({st.m, (float)st.sum_c, st.sum_s});
     const float lt = finish_side(p.out_t, t, st, has_id, bad_id);
-    uint8_t flags = (uint8_t)((st.member ? DVP_FLAG_IN_TRAIN : 0) | (has_id ? 0 : DVP_FLAG_NO_ID) |
-                              (bad_id ? DVP_FLAG_BAD_ID : 0));
-    if (p.infer) {
-      const float li = finish_side(p.out_i, t, si, has_id, bad_id);
-      if (si.member) flags |= DVP_FLAG_IN_INFER;
-      if (p.log_ratio)
-        p.log_ratio[t] = !(has_id && !bad_id)              ? __int_as_float(0x7fc00000)
-                         : (p.mode & DVP_MODE_FINITE_MASK) ? lt - li
-                                                           : log_ratio_of(st.member, si.member, lt, li);
+    if (p.side == kSideInfer) store_li(p, t, lt);
+    if (p.flags) {
+      const uint8_t in_infer = p.side == kSideTrain ? p.flags[t] & DVP_FLAG_IN_INFER : 0;
+      const uint8_t member = p.side == kSideInfer ? DVP_FLAG_IN_INFER : DVP_FLAG_IN_TRAIN;
+      p.flags[t] = (uint8_t)((st.member ? member : 0) | in_infer | (has_id ? 0 : DVP_FLAG_NO_ID) |
+                             (bad_id ? DVP_FLAG_BAD_ID : 0));
     }
-    if (p.flags) p.flags[t] = flags;
+    if (p.log_ratio) p.log_ratio[t] = a < 0 ? __int_as_float(0x7fc00000) : log_ratio_from(p.mode, st.member, lt, li);
   }
-  if (rank == 0) {  // the first block of a row's cluster writes the row's masks
-    if (mask_t) write_mask_row<TIn>(trow, V, st.tau, mask_t);
-    if (p.infer && p.out_i.mask)
-      write_mask_row<TIn>(reinterpret_cast<const TIn *>(p.infer) + t * p.ld_infer, V, si.tau,
-                          p.out_i.mask + t * ((p.V + 31) / 32));
-  }
+  if (p.out_t.mask && grp.part == 0) write_mask_row<TIn>(v.row, v.V, st.tau, p.out_t.mask + t * ((p.V + 31) / 32));
   // no block may leave while another one can still read its exchange slots
-  if constexpr (kCluster > 1) cluster_sync_all();
+  if (parts > 1 && !(kGrad != Grad::kNone && weighted)) {
+    __syncwarp();
+    cluster_wait();
+  }
 }
 
 // ---- scalar kernel: any row length --------------------------------------------
@@ -1020,32 +1250,86 @@ static inline bool aligned32(const void *base, long long ld, size_t elem) {
   return base == nullptr || (((uintptr_t)base % 32 == 0) && ((ld * (long long)elem) % 32 == 0));
 }
 
-template <typename TIn, typename TGrad, int kStage, int kThreads, int kBlocks, int kCluster, bool kWeighted = false,
-          bool kLoose = false>
-static cudaError_t launch_rows_vec(const RowParams &p, int threads, size_t smem, cudaStream_t s) {
-  auto k = dvp_row_kernel<TIn, TGrad, kStage, kThreads, kBlocks, kCluster, kWeighted, kLoose>;
+template <typename TIn, typename TGrad, int kBlk, Grad kGrad>
+static cudaError_t launch_rows_vec(const RowParams &p, long long t0, long long n, int log_parts, size_t smem,
+                                   cudaStream_t s) {
+  auto k = dvp_row_kernel<TIn, TGrad, kBlk, kGrad>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  if constexpr (kCluster == 1) {
-    k<<<(unsigned)p.T, threads, smem, s>>>(p);
-    return cudaGetLastError();
-  } else {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.T * kCluster), 1, 1);
-    cfg.blockDim = dim3((unsigned)threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kCluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, p);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n << log_parts), 1, 1);
+  cfg.blockDim = dim3(kBlk, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  cfg.attrs = attr;
+  cfg.numAttrs = 0;
+  if (log_parts > 0) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = 1u << log_parts;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs++].val.clusterDim.z = 1;
   }
+  if (p.side == kSideTrain) {  // may begin while the inference rows' launch ends
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, k, p, t0, log_parts);
+}
+
+template <typename TIn, typename TGrad, Grad kGrad>
+static cudaError_t launch_rows_blk(const RowParams &p, long long t0, long long n, int log_parts, int threads,
+                                   size_t smem, cudaStream_t s) {
+  switch (threads) {
+    case 64: return launch_rows_vec<TIn, TGrad, 64, kGrad>(p, t0, n, log_parts, smem, s);
+    case 128: return launch_rows_vec<TIn, TGrad, 128, kGrad>(p, t0, n, log_parts, smem, s);
+    case 256: return launch_rows_vec<TIn, TGrad, 256, kGrad>(p, t0, n, log_parts, smem, s);
+    default: return launch_rows_vec<TIn, TGrad, 512, kGrad>(p, t0, n, log_parts, smem, s);
+  }
+}
+
+// The inference rows, then the training rows.  ln pi^mp_infer(a) passes through the output that holds it, or
+// through one that the training rows' launch writes later: log_ratio, weight_out, or the start of the gradient
+// row (with a single 2-byte gradient element there is no room: V = 1, where ln pi^mp(a) is 0).
+template <typename TIn, typename TGrad>
+static cudaError_t launch_rows_both(const RowParams &p_in, bool loose, int log_parts, int threads, size_t smem,
+                                    cudaStream_t s) {
+  const long long per_launch = 0x7fffffffLL >> log_parts;  // a grid holds this many rows
+  for (long long t0 = 0; t0 < p_in.T; t0 += per_launch) {
+    const long long n = p_in.T - t0 < per_launch ? p_in.T - t0 : per_launch;
+    RowParams p = p_in;
+    p.side = kSideAlone;
+    if (p_in.infer) {
+      p.li_stride = sizeof(float);
+      p.li = reinterpret_cast<char *>(p_in.out_i.logp_mp ? p_in.out_i.logp_mp
+                                      : p_in.log_ratio   ? p_in.log_ratio
+                                                         : p_in.weight_out);
+      if (!p.li && p_in.weight_kind != DVP_WEIGHT_NONE && p_in.V * sizeof(TGrad) >= sizeof(float)) {
+        p.li = reinterpret_cast<char *>(p_in.grad);
+        p.li_stride = p_in.ld_grad * (long long)sizeof(TGrad);
+      }
+      RowParams q = p;
+      q.side = kSideInfer;
+      q.train = p_in.infer;
+      q.ld_train = p_in.ld_infer;
+      q.out_t = p_in.out_i;
+      q.infer = nullptr;
+      q.grad = nullptr;
+      q.log_ratio = nullptr;
+      q.weight_kind = DVP_WEIGHT_NONE;
+      const cudaError_t e = launch_rows_blk<TIn, TIn, Grad::kNone>(q, t0, n, log_parts, threads, smem, s);
+      if (e != cudaSuccess) return e;
+      p.side = kSideTrain;
+    }
+    const cudaError_t e =
+        !p.grad ? launch_rows_blk<TIn, TIn, Grad::kNone>(p, t0, n, log_parts, threads, smem, s)
+        : loose ? launch_rows_blk<TIn, TGrad, Grad::kLoose>(p, t0, n, log_parts, threads, smem, s)
+                : launch_rows_blk<TIn, TGrad, Grad::kGranules>(p, t0, n, log_parts, threads, smem, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // Shared memory one SM can give to `blocks` resident blocks (228 KB per SM, 1 KB of it
@@ -1109,16 +1393,19 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
     loose = shift % kA != 0 || (p.T > 1 && (p.ld_grad - p.ld_train) % kA != 0);
   }
   const long long n_gran_row = (p.V + kElems - 1) / kElems;
-  if (cluster == 0) cluster = 1;
-  const bool weighted = p.weight_kind != DVP_WEIGHT_NONE;  // one block per row only
-  if (weighted || loose) cluster = 1;
-  if (cluster > 1 && (n_gran_row < 4096 || p.T * cluster > 0x7fffffffLL)) cluster = 1;
-  const long long n_gran = (n_gran_row + cluster - 1) / cluster;  // granules per block
+  const bool weighted = p.weight_kind != DVP_WEIGHT_NONE;
+  int log_parts = cluster == 4 ? 2 : cluster == 2 ? 1 : 0;
+  while (log_parts > 0 && (n_gran_row >> log_parts) < 256) --log_parts;
+  const int parts = 1 << log_parts;
+  const long long n_gran = (n_gran_row + parts - 1) / parts;  // granules per block
   // shrink the block for short rows so that threads are not idle
+  int shape = 64;  // the largest of 64, 128, 256 and 512 threads that is not above the choice
+  while (2 * shape <= threads) shape *= 2;
+  threads = shape;
   while (threads > 64 && (long long)threads * stage / 2 >= n_gran) threads /= 2;
   const long long per = (long long)stage * threads;
   const size_t smem = (size_t)smem_words_fixed(threads) * 4 +
-                      (size_t)((n_gran + per - 1) / per) * per * sizeof(uint16_t);
+                      (size_t)((n_gran + per - 1) / per) * threads * 4;
   // 16-bit hot-list entries hold slot * 32 + lane: very long rows swept by few threads
   // would not fit them
   const bool hot_ok = ((n_gran + per - 1) / per) * stage * 32 <= 65536;
@@ -1126,7 +1413,7 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
     // stage byte 3 or 4: the kernel that keeps the candidates of the safe set on chip, with
     // three or four resident blocks per SM (measured slower than the kernel below; kept for
     // comparison)
-    if (vec_ok && cluster == 1 && (stage_hint == 3 || stage_hint == 4) && threads <= 256) {
+    if (vec_ok && parts == 1 && (stage_hint == 3 || stage_hint == 4) && threads <= 256) {
       const int n_steps = (int)((n_gran + per - 1) / per);
       cudaError_t e;
       if (weighted)
@@ -1139,23 +1426,7 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
     }
   }
   if (hot_ok && smem <= 200 * 1024) {
-    if (cluster == 4 && threads <= 256 && stage == 2)
-      return launch_rows_vec<TIn, TGrad, 2, 256, 4, 4>(p, threads, smem, s);
-    if (cluster == 2 && threads <= 256 && stage == 2)
-      return launch_rows_vec<TIn, TGrad, 2, 256, 4, 2>(p, threads, smem, s);
-    if (loose) {
-      if (weighted)
-        return threads > 256 ? launch_rows_vec<TIn, TGrad, 2, 512, 2, 1, true, true>(p, threads, smem, s)
-                             : launch_rows_vec<TIn, TGrad, 2, 256, 4, 1, true, true>(p, threads, smem, s);
-      return threads > 256 ? launch_rows_vec<TIn, TGrad, 2, 512, 2, 1, false, true>(p, threads, smem, s)
-                           : launch_rows_vec<TIn, TGrad, 2, 256, 4, 1, false, true>(p, threads, smem, s);
-    }
-    if (weighted) {
-      if (threads > 256) return launch_rows_vec<TIn, TGrad, 2, 512, 2, 1, true>(p, threads, smem, s);
-      return launch_rows_vec<TIn, TGrad, 2, 256, 4, 1, true>(p, threads, smem, s);
-    }
-    if (threads > 256) return launch_rows_vec<TIn, TGrad, 2, 512, 2, 1>(p, threads, smem, s);
-    return launch_rows_vec<TIn, TGrad, 2, 256, 4, 1>(p, threads, smem, s);
+    return launch_rows_both<TIn, TGrad>(p, loose, log_parts, threads, smem, s);
   }
   dvp_row_kernel_scalar<TIn, TGrad><<<(unsigned)p.T, 512, 0, s>>>(p);
   return cudaGetLastError();
