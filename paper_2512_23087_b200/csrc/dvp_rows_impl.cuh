@@ -1362,6 +1362,40 @@ static cudaError_t launch_rows_cs(const RowParams &p, int threads, int n_steps, 
   return cudaGetLastError();
 }
 
+// Threads of a block and blocks of a row, from the number of rows (both policies') and their length in
+// granules.  An SM holds 1,024 threads of the row kernel.
+//
+// A thread should have about 16 granules: each row costs it some 860 instructions beside the 250 of two
+// granules.  Measured, us, with the gradient, for 64 / 128 / 256 / 512 threads: 20,000 x 4,000 float32
+// 222 / 266 / 404 / 404; 4,000 x 8,001 float32 91 / 99 / 118 / 185; 8,000 x 20,000 bfloat16 226 at 128 against
+// 230 at 64 and 288 at 256; 2,000 x 32,000 float32 173 / 155 / 155 / 175.  Not above `most`, where rows of any
+// length run best: 256 for 2-byte logits (V = 151,936: 909 against 1207 at 128), 512 for float32 (V = 262,144:
+// 1904 against 2180 at 256).
+//
+// While all rows fit the chip at once, more threads a row are faster (100 x 20,000 bfloat16: 17.5 at 256
+// against 21.5 at 128 and 29.7 at 64), then more blocks a row (V = 151,936 bfloat16, 1 / 2 / 4 / 8 blocks:
+// T = 16 forward 36 / 28 / 21 / 19; T = 64 forward 38 / 32 / 28 / 34; T = 128 with the gradient
+// 65 / 50 / 48 / 60; T = 512 130 / 126 / 134 / 192; V = 50,000, T = 100: 30 / 24 / 28 / 38).  Blocks that share
+// a row need at least a step and a half of it each (V = 20,000: 13 / 15).
+struct RowShape {
+  int threads, log_parts;
+};
+static inline RowShape choose_shape(long long rows, long long n_gran, int most) {
+  const long long resident = 148 * 1024;
+  RowShape s = {64, 0};
+  while (s.threads < most && 16LL * s.threads < n_gran) s.threads *= 2;
+  while (s.threads < most && 2 * rows * s.threads <= resident && n_gran >= 2 * s.threads) s.threads *= 2;
+  while (s.log_parts < 3) {
+    const int lp = s.log_parts + 1;
+    const long long per = n_gran >> lp, total = (rows << lp) * s.threads;
+    const bool fits = lp == 1 ? total <= 4 * resident
+                              : total <= resident || (lp == 2 && total <= 2 * resident && per >= 8 * s.threads);
+    if (per < 3 * s.threads || !fits) break;
+    s.log_parts = lp;
+  }
+  return s;
+}
+
 template <typename TIn, typename TGrad>
 static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s) {
   constexpr int kElems = Granule<TIn>::kElems;
@@ -1378,9 +1412,6 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
     if (e != cudaErrorNotSupported) return e;
     cluster = 0;  // rows it cannot take: the streaming kernel below
   }
-  // measured on B200: 4-byte logits run best with 2 x 512 threads per SM, 2-byte
-  // logits (twice the exponentials per byte) with 4 x 256
-  if (threads == 0) threads = sizeof(TIn) == 4 ? 512 : 256;
   stage = 2;  // two granules per thread and pipeline stage
   const bool vec_ok = aligned32(p.train, p.ld_train, sizeof(TIn)) &&
                       aligned32(p.infer, p.ld_infer, sizeof(TIn)) &&
@@ -1394,15 +1425,23 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
   }
   const long long n_gran_row = (p.V + kElems - 1) / kElems;
   const bool weighted = p.weight_kind != DVP_WEIGHT_NONE;
-  int log_parts = cluster == 4 ? 2 : cluster == 2 ? 1 : 0;
-  while (log_parts > 0 && (n_gran_row >> log_parts) < 256) --log_parts;
+  const bool store_kernel = sizeof(TIn) == 2 && (stage_hint == 3 || stage_hint == 4);
+  int log_parts = 0;
+  if (threads == 0 && cluster == 0 && !store_kernel) {
+    const RowShape sh = choose_shape(p.T * (p.infer ? 2 : 1), n_gran_row, sizeof(TIn) == 4 ? 512 : 256);
+    threads = sh.threads;
+    log_parts = sh.log_parts;
+  } else {
+    if (threads == 0) threads = sizeof(TIn) == 4 ? 512 : 256;
+    log_parts = cluster == 8 ? 3 : cluster == 4 ? 2 : cluster == 2 ? 1 : 0;
+    while (log_parts > 0 && (n_gran_row >> log_parts) < 256) --log_parts;
+    int pow2 = 64;  // the largest of 64, 128, 256 and 512 threads that is not above the choice
+    while (2 * pow2 <= threads) pow2 *= 2;
+    threads = pow2;
+    while (threads > 64 && threads >= n_gran_row >> log_parts) threads /= 2;
+  }
   const int parts = 1 << log_parts;
   const long long n_gran = (n_gran_row + parts - 1) / parts;  // granules per block
-  // shrink the block for short rows so that threads are not idle
-  int shape = 64;  // the largest of 64, 128, 256 and 512 threads that is not above the choice
-  while (2 * shape <= threads) shape *= 2;
-  threads = shape;
-  while (threads > 64 && (long long)threads * stage / 2 >= n_gran) threads /= 2;
   const long long per = (long long)stage * threads;
   const size_t smem = (size_t)smem_words_fixed(threads) * 4 +
                       (size_t)((n_gran + per - 1) / per) * threads * 4;
@@ -1413,7 +1452,7 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
     // stage byte 3 or 4: the kernel that keeps the candidates of the safe set on chip, with
     // three or four resident blocks per SM (measured slower than the kernel below; kept for
     // comparison)
-    if (vec_ok && parts == 1 && (stage_hint == 3 || stage_hint == 4) && threads <= 256) {
+    if (store_kernel && vec_ok && parts == 1 && threads <= 256) {
       const int n_steps = (int)((n_gran + per - 1) / per);
       cudaError_t e;
       if (weighted)

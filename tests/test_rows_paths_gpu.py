@@ -1,0 +1,106 @@
+"""Paths of the row kernel that depend on sizes and on which outputs are asked for: a guess of the maximum that is far off,
+rows split over several blocks, and the places through which ln pi^mp_infer(a) passes between the two launches."""
+import ctypes
+import dataclasses
+
+import pytest
+import torch
+
+from paper_2512_23087_b200 import binding, inputs
+
+import oracle
+import parity
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+W = inputs.WORKLOADS
+
+
+def _check(batch, rho, V, **kw):
+    res = binding.dvp_forward(batch.train, batch.ids, rho, infer_logits=batch.infer, upstream=batch.upstream,
+                              want_mask=True, **kw)
+    torch.cuda.synchronize()
+    parity.check_forward(res, batch, rho, V, True)
+    return res
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("threads", [64, 256])
+def test_maximum_far_above_every_guess(dtype, threads):
+    """One token 200 above all others: e^200 overflows in the units of any earlier guess.  It sits in the first step, in a
+    later one, in the last piece, outside the pieces, or is (next to) the sampled token."""
+    V, places = 40003, [0, 70, 17000, 25001, 39990, 40002]
+    w = dataclasses.replace(W["c0_small_f32"], dtype=dtype, head_boost=0.0)
+    b = inputs.make_rows(w, seed=5, device=DEV, T=2 * len(places), V=V)
+    for i, k in enumerate(places):
+        for t in (2 * i, 2 * i + 1):
+            b.train[t, k] = 200.0
+            b.infer[t, k] = 201.0
+        b.ids[2 * i] = 12345
+        b.ids[2 * i + 1] = min(k + 1, V - 1)
+    for rho in (1e-3, 0.0):
+        _check(b, rho, V, launch_hint=threads)
+
+
+@pytest.mark.parametrize("dtype,T,V", [("bf16", 3, 151936), ("bf16", 150, 30001), ("f32", 2, 262144), ("f16", 40, 70000),
+                                       ("f32", 600, 515), ("bf16", 1, 12289), ("bf16", 1, 12287)])
+def test_default_shapes(dtype, T, V):
+    """Few rows take several blocks each, many short ones small blocks; sizes on both sides of the rules' lines."""
+    w = dataclasses.replace(W["c2_bf16_fwdbwd"], dtype=dtype)
+    b = inputs.make_rows(w, seed=V, device=DEV, T=T, V=V)
+    _check(b, 1e-4, V)
+
+
+@pytest.mark.parametrize("parts", [2, 4, 8])
+@pytest.mark.parametrize("V", [151936, 50021])
+def test_rows_split_over_blocks_with_weights(V, parts):
+    b = inputs.make_rows(W["c2_bf16_fwdbwd"], seed=parts, device=DEV, T=9, V=V)
+    weight = (oracle.WEIGHT_TRUNCATE, 0.0, 1.01)
+    res = binding.dvp_forward(b.train, b.ids, 1e-3, infer_logits=b.infer, upstream=b.upstream,
+                              weight_kind=weight[0], weight_lo=weight[1], weight_hi=weight[2],
+                              launch_hint=256 | (parts << 24))
+    torch.cuda.synchronize()
+    parity.check_weighted(res, b, 1e-3, V, weight)
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("V", [1, 2, 5003])
+@pytest.mark.parametrize("kept", [(), ("log_ratio",), ("flags",), ("weight",), ("log_ratio", "flags"), ("logp_mp_i",)])
+def test_outputs_left_out(kept, V, weighted):
+    """Any output may be missing; what is asked for is bit for bit what the full call gives."""
+    w = W["c2_bf16_fwdbwd"]
+    b = inputs.make_rows(dataclasses.replace(w, head_boost=2.0, head_max=1), seed=V, device=DEV, T=37, V=V)
+    b.ids[3], b.ids[4] = -1, V
+    kw = dict(weight_kind=binding.DVP_WEIGHT_TRUNCATE, weight_hi=1.01) if weighted else {}
+    full = binding.dvp_forward(b.train, b.ids, 1e-2, infer_logits=b.infer, upstream=b.upstream, **kw)
+    a = binding.ForwardArgs()
+    a.struct_size, a.logits_dtype, a.grad_dtype = ctypes.sizeof(binding.ForwardArgs), binding.DVP_BF16, binding.DVP_BF16
+    a.T, a.V, a.rho = 37, V, 1e-2
+    a.ld_train = a.ld_infer = a.ld_grad = V
+    grad = torch.full((37, V), 7.0, dtype=torch.bfloat16, device=DEV)
+    a.train_logits, a.infer_logits, a.ids = b.train.data_ptr(), b.infer.data_ptr(), b.ids.data_ptr()
+    a.upstream, a.grad_train = b.upstream.data_ptr(), grad.data_ptr()
+    out = {n: torch.empty(37, dtype=torch.uint8 if n == "flags" else torch.float32, device=DEV) for n in kept}
+    if "log_ratio" in out:
+        a.log_ratio = out["log_ratio"].data_ptr()
+    if "flags" in out:
+        a.flags = out["flags"].data_ptr()
+    if "weight" in out and weighted:
+        a.weight_out = out["weight"].data_ptr()
+    if "logp_mp_i" in out:
+        a.infer.logp_mp = out["logp_mp_i"].data_ptr()
+    if weighted:
+        a.weight_kind, a.weight_hi = binding.DVP_WEIGHT_TRUNCATE, 1.01
+    a.stream = torch.cuda.current_stream().cuda_stream
+    assert binding.load_library().dvp_forward(ctypes.byref(a)) == binding.DVP_OK
+    torch.cuda.synchronize()
+    same = lambda x, y: torch.equal(torch.nan_to_num(x.float(), nan=9e9), torch.nan_to_num(y.float(), nan=9e9))
+    assert same(grad, full.grad_train)
+    if "log_ratio" in out:
+        assert same(out["log_ratio"], full.log_ratio)
+    if "flags" in out:
+        assert same(out["flags"], full.flags)
+    if "weight" in out and weighted:
+        assert same(out["weight"], full.weight)
+    if "logp_mp_i" in out:
+        assert same(out["logp_mp_i"], full.infer.logp_mp)
