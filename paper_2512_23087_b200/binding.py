@@ -10,6 +10,7 @@ from __future__ import annotations
 import contextlib
 import ctypes
 import os
+import struct
 from types import SimpleNamespace
 
 import torch
@@ -180,6 +181,15 @@ class MonitorArgs(ctypes.Structure):
     ]
 
 
+# The hot entry points are called with their argument structs packed in one go: setting the fields of a ctypes
+# structure one by one costs several microseconds a call.
+_FORWARD_PACK = struct.Struct("=I3i5qd5Q18Q3QIIfIffQ")
+_BACKWARD_PACK = struct.Struct("=I3i4qd9QIIfI")
+_MONITOR_PACK = struct.Struct("=Ii4q7Q")
+_SEQUENCE_PACK = struct.Struct("=II2q2Qd9Q")
+assert _FORWARD_PACK.size == ctypes.sizeof(ForwardArgs) and _BACKWARD_PACK.size == ctypes.sizeof(BackwardArgs)
+assert _MONITOR_PACK.size == ctypes.sizeof(MonitorArgs) and _SEQUENCE_PACK.size == ctypes.sizeof(SequenceArgs)
+
 _lib = None
 
 
@@ -220,6 +230,11 @@ def load_library() -> ctypes.CDLL:
         lib.dvp_static_workspace_status.restype = ctypes.c_int
         lib.dvp_debug_bounds_status.argtypes = [ctypes.POINTER(ctypes.c_uint32)]
         lib.dvp_debug_bounds_status.restype = ctypes.c_int
+        lib.packed = {}   # the entry points that take a packed struct
+        for name in ("dvp_forward", "dvp_backward", "dvp_monitor", "dvp_sequence_aggregate"):
+            fn = lib[name]   # a function object of its own, with its own argtypes
+            fn.argtypes, fn.restype = [ctypes.c_char_p], ctypes.c_int
+            lib.packed[name] = fn
         _lib = lib
     return _lib
 
@@ -261,9 +276,13 @@ def _ptr(t: torch.Tensor | None):
     return None if t is None else t.data_ptr()
 
 
+def _address(t: torch.Tensor | None) -> int:
+    return 0 if t is None else t.data_ptr()
+
+
 def _stream(stream) -> int:
     if stream is None:
-        stream = torch.cuda.current_stream()
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream
 
 
@@ -274,14 +293,37 @@ def _check_matrix(name: str, x: torch.Tensor):
         raise ValueError(f"{name} must live on a CUDA device")
 
 
-def _side(device, T: int, V: int, want_mask: bool):
-    o = SimpleNamespace()
-    for n in ("max", "lse", "lse_safe", "logp", "logp_mp", "comp_mp", "log_cov"):
-        setattr(o, n, torch.empty(T, dtype=torch.float32, device=device))
-    o.count = torch.empty(T, dtype=torch.int32, device=device)
-    o.mask = torch.empty(T, (V + 31) // 32, dtype=torch.int32, device=device) if want_mask else None
-    s = SideOut(*(_ptr(getattr(o, n)) for n in _SIDE_FIELDS))
-    return o, s
+def _token_outputs(like: torch.Tensor, T: int, sides: int, floats: int):
+    """``sides`` side namespaces and ``floats`` further float32 vectors of T tokens, with their addresses.  All
+    float32 vectors are rows of one allocation, as are the counts: an allocator call costs about a
+    microsecond, a call of dvp_forward would make twenty."""
+    buf = like.new_empty((7 * sides + floats, T), dtype=torch.float32)
+    rows, base, step = buf.unbind(0), buf.data_ptr(), 4 * T
+    cnt = like.new_empty((sides, T), dtype=torch.int32)
+    counts, cbase = cnt.unbind(0), cnt.data_ptr()
+    out = []
+    for i in range(sides):
+        r, at = rows[7 * i:7 * i + 7], base + 7 * i * step
+        o = SimpleNamespace(max=r[0], lse=r[1], lse_safe=r[2], logp=r[3], logp_mp=r[4], comp_mp=r[5], log_cov=r[6],
+                            count=counts[i], mask=None)
+        # in the order of dvp_side_out
+        out.append((o, (at, at + step, at + 2 * step, at + 3 * step, at + 4 * step, at + 5 * step, cbase + i * step,
+                        0, at + 6 * step)))
+    return out, rows[7 * sides:]
+
+
+def _with_mask(side, like: torch.Tensor, T: int, V: int):
+    o, addresses = side
+    o.mask = like.new_empty((T, (V + 31) // 32), dtype=torch.int32)
+    return o, addresses[:7] + (o.mask.data_ptr(), addresses[8])
+
+
+_NO_SIDE = (0,) * 9
+
+
+def _float32(x: float) -> float:
+    """What a C float holds of x: struct refuses to pack a finite value beyond float32's range."""
+    return ctypes.c_float(x).value
 
 
 def _id_dtype(ids: torch.Tensor) -> int:
@@ -314,61 +356,51 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
     ``log_ratio``, ``flags`` and ``grad_train``.  Pass the namespace of an
     earlier call as ``out`` to reuse its buffers.
     """
-    lib = load_library()
+    packed = load_library().packed
     _check_matrix("train_logits", train_logits)
     T, V = train_logits.shape
-    dev = train_logits.device
-    a = ForwardArgs()
-    a.struct_size = ctypes.sizeof(ForwardArgs)
-    a.logits_dtype = _DTYPES[train_logits.dtype]
-    a.id_dtype = _id_dtype(ids)
-    a.T, a.V, a.rho = T, V, float(rho)
-    a.ld_train = train_logits.stride(0)
-    a.train_logits = _ptr(train_logits)
-    a.ids = _ptr(ids)
-    res = out if out is not None else SimpleNamespace(train=None, infer=None, log_ratio=None,
-                                                      flags=None, grad_train=None)
-    if out is None:
-        res.train, res._train_struct = _side(dev, T, V, want_mask)
-        res.flags = torch.empty(T, dtype=torch.uint8, device=dev)
-    a.train = res._train_struct
-    a.flags = _ptr(res.flags)
-    if infer_logits is not None:
+    dtype = train_logits.dtype
+    has_infer, weighted = infer_logits is not None, weight_kind != DVP_WEIGHT_NONE
+    if has_infer:
         _check_matrix("infer_logits", infer_logits)
-        if infer_logits.dtype != train_logits.dtype or infer_logits.shape != train_logits.shape:
+        if infer_logits.dtype != dtype or infer_logits.shape != train_logits.shape:
             raise ValueError("infer_logits must match train_logits in dtype and shape")
-        a.infer_logits = _ptr(infer_logits)
-        a.ld_infer = infer_logits.stride(0)
-        if out is None:
-            res.infer, res._infer_struct = _side(dev, T, V, want_mask)
-            res.log_ratio = torch.empty(T, dtype=torch.float32, device=dev)
-        a.infer = res._infer_struct
-        a.log_ratio = _ptr(res.log_ratio)
+    if out is not None:
+        res = out
+    else:
+        sides, rest = _token_outputs(train_logits, T, 2 if has_infer else 1, has_infer + weighted)
+        if want_mask:
+            sides = [_with_mask(side, train_logits, T, V) for side in sides]
+        res = SimpleNamespace(train=sides[0][0], infer=sides[1][0] if has_infer else None,
+                              log_ratio=rest[0] if has_infer else None,
+                              flags=train_logits.new_empty(T, dtype=torch.uint8), grad_train=None,
+                              _train_addresses=sides[0][1], _infer_addresses=sides[1][1] if has_infer else _NO_SIDE)
+        if weighted:
+            res.weight = rest[-1]
+    if weighted and getattr(res, "weight", None) is None:
+        res.weight = train_logits.new_empty(T, dtype=torch.float32)
+    grad_code = grad_ld = 0
     if upstream is not None:
         if upstream.dtype != torch.float32:
             raise TypeError("upstream must be float32")
         if grad_train is None:
             grad_train = res.grad_train
         if grad_train is None:
-            grad_train = torch.empty(T, V, dtype=grad_dtype or train_logits.dtype, device=dev)
+            grad_train = train_logits.new_empty((T, V), dtype=grad_dtype or dtype)
         _check_matrix("grad_train", grad_train)
         res.grad_train = grad_train
-        a.upstream = _ptr(upstream)
-        a.grad_train = _ptr(grad_train)
-        a.grad_dtype = _DTYPES[grad_train.dtype]
-        a.ld_grad = grad_train.stride(0)
-    a.stream = _stream(stream)
-    a.launch_hint = launch_hint
-    a.mode = (DVP_MODE_FINITE_MASK if mask_value is not None else 0) | \
+        grad_code, grad_ld = _DTYPES[grad_train.dtype], grad_train.stride(0)
+    else:
+        grad_train = None
+    mode = (DVP_MODE_FINITE_MASK if mask_value is not None else 0) | \
         (DVP_MODE_THRESHOLD_IN_LOGITS_DTYPE if threshold_in_logits_dtype else 0)
-    a.mask_value = float(mask_value) if mask_value is not None else 0.0
-    a.weight_kind = int(weight_kind)
-    a.weight_lo, a.weight_hi = float(weight_lo), float(weight_hi)
-    if weight_kind != DVP_WEIGHT_NONE:
-        if getattr(res, "weight", None) is None:
-            res.weight = torch.empty(T, dtype=torch.float32, device=dev)
-        a.weight_out = _ptr(res.weight)
-    st = lib.dvp_forward(ctypes.byref(a))
+    st = packed["dvp_forward"](_FORWARD_PACK.pack(
+        _FORWARD_PACK.size, _DTYPES[dtype], grad_code, _id_dtype(ids), T, V, train_logits.stride(0),
+        infer_logits.stride(0) if has_infer else 0, grad_ld, float(rho), train_logits.data_ptr(),
+        _address(infer_logits), ids.data_ptr(), _address(upstream), _address(grad_train), *res._train_addresses,
+        *(res._infer_addresses if has_infer else _NO_SIDE), res.log_ratio.data_ptr() if has_infer else 0,
+        res.flags.data_ptr(), _stream(stream), launch_hint, mode, _float32(mask_value) if mask_value is not None else 0.0,
+        int(weight_kind), _float32(weight_lo), _float32(weight_hi), res.weight.data_ptr() if weighted else 0))
     if st != DVP_OK:
         raise DvpError(st, "dvp_forward")
     return res
@@ -381,31 +413,20 @@ def dvp_backward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, upst
                  threshold_in_logits_dtype: bool = False) -> torch.Tensor:
     """dLoss/dlogits from the vectors an earlier ``dvp_forward`` saved
     (``saved`` = its result namespace) and a per-token upstream gradient."""
-    lib = load_library()
+    packed = load_library().packed
     _check_matrix("train_logits", train_logits)
     T, V = train_logits.shape
     if grad_train is None:
-        grad_train = torch.empty(T, V, dtype=grad_dtype or train_logits.dtype,
-                                 device=train_logits.device)
+        grad_train = train_logits.new_empty((T, V), dtype=grad_dtype or train_logits.dtype)
     _check_matrix("grad_train", grad_train)
-    a = BackwardArgs()
-    a.struct_size = ctypes.sizeof(BackwardArgs)
-    a.logits_dtype = _DTYPES[train_logits.dtype]
-    a.grad_dtype = _DTYPES[grad_train.dtype]
-    a.id_dtype = _id_dtype(ids)
-    a.T, a.V, a.rho = T, V, float(rho)
-    a.ld_train, a.ld_grad = train_logits.stride(0), grad_train.stride(0)
-    a.train_logits, a.ids, a.upstream = _ptr(train_logits), _ptr(ids), _ptr(upstream)
-    a.max_t, a.lse_safe_t = _ptr(saved.train.max), _ptr(saved.train.lse_safe)
-    a.comp_mp_t = _ptr(saved.train.comp_mp) if use_comp else None
-    a.flags = _ptr(saved.flags)
-    a.grad_train = _ptr(grad_train)
-    a.stream = _stream(stream)
-    a.launch_hint = launch_hint
-    a.mode = (DVP_MODE_FINITE_MASK if mask_value is not None else 0) | \
+    mode = (DVP_MODE_FINITE_MASK if mask_value is not None else 0) | \
         (DVP_MODE_THRESHOLD_IN_LOGITS_DTYPE if threshold_in_logits_dtype else 0)
-    a.mask_value = float(mask_value) if mask_value is not None else 0.0
-    st = lib.dvp_backward(ctypes.byref(a))
+    st = packed["dvp_backward"](_BACKWARD_PACK.pack(
+        _BACKWARD_PACK.size, _DTYPES[train_logits.dtype], _DTYPES[grad_train.dtype], _id_dtype(ids), T, V,
+        train_logits.stride(0), grad_train.stride(0), float(rho), train_logits.data_ptr(), ids.data_ptr(),
+        upstream.data_ptr(), saved.train.max.data_ptr(), saved.train.lse_safe.data_ptr(),
+        saved.train.comp_mp.data_ptr() if use_comp else 0, saved.flags.data_ptr(), grad_train.data_ptr(),
+        _stream(stream), launch_hint, mode, _float32(mask_value) if mask_value is not None else 0.0, 0))
     if st != DVP_OK:
         raise DvpError(st, "dvp_backward")
     return grad_train
@@ -469,7 +490,10 @@ def _fused_args(hidden, w_vocab, ids, rho, upstream, infer_logits, d_w, accumula
     a.ld_hidden, a.ld_w = hidden.stride(0), w_vocab.stride(0)
     a.hidden, a.w_vocab, a.ids, a.upstream = _ptr(hidden), _ptr(w_vocab), _ptr(ids), _ptr(upstream)
     res = SimpleNamespace(infer=None, log_ratio=None)
-    res.train, a.train = _side(dev, T, V, want_mask)
+    sides, rest = _token_outputs(hidden, T, 1 if infer_logits is None else 2, infer_logits is not None)
+    if want_mask:
+        sides[0] = _with_mask(sides[0], hidden, T, V)
+    res.train, a.train = sides[0][0], SideOut(*(x or None for x in sides[0][1]))
     res.flags = torch.empty(T, dtype=torch.uint8, device=dev)
     a.flags = _ptr(res.flags)
     if infer_logits is not None:
@@ -477,8 +501,8 @@ def _fused_args(hidden, w_vocab, ids, rho, upstream, infer_logits, d_w, accumula
         if infer_logits.dtype != torch.bfloat16:
             raise TypeError("infer_logits must be bfloat16")
         a.infer_logits, a.ld_infer = _ptr(infer_logits), infer_logits.stride(0)
-        res.infer, a.infer = _side(dev, T, V, False)
-        res.log_ratio = torch.empty(T, dtype=torch.float32, device=dev)
+        res.infer, a.infer = sides[1][0], SideOut(*(x or None for x in sides[1][1]))
+        res.log_ratio = rest[0]
         a.log_ratio = _ptr(res.log_ratio)
     res.d_hidden = torch.empty(T, H, dtype=torch.float32, device=dev)
     res.d_w = d_w if d_w is not None else torch.empty(V, H, dtype=torch.float32, device=dev)
@@ -565,32 +589,24 @@ def dvp_sequence_aggregate(log_ratio: torch.Tensor, seq_offsets: torch.Tensor,
     int64 device tensor of S + 1 non-decreasing token offsets.  With ``log_cov``
     (ln Z per token from ``dvp_forward``) also the minimum and the mean of the
     coverage Z over each sequence (Def. 5.2; the Z_min of Prop. 5.5)."""
-    lib = load_library()
+    packed = load_library().packed
     if log_ratio.dtype != torch.float32 or seq_offsets.dtype != torch.int64:
         raise TypeError("log_ratio must be float32 and seq_offsets int64")
+    has_cov = log_cov is not None
+    if has_cov and (log_cov.dtype != torch.float32 or log_cov.numel() != log_ratio.numel()):
+        raise TypeError("log_cov must be float32 with one entry per token")
     S = seq_offsets.numel() - 1
-    dev = log_ratio.device
-    res = SimpleNamespace(
-        seq_log_ratio=torch.empty(S, dtype=torch.float32, device=dev),
-        min_log_ratio=torch.empty(S, dtype=torch.float32, device=dev),
-        n_valid=torch.empty(S, dtype=torch.int32, device=dev),
-        n_zero_weight=torch.empty(S, dtype=torch.int32, device=dev),
-        veto=torch.empty(S, dtype=torch.uint8, device=dev))
-    a = SequenceArgs()
-    a.struct_size = ctypes.sizeof(SequenceArgs)
-    a.T, a.S = log_ratio.numel(), S
-    a.seq_offsets, a.log_ratio = _ptr(seq_offsets), _ptr(log_ratio)
-    a.veto_threshold = float(veto_threshold)
-    a.seq_log_ratio, a.min_log_ratio = _ptr(res.seq_log_ratio), _ptr(res.min_log_ratio)
-    a.n_valid, a.n_zero_weight, a.veto = _ptr(res.n_valid), _ptr(res.n_zero_weight), _ptr(res.veto)
-    a.stream = _stream(stream)
-    if log_cov is not None:
-        if log_cov.dtype != torch.float32 or log_cov.numel() != log_ratio.numel():
-            raise TypeError("log_cov must be float32 with one entry per token")
-        res.min_cov = torch.empty(S, dtype=torch.float32, device=dev)
-        res.mean_cov = torch.empty(S, dtype=torch.float32, device=dev)
-        a.log_cov, a.min_cov, a.mean_cov = _ptr(log_cov), _ptr(res.min_cov), _ptr(res.mean_cov)
-    st = lib.dvp_sequence_aggregate(ctypes.byref(a))
+    floats = log_ratio.new_empty((4 if has_cov else 2, S)).unbind(0)
+    counts = log_ratio.new_empty((2, S), dtype=torch.int32).unbind(0)
+    res = SimpleNamespace(seq_log_ratio=floats[0], min_log_ratio=floats[1], n_valid=counts[0], n_zero_weight=counts[1],
+                          veto=log_ratio.new_empty(S, dtype=torch.uint8))
+    if has_cov:
+        res.min_cov, res.mean_cov = floats[2], floats[3]
+    st = packed["dvp_sequence_aggregate"](_SEQUENCE_PACK.pack(
+        _SEQUENCE_PACK.size, 0, log_ratio.numel(), S, seq_offsets.data_ptr(), log_ratio.data_ptr(),
+        float(veto_threshold), floats[0].data_ptr(), floats[1].data_ptr(), counts[0].data_ptr(), counts[1].data_ptr(),
+        res.veto.data_ptr(), _stream(stream), _address(log_cov), floats[2].data_ptr() if has_cov else 0,
+        floats[3].data_ptr() if has_cov else 0))
     if st != DVP_OK:
         raise DvpError(st, "dvp_sequence_aggregate")
     return res
@@ -599,25 +615,19 @@ def dvp_sequence_aggregate(log_ratio: torch.Tensor, seq_offsets: torch.Tensor,
 def dvp_monitor(train_logits: torch.Tensor, infer_logits: torch.Tensor, stream=None):
     """Per-token KL(infer || train), KL(train || infer) and the two entropies over
     the full vocabulary (Sec. 6's stability metric), in nats."""
-    lib = load_library()
+    packed = load_library().packed
     _check_matrix("train_logits", train_logits)
     _check_matrix("infer_logits", infer_logits)
     if infer_logits.dtype != train_logits.dtype or infer_logits.shape != train_logits.shape:
         raise ValueError("infer_logits must match train_logits in dtype and shape")
     T, V = train_logits.shape
-    dev = train_logits.device
-    res = SimpleNamespace(**{n: torch.empty(T, dtype=torch.float32, device=dev)
-                             for n in ("kl_infer_train", "kl_train_infer", "entropy_train", "entropy_infer")})
-    a = MonitorArgs()
-    a.struct_size = ctypes.sizeof(MonitorArgs)
-    a.logits_dtype = _DTYPES[train_logits.dtype]
-    a.T, a.V = T, V
-    a.ld_train, a.ld_infer = train_logits.stride(0), infer_logits.stride(0)
-    a.train_logits, a.infer_logits = _ptr(train_logits), _ptr(infer_logits)
-    a.kl_infer_train, a.kl_train_infer = _ptr(res.kl_infer_train), _ptr(res.kl_train_infer)
-    a.entropy_train, a.entropy_infer = _ptr(res.entropy_train), _ptr(res.entropy_infer)
-    a.stream = _stream(stream)
-    st = lib.dvp_monitor(ctypes.byref(a))
+    buf = train_logits.new_empty((4, T), dtype=torch.float32)
+    rows, at, step = buf.unbind(0), buf.data_ptr(), 4 * T
+    st = packed["dvp_monitor"](_MONITOR_PACK.pack(
+        _MONITOR_PACK.size, _DTYPES[train_logits.dtype], T, V, train_logits.stride(0), infer_logits.stride(0),
+        train_logits.data_ptr(), infer_logits.data_ptr(), at, at + step, at + 2 * step, at + 3 * step,
+        _stream(stream)))
     if st != DVP_OK:
         raise DvpError(st, "dvp_monitor")
-    return res
+    return SimpleNamespace(kl_infer_train=rows[0], kl_train_infer=rows[1], entropy_train=rows[2],
+                           entropy_infer=rows[3])
