@@ -113,19 +113,6 @@ __global__ void grad_scale_kernel(const float *upstream, long long T, float fact
   }
 }
 
-// Merge the two sides: flags and the per-token log-ratio.
-__global__ void combine_sides_kernel(long long T, const float *lp_t, const float *lp_i,
-                                     const uint8_t *flags_i, uint8_t *flags, float *log_ratio) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= T) return;
-  const uint8_t ft = flags[t];
-  const bool in_t = ft & DVP_FLAG_IN_TRAIN, in_i = flags_i[t] & DVP_FLAG_IN_TRAIN;
-  flags[t] = (uint8_t)(ft | (in_i ? DVP_FLAG_IN_INFER : 0));
-  if (log_ratio)
-    log_ratio[t] = (ft & (DVP_FLAG_NO_ID | DVP_FLAG_BAD_ID)) ? __int_as_float(0x7fc00000)
-                                                             : log_ratio_of(in_t, in_i, lp_t[t], lp_i[t]);
-}
-
 namespace {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -133,7 +120,7 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 struct FusedLayout {
   long long Vp, Tp, panel;
   size_t off_scalars, off_lpt, off_lpi, off_fli, off_flt, off_wt, off_hs, off_z, off_g, off_rmax, off_rowscale,
-      off_hidscale, off_acoef, off_sort, total;
+      off_hidscale, off_acoef, total;
   long long max_pieces;
 };
 
@@ -170,7 +157,6 @@ bool fused_layout(const dvp_fused_args *a, FusedLayout *L) {
   L->off_rowscale = take((size_t)panel * 4);
   L->off_hidscale = take((size_t)panel * 4);
   L->off_acoef = take((size_t)panel * 4);
-  L->off_sort = take((size_t)panel::kSortChunk * 8);
   L->total = o;
   return true;
 }
@@ -272,7 +258,6 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
   float *row_scale = reinterpret_cast<float *>(ws + L.off_rowscale);  // [panel] factor of each row of P
   float *hid_scale = reinterpret_cast<float *>(ws + L.off_hidscale);  // [panel] the same times a power of two
   float *a_coef = reinterpret_cast<float *>(ws + L.off_acoef);        // [panel] coefficient of the 1[k = a] term
-  unsigned long long *sorted = reinterpret_cast<unsigned long long *>(ws + L.off_sort);
   const __nv_bfloat16 *hidden = static_cast<const __nv_bfloat16 *>(a->hidden);
   const __nv_bfloat16 *w = static_cast<const __nv_bfloat16 *>(a->w_vocab);
   const int T = (int)a->T, H = (int)a->H, V = (int)a->V;
@@ -300,8 +285,8 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     p.flags = fli;
     return launch_row_kernels(p, DVP_BF16, DVP_BF16, 0, s);
   };
-  // with an importance weight the training rows need the inference side first
-  if (weighted && infer_rows() != cudaSuccess) return DVP_ERR_CUDA;
+  // first: the training rows take the log-ratio (and an importance weight) from it
+  if (a->infer_logits && infer_rows() != cudaSuccess) return DVP_ERR_CUDA;
   int panel_index = 0;
   for (long long r0 = 0; r0 < a->T; r0 += L.panel, ++panel_index) {
     const int rows = (int)((a->T - r0 < L.panel) ? a->T - r0 : L.panel);
@@ -327,13 +312,16 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     p.out_t.logp_mp = lpt + r0;
     p.flags = flt + r0;
     p.bounds_status = bounds_status_word();
+    if (a->infer_logits) {
+      p.given_logp_mp_i = lpi + r0;
+      p.given_flags_i = fli + r0;
+      p.log_ratio = a->log_ratio ? a->log_ratio + r0 : nullptr;
+    }
     if (weighted) {
       p.weight_kind = (int)a->weight_kind;
       p.weight_lo = a->weight_lo;
       p.weight_hi = a->weight_hi;
       p.weight_out = a->weight_out ? a->weight_out + r0 : nullptr;
-      p.given_logp_mp_i = lpi + r0;
-      p.given_flags_i = fli + r0;
     }
     pp.row_max = rmax;
     pp.row_max_ld = L.max_pieces;
@@ -346,16 +334,32 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     pp.scale = &sc->scale;
     panel::dvp_panel_kernel<512, 2><<<(unsigned)rows, 512, 0, s>>>(pp);
     if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
-    // d_hidden[r0 : r0 + rows] = diag(c) P W, the factor applied per row in the epilogue
-    // few output tiles and a long K: two K ranges per tile fill the last wave of block pairs
-    const long long dh_tiles = ((rows + 255) / 256) * (long long)((H + 255) / 256);
-    e = gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, a->d_hidden + r0 * a->ld_dh, a->ld_dh, rows, H, V,
-                             false, 1.f, nullptr, false, &sc->status, sms, s, false, false,
-                             dh_tiles < 8LL * (sms / 2) ? 2 : 1, nullptr, 0, row_scale);
+    // d_hidden[r0 : r0 + rows] = diag(c) P W + q_t W[a_t]: the factor is applied per row and the 1[k = a] term
+    // added in fp32.  Few output tiles and a long K: each tile is computed as several K ranges, whose partial
+    // results go where the logits were (read for the last time by the row pass) and are summed in order.
+    const long long dh_tiles = ((rows + 255) / 256) * (long long)((H + 255) / 256), Hp = (H + 7) / 8 * 8;
+    const int room = (int)(L.panel * L.Vp / ((long long)rows * Hp) < 32 ? L.panel * L.Vp / ((long long)rows * Hp) : 32);
+    const int ranges = gemm::choose_ranges(dh_tiles, V, sms / 2, room > 1 ? room : 1, (double)rows * Hp * 4);
+    if (ranges > 1) {
+      e = gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, z, Hp, rows, H, V, false, 1.f, nullptr, false, &sc->status, sms,
+                               s, false, false, ranges, nullptr, 0, nullptr, rows * Hp);
+      if (e == cudaSuccess) {
+        panel::sum_ranges_kernel<<<(unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s>>>(
+            z, rows * Hp, Hp, ranges, row_scale, a->d_hidden + r0 * a->ld_dh, a->ld_dh, w, a->ld_w, p.ids, p.id_is_i32,
+            a_coef, H);
+        e = cudaGetLastError();
+      }
+    } else {
+      e = gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, a->d_hidden + r0 * a->ld_dh, a->ld_dh, rows, H, V, false, 1.f,
+                               nullptr, false, &sc->status, sms, s, false, false, 1, nullptr, 0, row_scale);
+      if (e == cudaSuccess) {
+        panel::sum_ranges_kernel<<<(unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s>>>(
+            a->d_hidden + r0 * a->ld_dh, 0, a->ld_dh, 1, nullptr, a->d_hidden + r0 * a->ld_dh, a->ld_dh, w, a->ld_w,
+            p.ids, p.id_is_i32, a_coef, H);
+        e = cudaGetLastError();
+      }
+    }
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
-    // ... + q_t W[a_t]: the 1[k = a] term in fp32
-    panel::add_sampled_rows_kernel<<<(unsigned)rows, 256, 0, s>>>(
-        a->d_hidden + r0 * a->ld_dh, a->ld_dh, w, a->ld_w, p.ids, p.id_is_i32, a_coef, H);
     // the panel's hidden rows times their factor (and 2^14 * scale / 512), transposed, in float16
     launch_transpose<__nv_bfloat16, __half>(hidden + r0 * a->ld_hidden, a->ld_hidden, hs16, L.panel, rows, H, s,
                                             hid_scale);
@@ -367,21 +371,16 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
                              s, false, true);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
     // ... + q_t hidden_t into row a_t of d_w: tokens that share a row are added in token order
-    for (int c0 = 0; c0 < rows; c0 += panel::kSortChunk) {
-      const int n = rows - c0 < panel::kSortChunk ? rows - c0 : panel::kSortChunk;
+    for (int c0 = 0; c0 < rows; c0 += panel::kIdChunk) {
+      const int n = rows - c0 < panel::kIdChunk ? rows - c0 : panel::kIdChunk;
       const void *ids_c = static_cast<const char *>(p.ids) + (long long)c0 * id_bytes;
-      panel::sort_sampled_ids_kernel<<<1, 1024, 0, s>>>(ids_c, p.id_is_i32, a_coef + c0, n, sorted);
-      panel::add_sampled_hidden_kernel<<<panel::kSortChunk, 256, 0, s>>>(
-          sorted, a_coef + c0, hidden + (r0 + c0) * a->ld_hidden, a->ld_hidden, a->d_w, a->ld_dw, H);
+      panel::add_sampled_hidden_kernel<<<(unsigned)n, 256, 0, s>>>(ids_c, p.id_is_i32, a_coef + c0, n,
+                                                                  hidden + (r0 + c0) * a->ld_hidden, a->ld_hidden,
+                                                                  a->d_w, a->ld_dw, H);
     }
     if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
   }
 
-  if (a->infer_logits) {
-    if (!weighted && infer_rows() != cudaSuccess) return DVP_ERR_CUDA;
-    combine_sides_kernel<<<(unsigned)((a->T + 255) / 256), 256, 0, s>>>(a->T, lpt, lpi, fli, flt,
-                                                                        a->log_ratio);
-  }
   return cudaGetLastError() == cudaSuccess ? DVP_OK : DVP_ERR_CUDA;
 }
 

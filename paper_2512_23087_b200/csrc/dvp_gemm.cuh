@@ -44,10 +44,11 @@ struct Params {
   int accumulate;          // C += instead of C =
   int *status;             // device word, set non-zero when a wait gives up
   int a_mn_major;          // A is stored transposed, [K, M] with M contiguous (pair kernel only)
-  int split_k;             // pair kernel: each tile's K range is cut into this many units whose
-                           // results are added to C with atomics (C zeroed or accumulated into)
+  int split_k;             // pair kernel: each tile's K range is cut into this many units (see range_stride)
   float *row_max;          // optional (pair kernel, no split, no accumulation): row_max[row * row_max_ld + tn]
   long long row_max_ld;    // = the maximum of row `row` of C over the columns of tile column tn
+  long long range_stride;  // split_k > 1: 0, the units' results are added to C with atomics (C zeroed or
+                           // accumulated into); otherwise K range i goes to C + i * range_stride (elements)
   const float *row_scale;  // optional (pair kernel): row `row` of the product is multiplied by row_scale[row]
 };
 
@@ -153,14 +154,64 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_wait_ld() {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// The registers pass through the wait: nothing may use them before it.
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                 "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                 "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
+                 "+r"(r[29])
+               :
+               : "memory");
+  asm volatile("" : "+r"(r[30]), "+r"(r[31])::"memory");
 }
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+
+// Thirty-two columns of a thread's accumulator row, times alpha, to C.  Every index is a constant: indexed
+// by a loop variable the accumulators went through local memory, half of all the bytes the epilogue stored
+// (a d_w contraction of 512 tokens x 32,000 x 1,024, which is bound by its epilogue: 68 us then).
+//   kStore  C = v     kAdd  C += v by vector reductions in L2: one addend per element and launch, so reruns
+//   are bit-identical; loads, additions and stores were 32 dependent round trips a tile
+enum class Out { kStore, kAdd };
+template <Out kOut>
+__device__ __forceinline__ void store_columns(float *c, const uint32_t (&r)[32], float alpha, int n_cols) {
+  if (n_cols >= 32) {
+#pragma unroll
+    for (int j = 0; j < 32; j += 8) {
+      float v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = alpha * __uint_as_float(r[j + e]);
+      if constexpr (kOut == Out::kStore) {
+        asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(c + j), "f"(v[0]), "f"(v[1]),
+                     "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                     : "memory");
+      } else {
+        asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(c + j), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                     "f"(v[3])
+                     : "memory");
+        asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(c + j + 4), "f"(v[4]), "f"(v[5]), "f"(v[6]),
+                     "f"(v[7])
+                     : "memory");
+      }
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      if (j < n_cols) {
+        const float v = alpha * __uint_as_float(r[j]);
+        if constexpr (kOut == Out::kStore)
+          c[j] = v;
+        else
+          atomicAdd(c + j, v);
+      }
+    }
+  }
 }
 
 struct Shared {
@@ -287,35 +338,13 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       for (int c0 = 0; c0 < kBN; c0 += 32) {
         uint32_t r[32];
         tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * kBN + c0, r);
-        tmem_wait_ld();
+        tmem_wait_ld(r);
         const int col = tn * kBN + c0;
         if (row < p.M && col < p.N) {
-          if (col + 32 <= p.N) {
-#pragma unroll
-            for (int j = 0; j < 32; j += 8) {
-              uint32_t w[8];
-              if (p.accumulate) {
-                const float4 o0 = *reinterpret_cast<const float4 *>(crow + col + j);
-                const float4 o1 = *reinterpret_cast<const float4 *>(crow + col + j + 4);
-                const float old[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
-#pragma unroll
-                for (int e = 0; e < 8; ++e)
-                  w[e] = __float_as_uint(fmaf(alpha, __uint_as_float(r[j + e]), old[e]));
-              } else {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) w[e] = __float_as_uint(alpha * __uint_as_float(r[j + e]));
-              }
-              asm volatile("st.global.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(crow + col + j),
-                           "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]),
-                           "r"(w[7])
-                           : "memory");
-            }
-          } else {
-            for (int j = 0; j < 32 && col + j < p.N; ++j) {
-              const float v = alpha * __uint_as_float(r[j]);
-              crow[col + j] = p.accumulate ? crow[col + j] + v : v;
-            }
-          }
+          if (p.accumulate)
+            store_columns<Out::kAdd>(crow + col, r, alpha, p.N - col);
+          else
+            store_columns<Out::kStore>(crow + col, r, alpha, p.N - col);
         }
       }
       tc_fence_before();
@@ -539,50 +568,42 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
       }
       tc_fence_after();
       const int row = tm * kPairBM + (int)rank * kBM + quarter * 32 + lane;
-      float *crow = p.C + (long long)row * p.ldc;
+      // a tile's K ranges meet in C by additions, or each range has a matrix of its own
+      const bool add_ranges = p.split_k > 1 && p.range_stride == 0;
+      float *crow = p.C + (long long)row * p.ldc + (long long)(unit / n_tiles) * p.range_stride;
       const float alpha = alpha_all * ((p.row_scale && row < p.M) ? p.row_scale[row] : 1.f);
       float row_hi = -__builtin_huge_valf();  // maximum of what this thread stores of its row
-#pragma unroll 1
-      for (int c0 = 0; c0 < kBN; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * kBN + c0, r);
-        tmem_wait_ld();
+      const uint32_t tmem_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * kBN;
+      // two groups of 32 columns in flight: the next is read from tensor memory while one is stored
+      uint32_t ra[32], rb[32];
+      auto emit = [&](const uint32_t (&r)[32], int c0) {
         const int col = tn * kBN + c0;
         if (p.row_max && row < p.M) {
+          if (col + 32 <= p.N) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (col + j < p.N) row_hi = fmaxf(row_hi, alpha * __uint_as_float(r[j]));
-        }
-        if (row < p.M && col < p.N) {
-          if (p.split_k > 1) {  // this unit holds a part of the sum: add it
-            for (int j = 0; j < 32 && col + j < p.N; ++j) atomicAdd(crow + col + j, alpha * __uint_as_float(r[j]));
-          } else if (col + 32 <= p.N) {
-#pragma unroll
-            for (int j = 0; j < 32; j += 8) {
-              uint32_t w[8];
-              if (p.accumulate) {
-                const float4 o0 = *reinterpret_cast<const float4 *>(crow + col + j);
-                const float4 o1 = *reinterpret_cast<const float4 *>(crow + col + j + 4);
-                const float old[8] = {o0.x, o0.y, o0.z, o0.w, o1.x, o1.y, o1.z, o1.w};
-#pragma unroll
-                for (int e = 0; e < 8; ++e)
-                  w[e] = __float_as_uint(fmaf(alpha, __uint_as_float(r[j + e]), old[e]));
-              } else {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) w[e] = __float_as_uint(alpha * __uint_as_float(r[j + e]));
-              }
-              asm volatile("st.global.v8.u32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(crow + col + j),
-                           "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]),
-                           "r"(w[7])
-                           : "memory");
-            }
+            for (int j = 0; j < 32; ++j) row_hi = fmaxf(row_hi, alpha * __uint_as_float(r[j]));
           } else {
-            for (int j = 0; j < 32 && col + j < p.N; ++j) {
-              const float v = alpha * __uint_as_float(r[j]);
-              crow[col + j] = p.accumulate ? crow[col + j] + v : v;
-            }
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (col + j < p.N) row_hi = fmaxf(row_hi, alpha * __uint_as_float(r[j]));
           }
         }
+        if (row < p.M && col < p.N) {
+          if (p.accumulate || add_ranges)
+            store_columns<Out::kAdd>(crow + col, r, alpha, p.N - col);
+          else
+            store_columns<Out::kStore>(crow + col, r, alpha, p.N - col);
+        }
+      };
+      tmem_ld32(tmem_row, ra);
+#pragma unroll 1
+      for (int c0 = 0; c0 < kBN; c0 += 64) {
+        tmem_wait_ld(ra);
+        tmem_ld32(tmem_row + c0 + 32, rb);
+        emit(ra, c0);
+        tmem_wait_ld(rb);
+        if (c0 + 64 < kBN) tmem_ld32(tmem_row + c0 + 64, ra);
+        emit(rb, c0 + 32);
       }
       if (p.row_max && row < p.M) p.row_max[(long long)row * p.row_max_ld + tn] = row_hi;
       tc_fence_before();
@@ -641,6 +662,33 @@ inline bool make_map(CUtensorMap *map, const void *base, long long rows, long lo
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The number of K ranges that a cut into `ranges` equal ones (in slices, rounded up) really has.
+inline int usable_ranges(int K, int ranges) {
+  const int slices = (K + kBK - 1) / kBK;
+  const int per = (slices + ranges - 1) / ranges;
+  return (slices + per - 1) / per;
+}
+
+// K ranges for a product of `tiles` output tiles on `pairs` pairs of blocks, at most `most`: the waves times the
+// slices of a unit, plus some 8 slices that a unit cannot overlap (its first loads and last stores), plus the
+// traffic of the partial results.  A slice takes about a third of a microsecond.  (512 x 1,024 x 32,000: 8 tiles
+// on 74 pairs took 110 us in two ranges each.)
+inline int choose_ranges(long long tiles, int K, int pairs, int most, double out_bytes) {
+  const int slices = (K + kBK - 1) / kBK;
+  int best = 1;
+  double best_cost = 1e300;
+  for (int r = 1; r <= most && slices >= 4 * r; ++r) {
+    if (usable_ranges(K, r) != r) continue;
+    const double waves = (double)((tiles * r + pairs - 1) / pairs);
+    const double cost = waves * ((slices + r - 1) / r + 8) + (r > 1 ? (r + 1) * out_bytes * 2 / 5e12 / 0.33e-6 : 0.0);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = r;
+    }
+  }
+  return best;
+}
+
 // C[M,N] (+)= alpha * A[M,K] * B[N,K]^T.  lda, ldb multiples of 8; ldc of 8; bases 16-byte
 // (A, B) and 32-byte (C) aligned.  Returns a CUDA error code; cudaErrorInvalidValue for
 // layouts it cannot take.
@@ -649,19 +697,25 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
                                   const float *alpha_dev, bool accumulate, int *status, int sm_count,
                                   cudaStream_t stream, bool single_block_tiles = false,
                                   bool a_mn_major = false, int split_k = 1, float *row_max = nullptr,
-                                  long long row_max_ld = 0, const float *row_scale = nullptr) {
+                                  long long row_max_ld = 0, const float *row_scale = nullptr,
+                                  long long range_stride = 0) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   if (lda % 8 || ldb % 8 || ldc % 8 || (uintptr_t)A % 16 || (uintptr_t)B % 16 || (uintptr_t)C % 32)
     return cudaErrorInvalidValue;
   if (a_mn_major && single_block_tiles) return cudaErrorInvalidValue;
-  // every K range of a split needs work; the split results meet in C by atomic adds
+  // every K range of a split needs work
   if (single_block_tiles || split_k < 1 || (K + kBK - 1) / kBK < 2 * split_k) split_k = 1;
+  if (range_stride != 0) {
+    if (usable_ranges(K, split_k) != split_k) return cudaErrorInvalidValue;
+  } else {
+    split_k = usable_ranges(K, split_k);
+  }
   // per-tile row maxima are those of the stored values: only where a tile is stored once, whole
   if (row_max && (single_block_tiles || split_k > 1 || accumulate)) return cudaErrorInvalidValue;
   if (row_scale && single_block_tiles) return cudaErrorInvalidValue;
   Params p{C, ldc, M, N, K, alpha, alpha_dev, accumulate ? 1 : 0, status, a_mn_major ? 1 : 0, split_k,
-           row_max, row_max_ld, row_scale};
-  if (split_k > 1 && !accumulate) {
+           row_max, row_max_ld, range_stride, row_scale};
+  if (split_k > 1 && !accumulate && range_stride == 0) {
     const cudaError_t z = cudaMemset2DAsync(C, (size_t)ldc * 4, 0, (size_t)N * 4, (size_t)M, stream);
     if (z != cudaSuccess) return z;
   }

@@ -150,9 +150,13 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_panel_kernel(const Pane
 
   if (threadIdx.x == 0) {
     finish_side(p.out_t, t, st, has_id, bad_id);
+    const bool in_i = p.given_flags_i && (p.given_flags_i[t] & DVP_FLAG_IN_TRAIN);  // of the inference rows' pass
     if (p.flags)
-      p.flags[t] = (uint8_t)((st.member ? DVP_FLAG_IN_TRAIN : 0) | (has_id ? 0 : DVP_FLAG_NO_ID) |
-                             (bad_id ? DVP_FLAG_BAD_ID : 0));
+      p.flags[t] = (uint8_t)((st.member ? DVP_FLAG_IN_TRAIN : 0) | (in_i ? DVP_FLAG_IN_INFER : 0) |
+                             (has_id ? 0 : DVP_FLAG_NO_ID) | (bad_id ? DVP_FLAG_BAD_ID : 0));
+    if (p.log_ratio)
+      p.log_ratio[t] = a < 0 ? __int_as_float(0x7fc00000)
+                             : log_ratio_of(st.member, in_i, logp_mp_of(st), p.given_logp_mp_i[t]);
     float g = p.upstream[t];
     if (p.weight_kind != DVP_WEIGHT_NONE) {
       const float w = row_weight_given(p, st, t, a >= 0);
@@ -181,70 +185,82 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_panel_kernel(const Pane
   }
 }
 
-// d_hidden[t, :] += q_t W[a_t, :]: the 1[k = a] term of the gradient row, in fp32.
-__global__ void __launch_bounds__(256) add_sampled_rows_kernel(float *d_hidden, long long ld_dh,
-                                                               const __nv_bfloat16 *w, long long ld_w,
-                                                               const void *ids, int id_is_i32, const float *a_coef,
-                                                               int H) {
-  const long long t = blockIdx.x;
-  const float q = a_coef[t];
-  if (q == 0.f) return;
-  const long long a = load_id(ids, id_is_i32, t);
-  const __nv_bfloat16 *wa = w + a * ld_w;
-  float *out = d_hidden + t * ld_dh;
-  for (int h = threadIdx.x; h < H; h += blockDim.x) out[h] = fmaf(q, __bfloat162float(wa[h]), out[h]);
-}
-
-// The tokens of a chunk (at most 4096) whose row has a gradient, sorted by (sampled id, token):
-// tokens that share a vocabulary row are then neighbours, in token order.  Keys: id << 12 | token;
-// the others sort to the end as all ones.
-constexpr int kSortChunk = 4096;
-__global__ void __launch_bounds__(1024) sort_sampled_ids_kernel(const void *ids, int id_is_i32, const float *a_coef,
-                                                                int rows, unsigned long long *sorted) {
-  __shared__ unsigned long long key[kSortChunk];
-  for (int i = threadIdx.x; i < kSortChunk; i += blockDim.x) {
-    unsigned long long k = ~0ull;
-    if (i < rows && a_coef[i] != 0.f) k = ((unsigned long long)load_id(ids, id_is_i32, i) << 12) | (unsigned)i;
-    key[i] = k;
-  }
-  __syncthreads();
-  for (int size = 2; size <= kSortChunk; size <<= 1) {  // bitonic network, ascending
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int i = threadIdx.x; i < kSortChunk / 2; i += blockDim.x) {
-        const int lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
-        const bool up = (lo & size) == 0;
-        const unsigned long long x = key[lo], y = key[hi];
-        if ((x > y) == up) {
-          key[lo] = y;
-          key[hi] = x;
-        }
-      }
-      __syncthreads();
+// d_hidden[t, :] = c_t sum_i part_i[t, :] + q_t W[a_t, :], the ranges in order: diag(c) P W from its K ranges and
+// the 1[k = a] term, in fp32.  One range: `part` may be d_hidden itself (c_t applied already: scale null).
+__global__ void __launch_bounds__(256) sum_ranges_kernel(const float *part, long long range_stride, long long ld_part,
+                                                         int ranges, const float *scale, float *d_hidden,
+                                                         long long ld_dh, const __nv_bfloat16 *w, long long ld_w,
+                                                         const void *ids, int id_is_i32, const float *a_coef, int H) {
+  const unsigned per_row = (unsigned)(H + 1023) / 1024;
+  const long long t = blockIdx.x / per_row;
+  const int h = (int)((blockIdx.x % per_row) * 1024 + threadIdx.x * 4);
+  if (h >= H) return;
+  const float q = a_coef[t], c = scale ? scale[t] : 1.f;
+  const __nv_bfloat16 *wa = q != 0.f ? w + load_id(ids, id_is_i32, t) * ld_w + h : nullptr;
+  const float *src = part + t * ld_part + h;
+  float *out = d_hidden + t * ld_dh + h;
+  if (h + 4 <= H) {  // strides are multiples of 8 elements
+    float4 acc = *reinterpret_cast<const float4 *>(src);
+    for (int i = 1; i < ranges; ++i) {
+      const float4 v = *reinterpret_cast<const float4 *>(src + i * range_stride);
+      acc.x += v.x, acc.y += v.y, acc.z += v.z, acc.w += v.w;
+    }
+    acc.x *= c, acc.y *= c, acc.z *= c, acc.w *= c;
+    if (wa) {
+      const uint2 raw = *reinterpret_cast<const uint2 *>(wa);
+      acc.x = fmaf(q, __uint_as_float(raw.x << 16), acc.x);
+      acc.y = fmaf(q, __uint_as_float(raw.x & 0xffff0000u), acc.y);
+      acc.z = fmaf(q, __uint_as_float(raw.y << 16), acc.z);
+      acc.w = fmaf(q, __uint_as_float(raw.y & 0xffff0000u), acc.w);
+    }
+    *reinterpret_cast<float4 *>(out) = acc;
+  } else {
+    for (int j = 0; h + j < H; ++j) {
+      float acc = src[j];
+      for (int i = 1; i < ranges; ++i) acc += src[i * range_stride + j];
+      acc *= c;
+      out[j] = wa ? fmaf(q, __bfloat162float(wa[j]), acc) : acc;
     }
   }
-  for (int i = threadIdx.x; i < kSortChunk; i += blockDim.x) sorted[i] = key[i];
 }
 
-// d_w[a, :] += sum over the tokens t of the chunk with a_t = a, in token order, of q_t hidden[t, :].
-// One block per sorted position; the block at the head of a run of equal ids does the run.
-__global__ void __launch_bounds__(256) add_sampled_hidden_kernel(const unsigned long long *sorted,
-                                                                 const float *a_coef, const __nv_bfloat16 *hidden,
+// d_w[a, :] += sum over the tokens t of the chunk (at most 4096) with a_t = a, in token order, of q_t hidden[t, :].
+// One block per token; the block of the first token with an id does all tokens with that id.  Each block looks
+// for its id among the others' itself: 33 MB of ids out of L2 for 4096 tokens.  (Sorting the ids took one block
+// 35 to 41 us first.)
+constexpr int kIdChunk = 4096;
+__global__ void __launch_bounds__(256) add_sampled_hidden_kernel(const void *ids, int id_is_i32, const float *a_coef,
+                                                                 int n, const __nv_bfloat16 *hidden,
                                                                  long long ld_hidden, float *d_w, long long ld_dw,
                                                                  int H) {
+  __shared__ uint32_t same[kIdChunk / 32];  // bit j: token j has this block's id
+  __shared__ int any;
   const int i = blockIdx.x;
-  const unsigned long long k = sorted[i];
-  if (k == ~0ull) return;
-  const unsigned long long a = k >> 12;
-  if (i > 0 && (sorted[i - 1] >> 12) == a) return;
-  float *out = d_w + (long long)a * ld_dw;
-  for (int h = threadIdx.x; h < H; h += blockDim.x) {
-    float acc = 0.f;
-    for (int j = i; j < kSortChunk; ++j) {
-      const unsigned long long kj = sorted[j];
-      if (kj == ~0ull || (kj >> 12) != a) break;
-      const int t = (int)(kj & 4095u);
-      acc = fmaf(a_coef[t], __bfloat162float(hidden[(long long)t * ld_hidden + h]), acc);
+  if (a_coef[i] == 0.f) return;
+  const long long a = load_id(ids, id_is_i32, i);
+  for (int k = threadIdx.x; k < kIdChunk / 32; k += blockDim.x) same[k] = 0;
+  if (threadIdx.x == 0) any = 0;
+  __syncthreads();
+  bool earlier = false;
+  for (int j = threadIdx.x; j < n; j += blockDim.x)
+    if (j != i && load_id(ids, id_is_i32, j) == a && a_coef[j] != 0.f) {
+      if (j < i) {
+        earlier = true;
+      } else {
+        atomicOr(&same[j >> 5], 1u << (j & 31));
+        any = 1;
+      }
     }
+  if (__syncthreads_or(earlier)) return;
+  float *out = d_w + a * ld_dw;
+  for (int h = threadIdx.x; h < H; h += blockDim.x) {
+    float acc = a_coef[i] * __bfloat162float(hidden[(long long)i * ld_hidden + h]);
+    if (any)
+      for (int k = i >> 5; k < (n + 31) / 32; ++k)
+        for (uint32_t m = same[k]; m; m &= m - 1) {
+          const int t = k * 32 + __ffs(m) - 1;
+          acc = fmaf(a_coef[t], __bfloat162float(hidden[(long long)t * ld_hidden + h]), acc);
+        }
     out[h] += acc;
   }
 }

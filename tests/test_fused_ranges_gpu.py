@@ -1,0 +1,37 @@
+"""d_hidden of few tokens: its few output tiles are computed as several ranges of the vocabulary, whose partial results
+are summed in order; and tokens that share a sampled id, whose rows of d_w are added in token order."""
+import pytest
+import torch
+
+from paper_2512_23087_b200 import binding, inputs
+
+import test_fused_gpu as fused
+
+pytestmark = pytest.mark.gpu
+
+
+# one tile with as many ranges as fit; H that ends inside a vector and inside a tile; V below H (no room for ranges);
+# two rows of tiles, the last of one token
+@pytest.mark.parametrize("T,H,V", [(24, 128, 9001), (33, 520, 8200), (16, 1032, 1000), (257, 264, 6000)])
+def test_ranges_of_the_vocabulary(T, H, V):
+    batch, res, want, rerun = fused._run_fused(T, H, V, 1e-3, seed=T)
+    fused._check_fused(batch, 1e-3, res, want, V, rerun=rerun)
+    again = rerun(batch.upstream)
+    assert torch.equal(again.d_hidden, res.d_hidden) and torch.equal(again.d_w, res.d_w)
+
+
+@pytest.mark.parametrize("n_ids", [1, 5])
+def test_many_tokens_of_one_id(n_ids):
+    w = inputs.WORKLOADS["c4_fused_lmhead"]
+    b = inputs.make_fused(w, seed=9, device=fused.DEV, T=300, H=256, V=2000)
+    b.ids.copy_(torch.arange(300, device=fused.DEV) % n_ids * 7)
+    r = [binding.dvp_fused_lmhead_forward_backward(b.hidden, b.w_vocab, b.ids, 0.0, b.upstream, infer_logits=b.infer)
+         for _ in range(2)]
+    torch.cuda.synchronize()
+    z = b.hidden.double() @ b.w_vocab.double().t()
+    g = -torch.softmax(z, 1) * b.upstream.double()[:, None]
+    g.scatter_add_(1, b.ids[:, None], b.upstream.double()[:, None])
+    want = g.t() @ b.hidden.double()
+    # float16 gradient panel: 2^-11 a term at most, tokens of one row add up
+    assert ((r[0].d_w.double() - want).norm(dim=1) <= 1e-3 * want.norm(dim=1) + 1e-6 * want.norm(dim=1).max()).all()
+    assert torch.equal(r[0].d_w, r[1].d_w)
