@@ -22,6 +22,7 @@
 #include "dvp_common.cuh"
 #include "dvp_gemm.cuh"
 #include "dvp_panel.cuh"
+#include "dvp_rows_two_sweeps.cuh"
 
 namespace dvp {
 
@@ -283,7 +284,8 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     p.out_t = a->infer;
     p.out_t.logp_mp = lpi;
     p.flags = fli;
-    return launch_row_kernels(p, DVP_BF16, DVP_BF16, 0, s);
+    p.bounds_status = bounds_status_word();
+    return two_sweeps::launch(p, s);
   };
   // first: the training rows take the log-ratio (and an importance weight) from it
   if (a->infer_logits && infer_rows() != cudaSuccess) return DVP_ERR_CUDA;

@@ -2,12 +2,20 @@
 // full-vocabulary inference and training policies and their entropies (the
 // stability metric of Sec. 6; the entropy Sec. 7 proposes to adapt rho to).
 //
-// Both rows are streamed together, once, in 32-byte granules.  Each thread keeps,
-// for each policy, an online log-sum-exp state in the base-2 domain extended by
-// two weighted sums: with w_k = 2^{z_k l - c},
+// Both rows are streamed together, once, in 32-byte granules, two of each in flight per thread.  Each thread
+// keeps, for each policy, an online log-sum-exp state in the base-2 domain extended by two weighted sums:
+// with w_k = 2^{z_k l - c},
 //   s = sum w_k,  a = sum w_k z_k,  b = sum w_k (z'_k - z_k),
 // from which  H = lse - a / s,  KL(train || infer) = -b/s - lse + lse',
-// KL(infer || train) = b'/s' - lse' + lse.  HBM-bound: it reads both matrices once.
+// KL(infer || train) = b'/s' - lse' + lse.
+//
+// Two logits go through one instruction (f32x2) and two granules through one check of the running maximum: with a
+// dozen instructions for every pair of logits the kernel is bound by issue and by its exponentials (0.7 of the
+// time that the bytes take), not by HBM.  T = 4096 x V = 151,936 bfloat16, 2.49 GB: 437 -> 418 us (374 at the
+// copy bandwidth); V = 50,021 with rows back to back, element by element before: 414 -> 172.  Blocks per SM:
+// bfloat16 418 / 423 at 4 / 3, float32 (2,000 x 262,144) 654 / 612.  One reference for the whole block, below the
+// maximum, would take 404 us but loses the divergence of rows with one dominant token (float32, V = 5,000,
+// heavy-tailed: relative error 3.6e-3 against 3.7e-4).
 #include "dvp_rows_impl.cuh"
 
 namespace dvp {
@@ -71,24 +79,82 @@ __device__ __forceinline__ Moments block_reduce(Moments v, float *scratch) {
   return r;
 }
 
-// Move the reference of a state to a larger maximum.
-__device__ __forceinline__ void raise(Moments &v, float new_max) {
-  if (new_max > v.m) {
-    const float cn = new_max * kLog2e;
-    const float f = ex2(v.c - cn);  // v.c = -inf at the start: factor 0
-    v.s *= f;
-    v.a *= f;
-    v.b *= f;
-    v.m = new_max;
-    v.c = cn;
+// The state of one policy over a thread's elements; the sums are pairs, of the even and the odd elements.
+struct PairMoments {
+  float m, c;
+  uint64_t s, a, b;
+
+  // Move the reference to a larger maximum.
+  __device__ __forceinline__ void raise(float new_max) {
+    if (new_max > m) {
+      const float cn = new_max * kLog2e;
+      const float f = ex2(c - cn);  // c = -inf at the start: factor 0
+      const uint64_t f2 = pack2(f, f);
+      s = mul2(s, f2);
+      a = mul2(a, f2);
+      b = mul2(b, f2);
+      m = new_max;
+      c = cn;
+    }
+  }
+  __device__ __forceinline__ void absorb(uint64_t x, uint64_t d) {
+    float w0, w1;
+    unpack2(fma2(x, pack2(kLog2e, kLog2e), pack2(-c, -c)), w0, w1);
+    const uint64_t w = pack2(ex2(w0), ex2(w1));
+    s = add2(s, w);
+    a = fma2(w, x, a);
+    b = fma2(w, d, b);
+  }
+  __device__ __forceinline__ Moments sum() const {
+    Moments r = {m, c, 0.f, 0.f, 0.f};
+    float lo, hi;
+    unpack2(s, lo, hi);
+    r.s = lo + hi;
+    unpack2(a, lo, hi);
+    r.a = lo + hi;
+    unpack2(b, lo, hi);
+    r.b = lo + hi;
+    return r;
+  }
+};
+
+template <typename TIn>
+__device__ __forceinline__ void absorb_granules(const Granule<TIn> &gt, const Granule<TIn> &gi, PairMoments &a,
+                                                PairMoments &b) {
+  constexpr int kElems = Granule<TIn>::kElems;
+  float x[kElems], y[kElems];
+  gt.get(x);
+  gi.get(y);
+#pragma unroll
+  for (int j = 0; j < kElems; j += 2) {
+    const uint64_t xx = pack2(x[j], x[j + 1]), yy = pack2(y[j], y[j + 1]);
+    const uint64_t d = fma2(xx, pack2(-1.f, -1.f), yy);
+    a.absorb(xx, d);
+    b.absorb(yy, d);
   }
 }
 
-__device__ __forceinline__ void absorb(Moments &v, float x, float d) {
-  const float w = ex2(fmaf(x, kLog2e, -v.c));
-  v.s += w;
-  v.a = fmaf(w, x, v.a);
-  v.b = fmaf(w, d, v.b);
+// The largest element of two granules.
+template <typename TIn>
+__device__ __forceinline__ float max_of(const Granule<TIn> &g, const Granule<TIn> &h) {
+  if constexpr (sizeof(TIn) == 4) {
+    return fmaxf(g.max(), h.max());
+  } else {
+    return SweepOps<TIn>::value(__hmax2(SweepOps<TIn>::tree(g), SweepOps<TIn>::tree(h)));
+  }
+}
+
+__device__ __forceinline__ void absorb_one(float x, float y, PairMoments &a, PairMoments &b) {
+  a.raise(x);
+  b.raise(y);
+  // the pair's other element: -inf has no weight, but it may not be multiplied
+  const float wa = ex2(fmaf(x, kLog2e, -a.c)), wb = ex2(fmaf(y, kLog2e, -b.c)), d = y - x;
+  a.s = add2(a.s, pack2(wa, 0.f));
+  a.a = fma2(pack2(wa, 0.f), pack2(x, 0.f), a.a);
+  a.b = fma2(pack2(wa, 0.f), pack2(d, 0.f), a.b);
+  b.s = add2(b.s, pack2(wb, 0.f));
+  b.a = fma2(pack2(wb, 0.f), pack2(y, 0.f), b.a);
+  b.b = fma2(pack2(wb, 0.f), pack2(d, 0.f), b.b);
 }
 
 struct MonitorParams {
@@ -112,83 +178,68 @@ __device__ __forceinline__ void monitor_finish(const MonitorParams &p, long long
   if (p.h_i) p.h_i[t] = (float)(lse_i - ez_i);
 }
 
+// kVector: the two rows of a token start alike against the 32-byte grid.  Granules are cut at the rows' own
+// boundaries; the elements in front of the first and behind the last whole granule are taken one per thread.
 template <typename TIn, bool kVector>
-__global__ void __launch_bounds__(256, 3) dvp_monitor_kernel(const MonitorParams p) {
+__global__ void __launch_bounds__(256, sizeof(TIn) == 2 ? 4 : 3) dvp_monitor_kernel(const MonitorParams p) {
   __shared__ float scratch[160];
   constexpr int kElems = Granule<TIn>::kElems;
   const long long t = blockIdx.x;
   const TIn *zt = reinterpret_cast<const TIn *>(p.train) + t * p.ld_train;
   const TIn *zi = reinterpret_cast<const TIn *>(p.infer) + t * p.ld_infer;
-  const int V = (int)p.V;
-  DVP_BOUNDS_BEGIN(p.bounds_status);
-  DVP_BOUNDS_SET(n_gran, (V + kElems - 1) / kElems);
-  DVP_BOUNDS_SET(V, V);
-  DVP_BOUNDS_SYNC();
-  Moments a = {kNegInf, kNegInf, 0.f, 0.f, 0.f}, b = a;
+  const int V = (int)p.V, tid = (int)threadIdx.x, n_thr = (int)blockDim.x;
+  PairMoments a = {kNegInf, kNegInf, 0, 0, 0}, b = a;
   if constexpr (kVector) {
-    // whole granules in the loop; the elements behind the last whole granule one per thread after
-    // it, so that the loop carries no element-wise code for a ragged granule
-    const int n_full = V / kElems;
-    for (int g = threadIdx.x; g < n_full; g += 2 * blockDim.x) {
-      const int g2 = g + blockDim.x;
-      Granule<TIn> ta, ia, tb, ib;  // two granules of each row in flight
+    const int mis = (int)(((uintptr_t)zt & 31u) / sizeof(TIn));
+    const int head = min(V, mis ? kElems - mis : 0), n_full = (V - head) / kElems;
+    DVP_BOUNDS_BEGIN(p.bounds_status);
+    DVP_BOUNDS_SET(n_gran, n_full);
+    DVP_BOUNDS_SET(V, (long long)n_full * kElems);
+    DVP_BOUNDS_SYNC();
+    const TIn *bt = zt + head, *bi = zi + head;
+    for (int g = tid; g < n_full; g += 2 * n_thr) {
+      Granule<TIn> t0, i0, t1, i1;
+      const int g1 = g + n_thr;
       if (!DVP_IN((long long)g * kElems + kElems - 1, V, DVP_OOB_GLOBAL)) break;
-      ta.load(zt + (size_t)g * kElems);
-      ia.load(zi + (size_t)g * kElems);
-      const bool second = g2 < n_full && DVP_IN((long long)g2 * kElems + kElems - 1, V, DVP_OOB_GLOBAL);
-      if (second) {
-        tb.load(zt + (size_t)g2 * kElems);
-        ib.load(zi + (size_t)g2 * kElems);
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (h == 1 && !second) break;
-        const Granule<TIn> &gt = h ? tb : ta, &gi = h ? ib : ia;
-        float x[kElems], y[kElems];
-        gt.get(x);
-        gi.get(y);
-        raise(a, gt.max());
-        raise(b, gi.max());
-#pragma unroll
-        for (int j = 0; j < kElems; ++j) {
-          const float d = y[j] - x[j];
-          absorb(a, x[j], d);
-          absorb(b, y[j], d);
-        }
-      }
+      const bool second = g1 < n_full && DVP_IN((long long)g1 * kElems + kElems - 1, V, DVP_OOB_GLOBAL);
+      t0.load(bt + (size_t)g * kElems);
+      i0.load(bi + (size_t)g * kElems);
+      t1.load(bt + (size_t)(second ? g1 : g) * kElems);
+      i1.load(bi + (size_t)(second ? g1 : g) * kElems);
+      a.raise(max_of<TIn>(t0, t1));
+      b.raise(max_of<TIn>(i0, i1));
+      absorb_granules<TIn>(t0, i0, a, b);
+      if (second) absorb_granules<TIn>(t1, i1, a, b);
     }
-    const int k_tail = n_full * kElems + (int)threadIdx.x;
-    if (k_tail < V) {
-      const float x = Storage<TIn>::widen(zt[k_tail]), y = Storage<TIn>::widen(zi[k_tail]);
-      raise(a, x);
-      raise(b, y);
-      absorb(a, x, y - x);
-      absorb(b, y, y - x);
-    }
+    const int k = tid < head ? tid : tid + n_full * kElems;  // fewer than 64 of them
+    if (k < V) absorb_one(Storage<TIn>::widen(zt[k]), Storage<TIn>::widen(zi[k]), a, b);
   } else {
     float mt = kNegInf, mi = kNegInf;
-    for (long long k = threadIdx.x; k < p.V; k += blockDim.x) {
+    for (long long k = tid; k < p.V; k += n_thr) {
       mt = fmaxf(mt, Storage<TIn>::widen(zt[k]));
       mi = fmaxf(mi, Storage<TIn>::widen(zi[k]));
     }
-    raise(a, mt);
-    raise(b, mi);
-    for (long long k = threadIdx.x; k < p.V; k += blockDim.x) {
-      const float x = Storage<TIn>::widen(zt[k]), y = Storage<TIn>::widen(zi[k]);
-      absorb(a, x, y - x);
-      absorb(b, y, y - x);
-    }
+    a.raise(mt);
+    b.raise(mi);
+    for (long long k = tid; k < p.V; k += n_thr)
+      absorb_one(Storage<TIn>::widen(zt[k]), Storage<TIn>::widen(zi[k]), a, b);
   }
-  const Moments ra = block_reduce(a, scratch);
-  const Moments rb = block_reduce(b, scratch);
+  const Moments ra = block_reduce(a.sum(), scratch);
+  const Moments rb = block_reduce(b.sum(), scratch);
   if (threadIdx.x == 0) monitor_finish(p, t, ra, rb);
 }
 
 template <typename TIn>
 static cudaError_t launch_monitor(const MonitorParams &p, cudaStream_t s) {
-  const bool vec = aligned32(p.train, p.ld_train, sizeof(TIn)) && aligned32(p.infer, p.ld_infer, sizeof(TIn));
-  if (vec)
-    dvp_monitor_kernel<TIn, true><<<(unsigned)p.T, 256, 0, s>>>(p);
+  const long long elem = sizeof(TIn);
+  const bool alike = ((long long)((uintptr_t)p.train % 32) - (long long)((uintptr_t)p.infer % 32)) % 32 == 0 &&
+                     (p.T == 1 || (p.ld_train - p.ld_infer) * elem % 32 == 0);
+  // some 16 granules of each row a thread, as in the row kernels
+  int threads = 64;
+  while (threads < 256 && 16LL * threads < p.V * elem / 32) threads *= 2;
+  while (threads < 256 && 2 * p.T * threads <= 148 * 1024) threads *= 2;
+  if (alike)
+    dvp_monitor_kernel<TIn, true><<<(unsigned)p.T, threads, 0, s>>>(p);
   else
     dvp_monitor_kernel<TIn, false><<<(unsigned)p.T, 256, 0, s>>>(p);
   return cudaGetLastError();

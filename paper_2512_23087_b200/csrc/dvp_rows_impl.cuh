@@ -685,7 +685,8 @@ __device__ __forceinline__ HotList build_hot_list(const uint32_t *bound, int n_s
 // Sweep 1 over (a part of) a row.
 //
 // The first guess of the maximum is the largest of `cand` (a value of the row: the sampled token's, which is
-// the maximum in most rows) and of what the first step loaded.  The block's threads exchange their maxima
+// the maximum in most rows) and of what the first two steps loaded (of the first one alone: T = 8192 x
+// V = 151,936 bfloat16 forward 892 against 864 us).  The block's threads exchange their maxima
 // every kSyncSteps steps: a larger one becomes the guess, and the masked sum starts again from there
 // (`first`).  All of it happens at fixed places, so that reruns are bit-identical.  `hole`: the granule
 // that reads as -inf (the sampled token's; its bound says that it can hold anything); xe: a value outside the
@@ -712,7 +713,10 @@ __device__ __forceinline__ void row_sweep1(const RowView<TIn> &v, int hole, floa
     if (second) s1.template load_block<kBlk>(row, n_full, step + 1);
     if (step == hole_step) s0.template punch<kBlk>(step, hole);
     if (step % kSyncSteps == 0) {
-      if (step == 0) (void)SweepOps<TIn>::bounds(s0, sw.mx);
+      if (step == 0) {
+        (void)SweepOps<TIn>::bounds(s0, sw.mx);
+        if (second) (void)SweepOps<TIn>::bounds(s1, sw.mx);
+      }
       const float m = red.max(SweepOps<TIn>::value(sw.mx));
       if (m > sw.guess) {
         if (step > 0 && m - sw.guess > kWide) sw.wide = true;
@@ -1376,7 +1380,8 @@ static cudaError_t launch_rows_cs(const RowParams &p, int threads, int n_steps, 
 // against 21.5 at 128 and 29.7 at 64), then more blocks a row (V = 151,936 bfloat16, 1 / 2 / 4 / 8 blocks:
 // T = 16 forward 36 / 28 / 21 / 19; T = 64 forward 38 / 32 / 28 / 34; T = 128 with the gradient
 // 65 / 50 / 48 / 60; T = 512 130 / 126 / 134 / 192; V = 50,000, T = 100: 30 / 24 / 28 / 38).  Blocks that share
-// a row need at least a step and a half of it each (V = 20,000: 13 / 15).
+// a row need at least a step and a half of it each (V = 20,000: 13 / 15), four steps where the chip is full
+// without them (T = 512, V = 32,000, one matrix: 26 / 31).
 struct RowShape {
   int threads, log_parts;
 };
@@ -1388,8 +1393,9 @@ static inline RowShape choose_shape(long long rows, long long n_gran, int most) 
   while (s.log_parts < 3) {
     const int lp = s.log_parts + 1;
     const long long per = n_gran >> lp, total = (rows << lp) * s.threads;
-    const bool fits = lp == 1 ? total <= 4 * resident
-                              : total <= resident || (lp == 2 && total <= 2 * resident && per >= 8 * s.threads);
+    const bool fits = total <= resident || (per >= 8 * s.threads && total <= (lp == 1   ? 4 * resident
+                                                                             : lp == 2 ? 2 * resident
+                                                                                       : resident));
     if (per < 3 * s.threads || !fits) break;
     s.log_parts = lp;
   }

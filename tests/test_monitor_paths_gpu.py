@@ -1,0 +1,40 @@
+"""The monitoring kernel on rows that start anywhere, and on rows with one value far above all others."""
+import pytest
+import torch
+
+from paper_2512_23087_b200 import binding
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _check(train, infer):
+    r = binding.dvp_monitor(train, infer)
+    torch.cuda.synchronize()
+    a, q = torch.log_softmax(train.double(), 1), torch.log_softmax(infer.double(), 1)
+    for got, want in ((r.kl_infer_train, (q.exp() * (q - a)).sum(1)), (r.kl_train_infer, (a.exp() * (a - q)).sum(1)),
+                      (r.entropy_train, -(a.exp() * a).sum(1)), (r.entropy_infer, -(q.exp() * q).sum(1))):
+        # float32 sums of terms of the logits' magnitude (at most 201)
+        assert (got.double() - want).abs().max().item() <= 2e-5 + 201 * 2.0 ** -20
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("V,pad_t,pad_i,off", [(5, 0, 0, 0), (31, 0, 0, 1), (1003, 0, 0, 3), (4099, 1, 1, 0),
+                                               (4099, 0, 2, 0), (50021, 0, 0, 0)])
+def test_rows_that_start_anywhere(V, pad_t, pad_i, off, dtype):
+    g = torch.Generator(device=DEV).manual_seed(V)
+    T = 7
+    z = torch.randn(T, V, generator=g, device=DEV) * 2
+    place = lambda x, ld: torch.full((off + T * ld,), 3e4, device=DEV, dtype=dtype)[off:].view(T, ld)[:, :V].copy_(x)
+    _check(place(z, V + pad_t), place(z + 0.1 * torch.randn(T, V, generator=g, device=DEV), V + pad_i))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_one_value_far_above_the_others(dtype):
+    g = torch.Generator(device=DEV).manual_seed(1)
+    z = torch.randn(4, 40003, generator=g, device=DEV)
+    for t, k in enumerate((0, 20000, 39999, 40002)):
+        z[t, k] = 200.0
+    zi = z.clone()
+    zi[1, 5] = 201.0
+    _check(z.to(dtype), zi.to(dtype))
