@@ -105,6 +105,30 @@ __device__ __forceinline__ void st_stream8(void *p, uint2 v) {
   asm volatile("st.global.cs.v2.u32 [%0], {%1,%2};" ::"l"(p), "r"(v.x), "r"(v.y) : "memory");
 }
 
+// ---- launches that overlap the end of the one before ------------------------------
+// A kernel launched by launch_after may begin while the previous kernel of the stream ends; it waits for that
+// kernel, and with it for all before, at begin_after, before it touches memory.  Kernels that call begin_after may
+// be launched in the ordinary way too.
+__device__ __forceinline__ void begin_after() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... Params, typename... Args>
+static cudaError_t launch_after(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem,
+                                cudaStream_t stream, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.blockDim = dim3(block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // ---- storage types ---------------------------------------------------------
 
 template <typename T>

@@ -34,7 +34,8 @@ __global__ void __launch_bounds__(256)
 transpose_convert_kernel(const TIn *in, long long ld_in, TOut *out, long long ld_out, int R, int C,
                          int vec_ok, const float *row_scale) {
   __shared__ TOut tile[64][66];
-  const int c0 = blockIdx.x * 64, r0 = blockIdx.y * 64;
+  begin_after();
+  const int per_row = (C + 63) / 64, c0 = (int)(blockIdx.x % per_row) * 64, r0 = (int)(blockIdx.x / per_row) * 64;
   const int tid = threadIdx.x;
   // load: 64 rows x 8 vectors of 8 elements, two vectors per thread
 #pragma unroll
@@ -79,8 +80,8 @@ template <typename TIn, typename TOut>
 static void launch_transpose(const TIn *in, long long ld_in, TOut *out, long long ld_out, int R, int C,
                              cudaStream_t s, const float *row_scale = nullptr) {
   const int vec_ok = ld_in % 8 == 0 && ld_out % 8 == 0 && (uintptr_t)in % 16 == 0 && (uintptr_t)out % 16 == 0;
-  transpose_convert_kernel<TIn, TOut>
-      <<<dim3((C + 63) / 64, (R + 63) / 64), 256, 0, s>>>(in, ld_in, out, ld_out, R, C, vec_ok, row_scale);
+  (void)launch_after(transpose_convert_kernel<TIn, TOut>, (unsigned)(((C + 63) / 64) * (long long)((R + 63) / 64)), 256, 0,
+                     s, in, ld_in, out, ld_out, R, C, vec_ok, row_scale);
 }
 
 struct FusedScalars {
@@ -297,7 +298,7 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     // then knows the threshold before it reads the panel
     cudaError_t e = gemm::launch_gemm_tn(hidden + r0 * a->ld_hidden, a->ld_hidden, w, a->ld_w, z, L.Vp,
                                          rows, V, H, true, 1.f, nullptr, false, &sc->status, sms, s, false,
-                                         false, 1, rmax, L.max_pieces);
+                                         false, 1, rmax, L.max_pieces, nullptr, 0, true);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
     // rows of the panel, one sweep: statistics, and the gradient panel up to a factor per row
     panel::PanelParams pp{};
@@ -334,8 +335,7 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     pp.hid_scale = hid_scale;
     pp.a_coef = a_coef;
     pp.scale = &sc->scale;
-    panel::dvp_panel_kernel<512, 2><<<(unsigned)rows, 512, 0, s>>>(pp);
-    if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
+    if (launch_after(panel::dvp_panel_kernel<512, 2>, (unsigned)rows, 512, 0, s, pp) != cudaSuccess) return DVP_ERR_CUDA;
     // d_hidden[r0 : r0 + rows] = diag(c) P W + q_t W[a_t]: the factor is applied per row and the 1[k = a] term
     // added in fp32.  Few output tiles and a long K: each tile is computed as several K ranges, whose partial
     // results go where the logits were (read for the last time by the row pass) and are summed in order.
@@ -344,21 +344,19 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     const int ranges = gemm::choose_ranges(dh_tiles, V, sms / 2, room > 1 ? room : 1, (double)rows * Hp * 4);
     if (ranges > 1) {
       e = gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, z, Hp, rows, H, V, false, 1.f, nullptr, false, &sc->status, sms,
-                               s, false, false, ranges, nullptr, 0, nullptr, rows * Hp);
+                               s, false, false, ranges, nullptr, 0, nullptr, rows * Hp, true);
       if (e == cudaSuccess) {
-        panel::sum_ranges_kernel<<<(unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s>>>(
+        e = launch_after(panel::sum_ranges_kernel, (unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s,
             z, rows * Hp, Hp, ranges, row_scale, a->d_hidden + r0 * a->ld_dh, a->ld_dh, w, a->ld_w, p.ids, p.id_is_i32,
             a_coef, H);
-        e = cudaGetLastError();
       }
     } else {
       e = gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, a->d_hidden + r0 * a->ld_dh, a->ld_dh, rows, H, V, false, 1.f,
-                               nullptr, false, &sc->status, sms, s, false, false, 1, nullptr, 0, row_scale);
+                               nullptr, false, &sc->status, sms, s, false, false, 1, nullptr, 0, row_scale, 0, true);
       if (e == cudaSuccess) {
-        panel::sum_ranges_kernel<<<(unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s>>>(
+        e = launch_after(panel::sum_ranges_kernel, (unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s,
             a->d_hidden + r0 * a->ld_dh, 0, a->ld_dh, 1, nullptr, a->d_hidden + r0 * a->ld_dh, a->ld_dh, w, a->ld_w,
             p.ids, p.id_is_i32, a_coef, H);
-        e = cudaGetLastError();
       }
     }
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
@@ -370,15 +368,14 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     // contiguous, as the transposed (MN-major) A operand of the contraction
     e = gemm::launch_gemm_tn(p16, L.Vp, hs16, L.panel, a->d_w, a->ld_dw, V, H, rows, false, 1.f / 32.f,
                              &sc->inv_scale, panel_index > 0 || a->accumulate_dw != 0, &sc->status, sms,
-                             s, false, true);
+                             s, false, true, 1, nullptr, 0, nullptr, 0, true);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
     // ... + q_t hidden_t into row a_t of d_w: tokens that share a row are added in token order
     for (int c0 = 0; c0 < rows; c0 += panel::kIdChunk) {
       const int n = rows - c0 < panel::kIdChunk ? rows - c0 : panel::kIdChunk;
       const void *ids_c = static_cast<const char *>(p.ids) + (long long)c0 * id_bytes;
-      panel::add_sampled_hidden_kernel<<<(unsigned)n, 256, 0, s>>>(ids_c, p.id_is_i32, a_coef + c0, n,
-                                                                  hidden + (r0 + c0) * a->ld_hidden, a->ld_hidden,
-                                                                  a->d_w, a->ld_dw, H);
+      (void)launch_after(panel::add_sampled_hidden_kernel, (unsigned)n, 256, 0, s, ids_c, p.id_is_i32, a_coef + c0, n,
+                         hidden + (r0 + c0) * a->ld_hidden, a->ld_hidden, a->d_w, a->ld_dw, H);
     }
     if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
   }

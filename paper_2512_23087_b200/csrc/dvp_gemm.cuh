@@ -19,6 +19,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "dvp_common.cuh"
+
 namespace dvp {
 namespace gemm {
 
@@ -478,6 +480,7 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   tc_fence_before();
   cluster_barrier();  // barriers of both blocks are initialised before anyone signals them
   tc_fence_after();
+  begin_after();
   const uint32_t tmem_base = sh->tmem_base;
   volatile int *abort_flag = &sh->abort_flag;
 
@@ -698,7 +701,7 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
                                   cudaStream_t stream, bool single_block_tiles = false,
                                   bool a_mn_major = false, int split_k = 1, float *row_max = nullptr,
                                   long long row_max_ld = 0, const float *row_scale = nullptr,
-                                  long long range_stride = 0) {
+                                  long long range_stride = 0, bool after = false) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   if (lda % 8 || ldb % 8 || ldc % 8 || (uintptr_t)A % 16 || (uintptr_t)B % 16 || (uintptr_t)C % 32)
     return cudaErrorInvalidValue;
@@ -736,13 +739,15 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = kSmemBytes2;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_after
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = after ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, gemm_tn_pair_kernel, map_a, map_b, p, is_bf16 ? 1u : 0u);
   }
   if (!make_map(&map_a, A, M, K, lda, kBM, is_bf16) || !make_map(&map_b, B, N, K, ldb, kBN, is_bf16))

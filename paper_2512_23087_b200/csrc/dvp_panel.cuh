@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_panel_kernel(const Pane
   __shared__ float scratch[96];
   const RowParams &p = pp.row;
   constexpr int kElems = 8, kStage = 2;
+  begin_after();
   const long long t = blockIdx.x;
   DVP_BOUNDS_BEGIN(p.bounds_status);
   DVP_BOUNDS_SET(n_gran, (p.V + kElems - 1) / kElems);
@@ -191,6 +192,7 @@ __global__ void __launch_bounds__(256) sum_ranges_kernel(const float *part, long
                                                          int ranges, const float *scale, float *d_hidden,
                                                          long long ld_dh, const __nv_bfloat16 *w, long long ld_w,
                                                          const void *ids, int id_is_i32, const float *a_coef, int H) {
+  begin_after();
   const unsigned per_row = (unsigned)(H + 1023) / 1024;
   const long long t = blockIdx.x / per_row;
   const int h = (int)((blockIdx.x % per_row) * 1024 + threadIdx.x * 4);
@@ -236,6 +238,7 @@ __global__ void __launch_bounds__(256) add_sampled_hidden_kernel(const void *ids
   __shared__ uint32_t same[kIdChunk / 32];  // bit j: token j has this block's id
   __shared__ int any;
   const int i = blockIdx.x;
+  begin_after();
   if (a_coef[i] == 0.f) return;
   const long long a = load_id(ids, id_is_i32, i);
   for (int k = threadIdx.x; k < kIdChunk / 32; k += blockDim.x) same[k] = 0;

@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(kBlk, 1024 / kBlk) dvp_two_sweeps_kernel(const
   float *scratch = smem;                                             // 96 floats
   uint16_t *hot_smem = reinterpret_cast<uint16_t *>(smem + 96);      // kHotCap per warp
   uint32_t *bound = reinterpret_cast<uint32_t *>(smem + 96 + (kBlk / 32) * kHotCap / 2);
+  begin_after();
   const long long t = blockIdx.x;
   const long long id = p.ids ? load_id(p.ids, p.id_is_i32, t) : -1;
   const bool has_id = id >= 0, bad_id = id >= p.V;
@@ -168,8 +169,7 @@ static cudaError_t launch_blk(const RowParams &p, size_t smem, cudaStream_t s) {
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  k<<<(unsigned)p.T, kBlk, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_after(k, (unsigned)p.T, kBlk, smem, s, p);
 }
 
 static inline cudaError_t launch(const RowParams &p, cudaStream_t s) {
