@@ -106,12 +106,18 @@ __device__ __forceinline__ void st_stream8(void *p, uint2 v) {
 }
 
 // ---- launches that overlap the end of the one before ------------------------------
-// A kernel launched by launch_after may begin while the previous kernel of the stream ends; it waits for that
-// kernel, and with it for all before, at begin_after, before it touches memory.  Kernels that call begin_after may
-// be launched in the ordinary way too.
-__device__ __forceinline__ void begin_after() {
+// A kernel launched by launch_after may begin while the previous kernel of the stream ends.  It waits for that
+// kernel, and with it for all before, in begin_after, before it touches memory; only then may the next one begin, so
+// that a kernel that begins finds everything before its predecessor complete.  A kernel that needs nothing of its
+// predecessor (and overwrites nothing that it reads) is `early`: it works first and waits in end_after, so that
+// whoever waits for it waits for both.  One thread of each block has to call end_after.  Kernels with these calls
+// may be launched in the ordinary way too.
+__device__ __forceinline__ void begin_after(bool early = false) {
+  if (!early) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void end_after(bool early) {
+  if (early) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 template <typename... Params, typename... Args>
 static cudaError_t launch_after(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem,

@@ -32,9 +32,9 @@ namespace dvp {
 template <typename TIn, typename TOut>
 __global__ void __launch_bounds__(256)
 transpose_convert_kernel(const TIn *in, long long ld_in, TOut *out, long long ld_out, int R, int C,
-                         int vec_ok, const float *row_scale) {
+                         int vec_ok, const float *row_scale, bool early) {
   __shared__ TOut tile[64][66];
-  begin_after();
+  begin_after(early);
   const int per_row = (C + 63) / 64, c0 = (int)(blockIdx.x % per_row) * 64, r0 = (int)(blockIdx.x / per_row) * 64;
   const int tid = threadIdx.x;
   // load: 64 rows x 8 vectors of 8 elements, two vectors per thread
@@ -74,6 +74,7 @@ transpose_convert_kernel(const TIn *in, long long ld_in, TOut *out, long long ld
       for (int j = 0; j < 8 && r + j < R; ++j) dst[j] = e[j];
     }
   }
+  if (tid == 0) end_after(early);
 }
 
 template <typename TIn, typename TOut>
@@ -81,7 +82,7 @@ static void launch_transpose(const TIn *in, long long ld_in, TOut *out, long lon
                              cudaStream_t s, const float *row_scale = nullptr) {
   const int vec_ok = ld_in % 8 == 0 && ld_out % 8 == 0 && (uintptr_t)in % 16 == 0 && (uintptr_t)out % 16 == 0;
   (void)launch_after(transpose_convert_kernel<TIn, TOut>, (unsigned)(((C + 63) / 64) * (long long)((R + 63) / 64)), 256, 0,
-                     s, in, ld_in, out, ld_out, R, C, vec_ok, row_scale);
+                     s, in, ld_in, out, ld_out, R, C, vec_ok, row_scale, row_scale == nullptr);
 }
 
 struct FusedScalars {
@@ -295,10 +296,11 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     const int rows = (int)((a->T - r0 < L.panel) ? a->T - r0 : L.panel);
     // logits of the panel: z = hidden[r0 : r0 + rows] x W^T (bf16 operands, fp32 accumulate)
     // its epilogue also leaves each row's maximum, one piece per tile column: the panel's row pass
-    // then knows the threshold before it reads the panel
+    // then knows the threshold before it reads the panel.  Early: the launch before it is the inference rows' pass
+    // or, from the second panel on, the last of d_w's, when nobody reads z or the maxima any more
     cudaError_t e = gemm::launch_gemm_tn(hidden + r0 * a->ld_hidden, a->ld_hidden, w, a->ld_w, z, L.Vp,
                                          rows, V, H, true, 1.f, nullptr, false, &sc->status, sms, s, false,
-                                         false, 1, rmax, L.max_pieces, nullptr, 0, true);
+                                         false, 1, rmax, L.max_pieces, nullptr, 0, gemm::Order::kEarly);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
     // rows of the panel, one sweep: statistics, and the gradient panel up to a factor per row
     panel::PanelParams pp{};
@@ -336,39 +338,33 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     pp.a_coef = a_coef;
     pp.scale = &sc->scale;
     if (launch_after(panel::dvp_panel_kernel<512, 2>, (unsigned)rows, 512, 0, s, pp) != cudaSuccess) return DVP_ERR_CUDA;
+    // the panel's hidden rows times their factor (and 2^14 * scale / 512), transposed, in float16
+    launch_transpose<__nv_bfloat16, __half>(hidden + r0 * a->ld_hidden, a->ld_hidden, hs16, L.panel, rows, H, s,
+                                            hid_scale);
+    if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
     // d_hidden[r0 : r0 + rows] = diag(c) P W + q_t W[a_t]: the factor is applied per row and the 1[k = a] term
     // added in fp32.  Few output tiles and a long K: each tile is computed as several K ranges, whose partial
     // results go where the logits were (read for the last time by the row pass) and are summed in order.
     const long long dh_tiles = ((rows + 255) / 256) * (long long)((H + 255) / 256), Hp = (H + 7) / 8 * 8;
     const int room = (int)(L.panel * L.Vp / ((long long)rows * Hp) < 32 ? L.panel * L.Vp / ((long long)rows * Hp) : 32);
     const int ranges = gemm::choose_ranges(dh_tiles, V, sms / 2, room > 1 ? room : 1, (double)rows * Hp * 4);
-    if (ranges > 1) {
-      e = gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, z, Hp, rows, H, V, false, 1.f, nullptr, false, &sc->status, sms,
-                               s, false, false, ranges, nullptr, 0, nullptr, rows * Hp, true);
-      if (e == cudaSuccess) {
-        e = launch_after(panel::sum_ranges_kernel, (unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s,
-            z, rows * Hp, Hp, ranges, row_scale, a->d_hidden + r0 * a->ld_dh, a->ld_dh, w, a->ld_w, p.ids, p.id_is_i32,
-            a_coef, H);
-      }
-    } else {
-      e = gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, a->d_hidden + r0 * a->ld_dh, a->ld_dh, rows, H, V, false, 1.f,
-                               nullptr, false, &sc->status, sms, s, false, false, 1, nullptr, 0, row_scale, 0, true);
-      if (e == cudaSuccess) {
-        e = launch_after(panel::sum_ranges_kernel, (unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s,
-            a->d_hidden + r0 * a->ld_dh, 0, a->ld_dh, 1, nullptr, a->d_hidden + r0 * a->ld_dh, a->ld_dh, w, a->ld_w,
-            p.ids, p.id_is_i32, a_coef, H);
-      }
-    }
+    float *dh = a->d_hidden + r0 * a->ld_dh;
+    e = ranges > 1 ? gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, z, Hp, rows, H, V, false, 1.f, nullptr, false,
+                                          &sc->status, sms, s, false, false, ranges, nullptr, 0, nullptr, rows * Hp,
+                                          gemm::Order::kAfter)
+                   : gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, dh, a->ld_dh, rows, H, V, false, 1.f, nullptr, false,
+                                          &sc->status, sms, s, false, false, 1, nullptr, 0, row_scale, 0,
+                                          gemm::Order::kAfter);
+    if (e == cudaSuccess)
+      e = launch_after(panel::sum_ranges_kernel, (unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s,
+                       ranges > 1 ? z : dh, rows * Hp, ranges > 1 ? Hp : a->ld_dh, ranges,
+                       ranges > 1 ? row_scale : nullptr, dh, a->ld_dh, w, a->ld_w, p.ids, p.id_is_i32, a_coef, H);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
-    // the panel's hidden rows times their factor (and 2^14 * scale / 512), transposed, in float16
-    launch_transpose<__nv_bfloat16, __half>(hidden + r0 * a->ld_hidden, a->ld_hidden, hs16, L.panel, rows, H, s,
-                                            hid_scale);
-    if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
     // d_w (+)= P^T x (scaled hidden rows) * 512 / (2^14 scale): P is read as it lies, [rows, V] with V
-    // contiguous, as the transposed (MN-major) A operand of the contraction
+    // contiguous, as the transposed (MN-major) A operand of the contraction; it needs nothing of sum_ranges_kernel
     e = gemm::launch_gemm_tn(p16, L.Vp, hs16, L.panel, a->d_w, a->ld_dw, V, H, rows, false, 1.f / 32.f,
                              &sc->inv_scale, panel_index > 0 || a->accumulate_dw != 0, &sc->status, sms,
-                             s, false, true, 1, nullptr, 0, nullptr, 0, true);
+                             s, false, true, 1, nullptr, 0, nullptr, 0, gemm::Order::kEarly);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
     // ... + q_t hidden_t into row a_t of d_w: tokens that share a row are added in token order
     for (int c0 = 0; c0 < rows; c0 += panel::kIdChunk) {

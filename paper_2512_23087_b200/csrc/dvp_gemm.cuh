@@ -51,6 +51,7 @@ struct Params {
   long long row_max_ld;    // = the maximum of row `row` of C over the columns of tile column tn
   long long range_stride;  // split_k > 1: 0, the units' results are added to C with atomics (C zeroed or
                            // accumulated into); otherwise K range i goes to C + i * range_stride (elements)
+  int early;               // pair kernel: see begin_after
   const float *row_scale;  // optional (pair kernel): row `row` of the product is multiplied by row_scale[row]
 };
 
@@ -480,7 +481,7 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   tc_fence_before();
   cluster_barrier();  // barriers of both blocks are initialised before anyone signals them
   tc_fence_after();
-  begin_after();
+  begin_after(p.early != 0);
   const uint32_t tmem_base = sh->tmem_base;
   volatile int *abort_flag = &sh->abort_flag;
 
@@ -622,6 +623,7 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     for (int i = 0; i < 2000; ++i) __nanosleep(500);
   }
   cluster_barrier();
+  if (threadIdx.x == 0) end_after(p.early != 0);
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols)
@@ -692,6 +694,10 @@ inline int choose_ranges(long long tiles, int K, int pairs, int most, double out
   return best;
 }
 
+// How the launch follows the one before: in the ordinary way; overlapping its end (launch_after); the same without
+// needing its results.
+enum class Order { kAlone, kAfter, kEarly };
+
 // C[M,N] (+)= alpha * A[M,K] * B[N,K]^T.  lda, ldb multiples of 8; ldc of 8; bases 16-byte
 // (A, B) and 32-byte (C) aligned.  Returns a CUDA error code; cudaErrorInvalidValue for
 // layouts it cannot take.
@@ -701,7 +707,7 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
                                   cudaStream_t stream, bool single_block_tiles = false,
                                   bool a_mn_major = false, int split_k = 1, float *row_max = nullptr,
                                   long long row_max_ld = 0, const float *row_scale = nullptr,
-                                  long long range_stride = 0, bool after = false) {
+                                  long long range_stride = 0, Order order = Order::kAlone) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   if (lda % 8 || ldb % 8 || ldc % 8 || (uintptr_t)A % 16 || (uintptr_t)B % 16 || (uintptr_t)C % 32)
     return cudaErrorInvalidValue;
@@ -717,7 +723,7 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
   if (row_max && (single_block_tiles || split_k > 1 || accumulate)) return cudaErrorInvalidValue;
   if (row_scale && single_block_tiles) return cudaErrorInvalidValue;
   Params p{C, ldc, M, N, K, alpha, alpha_dev, accumulate ? 1 : 0, status, a_mn_major ? 1 : 0, split_k,
-           row_max, row_max_ld, range_stride, row_scale};
+           row_max, row_max_ld, range_stride, order == Order::kEarly ? 1 : 0, row_scale};
   if (split_k > 1 && !accumulate && range_stride == 0) {
     const cudaError_t z = cudaMemset2DAsync(C, (size_t)ldc * 4, 0, (size_t)N * 4, (size_t)M, stream);
     if (z != cudaSuccess) return z;
@@ -747,7 +753,7 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_after
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = after ? 2 : 1;
+    cfg.numAttrs = order != Order::kAlone ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, gemm_tn_pair_kernel, map_a, map_b, p, is_bf16 ? 1u : 0u);
   }
   if (!make_map(&map_a, A, M, K, lda, kBM, is_bf16) || !make_map(&map_b, B, N, K, ldb, kBN, is_bf16))

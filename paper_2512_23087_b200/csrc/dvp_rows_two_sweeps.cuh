@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kBlk, 1024 / kBlk) dvp_two_sweeps_kernel(const
   float *scratch = smem;                                             // 96 floats
   uint16_t *hot_smem = reinterpret_cast<uint16_t *>(smem + 96);      // kHotCap per warp
   uint32_t *bound = reinterpret_cast<uint32_t *>(smem + 96 + (kBlk / 32) * kHotCap / 2);
-  begin_after();
+  begin_after(true);  // needs nothing of the fused entry's earlier launches
   const long long t = blockIdx.x;
   const long long id = p.ids ? load_id(p.ids, p.id_is_i32, t) : -1;
   const bool has_id = id >= 0, bad_id = id >= p.V;
@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(kBlk, 1024 / kBlk) dvp_two_sweeps_kernel(const
                              (bad_id ? DVP_FLAG_BAD_ID : 0));
   }
   if (p.out_t.mask) write_mask_row<T>(row, V, st.tau, p.out_t.mask + t * ((p.V + 31) / 32));
+  if (tid == 0) end_after(true);
 }
 
 template <int kBlk>
