@@ -187,6 +187,8 @@ _FORWARD_PACK = struct.Struct("=I3i5qd5Q18Q3QIIfIffQ")
 _BACKWARD_PACK = struct.Struct("=I3i4qd9QIIfI")
 _MONITOR_PACK = struct.Struct("=Ii4q7Q")
 _SEQUENCE_PACK = struct.Struct("=II2q2Qd9Q")
+_FUSED_PACK = struct.Struct("=Ii8qd7Qii18Q5QIff4xQ")
+assert _FUSED_PACK.size == ctypes.sizeof(FusedArgs)
 assert _FORWARD_PACK.size == ctypes.sizeof(ForwardArgs) and _BACKWARD_PACK.size == ctypes.sizeof(BackwardArgs)
 assert _MONITOR_PACK.size == ctypes.sizeof(MonitorArgs) and _SEQUENCE_PACK.size == ctypes.sizeof(SequenceArgs)
 
@@ -480,37 +482,28 @@ def _fused_args(hidden, w_vocab, ids, rho, upstream, infer_logits, d_w, accumula
     _check_matrix("w_vocab", w_vocab)
     T, H = hidden.shape
     V = w_vocab.shape[0]
-    dev = hidden.device
     if hidden.dtype != torch.bfloat16 or w_vocab.dtype != torch.bfloat16:
         raise TypeError("hidden and w_vocab must be bfloat16")
-    a = FusedArgs()
-    a.struct_size = ctypes.sizeof(FusedArgs)
-    a.id_dtype = _id_dtype(ids)
-    a.T, a.H, a.V, a.rho = T, H, V, float(rho)
-    a.ld_hidden, a.ld_w = hidden.stride(0), w_vocab.stride(0)
-    a.hidden, a.w_vocab, a.ids, a.upstream = _ptr(hidden), _ptr(w_vocab), _ptr(ids), _ptr(upstream)
-    res = SimpleNamespace(infer=None, log_ratio=None)
-    sides, rest = _token_outputs(hidden, T, 1 if infer_logits is None else 2, infer_logits is not None)
-    if want_mask:
-        sides[0] = _with_mask(sides[0], hidden, T, V)
-    res.train, a.train = sides[0][0], SideOut(*(x or None for x in sides[0][1]))
-    res.flags = torch.empty(T, dtype=torch.uint8, device=dev)
-    a.flags = _ptr(res.flags)
-    if infer_logits is not None:
+    has_infer = infer_logits is not None
+    if has_infer:
         _check_matrix("infer_logits", infer_logits)
         if infer_logits.dtype != torch.bfloat16:
             raise TypeError("infer_logits must be bfloat16")
-        a.infer_logits, a.ld_infer = _ptr(infer_logits), infer_logits.stride(0)
-        res.infer, a.infer = sides[1][0], SideOut(*(x or None for x in sides[1][1]))
-        res.log_ratio = rest[0]
-        a.log_ratio = _ptr(res.log_ratio)
-    res.d_hidden = torch.empty(T, H, dtype=torch.float32, device=dev)
-    res.d_w = d_w if d_w is not None else torch.empty(V, H, dtype=torch.float32, device=dev)
-    a.d_hidden, a.ld_dh = _ptr(res.d_hidden), res.d_hidden.stride(0)
-    a.d_w, a.ld_dw = _ptr(res.d_w), res.d_w.stride(0)
-    a.accumulate_dw = int(accumulate_dw)
-    a.panel_rows = int(panel_rows)
-    a.stream = _stream(stream)
+    sides, rest = _token_outputs(hidden, T, 2 if has_infer else 1, has_infer)
+    if want_mask:
+        sides[0] = _with_mask(sides[0], hidden, T, V)
+    res = SimpleNamespace(train=sides[0][0], infer=sides[1][0] if has_infer else None,
+                          log_ratio=rest[0] if has_infer else None,
+                          flags=hidden.new_empty(T, dtype=torch.uint8),
+                          d_hidden=hidden.new_empty((T, H), dtype=torch.float32),
+                          d_w=d_w if d_w is not None else hidden.new_empty((V, H), dtype=torch.float32))
+    a = FusedArgs.from_buffer_copy(_FUSED_PACK.pack(
+        _FUSED_PACK.size, _id_dtype(ids), T, H, V, hidden.stride(0), w_vocab.stride(0),
+        infer_logits.stride(0) if has_infer else 0, res.d_hidden.stride(0), res.d_w.stride(0), float(rho),
+        hidden.data_ptr(), w_vocab.data_ptr(), _address(infer_logits), ids.data_ptr(), _address(upstream),
+        res.d_hidden.data_ptr(), res.d_w.data_ptr(), int(accumulate_dw), int(panel_rows), *sides[0][1],
+        *(sides[1][1] if has_infer else _NO_SIDE), res.log_ratio.data_ptr() if has_infer else 0, res.flags.data_ptr(),
+        0, 0, _stream(stream), 0, 0.0, 0.0, 0))
     return a, res
 
 
