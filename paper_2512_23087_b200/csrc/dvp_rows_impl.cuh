@@ -238,27 +238,6 @@ __device__ __forceinline__ void granule_grad(const Granule<TIn> &gr, TGrad *grow
   }
 }
 
-// The same for a whole granule of the row kernel's sweeps (nothing is stored for any other index).
-template <typename TIn, typename TGrad>
-__device__ __forceinline__ void granule_grad_whole(const Granule<TIn> &gr, TGrad *grow, int n_full, int g, int a,
-                                                   float tau, float m, float coef, float g_a) {
-  constexpr int kElems = Granule<TIn>::kElems;
-  if (g < 0 || g >= n_full) {
-    if (g < 0) (void)DVP_IN(g, n_gran, DVP_OOB_GRANULE);
-    return;
-  }
-  float x[kElems], out[kElems];
-  gr.get(x);
-  const int ja = a - g * kElems;
-#pragma unroll
-  for (int j = 0; j < kElems; ++j) {
-    out[j] = x[j] >= tau ? coef * ex2((x[j] - m) * kLog2e) : 0.f;
-    if (j == ja) out[j] = g_a;
-  }
-  if (!DVP_IN((long long)g * kElems + kElems - 1, V, DVP_OOB_GLOBAL)) return;
-  store_granule<TGrad, kElems>(grow + (size_t)g * kElems, out);
-}
-
 // One pipeline stage of sweep 1: kStage granules of this thread.
 template <typename TIn, int kStage>
 struct Stage {
@@ -927,8 +906,49 @@ __device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *gro
   }
 }
 
-// Sweep 3: gradient of g * ln pi^mp(a) over the row.  Granules without a safe
-// token are written as zeros without being read.
+// Gradient entries coef 2^{z l - c} of a whole granule (c2: -c twice, coef2: coef twice), zeros below the threshold.
+template <typename TIn, typename TGrad>
+__device__ __forceinline__ void grad_granule(const Granule<TIn> &gr, TGrad *dst, float tau,
+                                             typename SweepOps<TIn>::Tau tau_p, uint64_t c2, uint64_t coef2) {
+  constexpr int kElems = Granule<TIn>::kElems;
+  const uint64_t l2 = pack2(kLog2e, kLog2e);
+  float x[kElems];
+  gr.get(x);
+  if constexpr (sizeof(TIn) == 2 && sizeof(TGrad) == 2) {
+    uint32_t w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float lo, hi;
+      unpack2(fma2(pack2(x[2 * i], x[2 * i + 1]), l2, c2), lo, hi);
+      unpack2(mul2(pack2(ex2(lo), ex2(hi)), coef2), lo, hi);
+      uint32_t v;
+      if constexpr (std::is_same<TGrad, __nv_bfloat16>::value) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+        v = *reinterpret_cast<const uint32_t *>(&h);
+      } else {
+        const __half2 h = __floats2half2_rn(lo, hi);
+        v = *reinterpret_cast<const uint32_t *>(&h);
+      }
+      w[i] = v & SweepOps<TIn>::reach(gr.w[i], tau_p);
+    }
+    st_stream32(dst, w);
+  } else {
+    float out[kElems];
+#pragma unroll
+    for (int j = 0; j < kElems; j += 2) {
+      float lo, hi;
+      unpack2(fma2(pack2(x[j], x[j + 1]), l2, c2), lo, hi);
+      unpack2(mul2(pack2(ex2(lo), ex2(hi)), coef2), lo, hi);
+      out[j] = x[j] >= tau ? lo : 0.f;
+      out[j + 1] = x[j + 1] >= tau ? hi : 0.f;
+    }
+    store_granule<TGrad, kElems>(dst, out);
+  }
+}
+
+// Sweep 3: gradient of g * ln pi^mp(a) over the row.  Granules without a safe token are written as zeros
+// without being read; the others are read again, the next pair while zeros are written and the last one
+// is worked on: the reads are scattered and the sweep waits for them.
 template <typename TIn, typename TGrad, int kBlk, bool kLoose>
 __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all, int a_row,
                                          const SideStats &st, float g, const uint32_t *bound,
@@ -946,9 +966,8 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
   const float coef = live ? -g / s_tot : 0.f;
   const float g_a = st.member ? g * ((st.s_x + st.s_mask) / s_tot) : 0.f;
   const int a_here = (live && st.member) ? a_row : -1;
-  const int a_live = a_here >= 0 ? v.rel(a_here) : -1;
   const bool listed = live && list.fits();
-  const float tau = live ? st.tau : -kNegInf;  // +inf: nothing passes
+  const float tau = live ? fmaxf(st.tau, -FLT_MAX) : -kNegInf;  // +inf: nothing passes
   const typename SweepOps<TIn>::Key key = SweepOps<TIn>::key(fmaxf(st.tau, -FLT_MAX));
 
   {  // the elements outside the granules, one per thread
@@ -961,49 +980,77 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
     }
   }
   if constexpr (kLoose) {
-    row_grad_loose<TIn, TGrad, kBlk>(v, grow_all, a_live, tau, key, live, st.m, coef, g_a, bound);
+    row_grad_loose<TIn, TGrad, kBlk>(v, grow_all, a_here >= 0 ? v.rel(a_here) : -1, tau, key, live, st.m, coef, g_a,
+                                     bound);
     return;
   }
-  for (int step = 0; step < n_steps; ++step) {
+  // zeros of one step's granules that hold no safe token
+  auto zeros = [&](int step) {
     const int wi = step * kBlk + tid;
-    if (!DVP_IN(wi, n_bound, DVP_OOB_BOUND)) break;
+    if (!DVP_IN(wi, n_bound, DVP_OOB_BOUND)) return;
     const uint32_t b = live ? SweepOps<TIn>::reach(bound[wi], key) : 0u;
     const int g0 = 2 * step * kBlk + tid, g1 = g0 + kBlk;
-    // granules that can hold safe tokens are written below
     if (!(b & 1u) && g0 < n_full && DVP_IN((long long)g0 * kElems + kElems - 1, V, DVP_OOB_GLOBAL))
       store_zero_granule<TGrad, kElems>(grow + (size_t)g0 * kElems);
     if (!(b & 0x10000u) && g1 < n_full && DVP_IN((long long)g1 * kElems + kElems - 1, V, DVP_OOB_GLOBAL))
       store_zero_granule<TGrad, kElems>(grow + (size_t)g1 * kElems);
+  };
+  // 2^{(z - m) l} = 2^{z l - c} 2^{c - m l}
+  const float c = st.m * kLog2e, cf = coef * ex2(-fmaf(st.m, kLog2e, -c));
+  const uint64_t c2 = pack2(-c, -c), cf2 = pack2(cf, cf);
+  const typename SweepOps<TIn>::Tau tau_p = SweepOps<TIn>::threshold(fmaxf(st.tau, -FLT_MAX));
+  const int g_here = a_here >= 0 ? v.granule_of(a_here) : -1;
+  // one granule; the sampled token's entry replaces the one that its granule's store left
+  auto emit = [&](const Granule<TIn> &gr, int g) {
+    if (!DVP_IN((long long)g * kElems + kElems - 1, V, DVP_OOB_GLOBAL)) return;
+    grad_granule<TIn, TGrad>(gr, grow + (size_t)g * kElems, tau, tau_p, c2, cf2);
+    if (g == g_here) grow_all[a_here] = Storage<TGrad>::narrow(g_a);
+  };
+  int step = 0;
+  if (listed) {
+    const int wbase = tid & ~31, lane = tid & 31;
+    // granule of list position q, -1 behind the end (with rho = 0 a list of float32 granules may name some
+    // behind the end of the row)
+    auto at = [&](int q) {
+      if (q >= list.count || !DVP_IN(q, n_hot, DVP_OOB_HOT)) return -1;
+      const uint32_t e = list.slots[q];
+      const int g = (int)(e >> 5) * kBlk + wbase + (int)(e & 31);
+      return g < n_full ? g : -1;
+    };
+    Granule<TIn> a0, a1, b0, b1;
+    int ga0 = at(lane), ga1 = at(lane + 32);
+    if (ga0 >= 0) a0.load_whole(row, n_full, ga0);
+    if (ga1 >= 0) a1.load_whole(row, n_full, ga1);
+    for (int q = lane; q < list.count; q += 128) {
+      const int gb0 = at(q + 64), gb1 = at(q + 96);
+      if (gb0 >= 0) b0.load_whole(row, n_full, gb0);
+      if (gb1 >= 0) b1.load_whole(row, n_full, gb1);
+      if (step < n_steps) zeros(step++);
+      if (ga0 >= 0) emit(a0, ga0);
+      if (ga1 >= 0) emit(a1, ga1);
+      ga0 = at(q + 128);
+      ga1 = at(q + 160);
+      if (ga0 >= 0) a0.load_whole(row, n_full, ga0);
+      if (ga1 >= 0) a1.load_whole(row, n_full, ga1);
+      if (step < n_steps) zeros(step++);
+      if (gb0 >= 0) emit(b0, gb0);
+      if (gb1 >= 0) emit(b1, gb1);
+    }
   }
+  for (; step < n_steps; ++step) zeros(step);
   if (live && !listed) {
     // a dense safe set: all of the thread's hot granules, a step's two at a time (both loads before either is used)
-    for (int step = 0; step < n_steps; ++step) {
+    for (step = 0; step < n_steps; ++step) {
       const int wi = step * kBlk + tid;
       if (!DVP_IN(wi, n_bound, DVP_OOB_BOUND)) break;
       const uint32_t h = SweepOps<TIn>::reach(bound[wi], key);
       const int g0 = 2 * step * kBlk + tid, g1 = g0 + kBlk;
-      const bool hot0 = h & 1u, hot1 = h & 0x10000u;
+      const bool hot0 = (h & 1u) && g0 < n_full, hot1 = (h & 0x10000u) && g1 < n_full;
       Granule<TIn> a0, a1;
       if (hot0) a0.load_whole(row, n_full, g0);
       if (hot1) a1.load_whole(row, n_full, g1);
-      if (hot0) granule_grad_whole<TIn, TGrad>(a0, grow, n_full, g0, a_live, tau, st.m, coef, g_a);
-      if (hot1) granule_grad_whole<TIn, TGrad>(a1, grow, n_full, g1, a_live, tau, st.m, coef, g_a);
-    }
-  }
-  if (listed) {
-    const int wbase = tid & ~31, lane = tid & 31;
-    for (int q = lane; q < list.count; q += 64) {
-      if (!DVP_IN(q, n_hot, DVP_OOB_HOT)) break;
-      const uint32_t e0 = list.slots[q];
-      const bool two = q + 32 < list.count && DVP_IN(q + 32, n_hot, DVP_OOB_HOT);
-      const uint32_t e1 = two ? list.slots[q + 32] : e0;
-      const int g0 = (int)(e0 >> 5) * kBlk + wbase + (int)(e0 & 31);
-      const int g1 = (int)(e1 >> 5) * kBlk + wbase + (int)(e1 & 31);
-      Granule<TIn> a0, a1;
-      a0.load_whole(row, n_full, g0);
-      if (two) a1.load_whole(row, n_full, g1);
-      granule_grad_whole<TIn, TGrad>(a0, grow, n_full, g0, a_live, tau, st.m, coef, g_a);
-      if (two) granule_grad_whole<TIn, TGrad>(a1, grow, n_full, g1, a_live, tau, st.m, coef, g_a);
+      if (hot0) emit(a0, g0);
+      if (hot1) emit(a1, g1);
     }
   }
 }
