@@ -193,6 +193,7 @@ assert _FORWARD_PACK.size == ctypes.sizeof(ForwardArgs) and _BACKWARD_PACK.size 
 assert _MONITOR_PACK.size == ctypes.sizeof(MonitorArgs) and _SEQUENCE_PACK.size == ctypes.sizeof(SequenceArgs)
 
 _lib = None
+_host = None
 
 
 def load_library() -> ctypes.CDLL:
@@ -203,6 +204,12 @@ def load_library() -> ctypes.CDLL:
             raise RuntimeError(
                 f"{LIB_PATH} is missing: build it with `python -m paper_2512_23087_b200.build`; "
                 "this package has no CPU or PyTorch fallback")
+        global _host
+        try:
+            from . import _host   # lays outputs over one allocation
+        except ImportError as e:
+            raise RuntimeError("the helper _host.so is missing or does not load: build it with "
+                               "`python -m paper_2512_23087_b200.build`") from e
         lib = ctypes.CDLL(LIB_PATH)
         lib.dvp_forward.argtypes = [ctypes.POINTER(ForwardArgs)]
         lib.dvp_forward.restype = ctypes.c_int
@@ -296,22 +303,17 @@ def _check_matrix(name: str, x: torch.Tensor):
 
 
 def _token_outputs(like: torch.Tensor, T: int, sides: int, floats: int):
-    """``sides`` side namespaces and ``floats`` further float32 vectors of T tokens, with their addresses.  All
-    float32 vectors are rows of one allocation, as are the counts: an allocator call costs about a
-    microsecond, a call of dvp_forward would make twenty."""
-    buf = like.new_empty((7 * sides + floats, T), dtype=torch.float32)
-    rows, base, step = buf.unbind(0), buf.data_ptr(), 4 * T
-    cnt = like.new_empty((sides, T), dtype=torch.int32)
-    counts, cbase = cnt.unbind(0), cnt.data_ptr()
-    out = []
+    """``sides`` side namespaces with their addresses in the order of ``dvp_side_out``, ``floats`` further float32
+    vectors of T tokens, and the flags.  All of them lie over one allocation."""
+    v, base, step = _host.outputs(like, T, 7 * sides + floats, sides)
+    out, n = [], 7 * sides + floats
     for i in range(sides):
-        r, at = rows[7 * i:7 * i + 7], base + 7 * i * step
+        r, at = v[7 * i:7 * i + 7], base + 7 * i * step
         o = SimpleNamespace(max=r[0], lse=r[1], lse_safe=r[2], logp=r[3], logp_mp=r[4], comp_mp=r[5], log_cov=r[6],
-                            count=counts[i], mask=None)
-        # in the order of dvp_side_out
-        out.append((o, (at, at + step, at + 2 * step, at + 3 * step, at + 4 * step, at + 5 * step, cbase + i * step,
+                            count=v[n + i], mask=None)
+        out.append((o, (at, at + step, at + 2 * step, at + 3 * step, at + 4 * step, at + 5 * step, base + (n + i) * step,
                         0, at + 6 * step)))
-    return out, rows[7 * sides:]
+    return out, v[7 * sides:n], v[-1]
 
 
 def _with_mask(side, like: torch.Tensor, T: int, V: int):
@@ -370,12 +372,12 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
     if out is not None:
         res = out
     else:
-        sides, rest = _token_outputs(train_logits, T, 2 if has_infer else 1, has_infer + weighted)
+        sides, rest, flags = _token_outputs(train_logits, T, 2 if has_infer else 1, has_infer + weighted)
         if want_mask:
             sides = [_with_mask(side, train_logits, T, V) for side in sides]
         res = SimpleNamespace(train=sides[0][0], infer=sides[1][0] if has_infer else None,
                               log_ratio=rest[0] if has_infer else None,
-                              flags=train_logits.new_empty(T, dtype=torch.uint8), grad_train=None,
+                              flags=flags, grad_train=None,
                               _train_addresses=sides[0][1], _infer_addresses=sides[1][1] if has_infer else _NO_SIDE)
         if weighted:
             res.weight = rest[-1]
@@ -489,12 +491,12 @@ def _fused_args(hidden, w_vocab, ids, rho, upstream, infer_logits, d_w, accumula
         _check_matrix("infer_logits", infer_logits)
         if infer_logits.dtype != torch.bfloat16:
             raise TypeError("infer_logits must be bfloat16")
-    sides, rest = _token_outputs(hidden, T, 2 if has_infer else 1, has_infer)
+    sides, rest, flags = _token_outputs(hidden, T, 2 if has_infer else 1, has_infer)
     if want_mask:
         sides[0] = _with_mask(sides[0], hidden, T, V)
     res = SimpleNamespace(train=sides[0][0], infer=sides[1][0] if has_infer else None,
                           log_ratio=rest[0] if has_infer else None,
-                          flags=hidden.new_empty(T, dtype=torch.uint8),
+                          flags=flags,
                           d_hidden=hidden.new_empty((T, H), dtype=torch.float32),
                           d_w=d_w if d_w is not None else hidden.new_empty((V, H), dtype=torch.float32))
     a = FusedArgs.from_buffer_copy(_FUSED_PACK.pack(
@@ -589,10 +591,10 @@ def dvp_sequence_aggregate(log_ratio: torch.Tensor, seq_offsets: torch.Tensor,
     if has_cov and (log_cov.dtype != torch.float32 or log_cov.numel() != log_ratio.numel()):
         raise TypeError("log_cov must be float32 with one entry per token")
     S = seq_offsets.numel() - 1
-    floats = log_ratio.new_empty((4 if has_cov else 2, S)).unbind(0)
-    counts = log_ratio.new_empty((2, S), dtype=torch.int32).unbind(0)
+    v, _, _ = _host.outputs(log_ratio, S, 4 if has_cov else 2, 2)
+    floats, counts = v[:-3], v[-3:-1]
     res = SimpleNamespace(seq_log_ratio=floats[0], min_log_ratio=floats[1], n_valid=counts[0], n_zero_weight=counts[1],
-                          veto=log_ratio.new_empty(S, dtype=torch.uint8))
+                          veto=v[-1])
     if has_cov:
         res.min_cov, res.mean_cov = floats[2], floats[3]
     st = packed["dvp_sequence_aggregate"](_SEQUENCE_PACK.pack(
@@ -614,8 +616,7 @@ def dvp_monitor(train_logits: torch.Tensor, infer_logits: torch.Tensor, stream=N
     if infer_logits.dtype != train_logits.dtype or infer_logits.shape != train_logits.shape:
         raise ValueError("infer_logits must match train_logits in dtype and shape")
     T, V = train_logits.shape
-    buf = train_logits.new_empty((4, T), dtype=torch.float32)
-    rows, at, step = buf.unbind(0), buf.data_ptr(), 4 * T
+    rows, at, step = _host.outputs(train_logits, T, 4, 0)
     st = packed["dvp_monitor"](_MONITOR_PACK.pack(
         _MONITOR_PACK.size, _DTYPES[train_logits.dtype], T, V, train_logits.stride(0), infer_logits.stride(0),
         train_logits.data_ptr(), infer_logits.data_ptr(), at, at + step, at + 2 * step, at + 3 * step,

@@ -1,7 +1,8 @@
 """Builds the CUDA library in-tree with nvcc for sm_100a.
 
-``build()`` compiles every ``csrc/*.cu`` to an object file (in parallel) and
-links ``libdvp_b200.so`` beside this file.  Objects are rebuilt only when a
+``build()`` compiles every ``csrc/*.cu`` to an object file (in parallel), links
+``libdvp_b200.so`` beside this file and compiles ``_host.so``, the Python helper
+that lays a call's outputs over one allocation.  Objects are rebuilt only when a
 source or header is newer.  Run as ``python -m paper_2512_23087_b200.build``;
 ``--debug-bounds`` builds the bounds-checking library instead.
 """
@@ -36,6 +37,30 @@ def _newest_header() -> float:
     hdrs = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
         glob.glob(os.path.join(ROOT, "include", "*.h"))
     return max(os.path.getmtime(h) for h in hdrs)
+
+
+HOST = os.path.join(HERE, "_host.so")
+
+
+def build_host() -> str:
+    """The Python helper ``_host`` (g++ against this interpreter's and torch's headers)."""
+    src = os.path.join(CSRC, "host_outputs.cpp")
+    if os.path.exists(HOST) and os.path.getmtime(HOST) >= os.path.getmtime(src):
+        return HOST
+    import sysconfig
+    import torch
+    base = os.path.join(os.path.dirname(torch.__file__))
+    tmp = HOST + f".{os.getpid()}.tmp"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", src, "-o", tmp,
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(base, "include"),
+           "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
+           "-L", os.path.join(base, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed: " + " ".join(cmd) + "\n" + r.stdout + r.stderr)
+    os.replace(tmp, HOST)
+    return HOST
 
 
 LIB_BOUNDS = os.path.join(HERE, "libdvp_b200_bounds.so")
@@ -77,6 +102,8 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
             for log in ex.map(run, jobs):
                 if verbose and log:
                     print(log, file=sys.stderr)
+    if not debug_bounds:
+        build_host()
     if jobs or not os.path.exists(lib):
         tmp = lib + f".{os.getpid()}.tmp"
         run([nvcc, "-shared", "-o", tmp, *objs, "-lcudart"])
