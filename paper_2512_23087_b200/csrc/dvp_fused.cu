@@ -318,8 +318,8 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     p.flags = flt + r0;
     p.bounds_status = bounds_status_word();
     if (a->infer_logits) {
-      p.given_logp_mp_i = lpi + r0;
-      p.given_flags_i = fli + r0;
+      pp.logp_mp_i = lpi + r0;
+      pp.flags_i = fli + r0;
       p.log_ratio = a->log_ratio ? a->log_ratio + r0 : nullptr;
     }
     if (weighted) {

@@ -23,6 +23,10 @@ constexpr float kPScale = 16384.f;  // 2^14: P uses float16's normal range for m
 
 struct PanelParams {
   RowParams row;       // train = the fp32 panel; ids, upstream, T, V, ld_train, log_rho, outputs, weights
+  // of the inference rows' pass, or null: ln pi^mp_infer(a) per token, and flags whose DVP_FLAG_IN_TRAIN bit
+  // says "a in V'_S"
+  const float *logp_mp_i;
+  const uint8_t *flags_i;
   const float *row_max;  // the row maxima that the logits contraction left, in pieces: the maximum of row t is
   long long row_max_ld;  // the largest of row_max[t * row_max_ld + i], i < row_max_n
   int row_max_n;
@@ -151,16 +155,16 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_panel_kernel(const Pane
 
   if (threadIdx.x == 0) {
     finish_side(p.out_t, t, st, has_id, bad_id);
-    const bool in_i = p.given_flags_i && (p.given_flags_i[t] & DVP_FLAG_IN_TRAIN);  // of the inference rows' pass
+    const bool in_i = pp.flags_i && (pp.flags_i[t] & DVP_FLAG_IN_TRAIN);
     if (p.flags)
       p.flags[t] = (uint8_t)((st.member ? DVP_FLAG_IN_TRAIN : 0) | (in_i ? DVP_FLAG_IN_INFER : 0) |
                              (has_id ? 0 : DVP_FLAG_NO_ID) | (bad_id ? DVP_FLAG_BAD_ID : 0));
-    if (p.log_ratio)
-      p.log_ratio[t] = a < 0 ? __int_as_float(0x7fc00000)
-                             : log_ratio_of(st.member, in_i, logp_mp_of(st), p.given_logp_mp_i[t]);
+    const float ratio = a >= 0 && pp.logp_mp_i ? log_ratio_of(st.member, in_i, logp_mp_of(st), pp.logp_mp_i[t])
+                                               : __int_as_float(0x7fc00000);
+    if (p.log_ratio) p.log_ratio[t] = ratio;
     float g = p.upstream[t];
     if (p.weight_kind != DVP_WEIGHT_NONE) {
-      const float w = row_weight_given(p, st, t, a >= 0);
+      const float w = token_weight(ratio, p.weight_kind, p.weight_lo, p.weight_hi);
       if (w == w) g *= w;
       if (p.weight_out) p.weight_out[t] = w;
     }

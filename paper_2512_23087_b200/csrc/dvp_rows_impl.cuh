@@ -1,17 +1,17 @@
 // Row kernels of Dynamic Vocabulary Pruning for sm_100a.
 //
-// One thread block owns one token row.  The row is streamed from HBM once
+// One thread block (or a cluster of them) owns one row.  The row is streamed from HBM once
 // (sweep 1) in 32-byte granules, one DRAM sector per lane and load, two
-// pipeline stages deep.  While it streams, every thread keeps an online
-// log-sum-exp of what it has seen and leaves in shared memory an upper bound
-// (bfloat16, rounded up) of the maximum of each granule it loaded.  Once the
-// row maximum, hence the threshold of Def. 5.1, is known, only granules whose
-// bound reaches the threshold can hold safe tokens: sweep 2 (masked sum and
-// count, Def. 5.2) and sweep 3 (gradient, Prop. 5.4) revisit just those, and
-// sweep 3 writes zeros for all the others without reading anything.  With a
-// sparse safe set a row costs one HBM read per logit matrix and one HBM write
-// of the gradient; with a dense safe set the same code degrades to three
-// sweeps, still correct.
+// pipeline stages deep.  While it streams, every thread adds up what it sees against a
+// guess of the row's maximum: the full sum, and the masked sum and count of Def. 5.2
+// under the guess's threshold; the maximum of each granule stays in shared memory
+// (float32: a bfloat16 upper bound).  Once the row maximum, hence the threshold of
+// Def. 5.1, is known, sweep 2 revisits only what came before the guess was the maximum,
+// and of it only granules whose bound reaches the threshold.  Sweep 3 (gradient,
+// Prop. 5.4) reads the granules with safe tokens again and writes zeros for all the
+// others without reading anything.
+// With a sparse safe set a row costs one HBM read per logit matrix and one HBM write
+// of the gradient; with a dense safe set sweep 3 reads the row a second time.
 #pragma once
 #include <float.h>
 #include <limits.h>
@@ -1211,7 +1211,7 @@ __global__ void dvp_row_kernel_scalar(const RowParams p) {
   if (irow) si = row_stats_scalar<TIn>(irow, p.V, a, p.log_rho, p.mode, p.mask_value, scratch, mask_i);
   float w = 1.f;
   if (p.weight_kind != DVP_WEIGHT_NONE)
-    w = irow ? row_weight(p, st, si, a >= 0) : row_weight_given(p, st, t, a >= 0);
+    w = row_weight(p, st, si, a >= 0);  // weights need inference rows
   if (p.weight_out && threadIdx.x == 0) p.weight_out[t] = w;
 
   if (p.grad) {
@@ -1469,7 +1469,7 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
   const int stage_hint = stage;
   // stage byte 0x11: the kernel that keeps the row in shared memory; 0x1e: the same with
   // block 0's first copy withheld (self-test of the wait limit)
-  if ((stage == 0x11 || stage == 0x1e) && !p.given_logp_mp_i) {
+  if (stage == 0x11 || stage == 0x1e) {
     const bool ok16 = aligned32(p.train, p.ld_train, sizeof(TIn)) &&
                       aligned32(p.infer, p.ld_infer, sizeof(TIn)) &&
                       aligned32(p.grad, p.ld_grad, sizeof(TGrad));

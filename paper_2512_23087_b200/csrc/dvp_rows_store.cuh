@@ -542,11 +542,9 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_row_kernel_cs(const Row
         float w;
         if (a < 0) {
           w = nan;
-        } else if (p.infer) {
+        } else {
           const float r = (p.mode & DVP_MODE_FINITE_MASK) ? lp - lp_i : log_ratio_of(s.member, mem_i, lp, lp_i);
           w = token_weight(r, p.weight_kind, p.weight_lo, p.weight_hi);
-        } else {
-          w = row_weight_given(p, s, t, true);
         }
         if (w == w) g *= w;
         if (p.weight_out && threadIdx.x == 0) p.weight_out[t] = w;
