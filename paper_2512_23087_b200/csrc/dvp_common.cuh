@@ -110,8 +110,9 @@ __device__ __forceinline__ void st_stream8(void *p, uint2 v) {
 // kernel, and with it for all before, in begin_after, before it touches memory; only then may the next one begin, so
 // that a kernel that begins finds everything before its predecessor complete.  A kernel that needs nothing of its
 // predecessor (and overwrites nothing that it reads) is `early`: it works first and waits in end_after, so that
-// whoever waits for it waits for both.  One thread of each block has to call end_after.  Kernels with these calls
-// may be launched in the ordinary way too.
+// whoever waits for it waits for both.  One thread of the grid has to call end_after: of the last block, where the
+// others should leave their place to the next blocks.  Kernels with these calls may be launched in the ordinary way
+// too.
 __device__ __forceinline__ void begin_after(bool early = false) {
   if (!early) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

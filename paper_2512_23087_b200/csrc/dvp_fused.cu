@@ -32,9 +32,9 @@ namespace dvp {
 template <typename TIn, typename TOut>
 __global__ void __launch_bounds__(256)
 transpose_convert_kernel(const TIn *in, long long ld_in, TOut *out, long long ld_out, int R, int C,
-                         int vec_ok, const float *row_scale, bool early) {
+                         int vec_ok, const float *row_scale) {
   __shared__ TOut tile[64][66];
-  begin_after(early);
+  begin_after(true);
   const int per_row = (C + 63) / 64, c0 = (int)(blockIdx.x % per_row) * 64, r0 = (int)(blockIdx.x / per_row) * 64;
   const int tid = threadIdx.x;
   // load: 64 rows x 8 vectors of 8 elements, two vectors per thread
@@ -74,7 +74,7 @@ transpose_convert_kernel(const TIn *in, long long ld_in, TOut *out, long long ld
       for (int j = 0; j < 8 && r + j < R; ++j) dst[j] = e[j];
     }
   }
-  if (tid == 0) end_after(early);
+  if (blockIdx.x == gridDim.x - 1 && tid == 0) end_after(true);  // the others leave their place to the next blocks
 }
 
 template <typename TIn, typename TOut>
@@ -82,7 +82,7 @@ static void launch_transpose(const TIn *in, long long ld_in, TOut *out, long lon
                              cudaStream_t s, const float *row_scale = nullptr) {
   const int vec_ok = ld_in % 8 == 0 && ld_out % 8 == 0 && (uintptr_t)in % 16 == 0 && (uintptr_t)out % 16 == 0;
   (void)launch_after(transpose_convert_kernel<TIn, TOut>, (unsigned)(((C + 63) / 64) * (long long)((R + 63) / 64)), 256, 0,
-                     s, in, ld_in, out, ld_out, R, C, vec_ok, row_scale, row_scale == nullptr);
+                     s, in, ld_in, out, ld_out, R, C, vec_ok, row_scale);
 }
 
 struct FusedScalars {
@@ -269,7 +269,6 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
 
   const bool weighted = a->weight_kind != DVP_WEIGHT_NONE;
   grad_scale_kernel<<<1, 1024, 0, s>>>(a->upstream, a->T, weighted ? fmaxf(1.f, a->weight_hi) : 1.f, sc);
-  launch_transpose<__nv_bfloat16, __half>(w, a->ld_w, wt16, L.Vp, V, H, s);
   if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
 
   const double log_rho = a->rho > 0.0 ? std::log(a->rho) : -HUGE_VAL;
@@ -289,19 +288,25 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     p.bounds_status = bounds_status_word();
     return two_sweeps::launch(p, s);
   };
-  // first: the training rows take the log-ratio (and an importance weight) from it
-  if (a->infer_logits && infer_rows() != cudaSuccess) return DVP_ERR_CUDA;
   int panel_index = 0;
   for (long long r0 = 0; r0 < a->T; r0 += L.panel, ++panel_index) {
     const int rows = (int)((a->T - r0 < L.panel) ? a->T - r0 : L.panel);
     // logits of the panel: z = hidden[r0 : r0 + rows] x W^T (bf16 operands, fp32 accumulate)
     // its epilogue also leaves each row's maximum, one piece per tile column: the panel's row pass
-    // then knows the threshold before it reads the panel.  Early: the launch before it is the inference rows' pass
-    // or, from the second panel on, the last of d_w's, when nobody reads z or the maxima any more
+    // then knows the threshold before it reads the panel.  Early: from the second panel on the launch before it is
+    // the last of d_w's, when nobody reads z or the maxima any more
     cudaError_t e = gemm::launch_gemm_tn(hidden + r0 * a->ld_hidden, a->ld_hidden, w, a->ld_w, z, L.Vp,
                                          rows, V, H, true, 1.f, nullptr, false, &sc->status, sms, s, false,
                                          false, 1, rmax, L.max_pieces, nullptr, 0, gemm::Order::kEarly);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
+    if (panel_index == 0) {
+      // Beside the first contraction, in the room that its blocks leave on an SM: the inference rows (the panel's
+      // rows take the log-ratio and the importance weight from them) and W^T.  512 x 1,024 x 32,000: 210 us a call
+      // with both in front of the contraction, 206 with the rows there, 199 with neither.
+      if (a->infer_logits && infer_rows() != cudaSuccess) return DVP_ERR_CUDA;
+      launch_transpose<__nv_bfloat16, __half>(w, a->ld_w, wt16, L.Vp, V, H, s);
+      if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
+    }
     // rows of the panel, one sweep: statistics, and the gradient panel up to a factor per row
     panel::PanelParams pp{};
     RowParams &p = pp.row;
@@ -338,10 +343,6 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     pp.a_coef = a_coef;
     pp.scale = &sc->scale;
     if (launch_after(panel::dvp_panel_kernel<512, 2>, (unsigned)rows, 512, 0, s, pp) != cudaSuccess) return DVP_ERR_CUDA;
-    // the panel's hidden rows times their factor (and 2^14 * scale / 512), transposed, in float16
-    launch_transpose<__nv_bfloat16, __half>(hidden + r0 * a->ld_hidden, a->ld_hidden, hs16, L.panel, rows, H, s,
-                                            hid_scale);
-    if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
     // d_hidden[r0 : r0 + rows] = diag(c) P W + q_t W[a_t]: the factor is applied per row and the 1[k = a] term
     // added in fp32.  Few output tiles and a long K: each tile is computed as several K ranges, whose partial
     // results go where the logits were (read for the last time by the row pass) and are summed in order.
@@ -355,6 +356,9 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
                    : gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, dh, a->ld_dh, rows, H, V, false, 1.f, nullptr, false,
                                           &sc->status, sms, s, false, false, 1, nullptr, 0, row_scale, 0,
                                           gemm::Order::kAfter);
+    // beside it: the panel's hidden rows times their factor (and 2^14 * scale / 512), transposed, in float16
+    launch_transpose<__nv_bfloat16, __half>(hidden + r0 * a->ld_hidden, a->ld_hidden, hs16, L.panel, rows, H, s,
+                                            hid_scale);
     if (e == cudaSuccess)
       e = launch_after(panel::sum_ranges_kernel, (unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s,
                        ranges > 1 ? z : dh, rows * Hp, ranges > 1 ? Hp : a->ld_dh, ranges,

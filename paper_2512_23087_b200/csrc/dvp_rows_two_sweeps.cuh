@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(kBlk, 1024 / kBlk) dvp_two_sweeps_kernel(const
                              (bad_id ? DVP_FLAG_BAD_ID : 0));
   }
   if (p.out_t.mask) write_mask_row<T>(row, V, st.tau, p.out_t.mask + t * ((p.V + 31) / 32));
-  if (tid == 0) end_after(true);
+  if (blockIdx.x == gridDim.x - 1 && tid == 0) end_after(true);  // the others leave their place to the next blocks
 }
 
 template <int kBlk>
