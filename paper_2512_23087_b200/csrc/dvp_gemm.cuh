@@ -181,37 +181,71 @@ __device__ __forceinline__ void tc_fence_after() {
 // (a d_w contraction of 512 tokens x 32,000 x 1,024, which is bound by its epilogue: 68 us then).
 //   kStore  C = v     kAdd  C += v by vector reductions in L2: one addend per element and launch, so reruns
 //   are bit-identical; loads, additions and stores were 32 dependent round trips a tile
+//
+// `exchange`: four neighbouring lanes exchange their rows' 32-byte pieces first, so that a store instruction of the
+// warp fills 8 whole lines instead of a piece of 32 of them.  With the pieces as they lie a 32,000 x 1,024 C leaves
+// the chip at 2.9 TB/s (zeroing it runs at 6.3), which bounds products with a short K; the exchange goes through the
+// shared-memory path that the MMAs read their operands by, which long ones are bound by.  us without / with it, K = 64,
+// 256, 512, 1,024, 2,048: 45.9 / 38.8, 49.4 / 41.2, 53.6 / 49.5, 67.3 / 69.2, 110 / 116; twice the epilogue
+// warps: no change.
+constexpr int kExchangeSlices = 8;  // up to this many slices of K in a unit
 enum class Out { kStore, kAdd };
+// c_own: where the thread's own row (`lane` of the warp's rows) begins; rows: how many of the warp's rows C has.
 template <Out kOut>
-__device__ __forceinline__ void store_columns(float *c, const uint32_t (&r)[32], float alpha, int n_cols) {
+__device__ __forceinline__ void store_columns(float *c_own, long long ldc, int lane, int rows, const uint32_t (&r)[32],
+                                              float alpha, int n_cols, bool exchange) {
   if (n_cols >= 32) {
+    float v[4][8];  // v[b]: columns 8 b .. 8 b + 7 of the thread's row
 #pragma unroll
-    for (int j = 0; j < 32; j += 8) {
-      float v[8];
+    for (int j = 0; j < 32; ++j) v[j >> 3][j & 7] = alpha * __uint_as_float(r[j]);
+    // a 4 x 4 transposition of pieces among the lanes 4 g + q: v[k] becomes piece q of row 4 g + k
+    if (exchange) {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = alpha * __uint_as_float(r[j + e]);
+      for (int s = 1; s <= 2; s *= 2) {
+        const bool odd = (lane & s) != 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          if (b & s) continue;
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const float got = __shfl_xor_sync(0xffffffffu, odd ? v[b][e] : v[b | s][e], s);
+            if (odd)
+              v[b][e] = got;
+            else
+              v[b | s][e] = got;
+          }
+        }
+      }
+    }
+    // piece k of the thread: of its own row, or piece `lane & 3` of row 4 g + k
+    const int first = exchange ? lane & ~3 : lane;
+    float *c = c_own + (long long)(first - lane) * ldc + (exchange ? 8 * (lane & 3) : 0);
+    const long long next = exchange ? ldc : 8;
+#pragma unroll
+    for (int k = 0; k < 4; ++k, c += next) {
+      if (first + (exchange ? k : 0) >= rows) break;
       if constexpr (kOut == Out::kStore) {
-        asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(c + j), "f"(v[0]), "f"(v[1]),
-                     "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+        asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(c), "f"(v[k][0]), "f"(v[k][1]),
+                     "f"(v[k][2]), "f"(v[k][3]), "f"(v[k][4]), "f"(v[k][5]), "f"(v[k][6]), "f"(v[k][7])
                      : "memory");
       } else {
-        asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(c + j), "f"(v[0]), "f"(v[1]), "f"(v[2]),
-                     "f"(v[3])
+        asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(c), "f"(v[k][0]), "f"(v[k][1]), "f"(v[k][2]),
+                     "f"(v[k][3])
                      : "memory");
-        asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(c + j + 4), "f"(v[4]), "f"(v[5]), "f"(v[6]),
-                     "f"(v[7])
+        asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(c + 4), "f"(v[k][4]), "f"(v[k][5]),
+                     "f"(v[k][6]), "f"(v[k][7])
                      : "memory");
       }
     }
-  } else {
+  } else if (lane < rows) {
 #pragma unroll
     for (int j = 0; j < 32; ++j) {
       if (j < n_cols) {
         const float v = alpha * __uint_as_float(r[j]);
         if constexpr (kOut == Out::kStore)
-          c[j] = v;
+          c_own[j] = v;
         else
-          atomicAdd(c + j, v);
+          atomicAdd(c_own + j, v);
       }
     }
   }
@@ -343,11 +377,11 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * kBN + c0, r);
         tmem_wait_ld(r);
         const int col = tn * kBN + c0;
-        if (row < p.M && col < p.N) {
+        if (col < p.N) {
           if (p.accumulate)
-            store_columns<Out::kAdd>(crow + col, r, alpha, p.N - col);
+            store_columns<Out::kAdd>(crow + col, p.ldc, lane, p.M - (row - lane), r, alpha, p.N - col, false);
           else
-            store_columns<Out::kStore>(crow + col, r, alpha, p.N - col);
+            store_columns<Out::kStore>(crow + col, p.ldc, lane, p.M - (row - lane), r, alpha, p.N - col, false);
         }
       }
       tc_fence_before();
@@ -559,14 +593,16 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   } else {
     // ---------------- epilogue (both blocks): own 128 rows of the pair's tile
     const int quarter = warp & 3;
+    const bool exchange = k_per <= kExchangeSlices;
     const float alpha_all = p.alpha * (p.alpha_dev ? *p.alpha_dev : 1.f);
     uint32_t local_tile = 0;
-    for (int unit = pair; unit < n_units && !*abort_flag; unit += n_pairs, ++local_tile) {
+    for (int unit = pair; unit < n_units; unit += n_pairs, ++local_tile) {
       const int tile = unit % n_tiles;
       const int tm = m_fastest ? tile % tiles_m : tile / tiles_n;
       const int tn = m_fastest ? tile / tiles_m : tile % tiles_n;
       const uint32_t buf = local_tile & 1, use = local_tile >> 1;
-      if (!mbar_wait(smem_u32(&sh->tmem_full[buf]), use & 1, abort_flag)) {
+      // the whole warp goes on or none of it: reading tensor memory and the exchange need every lane
+      if (!__all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_u32(&sh->tmem_full[buf]), use & 1, abort_flag))) {
         if (!*abort_flag) { *abort_flag = 1; atomicExch(p.status, kErrEpilogueWait); }
         break;
       }
@@ -592,11 +628,11 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
               if (col + j < p.N) row_hi = fmaxf(row_hi, alpha * __uint_as_float(r[j]));
           }
         }
-        if (row < p.M && col < p.N) {
+        if (col < p.N) {
           if (p.accumulate || add_ranges)
-            store_columns<Out::kAdd>(crow + col, r, alpha, p.N - col);
+            store_columns<Out::kAdd>(crow + col, p.ldc, lane, p.M - (row - lane), r, alpha, p.N - col, exchange);
           else
-            store_columns<Out::kStore>(crow + col, r, alpha, p.N - col);
+            store_columns<Out::kStore>(crow + col, p.ldc, lane, p.M - (row - lane), r, alpha, p.N - col, exchange);
         }
       };
       tmem_ld32(tmem_row, ra);

@@ -35,3 +35,23 @@ def test_many_tokens_of_one_id(n_ids):
     # float16 gradient panel: 2^-11 a term at most, tokens of one row add up
     assert ((r[0].d_w.double() - want).norm(dim=1) <= 1e-3 * want.norm(dim=1) + 1e-6 * want.norm(dim=1).max()).all()
     assert torch.equal(r[0].d_w, r[1].d_w)
+
+
+# products with a short k store exchanged pieces of four neighbouring rows (up to 8 slices of 64): ends inside the four
+# rows, the warp's 32 and the block's 128, columns that end inside a group of 32, and either side of the line
+@pytest.mark.parametrize("accumulate", [False, True])
+@pytest.mark.parametrize("k", [8, 512, 520])
+@pytest.mark.parametrize("m,n", [(1, 8), (3, 40), (35, 32), (130, 264), (513, 304)])
+def test_stores_of_short_products(m, n, k, accumulate):
+    g = torch.Generator(device=fused.DEV).manual_seed(m + n + k)
+    a = torch.randn(m, k, generator=g, device=fused.DEV).to(torch.bfloat16)
+    b = torch.randn(n, k, generator=g, device=fused.DEV).to(torch.bfloat16)
+    buf = torch.full((m + 4, n + 8), 3.0, device=fused.DEV)
+    out, status = binding.dvp_gemm_tn(a, b, alpha=0.5, out=buf[:m, :n], accumulate=accumulate)
+    torch.cuda.synchronize()
+    assert status.item() == 0
+    ref = 0.5 * (a.double() @ b.double().t()) + (3.0 if accumulate else 0.0)
+    # one rounding of the running sum per 16-wide step of k, one of the scaled value, one of the addition
+    bound = 2.0 ** -24 * (k / 16 + 2) * (a.double().abs() @ b.double().abs().t() + 3.0)
+    assert ((out.double() - ref).abs() <= bound).all()
+    assert (buf[m:] == 3.0).all() and (buf[:, n:] == 3.0).all()
