@@ -35,13 +35,13 @@ METRIC = "pruned_logprob_fwd_bwd_tokens_per_s"
 UNIT = "tokens/s"
 FALLBACK_HBM_GBS = 6650.0
 
-# DRAM bytes per launch of the row kernel (dram__bytes_read.sum + dram__bytes_write.sum
-# from one ncu capture of `bench.py --rows T ...`), keyed by (workload, rho); valid only for
+# DRAM bytes per call of the row kernel, two launches (dram__bytes_read.sum + dram__bytes_write.sum
+# of one ncu capture of a dvp_forward call on T rows of the workload), keyed by (workload, rho); valid only for
 # the kernel sources whose digest is recorded with it, scaled by rows to the full batch.
 NCU_TRAFFIC = {
-    ("c2_bf16_fwdbwd", 1e-4): {"digest": "47f036696d37ae2e", "T": 2048, "bytes": 1.663986e9 + 0.608635e9},
-    ("c2_bf16_fwdbwd", 1e-3): {"digest": "47f036696d37ae2e", "T": 2048, "bytes": 1.354420e9 + 0.603881e9},
-    ("c3_f32_heavy", 1e-4): {"digest": "47f036696d37ae2e", "T": 1024, "bytes": 2.148133e9 + 1.068105e9},
+    ("c2_bf16_fwdbwd", 1e-4): {"digest": "5e65b88e238fd975", "T": 2048, "bytes": 1.501346e9 + 0.573023e9},
+    ("c2_bf16_fwdbwd", 1e-3): {"digest": "5e65b88e238fd975", "T": 2048, "bytes": 1.313576e9 + 0.565076e9},
+    ("c3_f32_heavy", 1e-4): {"digest": "5e65b88e238fd975", "T": 1024, "bytes": 2.148167e9 + 1.017859e9},
 }
 
 

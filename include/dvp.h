@@ -148,10 +148,12 @@ typedef struct {
  *                 for a row without a valid sampled id)
  *   launch_hint   0 = library default; otherwise threads per block (a multiple
  *                 of 32, at most 512) in the low 16 bits, a kernel choice in the
- *                 next 8 bits, and the number of blocks that share one row (0, 1, 2
- *                 or 4; a thread-block cluster) in the top 8 bits.  Kernel choice:
- *                 0 or 2 the default kernel (one sweep, then revisits of the 32-byte
- *                 pieces of the row that can hold safe tokens); 3 or 4 (2-byte
+ *                 next 8 bits, and the number of blocks that share one row (0, 1, 2,
+ *                 4 or 8; a thread-block cluster) in the top 8 bits.  Kernel choice:
+ *                 0 or 2 the default kernel (64, 128, 256 or 512 threads, the largest
+ *                 not above the hint; one sweep with the masked sum under a guess of
+ *                 the maximum, then revisits of the 32-byte pieces of the row that can
+ *                 hold safe tokens); 3 or 4 (2-byte
  *                 logits, at most 256 threads, no cluster) the kernel that keeps
  *                 the candidates of the safe set in shared memory while the row
  *                 streams and reads nothing twice, with 3 or 4 blocks per SM;
