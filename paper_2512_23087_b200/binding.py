@@ -346,7 +346,7 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
                 weight_kind: int = DVP_WEIGHT_NONE, weight_lo: float = 0.0, weight_hi: float = float("inf")):
     """Pruned log-probabilities of the sampled tokens for the training and the
     inference logits (Def. 5.1, Def. 5.2), their log-ratio, and, when
-    ``upstream`` is given, dLoss/dlogits (Prop. 5.4) in the same launch.
+    ``upstream`` is given, dLoss/dlogits (Prop. 5.4) in the same call.
 
     ``mask_value`` (finite) switches to the App. A listing's semantics: pruned
     logits are replaced by it instead of by -inf; ``threshold_in_logits_dtype``
