@@ -58,9 +58,9 @@ def _kernel_digest(names=("dvp_common.cuh", "dvp_rows_impl.cuh")) -> str:
 # panels of 4096 rows): the first panel's three and a later panel's three (whose d_w contraction also reads
 # the d_w it adds to).  Valid for the sources whose digest is recorded; a step of P panels is taken as the
 # first panel's launches plus P - 1 times the later panel's.
-NCU_TRAFFIC_FUSED = {"digest": "607894dc2e40aeae", "H": 4096, "V": 151936, "panel": 4096,
-                     "first": (4.016951e9 + 2.557340e9) + (13.478416e9 + 0.144871e9) + (4.635654e9 + 2.545532e9),
-                     "later": (3.567931e9 + 2.542042e9) + (13.443569e9 + 0.145225e9) + (7.493283e9 + 2.471862e9)}
+NCU_TRAFFIC_FUSED = {"digest": "5009013b2377f941", "H": 4096, "V": 151936, "panel": 4096,
+                     "first": (4.615540e9 + 2.485369e9) + (13.608092e9 + 0.127318e9) + (5.593785e9 + 2.459819e9),
+                     "later": (4.840493e9 + 2.484551e9) + (12.678872e9 + 0.127140e9) + (8.013996e9 + 2.456163e9)}
 FUSED_SOURCES = ("dvp_gemm.cuh", "dvp_fused.cu", "dvp_panel.cuh")
 
 
