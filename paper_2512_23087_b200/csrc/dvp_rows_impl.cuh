@@ -450,6 +450,10 @@ struct Sweep1 {
     *bound = word;
     constexpr int kElems = Granule<TIn>::kElems;
     const uint64_t l2 = pack2(kLog2e, kLog2e), c2 = pack2(-c, -c);
+    // The step's terms are added up by themselves first: the thread that has met the maximum carries a sum of one or
+    // more, where every addition costs half a unit of 2^-23, whatever it adds.  (Term by term: ln Z of 700 rows of
+    // 151,936 bfloat16 1.8e-6 off at worst, 8e-7 this way; V = 151,936, forward, T = 8192: 930 / 931 us.)
+    uint64_t part = 0;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       float x[kElems], e[kElems];
@@ -459,7 +463,7 @@ struct Sweep1 {
         unpack2(fma2(pack2(x[j], x[j + 1]), l2, c2), e[j], e[j + 1]);
         e[j] = ex2(e[j]);
         e[j + 1] = ex2(e[j + 1]);
-        sum = add2(sum, pack2(e[j], e[j + 1]));
+        part = u + j == 0 ? pack2(e[j], e[j + 1]) : add2(part, pack2(e[j], e[j + 1]));
         // 2-byte logits: skipping the masked part where no lane of the warp has a safe token in the granule costs as
         // much as it saves (T = 8192 x V = 151,936: 996 against 986 us forward at 1e-4, 921 / 927 at 1e-3)
         if constexpr (sizeof(TIn) == 2)
@@ -473,6 +477,7 @@ struct Sweep1 {
         }
       }
     }
+    sum = add2(sum, part);
   }
 };
 

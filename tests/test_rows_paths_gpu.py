@@ -104,3 +104,29 @@ def test_outputs_left_out(kept, V, weighted):
         assert same(out["weight"], full.weight)
     if "logp_mp_i" in out:
         assert same(out["logp_mp_i"], full.infer.logp_mp)
+
+
+@pytest.mark.parametrize("dtype,V,hint", [("bf16", 151936, 64), ("bf16", 151936, 256), ("bf16", 151936, 256 | (2 << 24)),
+                                          ("f16", 50021, 64), ("f32", 262144, 512), ("f32", 40003, 64)])
+def test_full_sum_keeps_small_terms(dtype, V, hint):
+    """One token at 0 and all others at -17, where e^-17 = 0.69 * 2^-24 is lost when it is added to 1 by itself.  Each
+    step's terms (two granules a thread) are added up first: one rounding of the sum a step, log2(512) when the threads' sums
+    meet, and a few in the logarithm."""
+    elem = 4 if dtype == "f32" else 2
+    dt = inputs.torch_dtype(dtype)
+    train = torch.full((6, V), -17.0, dtype=dt, device=DEV)
+    for t, k in enumerate((3, 40, 700, 1023, 2047, 2050)):
+        train[t, k] = 0.0
+    ids = torch.tensor([3, V - 1, 5, 1023, -1, 2050], device=DEV)
+    res = binding.dvp_forward(train, ids, 1e-3, launch_hint=hint)
+    torch.cuda.synchronize()
+    z = train.double()
+    lse = torch.logsumexp(z, 1)
+    threads, parts = hint & 0xffff, max(1, hint >> 24)
+    steps = -(-V * elem // (64 * threads * parts))
+    bound = (steps + 9 + 4) * 2.0 ** -24
+    assert (res.train.lse.double() - lse).abs().max().item() <= bound
+    assert (res.train.log_cov.double() + lse).abs().max().item() <= bound   # the safe set is the one token: ln Z = -lse
+    has = ids >= 0
+    logp = z[has].gather(1, ids[has, None])[:, 0] - lse[has]
+    assert ((res.train.logp[has].double() - logp).abs() <= bound + 2.0 ** -24 * logp.abs()).all()
