@@ -20,6 +20,10 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
+// c = fl(m l), the reference of a sum of 2^{z l - c} whose largest z is m.  Clamped: m may be -inf or the lowest value of
+// its type, the fill of filtered logits, where m l is -inf and 2^{z l - c} would be +inf or NaN; clamped, it is 0.
+__device__ __forceinline__ float log2_reference(float m) { return fmaxf(m * kLog2e, -3.402823466e38f); }
+
 // ---- bounds-checking build (-DDVP_DEBUG_BOUNDS) ------------------------------------
 // Stands in for a memory checker: every shared-memory index of the row kernels' tables
 // (granule bounds, hot lists, candidate rings and lists, resident slots) and every global

@@ -431,7 +431,7 @@ struct Sweep1 {
   // the threshold is finite: rho = 0 keeps every finite logit, and the fill of a missing granule never passes
   __device__ __forceinline__ void set_guess(float m, double log_rho, int mode) {
     guess = m;
-    c = m * kLog2e;
+    c = log2_reference(m);
     const float t = fmaxf(threshold_of<TIn>(m, log_rho, mode), -FLT_MAX);
     tau = Ops::threshold(t);
     key = Ops::key(t);
@@ -717,7 +717,7 @@ __device__ __forceinline__ void row_sweep1(const RowView<TIn> &v, int hole, floa
       const float m = red.max(SweepOps<TIn>::value(sw.mx));
       if (m > sw.guess) {
         if (step > 0 && m - sw.guess > kWide) sw.wide = true;
-        const float f = ex2(sw.c - m * kLog2e);
+        const float f = ex2(sw.c - log2_reference(m));
         sw.sum = mul2(sw.sum, pack2(f, f));
         sw.set_guess(m, log_rho, mode);
         sw.first = step;
@@ -822,7 +822,7 @@ __device__ __forceinline__ SideStats row_stats(const RowView<TIn> &v, int a, dou
   st.member = has_a && st.z_a >= st.tau;
   st.e_a = st.member ? ex2((st.z_a - st.m) * kLog2e) : 0.f;
 
-  const float c = m * kLog2e;
+  const float c = log2_reference(m);
   float p0, p1;
   unpack2(sw.sum, p0, p1);
   float all = (p0 + p1) * ex2(sw.c - c) + ex2(fmaf(xe, kLog2e, -c));
