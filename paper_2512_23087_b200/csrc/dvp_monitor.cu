@@ -87,7 +87,7 @@ struct PairMoments {
   // Move the reference to a larger maximum.
   __device__ __forceinline__ void raise(float new_max) {
     if (new_max > m) {
-      const float cn = new_max * kLog2e;
+      const float cn = log2_reference(new_max);
       const float f = ex2(c - cn);  // c = -inf at the start: factor 0
       const uint64_t f2 = pack2(f, f);
       s = mul2(s, f2);

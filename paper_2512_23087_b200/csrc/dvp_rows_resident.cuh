@@ -451,7 +451,7 @@ __device__ __forceinline__ SideStats consume_side(const TIn *row, TGrad *grow, f
       if (valid[u]) cm = fmaxf(cm, v[u].max());
     if (cm > kNegInf) {
       if (cm > acc.m) {
-        const float cn = cm * kLog2e;
+        const float cn = log2_reference(cm);
         acc.s *= ex2(acc.c - cn);  // acc.c = -inf at the start: the factor is 0
         acc.m = cm;
         acc.c = cn;

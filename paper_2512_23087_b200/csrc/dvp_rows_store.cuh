@@ -256,7 +256,7 @@ __device__ __forceinline__ void absorb_stage_cs(const TIn *row, int V, const Sta
 
   if (cm > kNegInf) {
     if (cm > acc.m) {
-      const float cn = cm * kLog2e;
+      const float cn = log2_reference(cm);
       acc.s *= ex2(acc.c - cn);
       acc.m = cm;
       acc.c = cn;

@@ -24,7 +24,7 @@ __device__ __forceinline__ void absorb(const Stage<T, 2> &st, LogSum &acc, uint3
   const float cm = fmaxf(fmaxf(kNegInf, g0), g1);
   if (cm > kNegInf) {
     if (cm > acc.m) {
-      const float cn = cm * kLog2e;
+      const float cn = log2_reference(cm);
       acc.s *= ex2(acc.c - cn);  // acc.c = -inf at the start: the factor is 0
       acc.m = cm;
       acc.c = cn;
@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kBlk, 1024 / kBlk) dvp_two_sweeps_kernel(const
   const float x_tail = k_tail < V ? Storage<T>::widen(row[k_tail]) : kNegInf;
   if (x_tail > kNegInf) {
     if (x_tail > acc.m) {
-      const float cn = x_tail * kLog2e;
+      const float cn = log2_reference(x_tail);
       acc.s *= ex2(acc.c - cn);
       acc.m = x_tail;
       acc.c = cn;

@@ -55,3 +55,22 @@ def test_stores_of_short_products(m, n, k, accumulate):
     bound = 2.0 ** -24 * (k / 16 + 2) * (a.double().abs() @ b.double().abs().t() + 3.0)
     assert ((out.double() - ref).abs() <= bound).all()
     assert (buf[m:] == 3.0).all() and (buf[:, n:] == 3.0).all()
+
+
+@pytest.mark.parametrize("V", [32768, 32775])
+def test_inference_rows_of_mostly_fill(V):
+    """Filtered inference logits hold the lowest bfloat16, which times log2(e) is no float32; a thread may meet it first."""
+    w = inputs.WORKLOADS["c4_fused_lmhead"]
+    b = inputs.make_fused(w, seed=3, device=fused.DEV, T=24, H=128, V=V)
+    b.infer[:, :V // 2] = torch.finfo(torch.bfloat16).min
+    b.infer[1, :V - 3] = torch.finfo(torch.bfloat16).min
+    b.ids.copy_(torch.arange(24, device=fused.DEV) + V - 26)
+    r = binding.dvp_fused_lmhead_forward_backward(b.hidden, b.w_vocab, b.ids, 1e-4, b.upstream, infer_logits=b.infer)
+    torch.cuda.synchronize()
+    lse = torch.logsumexp(b.infer.double(), 1)
+    logp = b.infer.double().gather(1, b.ids[:, None])[:, 0] - lse
+    # float32 sums of at most 32775 terms and one rounding of the value itself
+    assert (r.infer.lse.double() - lse).abs().max().item() <= 4e-6
+    ok = logp > -1e30
+    assert ok.sum() >= 23 and (r.infer.logp.double() - logp)[ok].abs().max().item() <= 6e-6
+    assert torch.isfinite(r.d_hidden).all() and torch.isfinite(r.d_w).all()

@@ -38,3 +38,18 @@ def test_one_value_far_above_the_others(dtype):
     zi = z.clone()
     zi[1, 5] = 201.0
     _check(z.to(dtype), zi.to(dtype))
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("pad", [0, 1])
+def test_rows_of_mostly_fill(pad, dtype):
+    """Filtered logits hold the lowest value of their type, which times log2(e) is no float32; a thread may meet it first."""
+    V = 40000
+    g = torch.Generator(device=DEV).manual_seed(2)
+    z = torch.full((4, V), torch.finfo(dtype).min, dtype=torch.float64, device=DEV).to(dtype)
+    zi = torch.full((4, V + pad), torch.finfo(dtype).min, dtype=torch.float64, device=DEV).to(dtype)[:, :V]
+    for t, (lo, hi) in enumerate([(V // 2, V), (V - 5, V), (0, 9), (V // 3, V // 3 + 1000)]):
+        x = 2 * torch.randn(hi - lo, generator=g, device=DEV)
+        z[t, lo:hi] = x.to(dtype)
+        zi[t, lo:hi] = (x + 0.1 * torch.randn(hi - lo, generator=g, device=DEV)).to(dtype)
+    _check(z, zi)

@@ -49,3 +49,16 @@ def test_rows_of_mostly_fill(dtype, fill, hint, who):
             assert near(side.logp, (a - lse).clamp(min=-3.4028235e38) if fill == "lowest" else a - lse).all()
             inside = keep.gather(1, ids[:, None])[:, 0]
             assert near(side.logp_mp[inside], (a - lse_safe)[inside]).all() and (side.logp_mp[~inside] == -float("inf")).all()
+
+
+@pytest.mark.parametrize("hint", [0x11 << 16, 256 | (3 << 16), 256 | (4 << 16)])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_kernels_by_hint_on_rows_of_mostly_fill(dtype, hint):
+    V = 70016
+    z, windows = _filled(V, dtype, torch.finfo(dtype).min, seed=1)
+    ids = torch.tensor([lo for lo, _ in windows], device=DEV)
+    r = binding.dvp_forward(z, ids, 1e-3, infer_logits=z, launch_hint=hint)
+    torch.cuda.synchronize()
+    lse = torch.logsumexp(z.double(), 1)
+    assert ((r.train.lse.double() - lse).abs() <= 4e-6 + 2.0 ** -23 * lse.abs()).all()   # as above
+    assert torch.equal(r.train.lse, r.infer.lse) and torch.isfinite(r.train.log_cov).all()
