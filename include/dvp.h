@@ -137,7 +137,10 @@ typedef struct {
  *   upstream      device [T] float32: g_t = dLoss / d ln pi^mp_train(a_t)
  *   grad_train    device [T, ld_grad] of grad_dtype: g_t (1[k=a] - pi^mp(k))
  *                 on V_S, 0 off it, the whole row 0 when a is not in V_S;
- *                 rounded to nearest-even in grad_dtype
+ *                 rounded to nearest-even in grad_dtype.  It may take the
+ *                 place of train_logits or infer_logits (the same type, base
+ *                 and stride) when no `mask` is asked for; other overlaps
+ *                 with the logits are not allowed
  *   log_ratio     device [T] float32: ln pi^mp_train(a) - ln pi^mp_infer(a);
  *                 -inf when a is outside V_S (importance ratio zero, remark
  *                 after Thm. 5.3), +inf when a is in V_S but outside V'_S

@@ -1319,6 +1319,15 @@ static inline bool aligned32(const void *base, long long ld, size_t elem) {
   return base == nullptr || (((uintptr_t)base % 32 == 0) && ((ld * (long long)elem) % 32 == 0));
 }
 
+// Does the gradient take the place of (a part of) these logits?
+template <typename TIn, typename TGrad>
+static inline bool grad_over(const RowParams &p, const void *logits, long long ld) {
+  if (!p.grad || !logits) return false;
+  const uintptr_t g = (uintptr_t)p.grad, z = (uintptr_t)logits;
+  return g < z + (size_t)((p.T - 1) * ld + p.V) * sizeof(TIn) &&
+         z < g + (size_t)((p.T - 1) * p.ld_grad + p.V) * sizeof(TGrad);
+}
+
 template <typename TIn, typename TGrad, int kBlk, Grad kGrad>
 static cudaError_t launch_rows_vec(const RowParams &p, long long t0, long long n, int log_parts, size_t smem,
                                    cudaStream_t s) {
@@ -1341,7 +1350,8 @@ static cudaError_t launch_rows_vec(const RowParams &p, long long t0, long long n
     attr[cfg.numAttrs].val.clusterDim.y = 1;
     attr[cfg.numAttrs++].val.clusterDim.z = 1;
   }
-  if (p.side == kSideTrain) {  // may begin while the inference rows' launch ends
+  // may begin while the inference rows' launch ends; not where the gradient overwrites inference rows
+  if (p.side == kSideTrain && !grad_over<TIn, TGrad>(p, p.infer, p.ld_infer)) {
     attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
   }
@@ -1535,7 +1545,11 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
       if (e != cudaErrorNotSupported) return e;
     }
   }
-  if (hot_ok && smem <= 200 * 1024) {
+  // Weights with no output to pass ln pi^mp_infer(a) through (launch_rows_both) and a gradient in place of logits that
+  // it would be written over: both rows of a token in one block.
+  const bool no_place = weighted && !p.out_i.logp_mp && !p.log_ratio && !p.weight_out &&
+                        (grad_over<TIn, TGrad>(p, p.train, p.ld_train) || grad_over<TIn, TGrad>(p, p.infer, p.ld_infer));
+  if (hot_ok && smem <= 200 * 1024 && !no_place) {
     return launch_rows_both<TIn, TGrad>(p, loose, log_parts, threads, smem, s);
   }
   dvp_row_kernel_scalar<TIn, TGrad><<<(unsigned)p.T, 512, 0, s>>>(p);

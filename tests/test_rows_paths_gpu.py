@@ -130,3 +130,36 @@ def test_full_sum_keeps_small_terms(dtype, V, hint):
     has = ids >= 0
     logp = z[has].gather(1, ids[has, None])[:, 0] - lse[has]
     assert ((res.train.logp[has].double() - logp).abs() <= bound + 2.0 ** -24 * logp.abs()).all()
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("place", ["train", "infer"])
+@pytest.mark.parametrize("T,V", [(5, 151936), (700, 20000), (37, 5003)])
+def test_gradient_in_place_of_logits(T, V, place, weighted):
+    """The gradient may take the place of either matrix, also where ln pi^mp_infer(a) has no output to pass through."""
+    b = inputs.make_rows(W["c2_bf16_fwdbwd"], seed=T, device=DEV, T=T, V=V)
+    kw = dict(weight_kind=binding.DVP_WEIGHT_TRUNCATE, weight_hi=1.01) if weighted else {}
+    full = binding.dvp_forward(b.train, b.ids, 1e-3, infer_logits=b.infer, upstream=b.upstream, **kw)
+    train, infer = b.train.clone(), b.infer.clone()
+    grad = train if place == "train" else infer
+    res = binding.dvp_forward(train, b.ids, 1e-3, infer_logits=infer, upstream=b.upstream, grad_train=grad, **kw)
+    torch.cuda.synchronize()
+    assert torch.equal(grad, full.grad_train) and torch.equal(res.log_ratio, full.log_ratio)
+    assert torch.equal(res.train.lse, full.train.lse) and torch.equal(res.infer.lse, full.infer.lse)
+    train.copy_(b.train), infer.copy_(b.infer)
+    a = binding.ForwardArgs()
+    a.struct_size, a.logits_dtype, a.grad_dtype = ctypes.sizeof(binding.ForwardArgs), binding.DVP_BF16, binding.DVP_BF16
+    a.T, a.V, a.rho = T, V, 1e-3
+    a.ld_train = a.ld_infer = a.ld_grad = V
+    a.train_logits, a.infer_logits, a.ids = train.data_ptr(), infer.data_ptr(), b.ids.data_ptr()
+    a.upstream, a.grad_train = b.upstream.data_ptr(), grad.data_ptr()
+    if weighted:
+        a.weight_kind, a.weight_hi = binding.DVP_WEIGHT_TRUNCATE, 1.01
+    a.stream = torch.cuda.current_stream().cuda_stream
+    assert binding.load_library().dvp_forward(ctypes.byref(a)) == binding.DVP_OK
+    torch.cuda.synchronize()
+    if weighted:   # one kernel for both rows, sums in another order: one rounding of bfloat16 apart at most
+        d = (grad.float() - full.grad_train.float()).abs()
+        assert (d <= 2.0 ** -7 * full.grad_train.float().abs() + 1e-30).all()
+    else:
+        assert torch.equal(grad, full.grad_train)
