@@ -322,6 +322,11 @@ def _with_mask(side, like: torch.Tensor, T: int, V: int):
     return o, addresses[:7] + (o.mask.data_ptr(), addresses[8])
 
 
+def _addresses(side):
+    """The addresses of a side's tensors, in the order of ``dvp_side_out``."""
+    return tuple(_address(getattr(side, n)) for n in _SIDE_FIELDS)
+
+
 _NO_SIDE = (0,) * 9
 
 
@@ -371,14 +376,15 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
             raise ValueError("infer_logits must match train_logits in dtype and shape")
     if out is not None:
         res = out
+        at = [_addresses(res.train)] + ([_addresses(res.infer)] if has_infer else [])
     else:
         sides, rest, flags = _token_outputs(train_logits, T, 2 if has_infer else 1, has_infer + weighted)
         if want_mask:
             sides = [_with_mask(side, train_logits, T, V) for side in sides]
         res = SimpleNamespace(train=sides[0][0], infer=sides[1][0] if has_infer else None,
                               log_ratio=rest[0] if has_infer else None,
-                              flags=flags, grad_train=None,
-                              _train_addresses=sides[0][1], _infer_addresses=sides[1][1] if has_infer else _NO_SIDE)
+                              flags=flags, grad_train=None)
+        at = [addresses for _, addresses in sides]
         if weighted:
             res.weight = rest[-1]
     if weighted and getattr(res, "weight", None) is None:
@@ -401,8 +407,8 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
     st = packed["dvp_forward"](_FORWARD_PACK.pack(
         _FORWARD_PACK.size, _DTYPES[dtype], grad_code, _id_dtype(ids), T, V, train_logits.stride(0),
         infer_logits.stride(0) if has_infer else 0, grad_ld, float(rho), train_logits.data_ptr(),
-        _address(infer_logits), ids.data_ptr(), _address(upstream), _address(grad_train), *res._train_addresses,
-        *(res._infer_addresses if has_infer else _NO_SIDE), res.log_ratio.data_ptr() if has_infer else 0,
+        _address(infer_logits), ids.data_ptr(), _address(upstream), _address(grad_train), *at[0],
+        *(at[1] if has_infer else _NO_SIDE), res.log_ratio.data_ptr() if has_infer else 0,
         res.flags.data_ptr(), _stream(stream), launch_hint, mode, _float32(mask_value) if mask_value is not None else 0.0,
         int(weight_kind), _float32(weight_lo), _float32(weight_hi), res.weight.data_ptr() if weighted else 0))
     if st != DVP_OK:

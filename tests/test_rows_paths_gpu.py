@@ -1,5 +1,6 @@
 """Paths of the row kernel that depend on sizes and on which outputs are asked for: a guess of the maximum that is far off,
 rows split over several blocks, and the places through which ln pi^mp_infer(a) passes between the two launches."""
+import copy
 import ctypes
 import dataclasses
 
@@ -163,3 +164,21 @@ def test_gradient_in_place_of_logits(T, V, place, weighted):
         assert (d <= 2.0 ** -7 * full.grad_train.float().abs() + 1e-30).all()
     else:
         assert torch.equal(grad, full.grad_train)
+
+
+def test_out_names_the_tensors_it_holds():
+    """A copy of a result owns its buffers, and a tensor put into a result takes the next call's values."""
+    b, other = (inputs.make_rows(W["c2_bf16_fwdbwd"], seed=s, device=DEV, T=20, V=5003) for s in (1, 2))
+    first = binding.dvp_forward(b.train, b.ids, 1e-3, infer_logits=b.infer, want_mask=True)
+    kept = copy.deepcopy(first)
+    want = binding.dvp_forward(other.train, other.ids, 1e-3, infer_logits=other.infer, want_mask=True)
+    reused = copy.deepcopy(first)
+    old, reused.infer.lse = reused.infer.lse, torch.zeros_like(reused.infer.lse)
+    binding.dvp_forward(other.train, other.ids, 1e-3, infer_logits=other.infer, out=reused)
+    torch.cuda.synchronize()
+    for side in ("train", "infer"):
+        for n in ("max", "lse", "lse_safe", "logp", "logp_mp", "comp_mp", "count", "log_cov", "mask"):
+            assert torch.equal(getattr(getattr(reused, side), n), getattr(getattr(want, side), n)), n
+            assert torch.equal(getattr(getattr(first, side), n), getattr(getattr(kept, side), n)), n
+    assert torch.equal(reused.flags, want.flags) and torch.equal(reused.log_ratio, want.log_ratio)
+    assert torch.equal(old, kept.infer.lse)
