@@ -335,6 +335,16 @@ def _float32(x: float) -> float:
     return ctypes.c_float(x).value
 
 
+def _uint32(x) -> int:
+    """What a uint32_t holds of x, as ctypes takes it: struct refuses to pack what is out of range, where the library's
+    own check is to answer."""
+    return x & 0xffffffff
+
+
+def _int32(x) -> int:
+    return (int(x) + 0x80000000 & 0xffffffff) - 0x80000000
+
+
 def _id_dtype(ids: torch.Tensor) -> int:
     if ids.dtype == torch.int64:
         return DVP_ID_I64
@@ -409,8 +419,8 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
         infer_logits.stride(0) if has_infer else 0, grad_ld, float(rho), train_logits.data_ptr(),
         _address(infer_logits), ids.data_ptr(), _address(upstream), _address(grad_train), *at[0],
         *(at[1] if has_infer else _NO_SIDE), res.log_ratio.data_ptr() if has_infer else 0,
-        res.flags.data_ptr(), _stream(stream), launch_hint, mode, _float32(mask_value) if mask_value is not None else 0.0,
-        int(weight_kind), _float32(weight_lo), _float32(weight_hi), res.weight.data_ptr() if weighted else 0))
+        res.flags.data_ptr(), _stream(stream), _uint32(launch_hint), mode,
+        _float32(mask_value) if mask_value is not None else 0.0, _uint32(int(weight_kind)), _float32(weight_lo), _float32(weight_hi), res.weight.data_ptr() if weighted else 0))
     if st != DVP_OK:
         raise DvpError(st, "dvp_forward")
     return res
@@ -436,7 +446,7 @@ def dvp_backward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, upst
         train_logits.stride(0), grad_train.stride(0), float(rho), train_logits.data_ptr(), ids.data_ptr(),
         upstream.data_ptr(), saved.train.max.data_ptr(), saved.train.lse_safe.data_ptr(),
         saved.train.comp_mp.data_ptr() if use_comp else 0, saved.flags.data_ptr(), grad_train.data_ptr(),
-        _stream(stream), launch_hint, mode, _float32(mask_value) if mask_value is not None else 0.0, 0))
+        _stream(stream), _uint32(launch_hint), mode, _float32(mask_value) if mask_value is not None else 0.0, 0))
     if st != DVP_OK:
         raise DvpError(st, "dvp_backward")
     return grad_train
@@ -509,7 +519,7 @@ def _fused_args(hidden, w_vocab, ids, rho, upstream, infer_logits, d_w, accumula
         _FUSED_PACK.size, _id_dtype(ids), T, H, V, hidden.stride(0), w_vocab.stride(0),
         infer_logits.stride(0) if has_infer else 0, res.d_hidden.stride(0), res.d_w.stride(0), float(rho),
         hidden.data_ptr(), w_vocab.data_ptr(), _address(infer_logits), ids.data_ptr(), _address(upstream),
-        res.d_hidden.data_ptr(), res.d_w.data_ptr(), int(accumulate_dw), int(panel_rows), *sides[0][1],
+        res.d_hidden.data_ptr(), res.d_w.data_ptr(), _int32(accumulate_dw), _int32(panel_rows), *sides[0][1],
         *(sides[1][1] if has_infer else _NO_SIDE), res.log_ratio.data_ptr() if has_infer else 0, res.flags.data_ptr(),
         0, 0, _stream(stream), 0, 0.0, 0.0, 0))
     return a, res

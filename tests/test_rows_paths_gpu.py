@@ -182,3 +182,19 @@ def test_out_names_the_tensors_it_holds():
             assert torch.equal(getattr(getattr(first, side), n), getattr(getattr(kept, side), n)), n
     assert torch.equal(reused.flags, want.flags) and torch.equal(reused.log_ratio, want.log_ratio)
     assert torch.equal(old, kept.infer.lse)
+
+
+def test_numbers_beyond_their_c_type_are_the_library_s_to_refuse():
+    b = inputs.make_rows(W["c2_bf16_fwdbwd"], seed=1, device=DEV, T=4, V=512)
+    saved = binding.dvp_forward(b.train, b.ids, 1e-3, infer_logits=b.infer)
+    f = inputs.make_fused(W["c4_fused_lmhead"], seed=1, device=DEV, T=4, H=64, V=512)
+    for call in (lambda: binding.dvp_forward(b.train, b.ids, 1e-3, launch_hint=-1),
+                 lambda: binding.dvp_forward(b.train, b.ids, 1e-3, infer_logits=b.infer, upstream=b.upstream, weight_kind=-1),
+                 lambda: binding.dvp_backward(b.train, b.ids, 1e-3, b.upstream, saved, launch_hint=-1),
+                 lambda: binding.dvp_fused_lmhead_forward_backward(f.hidden, f.w_vocab, f.ids, 1e-3, f.upstream,
+                                                                   panel_rows=2 ** 31 + 128)):
+        with pytest.raises(binding.DvpError) as e:
+            call()
+        assert e.value.status == binding.DVP_ERR_INVALID_ARG
+    with pytest.raises(TypeError):
+        binding.dvp_forward(b.train, b.ids, 1e-3, launch_hint=256.0)
