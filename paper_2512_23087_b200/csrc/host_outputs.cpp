@@ -7,7 +7,9 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/object_ptr.h>
 
 namespace {
 
@@ -29,29 +31,28 @@ PyObject *outputs(PyObject *, PyObject *const *args, Py_ssize_t n_args) {
   }
   const int64_t T = PyLong_AsLongLong(args[1]), floats = PyLong_AsLongLong(args[2]), counts = PyLong_AsLongLong(args[3]);
   if (PyErr_Occurred()) return nullptr;
-  const int64_t rows = floats + counts + 1, stride = (T + 3) / 4 * 16;
-  try {
-    const at::Tensor buf =
-        at::empty({rows * stride}, THPVariable_Unpack(args[0]).options().dtype(at::kByte).requires_grad(false));
-    const c10::Storage &storage = buf.storage();
-    const c10::DispatchKeySet keys = buf.key_set();
-    PyObject *tensors = PyTuple_New(rows);
-    if (!tensors) return nullptr;
-    for (int64_t i = 0; i < rows; ++i) {
-      const at::ScalarType type = i < floats ? at::kFloat : i < floats + counts ? at::kInt : at::kByte;
-      PyObject *t = THPVariable_Wrap(row_view(storage, keys, type, i, stride, T));
-      if (!t) {
-        Py_DECREF(tensors);
-        return nullptr;
-      }
-      PyTuple_SET_ITEM(tensors, i, t);
-    }
-    return Py_BuildValue("(NLL)", tensors, static_cast<long long>(reinterpret_cast<uintptr_t>(buf.data_ptr())),
-                         static_cast<long long>(stride));
-  } catch (const std::exception &e) {
-    PyErr_SetString(PyExc_RuntimeError, e.what());
+  if (T < 0 || T >= (int64_t(1) << 56)) {
+    PyErr_Format(PyExc_RuntimeError, "outputs: there are no vectors of %lld elements", static_cast<long long>(T));
     return nullptr;
   }
+  // torch's own exception types reach Python, out-of-memory errors among them
+  HANDLE_TH_ERRORS
+  const int64_t rows = floats + counts + 1, stride = (T + 3) / 4 * 16;
+  const at::Tensor buf =
+      at::empty({rows * stride}, THPVariable_Unpack(args[0]).options().dtype(at::kByte).requires_grad(false));
+  const c10::Storage &storage = buf.storage();
+  const c10::DispatchKeySet keys = buf.key_set();
+  THPObjectPtr tensors(PyTuple_New(rows));
+  if (!tensors) return nullptr;
+  for (int64_t i = 0; i < rows; ++i) {
+    const at::ScalarType type = i < floats ? at::kFloat : i < floats + counts ? at::kInt : at::kByte;
+    PyObject *t = THPVariable_Wrap(row_view(storage, keys, type, i, stride, T));
+    if (!t) return nullptr;
+    PyTuple_SET_ITEM(tensors.get(), i, t);
+  }
+  return Py_BuildValue("(NLL)", tensors.release(), static_cast<long long>(reinterpret_cast<uintptr_t>(buf.data_ptr())),
+                       static_cast<long long>(stride));
+  END_HANDLE_TH_ERRORS
 }
 
 PyMethodDef methods[] = {{"outputs", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(outputs)), METH_FASTCALL,

@@ -28,3 +28,18 @@ def test_outputs_refuses_other_arguments():
     binding.load_library()
     with pytest.raises(TypeError):
         binding._host.outputs(1, 2, 3, 4)
+
+
+@pytest.mark.parametrize("T", [-1, -8, 2 ** 60])
+def test_outputs_refuses_lengths_no_vector_has(T):
+    binding.load_library()
+    with pytest.raises(RuntimeError, match="elements"):
+        binding._host.outputs(torch.empty(1), T, 3, 2)
+
+
+@pytest.mark.gpu
+def test_out_of_memory_keeps_its_type():
+    binding.load_library()
+    with pytest.raises(torch.OutOfMemoryError):   # 2^44 bytes: the allocator refuses
+        binding._host.outputs(torch.empty(1, device="cuda:0"), 2 ** 40, 3, 0)
+    assert binding._host.outputs(torch.empty(1, device="cuda:0"), 5, 3, 0)[2] == 32
