@@ -210,6 +210,10 @@ def load_library() -> ctypes.CDLL:
         except ImportError as e:
             raise RuntimeError("the helper _host.so is missing or does not load: build it with "
                                "`python -m paper_2512_23087_b200.build`") from e
+        from .build import host_target
+        if getattr(_host, "built_for", None) != f"[built for {host_target()}]":
+            raise RuntimeError(f"the helper _host.so was built for another interpreter or torch than {host_target()}: build "
+                               "it with `python -m paper_2512_23087_b200.build`")
         lib = ctypes.CDLL(LIB_PATH)
         lib.dvp_forward.argtypes = [ctypes.POINTER(ForwardArgs)]
         lib.dvp_forward.restype = ctypes.c_int

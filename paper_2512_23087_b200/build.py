@@ -3,7 +3,7 @@
 ``build()`` compiles every ``csrc/*.cu`` to an object file (in parallel), links
 ``libdvp_b200.so`` beside this file and compiles ``_host.so``, the Python helper
 that lays a call's outputs over one allocation.  Objects are rebuilt only when a
-source or header is newer.  Run as ``python -m paper_2512_23087_b200.build``;
+source or header is newer, ``_host.so`` also after a change of interpreter or torch.  Run as ``python -m paper_2512_23087_b200.build``;
 ``--debug-bounds`` builds the bounds-checking library instead.
 """
 from __future__ import annotations
@@ -42,17 +42,33 @@ def _newest_header() -> float:
 HOST = os.path.join(HERE, "_host.so")
 
 
-def build_host() -> str:
+def host_target() -> str:
+    """What ``_host.so`` has to be built for: it uses torch's C++ classes and this interpreter's, whose layouts differ from
+    version to version.  It carries this text, and ``binding.load_library`` refuses one built for something else."""
+    import torch
+    return f"{sys.implementation.cache_tag} torch {torch.__version__}"
+
+
+def _host_is_for(target: str) -> bool:
+    try:
+        with open(HOST, "rb") as f:
+            return f"[built for {target}]".encode() in f.read()
+    except OSError:
+        return False
+
+
+def build_host(force: bool = False) -> str:
     """The Python helper ``_host`` (g++ against this interpreter's and torch's headers)."""
     src = os.path.join(CSRC, "host_outputs.cpp")
-    if os.path.exists(HOST) and os.path.getmtime(HOST) >= os.path.getmtime(src):
+    target = host_target()
+    if not force and _host_is_for(target) and os.path.getmtime(HOST) >= os.path.getmtime(src):
         return HOST
     import sysconfig
     import torch
     base = os.path.join(os.path.dirname(torch.__file__))
     tmp = HOST + f".{os.getpid()}.tmp"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", src, "-o", tmp,
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           f'-DDVP_HOST_TARGET="{target}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
            "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(base, "include"),
            "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
            "-L", os.path.join(base, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"]
@@ -102,8 +118,7 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
             for log in ex.map(run, jobs):
                 if verbose and log:
                     print(log, file=sys.stderr)
-    if not debug_bounds:
-        build_host()
+    build_host(force and not debug_bounds)
     if jobs or not os.path.exists(lib):
         tmp = lib + f".{os.getpid()}.tmp"
         run([nvcc, "-shared", "-o", tmp, *objs, "-lcudart"])

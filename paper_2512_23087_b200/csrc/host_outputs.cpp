@@ -62,4 +62,13 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_host", nullptr, -1, methods, null
 
 }  // namespace
 
-extern "C" __attribute__((visibility("default"))) PyObject *PyInit__host() { return PyModule_Create(&module); }
+// PyInit__host: the module says what it was built for (build.py looks for the text in the file, binding.py asks the module)
+extern "C" __attribute__((visibility("default"))) PyObject *PyInit__host() {
+  static const char text[] = "[built for " DVP_HOST_TARGET "]";
+  PyObject *m = PyModule_Create(&module);
+  if (m && PyModule_AddStringConstant(m, "built_for", text) != 0) {
+    Py_DECREF(m);
+    return nullptr;
+  }
+  return m;
+}

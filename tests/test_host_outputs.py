@@ -43,3 +43,34 @@ def test_out_of_memory_keeps_its_type():
     with pytest.raises(torch.OutOfMemoryError):   # 2^44 bytes: the allocator refuses
         binding._host.outputs(torch.empty(1, device="cuda:0"), 2 ** 40, 3, 0)
     assert binding._host.outputs(torch.empty(1, device="cuda:0"), 5, 3, 0)[2] == 32
+
+
+def test_helper_is_rebuilt_for_another_torch(monkeypatch, tmp_path):
+    """A helper built against another torch (or interpreter) lays tensors over the wrong layout: it is neither kept by the
+    build nor used by the binding."""
+    monkeypatch.setattr(build, "HOST", str(tmp_path / "_host.so"))
+    monkeypatch.setattr(build.subprocess, "run", _fake_compiler(tmp_path))
+    build.build_host()
+    first = (tmp_path / "count").read_text()
+    build.build_host()
+    assert (tmp_path / "count").read_text() == first == "1"
+    monkeypatch.setattr(torch, "__version__", "9.9.9")
+    build.build_host()
+    assert (tmp_path / "count").read_text() == "2"
+    build.build_host(force=True)
+    assert (tmp_path / "count").read_text() == "3"
+    monkeypatch.setattr(binding, "_lib", None)
+    with pytest.raises(RuntimeError, match="built for another"):
+        binding.load_library()
+
+
+def _fake_compiler(tmp_path):
+    """Stands in for g++: writes the text that the helper would carry, and counts."""
+    def run(cmd, **kw):
+        n = tmp_path / "count"
+        n.write_text(str(int(n.read_text()) + 1 if n.exists() else 1))
+        define = next(c for c in cmd if c.startswith("-DDVP_HOST_TARGET="))
+        with open(cmd[cmd.index("-o") + 1], "wb") as f:
+            f.write(b"[built for " + define.split("=", 1)[1].strip('"').encode() + b"]")
+        return build.subprocess.CompletedProcess(cmd, 0, "", "")
+    return run
