@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kBlk, 1024 / kBlk) dvp_two_sweeps_kernel(const
       p.flags[t] = (uint8_t)((st.member ? DVP_FLAG_IN_TRAIN : 0) | (has_id ? 0 : DVP_FLAG_NO_ID) |
                              (bad_id ? DVP_FLAG_BAD_ID : 0));
   }
-  if (p.out_t.mask) write_mask_row<T>(row, V, st.tau, p.out_t.mask + t * ((p.V + 31) / 32));
+  if (p.out_t.mask) write_mask_row<T>(row, V, st.tau, p.out_t.mask + t * ((p.V + 31) / 32), 0, 1);
   if (blockIdx.x == gridDim.x - 1 && tid == 0) end_after(true);  // the others leave their place to the next blocks
 }
 

@@ -198,3 +198,17 @@ def test_numbers_beyond_their_c_type_are_the_library_s_to_refuse():
         assert e.value.status == binding.DVP_ERR_INVALID_ARG
     with pytest.raises(TypeError):
         binding.dvp_forward(b.train, b.ids, 1e-3, launch_hint=256.0)
+
+
+@pytest.mark.parametrize("hint", [0, 64, 256, 256 | (2 << 24), 512 | (8 << 24)])
+@pytest.mark.parametrize("V", [1, 31, 33, 1023, 1025, 32767, 70001])
+def test_mask_words(V, hint):
+    """Ends of words, of a warp's 32 words, and rows whose blocks share the mask; rho = 0 keeps everything."""
+    b = inputs.make_rows(W["c2_bf16_fwdbwd"], seed=V, device=DEV, T=3, V=V)
+    for rho in (1e-3, 0.0):
+        res = binding.dvp_forward(b.train, b.ids, rho, infer_logits=b.infer, want_mask=True, launch_hint=hint)
+        torch.cuda.synchronize()
+        for side, z in ((res.train, b.train), (res.infer, b.infer)):
+            z = z.double().cpu()
+            keep = z >= z.max(1, keepdim=True).values + (torch.log(torch.tensor(rho, dtype=torch.float64)) if rho else -float("inf"))
+            assert (parity.unpack_mask(side.mask, V) == keep.numpy()).all()
