@@ -144,9 +144,8 @@ __device__ __forceinline__ float max_of(const Granule<TIn> &g, const Granule<TIn
   }
 }
 
+// One element of each row, under references that are at least as large.
 __device__ __forceinline__ void absorb_one(float x, float y, PairMoments &a, PairMoments &b) {
-  a.raise(x);
-  b.raise(y);
   // the pair's other element: -inf has no weight, but it may not be multiplied
   const float wa = ex2(fmaf(x, kLog2e, -a.c)), wb = ex2(fmaf(y, kLog2e, -b.c)), d = y - x;
   a.s = add2(a.s, pack2(wa, 0.f));
@@ -212,7 +211,12 @@ __global__ void __launch_bounds__(256, sizeof(TIn) == 2 ? 4 : 3) dvp_monitor_ker
       if (second) absorb_granules<TIn>(t1, i1, a, b);
     }
     const int k = tid < head ? tid : tid + n_full * kElems;  // fewer than 64 of them
-    if (k < V) absorb_one(Storage<TIn>::widen(zt[k]), Storage<TIn>::widen(zi[k]), a, b);
+    if (k < V) {
+      const float x = Storage<TIn>::widen(zt[k]), y = Storage<TIn>::widen(zi[k]);
+      a.raise(x);
+      b.raise(y);
+      absorb_one(x, y, a, b);
+    }
   } else {
     float mt = kNegInf, mi = kNegInf;
     for (long long k = tid; k < p.V; k += n_thr) {
@@ -221,8 +225,17 @@ __global__ void __launch_bounds__(256, sizeof(TIn) == 2 ? 4 : 3) dvp_monitor_ker
     }
     a.raise(mt);
     b.raise(mi);
-    for (long long k = tid; k < p.V; k += n_thr)
-      absorb_one(Storage<TIn>::widen(zt[k]), Storage<TIn>::widen(zi[k]), a, b);
+    // the maximum is known: no reference moves in this pass, and two elements go through one instruction (bfloat16
+    // 700 x 20,000: 46 -> 33 us, 1,000 x 50,021: 167 -> 124; float32 700 x 20,000: 58 -> 43)
+    long long k = tid;
+    for (; k + n_thr < p.V; k += 2 * n_thr) {
+      const uint64_t xx = pack2(Storage<TIn>::widen(zt[k]), Storage<TIn>::widen(zt[k + n_thr]));
+      const uint64_t yy = pack2(Storage<TIn>::widen(zi[k]), Storage<TIn>::widen(zi[k + n_thr]));
+      const uint64_t d = fma2(xx, pack2(-1.f, -1.f), yy);
+      a.absorb(xx, d);
+      b.absorb(yy, d);
+    }
+    if (k < p.V) absorb_one(Storage<TIn>::widen(zt[k]), Storage<TIn>::widen(zi[k]), a, b);
   }
   const Moments ra = block_reduce(a.sum(), scratch);
   const Moments rb = block_reduce(b.sum(), scratch);
