@@ -79,25 +79,12 @@ __device__ __forceinline__ Moments block_reduce(Moments v, float *scratch) {
   return r;
 }
 
-// The state of one policy over a thread's elements; the sums are pairs, of the even and the odd elements.
-struct PairMoments {
-  float m, c;
+// The sums of one policy, as pairs: of the even and of the odd elements.
+struct PairSums {
   uint64_t s, a, b;
 
-  // Move the reference to a larger maximum.
-  __device__ __forceinline__ void raise(float new_max) {
-    if (new_max > m) {
-      const float cn = log2_reference(new_max);
-      const float f = ex2(c - cn);  // c = -inf at the start: factor 0
-      const uint64_t f2 = pack2(f, f);
-      s = mul2(s, f2);
-      a = mul2(a, f2);
-      b = mul2(b, f2);
-      m = new_max;
-      c = cn;
-    }
-  }
-  __device__ __forceinline__ void absorb(uint64_t x, uint64_t d) {
+  // two logits x, d = z' - z of both, reference c
+  __device__ __forceinline__ void absorb(uint64_t x, uint64_t d, float c) {
     float w0, w1;
     unpack2(fma2(x, pack2(kLog2e, kLog2e), pack2(-c, -c)), w0, w1);
     const uint64_t w = pack2(ex2(w0), ex2(w1));
@@ -105,32 +92,64 @@ struct PairMoments {
     a = fma2(w, x, a);
     b = fma2(w, d, b);
   }
+};
+
+// The state of one policy over a thread's elements.  The maximum itself is kept for float32 logits only: with 2-byte
+// logits the register is worth more (64 x 151,936: 24.6 -> 22.6 us; T = 4096: 471 -> 453), with float32 ones the code
+// without it spills (2,500 x 100,000: 310 against 314 us).
+template <typename TIn>
+struct PairMoments {
+  static constexpr bool kKeepMax = sizeof(TIn) == 4;
+  float m, c;
+  PairSums q;
+
+  // Move the reference to a larger maximum.
+  __device__ __forceinline__ void raise(float new_max) {
+    if constexpr (kKeepMax) {
+      if (new_max > m) {
+        rescale(log2_reference(new_max));
+        m = new_max;
+      }
+    } else {
+      const float cn = log2_reference(new_max);
+      if (cn > c) rescale(cn);
+    }
+  }
+  __device__ __forceinline__ void rescale(float cn) {
+    const float f = ex2(c - cn);  // c = -inf at the start: factor 0
+    const uint64_t f2 = pack2(f, f);
+    q.s = mul2(q.s, f2);
+    q.a = mul2(q.a, f2);
+    q.b = mul2(q.b, f2);
+    c = cn;
+  }
   __device__ __forceinline__ Moments sum() const {
-    Moments r = {m, c, 0.f, 0.f, 0.f};
+    Moments r = {kKeepMax ? m : c / kLog2e, c, 0.f, 0.f, 0.f};  // m: to float32 rounding, for a correction of 1e-8 of it
     float lo, hi;
-    unpack2(s, lo, hi);
+    unpack2(q.s, lo, hi);
     r.s = lo + hi;
-    unpack2(a, lo, hi);
+    unpack2(q.a, lo, hi);
     r.a = lo + hi;
-    unpack2(b, lo, hi);
+    unpack2(q.b, lo, hi);
     r.b = lo + hi;
     return r;
   }
 };
 
+__device__ __forceinline__ uint64_t difference(uint64_t x, uint64_t y) { return fma2(x, pack2(-1.f, -1.f), y); }
+
 template <typename TIn>
-__device__ __forceinline__ void absorb_granules(const Granule<TIn> &gt, const Granule<TIn> &gi, PairMoments &a,
-                                                PairMoments &b) {
+__device__ __forceinline__ void absorb_granules(const Granule<TIn> &gt, const Granule<TIn> &gi, float ca, float cb,
+                                                PairSums &a, PairSums &b) {
   constexpr int kElems = Granule<TIn>::kElems;
   float x[kElems], y[kElems];
   gt.get(x);
   gi.get(y);
 #pragma unroll
   for (int j = 0; j < kElems; j += 2) {
-    const uint64_t xx = pack2(x[j], x[j + 1]), yy = pack2(y[j], y[j + 1]);
-    const uint64_t d = fma2(xx, pack2(-1.f, -1.f), yy);
-    a.absorb(xx, d);
-    b.absorb(yy, d);
+    const uint64_t xx = pack2(x[j], x[j + 1]), yy = pack2(y[j], y[j + 1]), d = difference(xx, yy);
+    a.absorb(xx, d, ca);
+    b.absorb(yy, d, cb);
   }
 }
 
@@ -145,15 +164,17 @@ __device__ __forceinline__ float max_of(const Granule<TIn> &g, const Granule<TIn
 }
 
 // One element of each row, under references that are at least as large.
-__device__ __forceinline__ void absorb_one(float x, float y, PairMoments &a, PairMoments &b) {
+template <typename TIn>
+__device__ __forceinline__ void absorb_one(float x, float y, PairMoments<TIn> &a, PairMoments<TIn> &b) {
   // the pair's other element: -inf has no weight, but it may not be multiplied
   const float wa = ex2(fmaf(x, kLog2e, -a.c)), wb = ex2(fmaf(y, kLog2e, -b.c)), d = y - x;
-  a.s = add2(a.s, pack2(wa, 0.f));
-  a.a = fma2(pack2(wa, 0.f), pack2(x, 0.f), a.a);
-  a.b = fma2(pack2(wa, 0.f), pack2(d, 0.f), a.b);
-  b.s = add2(b.s, pack2(wb, 0.f));
-  b.a = fma2(pack2(wb, 0.f), pack2(y, 0.f), b.a);
-  b.b = fma2(pack2(wb, 0.f), pack2(d, 0.f), b.b);
+  const uint64_t wa2 = pack2(wa, 0.f), wb2 = pack2(wb, 0.f), d2 = pack2(d, 0.f);
+  a.q.s = add2(a.q.s, wa2);
+  a.q.a = fma2(wa2, pack2(x, 0.f), a.q.a);
+  a.q.b = fma2(wa2, d2, a.q.b);
+  b.q.s = add2(b.q.s, wb2);
+  b.q.a = fma2(wb2, pack2(y, 0.f), b.q.a);
+  b.q.b = fma2(wb2, d2, b.q.b);
 }
 
 struct MonitorParams {
@@ -177,9 +198,11 @@ __device__ __forceinline__ void monitor_finish(const MonitorParams &p, long long
   if (p.h_i) p.h_i[t] = (float)(lse_i - ez_i);
 }
 
-// kVector: the two rows of a token start alike against the 32-byte grid.  Granules are cut at the rows' own
-// boundaries; the elements in front of the first and behind the last whole granule are taken one per thread.
-template <typename TIn, bool kVector>
+// How a block reads its two rows.  kGranules: the rows of a token start alike against the 32-byte grid; granules are cut at
+// the rows' own boundaries, the elements in front of the first and behind the last whole granule are taken one per
+// thread.  kElementwise: any rows, in two passes.
+enum class Rows { kElementwise, kGranules };
+template <typename TIn, Rows kRows>
 __global__ void __launch_bounds__(256, sizeof(TIn) == 2 ? 4 : 3) dvp_monitor_kernel(const MonitorParams p) {
   __shared__ float scratch[160];
   constexpr int kElems = Granule<TIn>::kElems;
@@ -187,8 +210,8 @@ __global__ void __launch_bounds__(256, sizeof(TIn) == 2 ? 4 : 3) dvp_monitor_ker
   const TIn *zt = reinterpret_cast<const TIn *>(p.train) + t * p.ld_train;
   const TIn *zi = reinterpret_cast<const TIn *>(p.infer) + t * p.ld_infer;
   const int V = (int)p.V, tid = (int)threadIdx.x, n_thr = (int)blockDim.x;
-  PairMoments a = {kNegInf, kNegInf, 0, 0, 0}, b = a;
-  if constexpr (kVector) {
+  PairMoments<TIn> a = {kNegInf, kNegInf, {0, 0, 0}}, b = a;
+  if constexpr (kRows != Rows::kElementwise) {
     const int mis = (int)(((uintptr_t)zt & 31u) / sizeof(TIn));
     const int head = min(V, mis ? kElems - mis : 0), n_full = (V - head) / kElems;
     DVP_BOUNDS_BEGIN(p.bounds_status);
@@ -207,8 +230,8 @@ __global__ void __launch_bounds__(256, sizeof(TIn) == 2 ? 4 : 3) dvp_monitor_ker
       i1.load(bi + (size_t)(second ? g1 : g) * kElems);
       a.raise(max_of<TIn>(t0, t1));
       b.raise(max_of<TIn>(i0, i1));
-      absorb_granules<TIn>(t0, i0, a, b);
-      if (second) absorb_granules<TIn>(t1, i1, a, b);
+      absorb_granules<TIn>(t0, i0, a.c, b.c, a.q, b.q);
+      if (second) absorb_granules<TIn>(t1, i1, a.c, b.c, a.q, b.q);
     }
     const int k = tid < head ? tid : tid + n_full * kElems;  // fewer than 64 of them
     if (k < V) {
@@ -231,9 +254,9 @@ __global__ void __launch_bounds__(256, sizeof(TIn) == 2 ? 4 : 3) dvp_monitor_ker
     for (; k + n_thr < p.V; k += 2 * n_thr) {
       const uint64_t xx = pack2(Storage<TIn>::widen(zt[k]), Storage<TIn>::widen(zt[k + n_thr]));
       const uint64_t yy = pack2(Storage<TIn>::widen(zi[k]), Storage<TIn>::widen(zi[k + n_thr]));
-      const uint64_t d = fma2(xx, pack2(-1.f, -1.f), yy);
-      a.absorb(xx, d);
-      b.absorb(yy, d);
+      const uint64_t d = difference(xx, yy);
+      a.q.absorb(xx, d, a.c);
+      b.q.absorb(yy, d, b.c);
     }
     if (k < p.V) absorb_one(Storage<TIn>::widen(zt[k]), Storage<TIn>::widen(zi[k]), a, b);
   }
@@ -251,10 +274,10 @@ static cudaError_t launch_monitor(const MonitorParams &p, cudaStream_t s) {
   int threads = 64;
   while (threads < 256 && 16LL * threads < p.V * elem / 32) threads *= 2;
   while (threads < 256 && 2 * p.T * threads <= 148 * 1024) threads *= 2;
-  if (alike)
-    dvp_monitor_kernel<TIn, true><<<(unsigned)p.T, threads, 0, s>>>(p);
+  if (!alike)
+    dvp_monitor_kernel<TIn, Rows::kElementwise><<<(unsigned)p.T, 256, 0, s>>>(p);
   else
-    dvp_monitor_kernel<TIn, false><<<(unsigned)p.T, 256, 0, s>>>(p);
+    dvp_monitor_kernel<TIn, Rows::kGranules><<<(unsigned)p.T, threads, 0, s>>>(p);
   return cudaGetLastError();
 }
 
