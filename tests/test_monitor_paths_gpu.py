@@ -53,3 +53,18 @@ def test_rows_of_mostly_fill(pad, dtype):
         z[t, lo:hi] = x.to(dtype)
         zi[t, lo:hi] = (x + 0.1 * torch.randn(hi - lo, generator=g, device=DEV)).to(dtype)
     _check(z, zi)
+
+
+@pytest.mark.parametrize("V,dtype,steps", [(15000, torch.float16, 8), (16000, torch.bfloat16, 8), (6000, torch.float32, 6)])
+def test_sums_keep_small_terms_in_short_rows(V, dtype, steps):
+    """One token at 0 and all others at -17, where e^-17 = 0.69 * 2^-24 is lost when it is added to 1 by itself.  Each
+    step's terms are added up first: one rounding of the sum a step, one a pair of logits in the step of the maximum itself
+    (16 or 8), six where the 64 threads' sums meet, and a few in the logarithms."""
+    z = torch.full((1300, V), -17.0, dtype=dtype, device=DEV)   # fewer rows take more threads each
+    for t, k in enumerate((0, 33, 70)):
+        z[t::3, k] = 0.0
+    r = binding.dvp_monitor(z, z)
+    torch.cuda.synchronize()
+    a = torch.log_softmax(z.double(), 1)
+    err = (r.entropy_train.double() + (a.exp() * a).sum(1)).abs().max().item()
+    assert err <= (steps + 32 // z.element_size() + 6 + 4) * 2.0 ** -24
