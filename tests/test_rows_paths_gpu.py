@@ -212,3 +212,24 @@ def test_mask_words(V, hint):
             z = z.double().cpu()
             keep = z >= z.max(1, keepdim=True).values + (torch.log(torch.tensor(rho, dtype=torch.float64)) if rho else -float("inf"))
             assert (parity.unpack_mask(side.mask, V) == keep.numpy()).all()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
+@pytest.mark.parametrize("hint", [64, 256, 256 | (2 << 24), 256 | (4 << 24), 256 | (8 << 24)])
+def test_maxima_that_climb(dtype, hint):
+    """Maxima that rise by more than e^60 several times in a row, so that what was added up before them overflows, or nearly
+    so: in one exchange's steps, in neighbouring ones, in the last steps, in the last element; sampled tokens elsewhere,
+    at one of them, or none.  With several blocks a row each sees its own part of the climb."""
+    V = 70001
+    w = dataclasses.replace(W["c0_small_f32"], dtype=dtype, head_boost=0.0)
+    b = inputs.make_rows(w, seed=11, device=DEV, T=8, V=V)
+    places = [[40, 17000, 35000, 52000, 70000], [5000, 5001, 5040, 9000, 69990], [66000, 67000, 68000, 69000, 70000],
+              [70000, 60000, 40000, 20000, 3], [30000, 30001, 30002, 30003, 30004], [16383, 16384, 32767, 32768, 65535],
+              [0, 1024, 2048, 4096, 8192], [12000, 24000, 36000, 48000, 60000]]
+    for t, ks in enumerate(places):
+        for i, k in enumerate(ks):
+            b.train[t, k] = 62.0 * (i + 1) + t
+            b.infer[t, k] = 62.5 * (i + 1) + t
+    b.ids[:] = torch.tensor([1, 5040, 70000, -1, 30003, 16384, -1, 60001], device=DEV)
+    for rho in (1e-3, 0.0):
+        _check(b, rho, V, launch_hint=hint)
