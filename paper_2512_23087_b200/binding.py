@@ -339,13 +339,13 @@ def _float32(x: float) -> float:
     return ctypes.c_float(x).value
 
 
-def _uint32(x) -> int:
-    """What a uint32_t holds of x, as ctypes takes it: struct refuses to pack what is out of range, where the library's
-    own check is to answer."""
-    return x & 0xffffffff
+# What a uint32_t holds of a number, as ctypes takes it: struct refuses to pack what is out of range, where the library's
+# own check is to answer.
+_UINT32 = 0xffffffff
 
 
 def _int32(x) -> int:
+    """The same for an int32_t."""
     return (int(x) + 0x80000000 & 0xffffffff) - 0x80000000
 
 
@@ -390,7 +390,7 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
             raise ValueError("infer_logits must match train_logits in dtype and shape")
     if out is not None:
         res = out
-        at = [_addresses(res.train)] + ([_addresses(res.infer)] if has_infer else [])
+        train_at, infer_at = _addresses(res.train), _addresses(res.infer) if has_infer else _NO_SIDE
     else:
         sides, rest, flags = _token_outputs(train_logits, T, 2 if has_infer else 1, has_infer + weighted)
         if want_mask:
@@ -398,7 +398,7 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
         res = SimpleNamespace(train=sides[0][0], infer=sides[1][0] if has_infer else None,
                               log_ratio=rest[0] if has_infer else None,
                               flags=flags, grad_train=None)
-        at = [addresses for _, addresses in sides]
+        train_at, infer_at = sides[0][1], sides[1][1] if has_infer else _NO_SIDE
         if weighted:
             res.weight = rest[-1]
     if weighted and getattr(res, "weight", None) is None:
@@ -421,10 +421,10 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
     st = packed["dvp_forward"](_FORWARD_PACK.pack(
         _FORWARD_PACK.size, _DTYPES[dtype], grad_code, _id_dtype(ids), T, V, train_logits.stride(0),
         infer_logits.stride(0) if has_infer else 0, grad_ld, float(rho), train_logits.data_ptr(),
-        _address(infer_logits), ids.data_ptr(), _address(upstream), _address(grad_train), *at[0],
-        *(at[1] if has_infer else _NO_SIDE), res.log_ratio.data_ptr() if has_infer else 0,
-        res.flags.data_ptr(), _stream(stream), _uint32(launch_hint), mode,
-        _float32(mask_value) if mask_value is not None else 0.0, _uint32(int(weight_kind)), _float32(weight_lo), _float32(weight_hi), res.weight.data_ptr() if weighted else 0))
+        _address(infer_logits), ids.data_ptr(), _address(upstream), _address(grad_train), *train_at, *infer_at,
+        res.log_ratio.data_ptr() if has_infer else 0, res.flags.data_ptr(), _stream(stream), launch_hint & _UINT32, mode,
+        _float32(mask_value) if mask_value is not None else 0.0, int(weight_kind) & _UINT32, _float32(weight_lo),
+        _float32(weight_hi), res.weight.data_ptr() if weighted else 0))
     if st != DVP_OK:
         raise DvpError(st, "dvp_forward")
     return res
@@ -450,7 +450,7 @@ def dvp_backward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, upst
         train_logits.stride(0), grad_train.stride(0), float(rho), train_logits.data_ptr(), ids.data_ptr(),
         upstream.data_ptr(), saved.train.max.data_ptr(), saved.train.lse_safe.data_ptr(),
         saved.train.comp_mp.data_ptr() if use_comp else 0, saved.flags.data_ptr(), grad_train.data_ptr(),
-        _stream(stream), _uint32(launch_hint), mode, _float32(mask_value) if mask_value is not None else 0.0, 0))
+        _stream(stream), launch_hint & _UINT32, mode, _float32(mask_value) if mask_value is not None else 0.0, 0))
     if st != DVP_OK:
         raise DvpError(st, "dvp_backward")
     return grad_train
