@@ -233,3 +233,27 @@ def test_maxima_that_climb(dtype, hint):
     b.ids[:] = torch.tensor([1, 5040, 70000, -1, 30003, 16384, -1, 60001], device=DEV)
     for rho in (1e-3, 0.0):
         _check(b, rho, V, launch_hint=hint)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f16"])
+def test_float32_gradient_entries(dtype):
+    """Rows of two tokens that count, the sampled one and one exactly 1 above it: the other's entry is -g / (1 + e^-1), whose
+    only errors are e^-1's, the sum's and the quotient's, a unit of 2^-24 each at most.  It is made of differences of
+    logits that are exact here, so it is the same in every row, wherever the maximum lies."""
+    T, V = 4096, 800
+    g = torch.Generator(device=DEV).manual_seed(3)
+    m = (torch.randint(64, 8192, (T, 1), generator=g, device=DEV).float() / 256).to(torch.bfloat16).float().clamp(min=4.0)
+    m = torch.where(m >= 16, m.round(), (m * 16).round() / 16)   # m and m - 1 are exact in every type
+    z = torch.full((T, V), -40.0, device=DEV)
+    ids = torch.randint(0, V // 2, (T,), generator=g, device=DEV)
+    other = V // 2 + torch.randint(0, V // 2, (T,), generator=g, device=DEV)
+    z.scatter_(1, ids[:, None], m - 1)
+    z.scatter_(1, other[:, None], m)
+    z = z.to(inputs.torch_dtype(dtype))
+    up = torch.ones(T, device=DEV)
+    res = binding.dvp_forward(z, ids, 1e-3, upstream=up, grad_dtype=torch.float32)
+    torch.cuda.synchronize()
+    want = -1 / (1 + torch.exp(torch.tensor(-1.0, dtype=torch.float64)))
+    got = res.grad_train.gather(1, other[:, None])
+    assert (got.double() / want.item() - 1).abs().max().item() <= 3 * 2.0 ** -24
+    assert (got == got[0]).all()
