@@ -1,0 +1,100 @@
+"""Launches of a call may begin before their predecessor ends, and the fused entry's work beside one another.  Inputs that the
+stream has not written yet when the call is made, calls that share a workspace, and captured calls must give bit for
+bit what a call on finished inputs gives."""
+import pytest
+import torch
+
+from paper_2512_23087_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+W = inputs.WORKLOADS
+SIDE = ("max", "lse", "lse_safe", "logp", "logp_mp", "comp_mp", "count", "log_cov")
+
+
+def _results(r, more):
+    return {**{f"{s}.{n}": getattr(getattr(r, s), n) for s in ("train", "infer") for n in SIDE},
+            **{n: getattr(r, n) for n in ("log_ratio", "flags") + more}}
+
+
+def _same(got, want):
+    for n, x in want.items():
+        assert torch.equal(torch.nan_to_num(got[n].float(), nan=9e9), torch.nan_to_num(x.float(), nan=9e9)), n
+
+
+def _rows_call(b, weighted):
+    kw = dict(weight_kind=binding.DVP_WEIGHT_TRUNCATE, weight_hi=1.01) if weighted else {}
+    r = binding.dvp_forward(b.train, b.ids, 1e-3, infer_logits=b.infer, upstream=b.upstream, **kw)
+    return _results(r, ("grad_train", "weight") if weighted else ("grad_train",))
+
+
+def _fused_call(b, workspace=None):
+    r = binding.dvp_fused_lmhead_forward_backward(b.hidden, b.w_vocab, b.ids, 1e-3, b.upstream, infer_logits=b.infer,
+                                                  panel_rows=128, workspace=workspace)
+    return _results(r, ("d_hidden", "d_w")), r
+
+
+def _refill(b, other, names):
+    for n in names:
+        getattr(b, n).copy_(getattr(other, n))
+
+
+ROWS = ("train", "infer", "ids", "upstream")
+FUSED = ("hidden", "w_vocab", "infer", "ids", "upstream")
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("T,V", [(6, 151936), (900, 20000), (50, 3001)])
+def test_rows_behind_a_long_kernel(T, V, weighted):
+    first, second = (inputs.make_rows(W["c2_bf16_fwdbwd"], seed=s, device=DEV, T=T, V=V) for s in (1, 2))
+    want = _rows_call(second, weighted)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(20_000_000)   # some ten milliseconds; the inputs arrive behind it
+    _refill(first, second, ROWS)
+    got = _rows_call(first, weighted)
+    first.train.zero_(), first.infer.zero_(), first.ids.zero_()   # and are gone right after
+    torch.cuda.synchronize()
+    _same(got, want)
+
+
+@pytest.mark.parametrize("T,H,V", [(300, 256, 6000), (130, 128, 4099)])
+def test_fused_calls_share_a_workspace(T, H, V):
+    """Several panels a call; two problems in turn through one workspace, inputs behind a long kernel, no synchronisation."""
+    a, b, buf = (inputs.make_fused(W["c4_fused_lmhead"], seed=s, device=DEV, T=T, H=H, V=V) for s in (1, 2, 3))
+    want_a, r = _fused_call(a)
+    torch.cuda.synchronize()
+    want_b, _ = _fused_call(b)
+    torch.cuda.synchronize()
+    workspace = torch.empty_like(r.workspace)
+    torch.cuda._sleep(20_000_000)
+    got = []
+    for x in (a, b, a, b):
+        _refill(buf, x, FUSED)
+        got.append(_fused_call(buf, workspace)[0])
+    torch.cuda.synchronize()
+    assert workspace[:4].view(torch.int32).item() == 0
+    for g, w in zip(got, (want_a, want_b, want_a, want_b)):
+        _same(g, w)
+
+
+def test_captured_calls():
+    a, b = (inputs.make_rows(W["c2_bf16_fwdbwd"], seed=s, device=DEV, T=40, V=20000) for s in (1, 2))
+    fa, fb = (inputs.make_fused(W["c4_fused_lmhead"], seed=s, device=DEV, T=140, H=128, V=4000) for s in (1, 2))
+    wants = []
+    for x, f in ((a, fa), (b, fb)):
+        wants.append((_rows_call(x, True), _fused_call(f)[0]))
+        torch.cuda.synchronize()
+    x, f = (inputs.make_rows(W["c2_bf16_fwdbwd"], seed=3, device=DEV, T=40, V=20000),
+            inputs.make_fused(W["c4_fused_lmhead"], seed=3, device=DEV, T=140, H=128, V=4000))
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):   # once outside the capture
+        _rows_call(x, True), _fused_call(f)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        rows, (fused, keep) = _rows_call(x, True), _fused_call(f)
+    for (rw, fw), (xr, xf) in zip(wants, ((a, fa), (b, fb))):
+        _refill(x, xr, ROWS), _refill(f, xf, FUSED)
+        graph.replay()
+        torch.cuda.synchronize()
+        _same(rows, rw), _same(fused, fw)
