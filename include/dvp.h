@@ -28,7 +28,9 @@
  *   - Matrices are row-major with a row stride `ld*` counted in elements.
  *   - `struct_size` must equal sizeof of the struct the caller compiled with.
  *   - Logits must be finite.  Behaviour on NaN or infinite logits is
- *     unspecified (no fault, but the numbers mean nothing).
+ *     unspecified (no fault, but the numbers mean nothing).  Filtered logits may
+ *     hold the lowest value of their type as long as the row's maximum times log2(e)
+ *     is a float32.
  *   - rho lies in [0, 1].  rho = 0 keeps every token (full log-softmax);
  *     rho = 1 keeps the argmax and its exact ties.
  *   - The membership test is exact: it equals the comparison of the stored
@@ -137,10 +139,13 @@ typedef struct {
  *   upstream      device [T] float32: g_t = dLoss / d ln pi^mp_train(a_t)
  *   grad_train    device [T, ld_grad] of grad_dtype: g_t (1[k=a] - pi^mp(k))
  *                 on V_S, 0 off it, the whole row 0 when a is not in V_S;
- *                 rounded to nearest-even in grad_dtype.  It may take the
- *                 place of train_logits or infer_logits (the same type, base
- *                 and stride) when no `mask` is asked for; other overlaps
- *                 with the logits are not allowed
+ *                 rounded to nearest-even in grad_dtype.  With the default
+ *                 kernel it may take the place of train_logits or
+ *                 infer_logits (the same type, base and stride) when no
+ *                 `mask` is asked for; other overlaps with the logits are
+ *                 not allowed.  With weights and none of infer.logp_mp,
+ *                 log_ratio and weight_out, ln pi^mp_infer(a) passes
+ *                 through the first bytes of its rows meanwhile
  *   log_ratio     device [T] float32: ln pi^mp_train(a) - ln pi^mp_infer(a);
  *                 -inf when a is outside V_S (importance ratio zero, remark
  *                 after Thm. 5.3), +inf when a is in V_S but outside V'_S
@@ -154,7 +159,7 @@ typedef struct {
  *                 next 8 bits, and the number of blocks that share one row (0, 1, 2,
  *                 4 or 8; a thread-block cluster) in the top 8 bits.  Kernel choice:
  *                 0 or 2 the default kernel (64, 128, 256 or 512 threads, the largest
- *                 not above the hint; one sweep with the masked sum under a guess of
+ *                 not above the hint, 64 for a hint of 32; one sweep with the masked sum under a guess of
  *                 the maximum, then revisits of the 32-byte pieces of the row that can
  *                 hold safe tokens); 3 or 4 (2-byte
  *                 logits, at most 256 threads, no cluster) the kernel that keeps
@@ -162,7 +167,8 @@ typedef struct {
  *                 streams and reads nothing twice, with 3 or 4 blocks per SM;
  *                 0x11 (with zero elsewhere) the kernel that keeps the row itself
  *                 in shared memory (rows of up to 480 KB whose byte length is a
- *                 multiple of 16).  Rows a chosen kernel cannot take run the
+ *                 multiple of 16).  Choices 3, 4 and 0x11 need every row of every
+ *                 matrix on a 32-byte boundary.  Rows a chosen kernel cannot take run the
  *                 default one.  Tuning only: the safe set and counts do not
  *                 depend on it.
  *                 TEST ONLY: 0x1e in the second byte is a self-test of the 0x11
@@ -171,8 +177,9 @@ typedef struct {
  *                 a second, the launch ends by itself with undefined outputs and
  *                 dvp_row_wait_status reports code 1 or 2
  *
- * Any row stride and any base that is aligned to its element type is taken at full
- * width: rows are cut at their own 32-byte boundaries.  Needs no workspace.  Errors: DVP_ERR_INVALID_ARG for NULL required
+ * The default kernel takes any row stride and any base that is aligned to its element
+ * type at full width: rows are cut at their own 32-byte boundaries.  Needs no workspace.
+ * Errors: DVP_ERR_INVALID_ARG for NULL required
  * pointers, T < 0, V < 1, ld < V, rho outside [0,1] or NaN, upstream without
  * grad_train or the reverse, a malformed launch_hint; DVP_ERR_UNSUPPORTED
  * for unknown dtypes or V >= 2^31 - 256.  Rows too long for the on-chip row
@@ -370,9 +377,11 @@ int dvp_sequence_aggregate(const dvp_sequence_args *args);
  * quantity Sec. 7 proposes to adapt rho to), in nats:
  *   KL(p || q) = sum_k p_k (ln p_k - ln q_k),  H(p) = -sum_k p_k ln p_k,
  *   pi_train = softmax(train_logits[t]), pi_infer = softmax(infer_logits[t]).
- * Both matrices are read once.  Each output is a device [T] float32 array and
- * may be NULL.  Rows that start on 32-byte boundaries take the vectorised
- * kernel, other layouts a scalar one.  Errors as in dvp_forward.
+ * Each output is a device [T] float32 array and may be NULL.  Where the two rows of
+ * every token start alike against a 32-byte grid (at any element) both matrices are
+ * read once, 32 bytes at a time; otherwise twice, element by element.  Divergences
+ * are good to a few 1e-7 absolute, entropies to 2e-5 relative (1e-4 where they are
+ * below 0.1).  Errors as in dvp_forward.
  */
 typedef struct {
   uint32_t struct_size;

@@ -377,7 +377,9 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
 
     Returns a namespace with ``train`` / ``infer`` (per-token tensors),
     ``log_ratio``, ``flags`` and ``grad_train``.  Pass the namespace of an
-    earlier call as ``out`` to reuse its buffers.
+    earlier call as ``out`` to reuse its buffers.  The per-token tensors of a
+    call lie over one storage (at most eighty bytes a token): keeping one keeps
+    that storage, and ``torch.save`` of one writes all of it unless it is cloned.
     """
     packed = load_library().packed
     _check_matrix("train_logits", train_logits)

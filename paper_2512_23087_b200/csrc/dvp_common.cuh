@@ -560,8 +560,7 @@ struct BackwardParams {
   unsigned int *bounds_status;  // the bounds-checking build's status word; unused otherwise
 };
 
-// Launchers (dvp_rows.cu).  `hint`: threads per block in the low 16 bits,
-// 32-byte loads per thread and pipeline stage in the next 8 bits, 0 = default.
+// Launchers (dvp_rows.cu).  `hint`: launch_hint of dvp_forward_args; the backward takes its threads per block only.
 cudaError_t launch_row_kernels(const RowParams &p, int logits_dtype, int grad_dtype, uint32_t hint,
                                cudaStream_t s);
 cudaError_t launch_backward_kernel(const BackwardParams &p, int logits_dtype, int grad_dtype,

@@ -11,11 +11,17 @@
 //
 // Two logits go through one instruction (f32x2) and two granules through one check of the running maximum: with a
 // dozen instructions for every pair of logits the kernel is bound by issue and by its exponentials (0.7 of the
-// time that the bytes take), not by HBM.  T = 4096 x V = 151,936 bfloat16, 2.49 GB: 437 -> 418 us (374 at the
-// copy bandwidth); V = 50,021 with rows back to back, element by element before: 414 -> 172.  Blocks per SM:
-// bfloat16 418 / 423 at 4 / 3, float32 (2,000 x 262,144) 654 / 612.  One reference for the whole block, below the
-// maximum, would take 404 us but loses the divergence of rows with one dominant token (float32, V = 5,000,
-// heavy-tailed: relative error 3.6e-3 against 3.7e-4).
+// time that the bytes take), not by HBM.  T = 4096 x V = 151,936 bfloat16, 2.49 GB, in bursts in turn with the form
+// that takes one logit an instruction: 483 -> 450 us (386 at the copy bandwidth); 1,000 x 50,021 with rows back to
+// back, element by element there: 129 -> 46.  Blocks per SM: bfloat16 446 / 459 at 4 / 3, float32 (2,000 x 262,144)
+// 661 / 606.  Loads of the next granules before the last ones are worked on are slower (few rows 31 against 23 us,
+// 4,096 rows 487 against 450): the code spills or runs with fewer warps.  One reference for the whole block, below
+// the maximum, loses the divergence of rows with one dominant token (float32, V = 5,000, heavy-tailed: relative error
+// 3.6e-3 against 3.7e-4).
+//
+// Accuracy against float64, relative 2-norm over a batch: entropies 1e-6 to 2e-6 (one dominant token and heavy tails,
+// where the entropy itself is small: 2e-5 to 1e-4); divergences are differences of sums of order one, good to some
+// 2e-7 absolute, 1e-3 relative where they are 2e-4.
 #include "dvp_rows_impl.cuh"
 
 namespace dvp {

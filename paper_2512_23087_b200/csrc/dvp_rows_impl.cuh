@@ -686,10 +686,10 @@ __device__ __forceinline__ HotList build_hot_list(const uint32_t *bound, int n_s
 // every kSyncSteps steps: a larger one becomes the guess, and the masked sum starts again from there
 // (`first`).  A value more than kWide above the guess may have overflowed the sum of the steps since the last exchange,
 // and what came before is nothing against it (V e^-60): the sweep goes back to that exchange and starts its sums there.
-// (Back to the start of the row, heavy-tailed rows without a sampled token took 259 us
-// where they take 210: 2,500 x 100,000 bfloat16, both policies.)  All of it happens at fixed
-// places, so that reruns are bit-identical.  `start`: the exchange to begin at; `hole`: the granule that reads as -inf
-// (the sampled token's; its bound says that it can hold anything); xe: a value outside the granules.
+// (Back to the start of the row, heavy-tailed rows without a sampled token took 259 us where they take 210: 2,500 x
+// 100,000 bfloat16, both policies.)  All of it happens at fixed places, so that reruns are bit-identical.  `start`: the
+// exchange to begin at; `hole`: the granule that reads as -inf (the sampled token's; its bound says that it can hold
+// anything); xe: a value outside the granules.
 constexpr int kSyncSteps = 4;
 constexpr float kWide = 60.f;  // e^60 times the longest row is far from overflow
 template <typename TIn, int kBlk>
