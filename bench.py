@@ -39,9 +39,9 @@ FALLBACK_HBM_GBS = 6650.0
 # of one ncu capture of a dvp_forward call on T rows of the workload), keyed by (workload, rho); valid only for
 # the kernel sources whose digest is recorded with it, scaled by rows to the full batch.
 NCU_TRAFFIC = {
-    ("c2_bf16_fwdbwd", 1e-4): {"digest": "5e65b88e238fd975", "T": 2048, "bytes": 1.501346e9 + 0.573023e9},
-    ("c2_bf16_fwdbwd", 1e-3): {"digest": "5e65b88e238fd975", "T": 2048, "bytes": 1.313576e9 + 0.565076e9},
-    ("c3_f32_heavy", 1e-4): {"digest": "5e65b88e238fd975", "T": 1024, "bytes": 2.148167e9 + 1.017859e9},
+    ("c2_bf16_fwdbwd", 1e-4): {"digest": "31a815c921717097", "T": 2048, "bytes": 1.495590e9 + 0.571554e9},
+    ("c2_bf16_fwdbwd", 1e-3): {"digest": "31a815c921717097", "T": 2048, "bytes": 1.310682e9 + 0.564589e9},
+    ("c3_f32_heavy", 1e-4): {"digest": "31a815c921717097", "T": 1024, "bytes": 2.147990e9 + 1.013474e9},
 }
 
 
@@ -58,7 +58,7 @@ def _kernel_digest(names=("dvp_common.cuh", "dvp_rows_impl.cuh")) -> str:
 # panels of 4096 rows): the first panel's three and a later panel's three (whose d_w contraction also reads
 # the d_w it adds to).  Valid for the sources whose digest is recorded; a step of P panels is taken as the
 # first panel's launches plus P - 1 times the later panel's.
-NCU_TRAFFIC_FUSED = {"digest": "5009013b2377f941", "H": 4096, "V": 151936, "panel": 4096,
+NCU_TRAFFIC_FUSED = {"digest": "5d40d86b109ab9fb", "H": 4096, "V": 151936, "panel": 4096,
                      "first": (4.615540e9 + 2.485369e9) + (13.608092e9 + 0.127318e9) + (5.593785e9 + 2.459819e9),
                      "later": (4.840493e9 + 2.484551e9) + (12.678872e9 + 0.127140e9) + (8.013996e9 + 2.456163e9)}
 FUSED_SOURCES = ("dvp_gemm.cuh", "dvp_fused.cu", "dvp_panel.cuh")
