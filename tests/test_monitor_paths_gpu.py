@@ -29,6 +29,17 @@ def test_rows_that_start_anywhere(V, pad_t, pad_i, off, dtype):
     _check(place(z, V + pad_t), place(z + 0.1 * torch.randn(T, V, generator=g, device=DEV), V + pad_i))
 
 
+@pytest.mark.parametrize("T,V", [(5, 24575), (5, 24576), (3, 49151), (3, 49169), (2, 98303), (2, 98305), (297, 24576),
+                                 (149, 49152), (74, 98305)])
+@pytest.mark.parametrize("off", [0, 5])
+def test_rows_shared_by_several_blocks(T, V, off):
+    """Rows of 1,536, 3,072 and 6,144 pieces take two, four and eight blocks while as many fit the chip at once."""
+    g = torch.Generator(device=DEV).manual_seed(V)
+    z = torch.randn(T, V, generator=g, device=DEV) * 2
+    place = lambda x: torch.full((off + T * V,), 3e4, device=DEV, dtype=torch.bfloat16)[off:].view(T, V).copy_(x)
+    _check(place(z), place(z + 0.1 * torch.randn(T, V, generator=g, device=DEV)))
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_one_value_far_above_the_others(dtype):
     g = torch.Generator(device=DEV).manual_seed(1)
