@@ -885,87 +885,144 @@ __host__ __device__ constexpr int grad_align() {
   return Granule<TIn>::kElems < 32 / (int)sizeof(TGrad) ? Granule<TIn>::kElems : 32 / (int)sizeof(TGrad);
 }
 
-// Sweep 3 when the gradient row lies differently than its logits row (another row stride or base):
-// zeros first, in the gradient row's own 32-byte pieces, then the safe tokens one by one.
-template <typename TIn, typename TGrad, int kBlk>
-__device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *grow, int a, float tau,
-                                               typename SweepOps<TIn>::Key key, bool live, float m, float coef,
-                                               float g_a, const uint32_t *bound) {
-  constexpr int kElems = Granule<TIn>::kElems, kOut = 32 / (int)sizeof(TGrad);
-  const int tid = threadIdx.x, n_thr = kBlk;
-  const int k0 = v.head + v.g_first * kElems, k1 = k0 + v.n_full * kElems;  // this block's granules, as elements
-  TGrad *dst = grow + k0;
-  const int n = k1 - k0;
-  const int mis = (int)(((uintptr_t)dst & 31u) / sizeof(TGrad));
-  const int head = min(n, mis ? kOut - mis : 0), n_vec = (n - head) / kOut;
-  const uint32_t z[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  if (tid < head) dst[tid] = Storage<TGrad>::narrow(0.f);
-  for (int i = tid; i < n_vec; i += n_thr) st_stream32(dst + head + (size_t)i * kOut, z);
-  const int k_rest = head + n_vec * kOut + tid;
-  if (k_rest < n) dst[k_rest] = Storage<TGrad>::narrow(0.f);
-  __syncthreads();  // the zeros of this block's part are in place before single elements replace them
-  if (!live) return;
-  for (int i = 0;; ++i) {
-    const int g = i * n_thr + tid, wi = (i >> 1) * n_thr + tid;
-    if (g >= v.n_full || !DVP_IN(wi, n_bound, DVP_OOB_BOUND)) break;
-    if (!((SweepOps<TIn>::reach(bound[wi], key) >> (16 * (i & 1))) & 1u)) continue;
-    Granule<TIn> gr;
-    gr.load_whole(v.base, v.n_full, g);
-    float x[kElems];
-    gr.get(x);
-    const int ja = a - g * kElems;
-#pragma unroll
-    for (int j = 0; j < kElems; ++j)
-      if (x[j] >= tau)
-        dst[(size_t)g * kElems + j] =
-            Storage<TGrad>::narrow(j == ja ? g_a : coef * ex2((x[j] - m) * kLog2e));
-  }
-}
-
 // 2^{(z - m) l} as 2^{z l - c} 2^{c - m l}, the second factor in the coefficient: one instruction less, and one rounding
 // more, which entries of 16 bits do not show (float32 entries of 333 x 50,021 logits: relative error 5.9e-8 with it,
 // 5.0e-8 without).
 template <typename TIn, typename TGrad>
 constexpr bool kFoldedGrad = sizeof(TIn) == 2 && sizeof(TGrad) == 2;
 
+// The words of memory that a granule's gradient entries fill.
+template <typename TIn, typename TGrad>
+constexpr int kGradWords = Granule<TIn>::kElems * (int)sizeof(TGrad) / 4;
+
 // Gradient entries coef 2^{(z - m) l} of a whole granule (m2: -m twice, coef2: coef twice), zeros below the threshold.
 // 16-bit logits and entries: coef 2^{z l - m2}, one instruction less for two of them (see kFoldedGrad).
 template <typename TIn, typename TGrad>
-__device__ __forceinline__ void grad_granule(const Granule<TIn> &gr, TGrad *dst, float tau,
-                                             typename SweepOps<TIn>::Tau tau_p, uint64_t m2, uint64_t coef2) {
+__device__ __forceinline__ void grad_words(const Granule<TIn> &gr, float tau, typename SweepOps<TIn>::Tau tau_p,
+                                           uint64_t m2, uint64_t coef2, uint32_t (&w)[kGradWords<TIn, TGrad>]) {
   constexpr int kElems = Granule<TIn>::kElems;
   const uint64_t l2 = pack2(kLog2e, kLog2e);
   float x[kElems];
   gr.get(x);
-  if constexpr (kFoldedGrad<TIn, TGrad>) {
-    uint32_t w[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      float lo, hi;
-      unpack2(fma2(pack2(x[2 * i], x[2 * i + 1]), l2, m2), lo, hi);
-      unpack2(mul2(pack2(ex2(lo), ex2(hi)), coef2), lo, hi);
-      uint32_t v;
-      if constexpr (std::is_same<TGrad, __nv_bfloat16>::value) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
-        v = *reinterpret_cast<const uint32_t *>(&h);
-      } else {
-        const __half2 h = __floats2half2_rn(lo, hi);
-        v = *reinterpret_cast<const uint32_t *>(&h);
-      }
-      w[i] = v & SweepOps<TIn>::reach(gr.w[i], tau_p);
+  for (int j = 0; j < kElems; j += 2) {
+    float lo, hi;
+    unpack2(kFoldedGrad<TIn, TGrad> ? fma2(pack2(x[j], x[j + 1]), l2, m2) : mul2(add2(pack2(x[j], x[j + 1]), m2), l2), lo, hi);
+    unpack2(mul2(pack2(ex2(lo), ex2(hi)), coef2), lo, hi);
+    if constexpr (!kFoldedGrad<TIn, TGrad>) {
+      lo = x[j] >= tau ? lo : 0.f;
+      hi = x[j + 1] >= tau ? hi : 0.f;
     }
-    st_stream32(dst, w);
+    if constexpr (sizeof(TGrad) == 4) {
+      w[j] = __float_as_uint(lo);
+      w[j + 1] = __float_as_uint(hi);
+    } else if constexpr (std::is_same<TGrad, __nv_bfloat16>::value) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+      w[j / 2] = *reinterpret_cast<const uint32_t *>(&h);
+    } else {
+      const __half2 h = __floats2half2_rn(lo, hi);
+      w[j / 2] = *reinterpret_cast<const uint32_t *>(&h);
+    }
+    if constexpr (kFoldedGrad<TIn, TGrad>) w[j / 2] &= SweepOps<TIn>::reach(gr.w[j / 2], tau_p);
+  }
+}
+template <typename TIn, typename TGrad>
+__device__ __forceinline__ void grad_granule(const Granule<TIn> &gr, TGrad *dst, float tau,
+                                             typename SweepOps<TIn>::Tau tau_p, uint64_t m2, uint64_t coef2) {
+  constexpr int kWords = kGradWords<TIn, TGrad>;
+  uint32_t w[kWords];
+  grad_words<TIn, TGrad>(gr, tau, tau_p, m2, coef2, w);
+  if constexpr (kWords == 4) {
+    st_stream16(dst, make_uint4(w[0], w[1], w[2], w[3]));
   } else {
-    float out[kElems];
 #pragma unroll
-    for (int j = 0; j < kElems; j += 2) {
-      float lo, hi;
-      unpack2(mul2(add2(pack2(x[j], x[j + 1]), m2), l2), lo, hi);
-      unpack2(mul2(pack2(ex2(lo), ex2(hi)), coef2), lo, hi);
-      out[j] = x[j] >= tau ? lo : 0.f;
-      out[j + 1] = x[j + 1] >= tau ? hi : 0.f;
+    for (int i = 0; i < kWords; i += 8) {
+      uint32_t v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = w[i + k];
+      st_stream32(reinterpret_cast<uint32_t *>(dst) + i, v);
     }
-    store_granule<TGrad, kElems>(dst, out);
+  }
+}
+
+// The same for a gradient row that lies differently than its logits row (another row stride or base): the entries of `n`
+// neighbouring granules, one a lane from lane 0 on, to `dst`, where those of the first begin, at any alignment of theirs.
+// They pass through 512 bytes of the warp's shared memory, so that 32 lanes store 32 neighbouring words, put together from
+// the halves of two where 2-byte entries begin at an odd one.  `any`: some lane's granule has a safe token; a lane whose
+// granule has none holds zeros.
+constexpr int kShiftWords = 128;  // of shared memory, a warp
+template <int kWords, typename TGrad>
+__device__ __forceinline__ void store_shifted(const uint32_t (&w)[kWords], bool any, TGrad *dst, int n, uint32_t *smem) {
+  constexpr int kLanes = 32 * kWords <= kShiftWords ? 32 : kShiftWords / kWords;  // whose entries fit at once
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = 0; h < 32 / kLanes; ++h) {
+    const int n_words = min(kLanes, n - h * kLanes) * kWords;
+    if (n_words <= 0) break;
+    if (any) {
+      __syncwarp();  // the words before are stored
+      if (lane / kLanes == h) {
+        uint32_t *mine = smem + (lane % kLanes) * kWords;
+        if constexpr (kWords == 2) {
+          *reinterpret_cast<uint2 *>(mine) = make_uint2(w[0], w[1]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < kWords; i += 4)
+            *reinterpret_cast<uint4 *>(mine + i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
+        }
+      }
+      __syncwarp();
+    }
+    uint32_t *out = reinterpret_cast<uint32_t *>(dst) + h * kLanes * kWords;
+    if (sizeof(TGrad) == 4 || ((uintptr_t)dst & 3u) == 0) {
+#pragma unroll
+      for (int k = lane; k < kLanes * kWords; k += 32)
+        if (k < n_words) st_stream4(out + k, any ? smem[k] : 0u);
+    } else {
+      uint16_t *half = reinterpret_cast<uint16_t *>(out);
+#pragma unroll
+      for (int k = lane; k < kLanes * kWords; k += 32) {
+        if (k + 1 < n_words) st_stream4(half + 2 * k + 1, any ? __byte_perm(smem[k], smem[k + 1], 0x5432) : 0u);
+        if (k + 1 == n_words) half[2 * k + 1] = any ? (uint16_t)(smem[k] >> 16) : (uint16_t)0;
+      }
+      if (lane == 0) half[0] = any ? (uint16_t)smem[0] : (uint16_t)0;
+    }
+  }
+}
+
+// Sweep 3 when the gradient row lies differently than its logits row: every granule in turn, a step's two at a time
+// (both loads before either is used).  `smem`: kShiftWords a warp.
+template <typename TIn, typename TGrad, int kBlk>
+__device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *grow, TGrad *entry_a, int g_a, float out_a,
+                                               float tau, typename SweepOps<TIn>::Tau tau_p,
+                                               typename SweepOps<TIn>::Key key, bool live, uint64_t m2, uint64_t coef2,
+                                               const uint32_t *bound, uint32_t *smem) {
+  constexpr int kElems = Granule<TIn>::kElems, kWords = kGradWords<TIn, TGrad>;
+  const int tid = threadIdx.x, first = tid & ~31, lane = tid & 31;
+  smem += (tid >> 5) * kShiftWords;
+  for (int step = 0; 2 * step * kBlk + first < v.n_full; ++step) {
+    const int wi = step * kBlk + tid, g0 = 2 * step * kBlk + tid;
+    const uint32_t b = live && DVP_IN(wi, n_bound, DVP_OOB_BOUND) ? SweepOps<TIn>::reach(bound[wi], key) : 0u;
+    Granule<TIn> gr[2];
+    const bool hot[2] = {(b & 1u) && g0 < v.n_full, (b & 0x10000u) && g0 + kBlk < v.n_full};
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (hot[u]) gr[u].load_whole(v.base, v.n_full, g0 + u * kBlk);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int g = g0 + u * kBlk, n = min(32, v.n_full - (g - lane));
+      if (n <= 0 || !DVP_IN((long long)(g - lane + n) * kElems - 1, V, DVP_OOB_GLOBAL)) break;
+      uint32_t w[kWords];
+      if (hot[u]) {
+        grad_words<TIn, TGrad>(gr[u], tau, tau_p, m2, coef2, w);
+      } else {
+#pragma unroll
+        for (int i = 0; i < kWords; ++i) w[i] = 0;
+      }
+      store_shifted(w, __any_sync(0xffffffffu, hot[u]), grow + (size_t)(g - lane) * kElems, n, smem);
+      __syncwarp();  // the sampled token's entry replaces what a lane of the warp stored there
+      if (g == g_a) *entry_a = Storage<TGrad>::narrow(out_a);
+    }
   }
 }
 
@@ -975,7 +1032,7 @@ __device__ __forceinline__ void grad_granule(const Granule<TIn> &gr, TGrad *dst,
 template <typename TIn, typename TGrad, int kBlk, bool kLoose>
 __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all, int a_row,
                                          const SideStats &st, float g, const uint32_t *bound,
-                                         const HotList &list) {
+                                         const HotList &list, uint16_t *hot_smem) {
   constexpr int kElems = Granule<TIn>::kElems;
   const TIn *row = v.base;
   const int n_full = v.n_full;
@@ -1002,11 +1059,6 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
       grow_all[k_extra] = Storage<TGrad>::narrow(out);
     }
   }
-  if constexpr (kLoose) {
-    row_grad_loose<TIn, TGrad, kBlk>(v, grow_all, a_here >= 0 ? v.rel(a_here) : -1, tau, key, live, st.m, coef, g_a,
-                                     bound);
-    return;
-  }
   // zeros of one step's granules that hold no safe token
   auto zeros = [&](int step) {
     const int wi = step * kBlk + tid;
@@ -1026,6 +1078,11 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
   const uint64_t m2 = pack2(-mc, -mc), cf2 = pack2(cf, cf);
   const typename SweepOps<TIn>::Tau tau_p = SweepOps<TIn>::threshold(fmaxf(st.tau, -FLT_MAX));
   const int g_here = a_here >= 0 ? v.granule_of(a_here) : -1;
+  if constexpr (kLoose) {
+    row_grad_loose<TIn, TGrad, kBlk>(v, grow, grow_all + a_here, g_here, g_a, tau, tau_p, key, live, m2, cf2, bound,
+                                     reinterpret_cast<uint32_t *>(hot_smem));
+    return;
+  }
   // one granule; the sampled token's entry replaces the one that its granule's store left
   auto emit = [&](const Granule<TIn> &gr, int g) {
     if (!DVP_IN((long long)g * kElems + kElems - 1, V, DVP_OOB_GLOBAL)) return;
@@ -1083,6 +1140,7 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
 
 // Shared-memory layout of the row kernel, in 4-byte words: the block reductions, 8 for what blocks of a
 // cluster exchange, then the hot lists, then the bounds.
+static_assert(kShiftWords * 4 <= kHotCap * sizeof(uint16_t), "store_shifted uses the place of a warp's hot list");
 __host__ __device__ inline int smem_words_fixed(int threads) {
   return kRedWords + 8 + (threads / 32) * kHotCap / 2;
 }
@@ -1142,7 +1200,7 @@ dvp_row_kernel(const __grid_constant__ RowParams p, const long long t0, const in
       if (p.weight_out && writer) p.weight_out[t] = w;
     }
     row_grad<TIn, TGrad, kBlk, kGrad == Grad::kLoose>(v, reinterpret_cast<TGrad *>(p.grad) + t * p.ld_grad, a, st, g,
-                                                      bound, list);
+                                                      bound, list, hot_smem);
   }
   if (writer) {
     if (p.side == kSideTrain && !weighted) {
@@ -1275,56 +1333,83 @@ __global__ void dvp_row_kernel_scalar(const RowParams p) {
 
 // ---- stand-alone backward: a streaming map from saved row statistics ---------
 
-template <typename TIn, typename TGrad, int kStage, bool kVector>
-__global__ void dvp_backward_kernel(const BackwardParams p) {
-  const long long t = blockIdx.x;
-  DVP_BOUNDS_BEGIN(p.bounds_status);
-  DVP_BOUNDS_SET(n_gran, (p.V + Granule<TIn>::kElems - 1) / Granule<TIn>::kElems);
-  DVP_BOUNDS_SET(V, p.V);
-  DVP_BOUNDS_SYNC();
+// A row is shared by 2^log_parts blocks; nothing passes between them.  Granules are cut as in the row kernel (RowView),
+// so that rows may start at any element; kLoose: gradient rows that lie differently (store_shifted).  A step is two
+// granules a thread, both loads in flight, the first step's before the row's scalars are read.  Granules of a warp
+// without a safe token are written as zeros without an exponential.
+template <typename TIn, typename TGrad, bool kLoose>
+__global__ void __launch_bounds__(512, 2) dvp_backward_kernel(const __grid_constant__ BackwardParams p, const int log_parts) {
+  constexpr int kElems = Granule<TIn>::kElems, kWords = kGradWords<TIn, TGrad>;
+  extern __shared__ __align__(16) uint32_t shift_smem[];  // kLoose: kShiftWords a warp
+  const long long t = blockIdx.x >> log_parts;
+  const int tid = (int)threadIdx.x, n_thr = (int)blockDim.x, lane = tid & 31;
   const TIn *row = reinterpret_cast<const TIn *>(p.train) + t * p.ld_train;
   TGrad *grow = reinterpret_cast<TGrad *>(p.grad) + t * p.ld_grad;
+  RowView<TIn> v;
+  v.set(row, (int)p.V, (int)blockIdx.x & ((1 << log_parts) - 1), log_parts);
+  DVP_BOUNDS_BEGIN(p.bounds_status);
+  DVP_BOUNDS_SET(n_gran, v.n_full);
+  DVP_BOUNDS_SET(V, (long long)v.n_full * kElems);
+  DVP_BOUNDS_SYNC();
+  const int n_full = v.n_full;
+  Granule<TIn> gr[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+    if (tid + u * n_thr < n_full) gr[u].load_whole(v.base, n_full, tid + u * n_thr);
+
   const long long id = load_id(p.ids, p.id_is_i32, t);
-  const bool member = (p.flags[t] & DVP_FLAG_IN_TRAIN) && id >= 0 && id < p.V;
+  const bool valid = id >= 0 && id < p.V;
+  const bool member = (p.flags[t] & DVP_FLAG_IN_TRAIN) && valid;
   // with a finite mask value a pruned sampled token still has a gradient on the kept positions
-  const bool live = member || ((p.mode & DVP_MODE_FINITE_MASK) && id >= 0 && id < p.V);
-  const long long a = member ? id : -1;
+  const bool live = member || ((p.mode & DVP_MODE_FINITE_MASK) && valid);
+  const int a = member ? (int)id : -1;
   const float g = p.upstream[t], m = p.max_t[t];
-  const float tau = live ? threshold_of<TIn>(m, p.log_rho, p.mode) : -kNegInf;
+  const float tau = fmaxf(threshold_of<TIn>(m, p.log_rho, p.mode), -FLT_MAX);
   // e^{z - lse_safe} = e^{z - m} e^{m - lse_safe}; the second factor is 1 / s_safe
   const float coef = live ? -g * ex2((m - p.lse_safe_t[t]) * kLog2e) : 0.f;
-  float g_a = 0.f;
+  float out_a = 0.f;
   if (member) {
-    const float comp = p.comp_mp_t ? p.comp_mp_t[t]
-                                   : -expm1f(Storage<TIn>::widen(row[a]) - p.lse_safe_t[t]);
-    g_a = g * comp;
+    const float comp = p.comp_mp_t ? p.comp_mp_t[t] : -expm1f(Storage<TIn>::widen(row[a]) - p.lse_safe_t[t]);
+    out_a = g * comp;
   }
-  if constexpr (kVector) {
-    constexpr int kElems = Granule<TIn>::kElems;
-    const int V = (int)p.V;
-    const int n_full = V / kElems;
-    const int n_gran = (V + kElems - 1) / kElems;
-    const int per_step = kStage * (int)blockDim.x;
-    for (int gb = 0; gb < n_gran; gb += per_step) {
-      Granule<TIn> gr[kStage];
+  const int k_extra = tid < 32 ? v.extra() : v.V;  // V may be close to INT_MAX here
+  if (k_extra < v.V) {
+    const float x = Storage<TIn>::widen(row[k_extra]);
+    const float out = live && x >= tau ? coef * ex2((x - m) * kLog2e) : 0.f;
+    grow[k_extra] = Storage<TGrad>::narrow(k_extra == a ? out_a : out);
+  }
+  float mc = m, cf = coef;
+  if constexpr (kFoldedGrad<TIn, TGrad>) {
+    mc = m * kLog2e;
+    cf = coef * ex2(-fmaf(m, kLog2e, -mc));
+  }
+  const uint64_t m2 = pack2(-mc, -mc), cf2 = pack2(cf, cf);
+  const typename SweepOps<TIn>::Tau tau_p = SweepOps<TIn>::threshold(tau);
+  const int g_a = a >= 0 ? v.granule_of(a) : -1;
+  TGrad *gbase = grow + (v.base - row);
+  // whole warps stay: a lane past the end has nothing to store
+  for (int g0 = tid; g0 - lane < n_full; g0 += 2 * n_thr) {
 #pragma unroll
-      for (int u = 0; u < kStage; ++u) {
-        const int gi = gb + u * (int)blockDim.x + threadIdx.x;
-        if (gi < n_gran) gr[u].load_any(row, V, n_full, gi);
-      }
+    for (int u = 0; u < 2; ++u) {
+      const int gi = g0 + u * n_thr, n = min(32, n_full - (gi - lane));
+      if (n <= 0 || !DVP_IN((long long)(gi - lane + n) * kElems - 1, V, DVP_OOB_GLOBAL)) break;
+      const bool hot = live && lane < n && gr[u].max() >= tau, any = __any_sync(0xffffffffu, hot);
+      TGrad *dst = gbase + (size_t)gi * kElems;
+      if constexpr (kLoose) {
+        uint32_t w[kWords];
 #pragma unroll
-      for (int u = 0; u < kStage; ++u) {
-        const int gi = gb + u * (int)blockDim.x + threadIdx.x;
-        if (gi < n_gran)
-          granule_grad<TIn, TGrad>(gr[u], grow, V, n_full, gi, (int)a, tau, m, coef, g_a);
+        for (int i = 0; i < kWords; ++i) w[i] = 0;
+        if (hot) grad_words<TIn, TGrad>(gr[u], tau, tau_p, m2, cf2, w);
+        store_shifted(w, any, dst - lane * kElems, n, shift_smem + (tid >> 5) * kShiftWords);
+        __syncwarp();  // the sampled token's entry replaces what a lane of the warp stored there
+      } else if (lane < n) {
+        if (any)
+          grad_granule<TIn, TGrad>(gr[u], dst, tau, tau_p, m2, cf2);
+        else
+          store_zero_granule<TGrad, kElems>(dst);
       }
-    }
-  } else {
-    for (long long k = threadIdx.x; k < p.V; k += blockDim.x) {
-      const float z = Storage<TIn>::widen(row[k]);
-      float out = z >= tau ? coef * ex2((z - m) * kLog2e) : 0.f;
-      if (k == a) out = g_a;
-      grow[k] = Storage<TGrad>::narrow(out);
+      if (gi == g_a) grow[a] = Storage<TGrad>::narrow(out_a);
+      if (gi + 2 * n_thr < n_full) gr[u].load_whole(v.base, n_full, gi + 2 * n_thr);
     }
   }
 }
@@ -1339,6 +1424,14 @@ namespace dvp {
 
 static inline bool aligned32(const void *base, long long ld, size_t elem) {
   return base == nullptr || (((uintptr_t)base % 32 == 0) && ((ld * (long long)elem) % 32 == 0));
+}
+
+// Do the gradient's granules start on store boundaries wherever the logits' do?
+template <typename TIn, typename TGrad>
+static inline bool grad_loose(const void *logits, long long ld, const void *grad, long long ld_grad, long long T) {
+  constexpr long long kA = grad_align<TIn, TGrad>();
+  const long long shift = (long long)((uintptr_t)grad / sizeof(TGrad) % kA) - (long long)((uintptr_t)logits / sizeof(TIn) % kA);
+  return shift % kA != 0 || (T > 1 && (ld_grad - ld) % kA != 0);
 }
 
 // Does the gradient take the place of (a part of) these logits?
@@ -1519,13 +1612,7 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
   const bool vec_ok = aligned32(p.train, p.ld_train, sizeof(TIn)) &&
                       aligned32(p.infer, p.ld_infer, sizeof(TIn)) &&
                       aligned32(p.grad, p.ld_grad, sizeof(TGrad));
-  bool loose = false;
-  if (p.grad) {  // do the gradient's granules start on store boundaries wherever the logits' do?
-    constexpr long long kA = grad_align<TIn, TGrad>();
-    const long long shift = (long long)((uintptr_t)p.grad / sizeof(TGrad) % kA) -
-                            (long long)((uintptr_t)p.train / sizeof(TIn) % kA);
-    loose = shift % kA != 0 || (p.T > 1 && (p.ld_grad - p.ld_train) % kA != 0);
-  }
+  const bool loose = p.grad && grad_loose<TIn, TGrad>(p.train, p.ld_train, p.grad, p.ld_grad, p.T);
   const long long n_gran_row = (p.V + kElems - 1) / kElems;
   const bool weighted = p.weight_kind != DVP_WEIGHT_NONE;
   const bool store_kernel = sizeof(TIn) == 2 && (stage_hint == 3 || stage_hint == 4);
@@ -1587,16 +1674,24 @@ static cudaError_t launch_rows_g(const RowParams &p, int grad_dtype, uint32_t hi
   }
 }
 
+// Blocks of a row: as many as bring some 16 warps to every SM (four times its 2,048 threads' worth of rows are enough),
+// while each has a step or more.
 template <typename TIn, typename TGrad>
 static cudaError_t launch_bwd(const BackwardParams &p, uint32_t hint, cudaStream_t s) {
-  int threads = hint & 0xffff;
-  if (threads == 0) threads = 256;
-  const bool vec_ok =
-      aligned32(p.train, p.ld_train, sizeof(TIn)) && aligned32(p.grad, p.ld_grad, sizeof(TGrad));
-  if (vec_ok)
-    dvp_backward_kernel<TIn, TGrad, 2, true><<<(unsigned)p.T, threads, 0, s>>>(p);
+  const long long n_gran = p.V / Granule<TIn>::kElems;
+  int threads = hint & 0xffff, log_parts = 0;
+  if (threads == 0) {
+    threads = 256;
+    while (threads > 64 && threads >= n_gran) threads /= 2;
+  }
+  while (log_parts < 10 && (p.T << log_parts) * threads < 4 * 148 * 1024 && n_gran >> (log_parts + 1) >= 2 * threads)
+    ++log_parts;
+  const bool loose = grad_loose<TIn, TGrad>(p.train, p.ld_train, p.grad, p.ld_grad, p.T);
+  const unsigned grid = (unsigned)(p.T << log_parts);
+  if (loose)
+    dvp_backward_kernel<TIn, TGrad, true><<<grid, threads, threads / 32 * kShiftWords * 4, s>>>(p, log_parts);
   else
-    dvp_backward_kernel<TIn, TGrad, 1, false><<<(unsigned)p.T, threads, 0, s>>>(p);
+    dvp_backward_kernel<TIn, TGrad, false><<<grid, threads, 0, s>>>(p, log_parts);
   return cudaGetLastError();
 }
 

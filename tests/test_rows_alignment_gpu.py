@@ -2,6 +2,7 @@
 and gradient matrices that lie differently than their logits.  The row kernels cut each row at its own
 32-byte boundaries; the elements in front of the first and behind the last whole piece, and the pieces
 themselves, must all be taken exactly once, and nothing outside the rows may be written."""
+import contextlib
 import dataclasses
 
 import pytest
@@ -57,6 +58,32 @@ def test_rows_that_start_anywhere(dtype, grad_dtype, V, pad, offset, grad_pad, g
         else:
             res = run(rho)
         parity.check_forward(res, b, rho, V, True)
+        outside = torch.ones_like(buf, dtype=torch.bool)
+        outside[grad_offset:grad_offset + T * ld].view(T, ld)[:, :V] = False
+        assert (buf[outside] == 7.0).all(), "written outside the gradient's rows"
+
+
+# few and long rows are shared by several blocks each
+@pytest.mark.parametrize("pad,offset,grad_pad,grad_offset", [(0, 0, 0, 0), (3, 5, 3, 5), (1, 8, 0, 3), (16, 1, 8, 0)])
+@pytest.mark.parametrize("T,V", [(13, 5), (13, 31), (13, 47), (13, 2999), (600, 4097), (3, 50021)])
+@pytest.mark.parametrize("dtype,grad_dtype", [("bf16", torch.bfloat16), ("f16", torch.float32), ("f32", torch.float32),
+                                              ("f32", torch.bfloat16)])
+@pytest.mark.parametrize("checks", [False, True], ids=["", "bounds"])
+def test_backward_rows_that_start_anywhere(dtype, grad_dtype, T, V, pad, offset, grad_pad, grad_offset, checks):
+    w = dataclasses.replace(W["c0_small_f32"], dtype=dtype, head_boost=5.0)
+    b = inputs.make_rows(w, seed=V + pad, device=DEV, T=T, V=V)
+    b = dataclasses.replace(b, train=_place(b.train, V + pad, offset))
+    ld = V + grad_pad
+    for rho in (1e-3, 0.0):
+        buf = torch.full((grad_offset + T * ld + 64,), 7.0, dtype=grad_dtype, device=DEV)
+        grad = buf[grad_offset:grad_offset + T * ld].view(T, ld)[:, :V]
+        saved = binding.dvp_forward(b.train, b.ids, rho, infer_logits=b.infer)
+        with binding.bounds_checking_library() if checks else contextlib.nullcontext():
+            binding.dvp_backward(b.train, b.ids, rho, b.upstream, saved, grad_train=grad)
+            torch.cuda.synchronize()
+            assert not checks or binding.dvp_debug_bounds_status() == 0, "an index was out of range"
+        want = parity.run_oracle(b.train, b.infer, b.ids, rho, b.upstream)
+        parity.check_grad(grad, want.grad, {})
         outside = torch.ones_like(buf, dtype=torch.bool)
         outside[grad_offset:grad_offset + T * ld].view(T, ld)[:, :V] = False
         assert (buf[outside] == 7.0).all(), "written outside the gradient's rows"
