@@ -963,13 +963,9 @@ __device__ __forceinline__ void store_shifted(const uint32_t (&w)[kWords], bool 
       __syncwarp();  // the words before are stored
       if (lane / kLanes == h) {
         uint32_t *mine = smem + (lane % kLanes) * kWords;
-        if constexpr (kWords == 2) {
-          *reinterpret_cast<uint2 *>(mine) = make_uint2(w[0], w[1]);
-        } else {
 #pragma unroll
-          for (int i = 0; i < kWords; i += 4)
-            *reinterpret_cast<uint4 *>(mine + i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
-        }
+        for (int i = 0; i < kWords; i += 4)
+          *reinterpret_cast<uint4 *>(mine + i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
       }
       __syncwarp();
     }
@@ -990,39 +986,42 @@ __device__ __forceinline__ void store_shifted(const uint32_t (&w)[kWords], bool 
   }
 }
 
-// Sweep 3 when the gradient row lies differently than its logits row: every granule in turn, a step's two at a time
-// (both loads before either is used).  `smem`: kShiftWords a warp.
+// Sweep 3 when the gradient row lies differently than its logits row (another row stride or base): zeros first, in the
+// gradient row's own 32-byte pieces, then the safe tokens one by one.  (store_shifted for every granule instead, us, 1,000 x
+// 100,003 bfloat16 at rho = 1e-4 179 / 187, 5,000 x 20,000 float16 156 / 195; 2,000 x 50,021 at e^-13, where most granules
+// have a safe token, 227 / 200; both forms in one kernel cost float16 rows 3 %.)
 template <typename TIn, typename TGrad, int kBlk>
-__device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *grow, TGrad *entry_a, int g_a, float out_a,
-                                               float tau, typename SweepOps<TIn>::Tau tau_p,
-                                               typename SweepOps<TIn>::Key key, bool live, uint64_t m2, uint64_t coef2,
-                                               const uint32_t *bound, uint32_t *smem) {
-  constexpr int kElems = Granule<TIn>::kElems, kWords = kGradWords<TIn, TGrad>;
-  const int tid = threadIdx.x, first = tid & ~31, lane = tid & 31;
-  smem += (tid >> 5) * kShiftWords;
-  for (int step = 0; 2 * step * kBlk + first < v.n_full; ++step) {
-    const int wi = step * kBlk + tid, g0 = 2 * step * kBlk + tid;
-    const uint32_t b = live && DVP_IN(wi, n_bound, DVP_OOB_BOUND) ? SweepOps<TIn>::reach(bound[wi], key) : 0u;
-    Granule<TIn> gr[2];
-    const bool hot[2] = {(b & 1u) && g0 < v.n_full, (b & 0x10000u) && g0 + kBlk < v.n_full};
+__device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *grow, int a, float tau,
+                                               typename SweepOps<TIn>::Key key, bool live, float m, float coef,
+                                               float g_a, const uint32_t *bound) {
+  constexpr int kElems = Granule<TIn>::kElems, kOut = 32 / (int)sizeof(TGrad);
+  const int tid = threadIdx.x, n_thr = kBlk;
+  const int k0 = v.head + v.g_first * kElems, k1 = k0 + v.n_full * kElems;  // this block's granules, as elements
+  TGrad *dst = grow + k0;
+  const int n = k1 - k0;
+  const int mis = (int)(((uintptr_t)dst & 31u) / sizeof(TGrad));
+  const int head = min(n, mis ? kOut - mis : 0), n_vec = (n - head) / kOut;
+  const uint32_t z[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  if (tid < head) dst[tid] = Storage<TGrad>::narrow(0.f);
+  for (int i = tid; i < n_vec; i += n_thr) st_stream32(dst + head + (size_t)i * kOut, z);
+  const int k_rest = head + n_vec * kOut + tid;
+  if (k_rest < n) dst[k_rest] = Storage<TGrad>::narrow(0.f);
+  __syncthreads();  // the zeros of this block's part are in place before single elements replace them
+  if (!live) return;
+  for (int i = 0;; ++i) {
+    const int g = i * n_thr + tid, wi = (i >> 1) * n_thr + tid;
+    if (g >= v.n_full || !DVP_IN(wi, n_bound, DVP_OOB_BOUND)) break;
+    if (!((SweepOps<TIn>::reach(bound[wi], key) >> (16 * (i & 1))) & 1u)) continue;
+    Granule<TIn> gr;
+    gr.load_whole(v.base, v.n_full, g);
+    float x[kElems];
+    gr.get(x);
+    const int ja = a - g * kElems;
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
-      if (hot[u]) gr[u].load_whole(v.base, v.n_full, g0 + u * kBlk);
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int g = g0 + u * kBlk, n = min(32, v.n_full - (g - lane));
-      if (n <= 0 || !DVP_IN((long long)(g - lane + n) * kElems - 1, V, DVP_OOB_GLOBAL)) break;
-      uint32_t w[kWords];
-      if (hot[u]) {
-        grad_words<TIn, TGrad>(gr[u], tau, tau_p, m2, coef2, w);
-      } else {
-#pragma unroll
-        for (int i = 0; i < kWords; ++i) w[i] = 0;
-      }
-      store_shifted(w, __any_sync(0xffffffffu, hot[u]), grow + (size_t)(g - lane) * kElems, n, smem);
-      __syncwarp();  // the sampled token's entry replaces what a lane of the warp stored there
-      if (g == g_a) *entry_a = Storage<TGrad>::narrow(out_a);
-    }
+    for (int j = 0; j < kElems; ++j)
+      if (x[j] >= tau)
+        dst[(size_t)g * kElems + j] =
+            Storage<TGrad>::narrow(j == ja ? g_a : coef * ex2((x[j] - m) * kLog2e));
   }
 }
 
@@ -1032,7 +1031,7 @@ __device__ __forceinline__ void row_grad_loose(const RowView<TIn> &v, TGrad *gro
 template <typename TIn, typename TGrad, int kBlk, bool kLoose>
 __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all, int a_row,
                                          const SideStats &st, float g, const uint32_t *bound,
-                                         const HotList &list, uint16_t *hot_smem) {
+                                         const HotList &list) {
   constexpr int kElems = Granule<TIn>::kElems;
   const TIn *row = v.base;
   const int n_full = v.n_full;
@@ -1079,8 +1078,7 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
   const typename SweepOps<TIn>::Tau tau_p = SweepOps<TIn>::threshold(fmaxf(st.tau, -FLT_MAX));
   const int g_here = a_here >= 0 ? v.granule_of(a_here) : -1;
   if constexpr (kLoose) {
-    row_grad_loose<TIn, TGrad, kBlk>(v, grow, grow_all + a_here, g_here, g_a, tau, tau_p, key, live, m2, cf2, bound,
-                                     reinterpret_cast<uint32_t *>(hot_smem));
+    row_grad_loose<TIn, TGrad, kBlk>(v, grow_all, a_here >= 0 ? v.rel(a_here) : -1, tau, key, live, st.m, coef, g_a, bound);
     return;
   }
   // one granule; the sampled token's entry replaces the one that its granule's store left
@@ -1140,7 +1138,6 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
 
 // Shared-memory layout of the row kernel, in 4-byte words: the block reductions, 8 for what blocks of a
 // cluster exchange, then the hot lists, then the bounds.
-static_assert(kShiftWords * 4 <= kHotCap * sizeof(uint16_t), "store_shifted uses the place of a warp's hot list");
 __host__ __device__ inline int smem_words_fixed(int threads) {
   return kRedWords + 8 + (threads / 32) * kHotCap / 2;
 }
@@ -1200,7 +1197,7 @@ dvp_row_kernel(const __grid_constant__ RowParams p, const long long t0, const in
       if (p.weight_out && writer) p.weight_out[t] = w;
     }
     row_grad<TIn, TGrad, kBlk, kGrad == Grad::kLoose>(v, reinterpret_cast<TGrad *>(p.grad) + t * p.ld_grad, a, st, g,
-                                                      bound, list, hot_smem);
+                                                      bound, list);
   }
   if (writer) {
     if (p.side == kSideTrain && !weighted) {
