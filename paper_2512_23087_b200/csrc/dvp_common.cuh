@@ -405,11 +405,13 @@ struct RowParams {
   float *weight_out;
   unsigned int *bounds_status;  // the bounds-checking build's status word; unused otherwise
   // the row kernel sweeps one row per token (`train`, `out_t`); with two launches for a call:
-  int side;  // kSide*
-  char *li;  // where ln pi^mp_infer(a) of token t passes from one to the other: two 2-byte halves at t * li_stride
+  int side;   // kSide*
+  int order;  // kOrder*
+  char *li;   // where ln pi^mp(a) of token t passes from the first to the second: two 2-byte halves at t * li_stride
   long long li_stride;
 };
-enum { kSideAlone = 0, kSideInfer = 1, kSideTrain = 2 };
+enum { kSideTrain = 0, kSideInfer = 1 };
+enum { kOrderAlone = 0, kOrderFirst = 1, kOrderSecond = 2, kOrderApart = 3 };
 
 __device__ __forceinline__ long long load_id(const void *ids, int is_i32, long long t) {
   return is_i32 ? (long long)reinterpret_cast<const int *>(ids)[t]
@@ -568,6 +570,9 @@ cudaError_t launch_row_kernels(const RowParams &p, int logits_dtype, int grad_dt
                                cudaStream_t s);
 cudaError_t launch_backward_kernel(const BackwardParams &p, int logits_dtype, int grad_dtype,
                                    uint32_t hint, cudaStream_t s);
+
+// The last of three launches for a call (kOrderApart): log-ratios and flags from what the other two have left.
+cudaError_t launch_ratio_kernel(const RowParams &p, long long t0, long long n, cudaStream_t s);
 
 // Synchronises the current device, reads the resident-row kernel's status word and clears it.
 cudaError_t read_and_clear_row_status(uint32_t *host_out);

@@ -66,6 +66,22 @@ cudaError_t read_and_clear_bounds_status(uint32_t *host_out) {
   return cudaMemcpyToSymbol(g_bounds_status, &zero, sizeof(zero));
 }
 
+// ln pi^mp of both policies and the training rows' flags are in place; log_ratio holds the inference rows' membership.
+__global__ void __launch_bounds__(256) dvp_ratio_kernel(const RowParams p, const long long t0, const long long n) {
+  begin_after();
+  const long long i = blockIdx.x * 256LL + threadIdx.x;
+  if (i >= n) return;
+  const long long t = t0 + i, id = p.ids ? load_id(p.ids, p.id_is_i32, t) : -1;
+  const bool valid = id >= 0 && id < p.V, in_infer = p.log_ratio[t] != 0.f;
+  const float lt = p.out_t.logp_mp[t], li = p.out_i.logp_mp[t];
+  p.log_ratio[t] = valid ? log_ratio_from(p.mode, lt > kNegInf, lt, li) : __int_as_float(0x7fc00000);
+  if (p.flags && in_infer) p.flags[t] |= DVP_FLAG_IN_INFER;
+}
+
+cudaError_t launch_ratio_kernel(const RowParams &p, long long t0, long long n, cudaStream_t s) {
+  return launch_after(dvp_ratio_kernel, (unsigned)((n + 255) / 256), 256, 0, s, p, t0, n);
+}
+
 cudaError_t launch_row_kernels(const RowParams &p_in, int logits_dtype, int grad_dtype, uint32_t hint,
                                cudaStream_t s) {
   RowParams p = p_in;

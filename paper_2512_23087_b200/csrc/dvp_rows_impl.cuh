@@ -507,7 +507,10 @@ __device__ __forceinline__ float ld_cluster_f32(const float *local, uint32_t ran
 }
 struct RowGroup {
   int parts, part;
-  float *slots;  // 4 floats of shared memory, each written once per kernel
+  float *slots;  // 6 floats of shared memory, each written once per kernel
+
+  // rank in the cluster of the row's first block: 0, or behind a token's other row
+  __device__ __forceinline__ uint32_t first() const { return cluster_rank() & (uint32_t)parts; }
 
   __device__ __forceinline__ float max(float m) const {
     if (parts == 1) return m;
@@ -516,7 +519,8 @@ struct RowGroup {
     cluster_arrive();
     cluster_wait();
     float hi = kNegInf;
-    for (int k = 0; k < parts; ++k) hi = fmaxf(hi, ld_cluster_f32(slots + 0, (uint32_t)k));
+    const uint32_t r0 = first();
+    for (int k = 0; k < parts; ++k) hi = fmaxf(hi, ld_cluster_f32(slots + 0, r0 + k));
     return hi;
   }
   __device__ __forceinline__ void sums(float &all, SumCount &safe) const {
@@ -531,10 +535,11 @@ struct RowGroup {
     cluster_wait();
     all = 0.f;
     safe = {0.f, 0};
+    const uint32_t r0 = first();
     for (int k = 0; k < parts; ++k) {  // in order: same result in every block
-      all += ld_cluster_f32(slots + 1, (uint32_t)k);
-      safe.s += ld_cluster_f32(slots + 2, (uint32_t)k);
-      safe.n += __float_as_int(ld_cluster_f32(slots + 3, (uint32_t)k));
+      all += ld_cluster_f32(slots + 1, r0 + k);
+      safe.s += ld_cluster_f32(slots + 2, r0 + k);
+      safe.n += __float_as_int(ld_cluster_f32(slots + 3, r0 + k));
     }
   }
 };
@@ -1148,12 +1153,14 @@ enum class Grad { kNone, kGranules, kLoose };
 // One row per block, or per cluster of 2^log_parts blocks.  kBlk: threads of a block, 1024 of them on an SM;
 // a compile-time constant, because it makes the sweeps' indices immediate operands.
 //
-// A token's two rows are swept by two launches, the inference rows' first: two copies of the sweeps in one
-// kernel stall on instruction fetches, a loop over the two rows spills 460 bytes a thread (rows 12 to 17 %
-// slower), and pairs of blocks in a cluster wait for two free places at once (18 % slower with two blocks
-// per SM).  The training rows' launch may begin while the last inference rows are still swept; it waits for
-// them where it needs ln pi^mp_infer(a) and the membership, which they leave at p.li and in p.flags.
-template <typename TIn, typename TGrad, int kBlk, Grad kGrad>
+// A batch that fills the chip is swept by two launches, one a policy: two copies of the sweeps in one kernel stall on
+// instruction fetches, a loop over the two rows spills 460 bytes a thread (rows 12 to 17 % slower), and pairs of blocks in
+// a cluster wait for two free places at once (18 % slower with two blocks per SM).  The second launch may begin while the
+// last rows of the first are still swept (launch_rows_both says which is first and how the two meet).
+//
+// Small calls are one launch, a token's two rows in one cluster (kTogether): ln pi^mp_infer(a) and the membership pass
+// through shared memory.
+template <typename TIn, typename TGrad, int kBlk, Grad kGrad, bool kTogether>
 __global__ void __launch_bounds__(kBlk, 1024 / kBlk)
 dvp_row_kernel(const __grid_constant__ RowParams p, const long long t0, const int log_parts) {
   extern __shared__ __align__(16) float smem[];
@@ -1162,63 +1169,104 @@ dvp_row_kernel(const __grid_constant__ RowParams p, const long long t0, const in
   uint32_t *bound = reinterpret_cast<uint32_t *>(smem + smem_words_fixed(kBlk));
 
   DVP_BOUNDS_BEGIN(p.bounds_status);
-  if (p.side == kSideInfer) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (p.order == kOrderFirst) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  constexpr int both = kTogether;
   const int parts = 1 << log_parts;
-  const RowGroup grp{parts, parts > 1 ? (int)cluster_rank() : 0, smem + kRedWords};
-  const long long t = t0 + (blockIdx.x >> log_parts);
+  // with both rows of a token in a cluster, the second half of its blocks has the inference row
+  auto other_half = [&] { return both && (int)cluster_rank() >= parts; };
+  // the rows of a launch with a gradient are the training rows
+  constexpr bool any_side = kGrad == Grad::kNone;
+  float *slots = smem + kRedWords;
+  const RowGroup grp{parts, parts > 1 ? (int)cluster_rank() & (parts - 1) : 0, slots};
+  const long long t = t0 + (blockIdx.x >> (log_parts + both));
   const long long id = p.ids ? load_id(p.ids, p.id_is_i32, t) : -1;
   const bool has_id = id >= 0, bad_id = id >= p.V;
   const int a = (has_id && !bad_id) ? (int)id : -1;
   const bool writer = threadIdx.x == 0 && grp.part == 0;
   RowView<TIn> v;
-  v.set(reinterpret_cast<const TIn *>(p.train) + t * p.ld_train, (int)p.V, grp.part, log_parts);
+  v.set(other_half() ? reinterpret_cast<const TIn *>(p.infer) + t * p.ld_infer
+                      : reinterpret_cast<const TIn *>(p.train) + t * p.ld_train,
+        (int)p.V, grp.part, log_parts);
   HotList list;
-  SideStats st = row_stats<TIn, kBlk>(v, a, p.log_rho, p.mode, p.mask_value, kGrad == Grad::kGranules, bound, red,
-                                      grp, hot_smem, list);
-  if (parts > 1) cluster_arrive();  // this block has read the others' slots
-  float li = 0.f;
+  SideStats st = row_stats<TIn, kBlk>(v, a, p.log_rho, p.mode, p.mask_value, kGrad == Grad::kGranules && !other_half(),
+                                      bound, red, grp, hot_smem, list);
   const bool weighted = p.weight_kind != DVP_WEIGHT_NONE;
-  if constexpr (kGrad != Grad::kNone) {
-    float g = p.upstream[t];
-    if (weighted) {
-      asm volatile("griddepcontrol.wait;" ::: "memory");
-      li = load_li(p, t);
-      const float w = a < 0 ? __int_as_float(0x7fc00000)
-                            : token_weight(log_ratio_from(p.mode, st.member, logp_mp_of(st), li), p.weight_kind,
-                                           p.weight_lo, p.weight_hi);
-      if (w == w) g *= w;
-      if (parts > 1) {  // every block of the row has li before the place that holds it is overwritten
-        cluster_wait();
-        cluster_arrive();
-        cluster_wait();
-      } else {
-        __syncthreads();
+  float li = 0.f;
+  if (both) {  // ln pi^mp_infer(a) and the membership; and the inference row has been read
+    if (other_half() && writer) {
+      slots[4] = logp_mp_of(st);
+      slots[5] = st.member ? 1.f : 0.f;
+    }
+    __syncthreads();
+    cluster_arrive();
+    cluster_wait();
+    if (!other_half()) {
+      li = ld_cluster_f32(slots + 4, (uint32_t)parts);
+      if (writer) {
+        slots[4] = li;
+        slots[5] = ld_cluster_f32(slots + 5, (uint32_t)parts);
       }
-      if (p.weight_out && writer) p.weight_out[t] = w;
     }
-    row_grad<TIn, TGrad, kBlk, kGrad == Grad::kLoose>(v, reinterpret_cast<TGrad *>(p.grad) + t * p.ld_grad, a, st, g,
-                                                      bound, list);
   }
+  if (parts > 1 || both) cluster_arrive();  // this block has read the others' slots
+  if constexpr (kGrad != Grad::kNone) {
+    if (!other_half()) {
+      float g = p.upstream[t];
+      if (weighted) {
+        if (!both) {
+          asm volatile("griddepcontrol.wait;" ::: "memory");
+          li = load_li(p, t);
+        }
+        const float w = a < 0 ? __int_as_float(0x7fc00000)
+                              : token_weight(log_ratio_from(p.mode, st.member, logp_mp_of(st), li), p.weight_kind,
+                                             p.weight_lo, p.weight_hi);
+        if (w == w) g *= w;
+        if (!both) {
+          if (parts > 1) {  // every block of the row has li before the place that holds it is overwritten
+            cluster_wait();
+            cluster_arrive();
+            cluster_wait();
+          } else {
+            __syncthreads();
+          }
+        }
+        if (p.weight_out && writer) p.weight_out[t] = w;
+      }
+      row_grad<TIn, TGrad, kBlk, kGrad == Grad::kLoose>(v, reinterpret_cast<TGrad *>(p.grad) + t * p.ld_grad, a, st, g,
+                                                        bound, list);
+    }
+  }
+  const bool second_half = other_half();
+  const dvp_side_out &out = second_half ? p.out_i : p.out_t;
   if (writer) {
-    if (p.side == kSideTrain && !weighted) {
+    if (p.order == kOrderSecond && !weighted) {
       asm volatile("griddepcontrol.wait;" ::: "memory");
       li = load_li(p, t);
     }
+    if (both) li = slots[4];
     st.lse = lse_from_logsum({st.m, (float)st.sum_c, st.sum_s});
-    const float lt = finish_side(p.out_t, t, st, has_id, bad_id);
-    if (p.side == kSideInfer) store_li(p, t, lt);
-    if (p.flags) {
-      const uint8_t in_infer = p.side == kSideTrain ? p.flags[t] & DVP_FLAG_IN_INFER : 0;
-      const uint8_t member = p.side == kSideInfer ? DVP_FLAG_IN_INFER : DVP_FLAG_IN_TRAIN;
-      p.flags[t] = (uint8_t)((st.member ? member : 0) | in_infer | (has_id ? 0 : DVP_FLAG_NO_ID) |
+    const float own = finish_side(out, t, st, has_id, bad_id);
+    if (p.order == kOrderFirst) store_li(p, t, own);
+    if (p.flags && !second_half) {
+      const uint8_t theirs = any_side && p.side == kSideInfer ? DVP_FLAG_IN_TRAIN : DVP_FLAG_IN_INFER;
+      const uint8_t before = p.order == kOrderSecond ? p.flags[t] & theirs : both && slots[5] != 0.f ? theirs : 0;
+      const uint8_t member = any_side && p.side == kSideInfer ? DVP_FLAG_IN_INFER : DVP_FLAG_IN_TRAIN;
+      p.flags[t] = (uint8_t)((st.member ? member : 0) | before | (has_id ? 0 : DVP_FLAG_NO_ID) |
                              (bad_id ? DVP_FLAG_BAD_ID : 0));
     }
-    if (p.log_ratio) p.log_ratio[t] = a < 0 ? __int_as_float(0x7fc00000) : log_ratio_from(p.mode, st.member, lt, li);
+    if (p.log_ratio && !second_half)
+      p.log_ratio[t] = any_side && p.order == kOrderApart     ? (st.member ? 1.f : 0.f)
+                       : a < 0                                ? __int_as_float(0x7fc00000)
+                       : any_side && p.side == kSideInfer     ? log_ratio_from(p.mode, li > kNegInf, li, own)
+                                                              : log_ratio_from(p.mode, st.member, own, li);
   }
-  if (p.out_t.mask)
-    write_mask_row<TIn>(v.row, v.V, st.tau, p.out_t.mask + t * ((p.V + 31) / 32), grp.part, parts);
+  if (out.mask)
+    write_mask_row<TIn>(v.row, v.V, st.tau, out.mask + t * ((p.V + 31) / 32), grp.part, parts);
+  // whoever waits for this launch waits for the one before too
+  if (any_side && p.order == kOrderApart && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
   // no block may leave while another one can still read its exchange slots
-  if (parts > 1 && !(kGrad != Grad::kNone && weighted)) {
+  if (both || (parts > 1 && !(kGrad != Grad::kNone && weighted))) {
     __syncwarp();
     cluster_wait();
   }
@@ -1440,84 +1488,138 @@ static inline bool grad_over(const RowParams &p, const void *logits, long long l
          z < g + (size_t)((p.T - 1) * p.ld_grad + p.V) * sizeof(TGrad);
 }
 
-template <typename TIn, typename TGrad, int kBlk, Grad kGrad>
+template <typename TIn, typename TGrad, int kBlk, Grad kGrad, bool kTogether>
 static cudaError_t launch_rows_vec(const RowParams &p, long long t0, long long n, int log_parts, size_t smem,
                                    cudaStream_t s) {
-  auto k = dvp_row_kernel<TIn, TGrad, kBlk, kGrad>;
+  auto k = dvp_row_kernel<TIn, TGrad, kBlk, kGrad, kTogether>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(n << log_parts), 1, 1);
+  const int log_cluster = log_parts + (kTogether ? 1 : 0);
+  cfg.gridDim = dim3((unsigned)(n << log_cluster), 1, 1);
   cfg.blockDim = dim3(kBlk, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   cfg.attrs = attr;
   cfg.numAttrs = 0;
-  if (log_parts > 0) {
+  if (log_cluster > 3) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  if (log_cluster > 0) {
     attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
-    attr[cfg.numAttrs].val.clusterDim.x = 1u << log_parts;
+    attr[cfg.numAttrs].val.clusterDim.x = 1u << log_cluster;
     attr[cfg.numAttrs].val.clusterDim.y = 1;
     attr[cfg.numAttrs++].val.clusterDim.z = 1;
   }
-  // may begin while the inference rows' launch ends; not where the gradient overwrites inference rows
-  if (p.side == kSideTrain && !grad_over<TIn, TGrad>(p, p.infer, p.ld_infer)) {
+  // may begin while the first launch ends; not where the gradient overwrites inference rows
+  if ((p.order == kOrderSecond || p.order == kOrderApart) && !grad_over<TIn, TGrad>(p, p.infer, p.ld_infer)) {
     attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
   }
   return cudaLaunchKernelEx(&cfg, k, p, t0, log_parts);
 }
 
-template <typename TIn, typename TGrad, Grad kGrad>
+template <typename TIn, typename TGrad, Grad kGrad, bool kTogether>
 static cudaError_t launch_rows_blk(const RowParams &p, long long t0, long long n, int log_parts, int threads,
                                    size_t smem, cudaStream_t s) {
   switch (threads) {
-    case 64: return launch_rows_vec<TIn, TGrad, 64, kGrad>(p, t0, n, log_parts, smem, s);
-    case 128: return launch_rows_vec<TIn, TGrad, 128, kGrad>(p, t0, n, log_parts, smem, s);
-    case 256: return launch_rows_vec<TIn, TGrad, 256, kGrad>(p, t0, n, log_parts, smem, s);
-    default: return launch_rows_vec<TIn, TGrad, 512, kGrad>(p, t0, n, log_parts, smem, s);
+    case 64:
+      if constexpr (kTogether) return cudaErrorNotSupported;  // rows of less than 128 granules
+      return launch_rows_vec<TIn, TGrad, 64, kGrad, false>(p, t0, n, log_parts, smem, s);
+    case 128: return launch_rows_vec<TIn, TGrad, 128, kGrad, kTogether>(p, t0, n, log_parts, smem, s);
+    case 256: return launch_rows_vec<TIn, TGrad, 256, kGrad, kTogether>(p, t0, n, log_parts, smem, s);
+    default: return launch_rows_vec<TIn, TGrad, 512, kGrad, kTogether>(p, t0, n, log_parts, smem, s);
   }
 }
 
-// The inference rows, then the training rows.  ln pi^mp_infer(a) passes through the output that holds it, or
-// through one that the training rows' launch writes later: log_ratio, weight_out, or the start of the gradient
-// row (with a single 2-byte gradient element there is no room: V = 1, where ln pi^mp(a) is 0).
+// Does the gradient lie in the place of the inference rows, row for row?  (Not in other places of theirs.)
+template <typename TIn, typename TGrad>
+static inline bool grad_over_its_infer_row(const RowParams &p) {
+  return p.grad == p.infer && sizeof(TGrad) == sizeof(TIn) && (p.T == 1 || p.ld_grad == p.ld_infer);
+}
+
+// Both policies' rows, in one launch, two or three; the second may begin while the first ends.
+//
+// One launch for calls that fill half of the chip at most, bound by the chain of their phases and by
+// what a launch costs on the host (2 of 17 us).  Device time of 64 x 4,096 float32, forward / with the gradient, two
+// launches and one: 6.5 / 8.5 and 5.8 / 7.9 us; 8 x 151,936 bfloat16 10.5 / 12.6 and 9.3 / 12.1; weighted 148 x 2,312 float32 10.1 and
+// 7.8.  Above, clusters wait for free places: 1,100 x 2,500 bfloat16 10.1 / 12.8 and 12.5 / 17.4, 32 x 151,936 (clusters
+// of 16) 13.7 / 17.6 and 16.6 / 22.1.
+// Otherwise the rows with a gradient come first: the chip's last wave then has the short rows.  While all rows fit the chip
+// at once the inference rows wait for the training rows at their end; in larger batches they would hold their places
+// idle, so that neither launch waits for the other and a third one forms the log-ratios and flags (the inference rows'
+// membership passes through log_ratio).  us, with the gradient, inference rows first / now: V = 151,936 bfloat16, T = 256
+// 72 / 64, 512 122 / 112, 800 177 / 157, 2,048 379 / 358, 4,096 707 / 684; 1,000 x 65,536 99 / 89; float32 1,000 x 50,021
+// 129 / 122, 2,000 x 100,000 428 / 418.  (Waiting in larger batches: T = 800 187, 2,048 388.)  The third launch costs some
+// 4 us, the last wave of 32,768 bfloat16 rows 40 (5,537 / 5,513); that of float32 rows, which are bound by their bytes
+// alone, less than that from some 16 waves on (4,096 x 262,144, 28 waves: 1,892 / 1,897).
+// The inference rows come first where the training rows need them, for weights, where the gradient takes their place, and
+// without a gradient; and in larger batches where a third launch does not pay or an output that it needs is missing.
+//
+// Between a first and a second launch ln pi^mp(a) passes through the output that holds it, or through one that the second
+// launch writes later: log_ratio, weight_out, or the start of the gradient row (with a single 2-byte gradient element
+// there is no room: V = 1, where ln pi^mp(a) is 0).
 template <typename TIn, typename TGrad>
 static cudaError_t launch_rows_both(const RowParams &p_in, bool loose, int log_parts, int threads, size_t smem,
                                     cudaStream_t s) {
+  const bool weighted = p_in.weight_kind != DVP_WEIGHT_NONE;
+  const bool over_infer = grad_over<TIn, TGrad>(p_in, p_in.infer, p_in.ld_infer);
+  const bool resident = (p_in.T << (log_parts + 1)) * threads <= 148 * 1024;
+  auto launch = [&](const RowParams &p, long long t0, long long n, auto together) {
+    constexpr bool kTogether = decltype(together)::value;
+    return !p.grad ? launch_rows_blk<TIn, TIn, Grad::kNone, kTogether>(p, t0, n, log_parts, threads, smem, s)
+           : loose ? launch_rows_blk<TIn, TGrad, Grad::kLoose, kTogether>(p, t0, n, log_parts, threads, smem, s)
+                   : launch_rows_blk<TIn, TGrad, Grad::kGranules, kTogether>(p, t0, n, log_parts, threads, smem, s);
+  };
+  if (p_in.infer && (p_in.T << (log_parts + 1)) * threads <= 74 * 1024 &&
+      (!over_infer || grad_over_its_infer_row<TIn, TGrad>(p_in))) {
+    RowParams p = p_in;
+    const cudaError_t e = launch(p, 0, p.T, std::true_type{});
+    if (e == cudaSuccess) return e;
+    (void)cudaGetLastError();  // very short rows, or a cluster of 16 blocks that the device does not take: two launches
+  }
   const long long per_launch = 0x7fffffffLL >> log_parts;  // a grid holds this many rows
+  const bool pays = sizeof(TIn) == 2 || (p_in.T << (log_parts + 1)) * threads <= 16 * 148 * 1024LL;
+  const bool train_first = p_in.infer && p_in.grad && !weighted && !over_infer &&
+                           (resident || (pays && p_in.log_ratio && p_in.out_t.logp_mp && p_in.out_i.logp_mp));
   for (long long t0 = 0; t0 < p_in.T; t0 += per_launch) {
     const long long n = p_in.T - t0 < per_launch ? p_in.T - t0 : per_launch;
-    RowParams p = p_in;
-    p.side = kSideAlone;
+    RowParams p = p_in, q = p_in;  // the training rows' launch, the inference rows'
+    p.side = kSideTrain;
+    q.side = kSideInfer;
+    q.train = p_in.infer;
+    q.ld_train = p_in.ld_infer;
+    q.out_t = p_in.out_i;
+    q.infer = nullptr;
+    q.grad = nullptr;
+    q.weight_kind = DVP_WEIGHT_NONE;
+    RowParams &first = train_first ? p : q, &second = train_first ? q : p;
+    cudaError_t e = cudaSuccess;
     if (p_in.infer) {
-      p.li_stride = sizeof(float);
-      p.li = reinterpret_cast<char *>(p_in.out_i.logp_mp ? p_in.out_i.logp_mp
-                                      : p_in.log_ratio   ? p_in.log_ratio
-                                                         : p_in.weight_out);
-      if (!p.li && p_in.weight_kind != DVP_WEIGHT_NONE && p_in.V * sizeof(TGrad) >= sizeof(float)) {
-        p.li = reinterpret_cast<char *>(p_in.grad);
-        p.li_stride = p_in.ld_grad * (long long)sizeof(TGrad);
+      first.order = kOrderFirst;
+      first.log_ratio = nullptr;
+      second.order = train_first && !resident ? kOrderApart : kOrderSecond;
+      if (second.order == kOrderApart) {
+        second.flags = nullptr;
+      } else {
+        char *place = reinterpret_cast<char *>(first.out_t.logp_mp ? first.out_t.logp_mp
+                                               : p_in.log_ratio    ? p_in.log_ratio
+                                                                   : p_in.weight_out);
+        p.li_stride = q.li_stride = sizeof(float);
+        if (!place && weighted && p_in.V * sizeof(TGrad) >= sizeof(float)) {
+          place = reinterpret_cast<char *>(p_in.grad);
+          p.li_stride = q.li_stride = p_in.ld_grad * (long long)sizeof(TGrad);
+        }
+        p.li = q.li = place;
       }
-      RowParams q = p;
-      q.side = kSideInfer;
-      q.train = p_in.infer;
-      q.ld_train = p_in.ld_infer;
-      q.out_t = p_in.out_i;
-      q.infer = nullptr;
-      q.grad = nullptr;
-      q.log_ratio = nullptr;
-      q.weight_kind = DVP_WEIGHT_NONE;
-      const cudaError_t e = launch_rows_blk<TIn, TIn, Grad::kNone>(q, t0, n, log_parts, threads, smem, s);
-      if (e != cudaSuccess) return e;
-      p.side = kSideTrain;
+      e = launch(first, t0, n, std::false_type{});
     }
-    const cudaError_t e =
-        !p.grad ? launch_rows_blk<TIn, TIn, Grad::kNone>(p, t0, n, log_parts, threads, smem, s)
-        : loose ? launch_rows_blk<TIn, TGrad, Grad::kLoose>(p, t0, n, log_parts, threads, smem, s)
-                : launch_rows_blk<TIn, TGrad, Grad::kGranules>(p, t0, n, log_parts, threads, smem, s);
+    if (e == cudaSuccess) e = launch(second, t0, n, std::false_type{});
+    if (e == cudaSuccess && second.order == kOrderApart) e = launch_ratio_kernel(p_in, t0, n, s);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

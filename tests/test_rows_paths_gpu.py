@@ -107,6 +107,38 @@ def test_outputs_left_out(kept, V, weighted):
         assert same(out["logp_mp_i"], full.infer.logp_mp)
 
 
+@pytest.mark.parametrize("T,V,dtype", [(1, 5003, "bf16"), (148, 5003, "bf16"), (149, 5003, "bf16"), (592, 5003, "bf16"),
+                                       (1300, 5003, "bf16"), (5, 151936, "bf16"), (37, 151936, "f16"), (74, 4096, "f32"),
+                                       (75, 4096, "f32"), (9, 262143, "f32")])
+def test_launches_of_a_call(T, V, dtype):
+    """Both policies' rows in one launch, in two with either first, and in three, on both sides of the rules' lines.  Without
+    some of the outputs, or with the gradient over the inference rows, the order is another one and the results the same."""
+    w = dataclasses.replace(W["c2_bf16_fwdbwd"], dtype=dtype, head_boost=2.0, head_max=1)
+    b = inputs.make_rows(w, seed=T, device=DEV, T=T, V=V)
+    full = _check(b, 1e-2, V)
+    again = binding.dvp_forward(b.train, b.ids, 1e-2, infer_logits=b.infer, upstream=b.upstream)
+    over = b.infer.clone()
+    placed = binding.dvp_forward(b.train, b.ids, 1e-2, infer_logits=over, upstream=b.upstream, grad_train=over)
+    some, a = {"log_ratio": torch.empty(T, device=DEV), "flags": torch.empty(T, dtype=torch.uint8, device=DEV)}, binding.ForwardArgs()
+    grad = torch.empty_like(b.train)
+    code = binding._DTYPES[b.train.dtype]
+    a.struct_size, a.logits_dtype, a.grad_dtype = ctypes.sizeof(binding.ForwardArgs), code, code
+    a.T, a.V, a.rho = T, V, 1e-2
+    a.ld_train = a.ld_infer = a.ld_grad = V
+    a.train_logits, a.infer_logits, a.ids = b.train.data_ptr(), b.infer.data_ptr(), b.ids.data_ptr()
+    a.upstream, a.grad_train = b.upstream.data_ptr(), grad.data_ptr()
+    a.log_ratio, a.flags = some["log_ratio"].data_ptr(), some["flags"].data_ptr()
+    a.stream = torch.cuda.current_stream().cuda_stream
+    assert binding.load_library().dvp_forward(ctypes.byref(a)) == binding.DVP_OK
+    torch.cuda.synchronize()
+    for got in (again.grad_train, placed.grad_train, grad):
+        assert torch.equal(got, full.grad_train)
+    for n, x in some.items():
+        assert all(torch.equal(y, getattr(full, n)) for y in (getattr(again, n), getattr(placed, n), x)), n
+    for n in ("lse", "logp_mp", "log_cov", "count"):
+        assert all(torch.equal(getattr(r.infer, n), getattr(full.infer, n)) for r in (again, placed)), n
+
+
 @pytest.mark.parametrize("dtype,V,hint", [("bf16", 151936, 64), ("bf16", 151936, 256), ("bf16", 151936, 256 | (2 << 24)),
                                           ("f16", 50021, 64), ("f32", 262144, 512), ("f32", 40003, 64)])
 def test_full_sum_keeps_small_terms(dtype, V, hint):
