@@ -1666,26 +1666,40 @@ static cudaError_t launch_rows_cs(const RowParams &p, int threads, int n_steps, 
 // 1904 against 2180 at 256).
 //
 // While all rows fit the chip at once, more threads a row are faster (100 x 20,000 bfloat16: 17.5 at 256
-// against 21.5 at 128 and 29.7 at 64), then more blocks a row (V = 151,936 bfloat16, 1 / 2 / 4 / 8 blocks:
-// T = 16 forward 36 / 28 / 21 / 19; T = 64 forward 38 / 32 / 28 / 34; T = 128 with the gradient
-// 65 / 50 / 48 / 60; T = 512 130 / 126 / 134 / 192; V = 50,000, T = 100: 30 / 24 / 28 / 38).  Blocks that share
-// a row need at least a step and a half of it each (V = 20,000: 13 / 15), four steps where the chip is full
-// without them (T = 512, V = 32,000, one matrix: 26 / 31).
+// against 21.5 at 128 and 29.7 at 64); so they are while the rows that come first do, and a thread has four granules (300 x
+// 32,000 bfloat16 with the gradient 26.7 -> 22.6; 1,000 x 20,000, which do not fit, 37.1 / 43.2), 2-byte rows up to a few
+// more than fit (600 x 32,000 42.5 -> 35.4; 300 x 27,652 float32 28.3 / 28.9).
+//
+// Then more blocks a row, V = 151,936 bfloat16, 1 / 2 / 4 / 8 blocks: T = 16 forward 36 / 28 / 21 / 19; T = 128 with the
+// gradient 57 / 47 / 41.  Blocks that share a row need at least a step and a half of it each (V = 20,000: 13 / 15), without
+// a gradient two and a half where they fill more than half of the chip (100 x 32,000 12.4 / 14.1).
+//
+// With the gradient they pay also beyond the chip, the further the longer a thread's part of a row is, because the last
+// wave is shorter.  us, 1 block / 2, at about 2, 3.5, 4.7 and 6.9 times the chip: 64 granules a thread (V = 262,144) 101 / 74,
+// 203 / 180, 264 / 237, 358 / 331; 37 (V = 151,936) 64 / 50, 117 / 113, 146 / 146, 198 / 200; 24 (V = 100,000 float32) 57 / 55, 80 / 79,
+// 114 / 126; with weights 37 granules 171 / 164 at 4.7, 24 91 / 86 at 3.5; 12 (V = 50,021) 29 / 31 at 1.4.  2 blocks / 4 at 2, 2.7
+// and 4: 64 granules 74 / 68, 90 / 81, 113 / 111; 37 50 / 49, 56 / 58, 75 / 81; 24 28 / 30 at 1.7.
+// Without a gradient only very long rows gain by it: V = 262,144 140 / 130 and 196 / 169 at 3.5 and 4.7 times the chip;
+// V = 151,936 65 / 81 and 77 / 88 at 2.7 and 3.5, V = 100,000 float32 44 / 55 at 2.7.
 struct RowShape {
   int threads, log_parts;
 };
-static inline RowShape choose_shape(long long rows, long long n_gran, int most) {
-  const long long resident = 148 * 1024;
+// `first`: the rows, of `rows`, that are swept first (with weights taken like without, so that their statistics are the same).
+static inline RowShape choose_shape(long long rows, long long first, long long n_gran, int most, bool grad) {
+  const long long chip = 148 * 1024, nearly = most == 256 ? 152 * 1024 : chip;  // 256: 2-byte rows
   RowShape s = {64, 0};
   while (s.threads < most && 16LL * s.threads < n_gran) s.threads *= 2;
-  while (s.threads < most && 2 * rows * s.threads <= resident && n_gran >= 2 * s.threads) s.threads *= 2;
+  while (s.threads < most && 2 * rows * s.threads <= chip && n_gran >= 2 * s.threads) s.threads *= 2;
+  while (s.threads < most && 2 * first * s.threads <= nearly && n_gran >= 8 * s.threads) s.threads *= 2;
   while (s.log_parts < 3) {
     const int lp = s.log_parts + 1;
-    const long long per = n_gran >> lp, total = (rows << lp) * s.threads;
-    const bool fits = total <= resident || (per >= 8 * s.threads && total <= (lp == 1   ? 4 * resident
-                                                                             : lp == 2 ? 2 * resident
-                                                                                       : resident));
-    if (per < 3 * s.threads || !fits) break;
+    const long long per = n_gran >> lp, total = (rows << lp) * s.threads, steps = n_gran / s.threads;
+    const long long least = grad || 2 * total <= chip ? 3 : 5;
+    // total / chip: at most steps / 6, but 8 (2 blocks), or steps / 16 (4); steps / 12 or / 24 without a gradient
+    const long long scale = grad ? (lp == 1 ? 6 : 16) : 6 << lp;
+    const bool beyond =
+        lp < 3 && steps >= (grad ? 20 : 48) && total * scale <= steps * chip && total <= 8 * chip;
+    if (per < least * s.threads || !(total <= chip || beyond)) break;
     s.log_parts = lp;
   }
   return s;
@@ -1717,7 +1731,8 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
   const bool store_kernel = sizeof(TIn) == 2 && (stage_hint == 3 || stage_hint == 4);
   int log_parts = 0;
   if (threads == 0 && cluster == 0 && !store_kernel) {
-    const RowShape sh = choose_shape(p.T * (p.infer ? 2 : 1), n_gran_row, sizeof(TIn) == 4 ? 512 : 256);
+    const RowShape sh = choose_shape(p.T * (p.infer ? 2 : 1), p.T * (p.infer && !p.grad ? 2 : 1), n_gran_row,
+                                     sizeof(TIn) == 4 ? 512 : 256, p.grad != nullptr);
     threads = sh.threads;
     log_parts = sh.log_parts;
   } else {
@@ -1773,15 +1788,17 @@ static cudaError_t launch_rows_g(const RowParams &p, int grad_dtype, uint32_t hi
   }
 }
 
-// Blocks of a row: as many as bring some 16 warps to every SM (four times its 2,048 threads' worth of rows are enough),
-// while each has a step or more.
+// Threads: up to eight granules each (64 / 128 / 256 threads, us: 20,000 x 4,001 bfloat16 57 / 68 / 98, 10,000 x 2,500 with
+// float32 entries 30 / 35 / 47, 3,130 x 7,488 float16 15.3 / 17.8 / 18.6, 10,400 x 21,440 bfloat16 144 / 140 / 140).  Blocks of a row:
+// as many as bring some 16 warps to every SM (four times its 1,024 threads' worth of rows are enough), while each has a
+// step or more.
 template <typename TIn, typename TGrad>
 static cudaError_t launch_bwd(const BackwardParams &p, uint32_t hint, cudaStream_t s) {
   const long long n_gran = p.V / Granule<TIn>::kElems;
   int threads = hint & 0xffff, log_parts = 0;
   if (threads == 0) {
-    threads = 256;
-    while (threads > 64 && threads >= n_gran) threads /= 2;
+    threads = 64;
+    while (threads < 256 && n_gran > 8 * threads) threads *= 2;
   }
   while (log_parts < 10 && (p.T << log_parts) * threads < 4 * 148 * 1024 && n_gran >> (log_parts + 1) >= 2 * threads)
     ++log_parts;
