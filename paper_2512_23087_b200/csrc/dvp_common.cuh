@@ -249,9 +249,8 @@ __device__ __forceinline__ MaxSum combine(MaxSum a, MaxSum b) {
   return r;
 }
 
-// scratch: 64 floats of shared memory.  Result valid in every thread.
-__device__ __forceinline__ MaxSum block_reduce_maxsum(MaxSum v, float *scratch) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
+__device__ __forceinline__ MaxSum warp_reduce(MaxSum v) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     MaxSum other;
@@ -260,6 +259,13 @@ __device__ __forceinline__ MaxSum block_reduce_maxsum(MaxSum v, float *scratch) 
     // keep operand order independent of the lane so both partners agree
     v = (lane & o) ? combine(other, v) : combine(v, other);
   }
+  return v;
+}
+
+// scratch: 64 floats of shared memory.  Result valid in every thread.
+__device__ __forceinline__ MaxSum block_reduce_maxsum(MaxSum v, float *scratch) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
+  v = warp_reduce(v);
   __syncthreads();  // scratch may still be read from an earlier reduction
   if (lane == 0) {
     scratch[warp] = v.m;
@@ -269,14 +275,7 @@ __device__ __forceinline__ MaxSum block_reduce_maxsum(MaxSum v, float *scratch) 
   MaxSum r;
   r.m = lane < nwarp ? scratch[lane] : kNegInf;
   r.s = lane < nwarp ? scratch[32 + lane] : 0.f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    MaxSum other;
-    other.m = __shfl_xor_sync(0xffffffffu, r.m, o);
-    other.s = __shfl_xor_sync(0xffffffffu, r.s, o);
-    r = (lane & o) ? combine(other, r) : combine(r, other);
-  }
-  return r;
+  return warp_reduce(r);
 }
 
 // Log-sum-exp state kept in the base-2 domain so that each term costs one FMA
@@ -344,8 +343,8 @@ struct SumCount {
   int n;
 };
 
-__device__ __forceinline__ SumCount block_reduce_sumcount(SumCount v, float *scratch) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
+__device__ __forceinline__ SumCount warp_reduce(SumCount v) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float os = __shfl_xor_sync(0xffffffffu, v.s, o);
@@ -353,6 +352,12 @@ __device__ __forceinline__ SumCount block_reduce_sumcount(SumCount v, float *scr
     v.s = (lane & o) ? os + v.s : v.s + os;
     v.n += on;
   }
+  return v;
+}
+
+__device__ __forceinline__ SumCount block_reduce_sumcount(SumCount v, float *scratch) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = (blockDim.x + 31) >> 5;
+  v = warp_reduce(v);
   __syncthreads();
   if (lane == 0) {
     scratch[warp] = v.s;
@@ -362,14 +367,7 @@ __device__ __forceinline__ SumCount block_reduce_sumcount(SumCount v, float *scr
   SumCount r;
   r.s = lane < nwarp ? scratch[lane] : 0.f;
   r.n = lane < nwarp ? reinterpret_cast<int *>(scratch)[32 + lane] : 0;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float os = __shfl_xor_sync(0xffffffffu, r.s, o);
-    const int on = __shfl_xor_sync(0xffffffffu, r.n, o);
-    r.s = (lane & o) ? os + r.s : r.s + os;
-    r.n += on;
-  }
-  return r;
+  return warp_reduce(r);
 }
 
 // Maximum over the block.  scratch: 32 floats.  Result valid in every thread.
