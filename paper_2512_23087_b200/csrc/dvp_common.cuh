@@ -93,6 +93,14 @@ __device__ __forceinline__ void ld_stream32(const void *p, uint32_t (&w)[8]) {
                : "l"(p));
 }
 
+// The same for what nobody reads again: the first that L2 gives up.
+__device__ __forceinline__ void ld_last32(const void *p, uint32_t (&w)[8]) {
+  asm volatile("ld.global.nc.L1::no_allocate.L2::evict_first.v8.u32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]),
+                 "=r"(w[7])
+               : "l"(p));
+}
+
 // Streaming stores (evict-first): the gradient is written once and not read
 // again by this library.
 __device__ __forceinline__ void st_stream16(void *p, uint4 v) {

@@ -347,7 +347,13 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     pp.hid_scale = hid_scale;
     pp.a_coef = a_coef;
     pp.scale = &sc->scale;
-    if (launch_after(panel::dvp_panel_kernel<512, 2>, (unsigned)rows, 512, 0, s, pp) != cudaSuccess) return DVP_ERR_CUDA;
+    // Few rows: as many threads a row as it has sums.  More than fill the chip: half of them, so that one row's reductions
+    // and results pass beside the sweeps of three others.  us a call with the first form / the second: 163 x 416 x 45,277
+    // 138 / 146, 767 x 1,448 x 10,474 172 / 170, 4,727 x 2,864 x 12,179 1,274 / 1,224, 3,891 x 2,752 x 58,933 4,220 / 3,997.
+    const cudaError_t pe = rows < 4 * 148
+                               ? launch_after(panel::dvp_panel_kernel<1, 4>, (unsigned)rows, panel::kSums, 0, s, pp)
+                               : launch_after(panel::dvp_panel_kernel<2, 1>, (unsigned)rows, panel::kSums / 2, 0, s, pp);
+    if (pe != cudaSuccess) return DVP_ERR_CUDA;
     // d_hidden[r0 : r0 + rows] = diag(c) P W + q_t W[a_t]: the factor is applied per row and the 1[k = a] term
     // added in fp32.  Few output tiles and a long K: each tile is computed as several K ranges, whose partial
     // results go where the logits were (read for the last time by the row pass) and are summed in order.

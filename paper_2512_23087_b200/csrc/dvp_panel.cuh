@@ -44,8 +44,9 @@ struct PanelSums {
   int n;                  // |V_S|
 };
 
-__device__ __forceinline__ void absorb_panel(const Granule<float> &gr, int g, int n_full, int V, int a, float m,
-                                             float tau, PanelSums &acc, __half *prow) {
+template <bool kWhole>
+__device__ __forceinline__ void absorb_panel(const Granule<float> &gr, int g, int V, int a, float m, float tau,
+                                             PanelSums &acc, __half *prow) {
   constexpr int kElems = 8;
   float x[kElems];
   gr.get(x);
@@ -73,8 +74,8 @@ __device__ __forceinline__ void absorb_panel(const Granule<float> &gr, int g, in
     w[j / 2] = *reinterpret_cast<const uint32_t *>(&h2);
   }
   acc.s_all += all;
-  if (g < n_full) {
-    st_stream16(prow + (size_t)g * kElems, make_uint4(w[0], w[1], w[2], w[3]));
+  if constexpr (kWhole) {
+    *reinterpret_cast<uint4 *>(prow + (size_t)g * kElems) = make_uint4(w[0], w[1], w[2], w[3]);
   } else {
     const __half *h = reinterpret_cast<const __half *>(w);
 #pragma unroll
@@ -85,27 +86,42 @@ __device__ __forceinline__ void absorb_panel(const Granule<float> &gr, int g, in
   }
 }
 
-template <int kThreads, int kBlocks>
-__global__ void __launch_bounds__(kThreads, kBlocks) dvp_panel_kernel(const PanelParams pp) {
+// The sums of a row are 512 partial ones, kSets of them a thread: the i-th over the granules i, i + 512, ..., however many
+// threads a block has.  Every set has kAhead granules in flight, the first of them while the row's maximum is found.
+constexpr int kSums = 512;
+template <int kSets, int kAhead>
+__global__ void __launch_bounds__(kSums / kSets, 2 * kSets) dvp_panel_kernel(const PanelParams pp) {
   __shared__ float scratch[96];
   const RowParams &p = pp.row;
-  constexpr int kElems = 8, kStage = 2;
+  constexpr int kElems = 8, kThreads = kSums / kSets;
   begin_after();
   const long long t = blockIdx.x;
   DVP_BOUNDS_BEGIN(p.bounds_status);
   DVP_BOUNDS_SET(n_gran, (p.V + kElems - 1) / kElems);
   DVP_BOUNDS_SET(V, p.V);
   DVP_BOUNDS_SYNC();
+  const int V = (int)p.V, tid = (int)threadIdx.x;
+  const float *row = reinterpret_cast<const float *>(p.train) + t * p.ld_train;
+  __half *prow = pp.P + t * pp.ld_p;
+  const int n_full = V / kElems;
+  // the logits are not read again, the gradient panel is, by two contractions: L2 keeps the latter (without: 3,891 x 2,752
+  // x 58,933 3,894 us a call, 3,710 with; 4,727 x 2,864 x 12,179 1,233 / 1,196)
+  auto load_last = [&](Granule<float> &gr, int g) {
+    if (DVP_IN((long long)g * kElems + kElems - 1, V, DVP_OOB_GLOBAL)) ld_last32(row + (size_t)g * kElems, gr.w);
+  };
+  Granule<float> gr[kAhead][kSets];
+#pragma unroll
+  for (int u = 0; u < kAhead; ++u)
+#pragma unroll
+    for (int v = 0; v < kSets; ++v)
+      if (tid + v * kThreads + u * kSums < n_full) load_last(gr[u][v], tid + v * kThreads + u * kSums);
   const long long id = load_id(p.ids, p.id_is_i32, t);
   const bool has_id = id >= 0, bad_id = id >= p.V;
   const int a = (has_id && !bad_id) ? (int)id : -1;
-  const int V = (int)p.V;
-  const float *row = reinterpret_cast<const float *>(p.train) + t * p.ld_train;
-  __half *prow = pp.P + t * pp.ld_p;
 
   const float *pieces = pp.row_max + t * pp.row_max_ld;
   float mx = kNegInf;
-  for (int i = threadIdx.x; i < pp.row_max_n; i += blockDim.x) mx = fmaxf(mx, pieces[i]);
+  for (int i = tid; i < pp.row_max_n; i += kThreads) mx = fmaxf(mx, pieces[i]);
   const float m = block_reduce_max(mx, scratch);
 
   SideStats st;
@@ -116,41 +132,52 @@ __global__ void __launch_bounds__(kThreads, kBlocks) dvp_panel_kernel(const Pane
   st.member = has_a && st.z_a >= st.tau;
   st.e_a = st.member ? ex2((st.z_a - m) * kLog2e) : 0.f;
 
-  const int n_full = V / kElems;
-  const int n_gran = (V + kElems - 1) / kElems;
-  const int per_step = kStage * (int)blockDim.x;
-  const int n_steps = (n_gran + per_step - 1) / per_step;
-  PanelSums acc = {0.f, 0.f, 0};
-  if (n_steps > 0) {  // two stages in flight, as in the row kernels
-    Stage<float, kStage> s0, s1;
-    s0.load(row, V, n_full, 0);
-    int step = 0;
-    for (; step + 1 < n_steps; step += 2) {
-      s1.load(row, V, n_full, step + 1);
+  PanelSums acc[kSets];
 #pragma unroll
-      for (int u = 0; u < kStage; ++u)
-        absorb_panel(s0.g[u], (step * kStage + u) * (int)blockDim.x + (int)threadIdx.x, n_full, V, a, m, st.tau, acc,
-                     prow);
-      if (step + 2 < n_steps) s0.load(row, V, n_full, step + 2);
+  for (int v = 0; v < kSets; ++v) acc[v] = {0.f, 0.f, 0};
+  for (int g0 = tid; g0 < n_full; g0 += kAhead * kSums) {
 #pragma unroll
-      for (int u = 0; u < kStage; ++u)
-        absorb_panel(s1.g[u], ((step + 1) * kStage + u) * (int)blockDim.x + (int)threadIdx.x, n_full, V, a, m,
-                     st.tau, acc, prow);
-    }
-    if (step < n_steps) {
+    for (int u = 0; u < kAhead; ++u) {
 #pragma unroll
-      for (int u = 0; u < kStage; ++u)
-        absorb_panel(s0.g[u], (step * kStage + u) * (int)blockDim.x + (int)threadIdx.x, n_full, V, a, m, st.tau, acc,
-                     prow);
+      for (int v = 0; v < kSets; ++v) {
+        const int g = g0 + u * kSums + v * kThreads;
+        if (g < n_full) absorb_panel<true>(gr[u][v], g, V, a, m, st.tau, acc[v], prow);
+        if (g + kAhead * kSums < n_full) load_last(gr[u][v], g + kAhead * kSums);
+      }
     }
   }
-  const SumCount safe = block_reduce_sumcount({acc.s_safe_x, acc.n}, scratch);
-  const SumCount all = block_reduce_sumcount({acc.s_all, 0}, scratch);
-  st.s_x = safe.s;
-  st.n = safe.n;
-  st.lse = (double)m + (double)logf(all.s);
+#pragma unroll
+  for (int v = 0; v < kSets; ++v) {
+    if (n_full * kElems < V && n_full % kSums == tid + v * kThreads) {  // the ragged last granule
+      gr[0][0].load_any(row, V, n_full, n_full);
+      absorb_panel<false>(gr[0][0], n_full, V, a, m, st.tau, acc[v], prow);
+    }
+  }
+  {  // the partial sums by warps of 32, then the 16 of those, in a fixed order
+    const int lane = tid & 31, warp = tid >> 5;
+    constexpr int kParts = kSums / 32;
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < kSets; ++v) {
+      const SumCount x = warp_reduce(SumCount{acc[v].s_safe_x, acc[v].n});
+      const SumCount y = warp_reduce(SumCount{acc[v].s_all, 0});
+      if (lane == 0) {
+        const int at = warp + v * (kThreads / 32);
+        scratch[at] = x.s;
+        scratch[32 + at] = y.s;
+        scratch[64 + at] = __int_as_float(x.n);
+      }
+    }
+    __syncthreads();
+    const SumCount safe = warp_reduce(
+        lane < kParts ? SumCount{scratch[lane], __float_as_int(scratch[64 + lane])} : SumCount{0.f, 0});
+    const SumCount all = warp_reduce(SumCount{lane < kParts ? scratch[32 + lane] : 0.f, 0});
+    st.s_x = safe.s;
+    st.n = safe.n;
+    st.sum_s = all.s;
+  }
+  st.lse = (double)m + (double)logf(st.sum_s);
   st.sum_c = (double)m * (double)kLog2e;
-  st.sum_s = all.s;
   set_mask_mass(st, V, 0, 0.f, has_a);
 
   if (threadIdx.x == 0) {
