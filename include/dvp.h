@@ -271,7 +271,8 @@ int dvp_backward(const dvp_backward_args *args);
  *                 Its first 32-bit word is a status: 0 after a run in which
  *                 every tensor-core kernel finished, non-zero if one gave up
  *                 waiting (results are then invalid).
- *   panel_rows    0 = library default (at most 4096); otherwise a multiple of 128
+ *   panel_rows    0 = library default (4096, or more where 6 V panel_rows bytes are
+ *                 at most 1 GiB and the workspace has room); otherwise a multiple of 128
  *   weight_kind   DVP_WEIGHT_NONE, DVP_WEIGHT_TRUNCATE or DVP_WEIGHT_MASK, as in
  *                 dvp_forward: each token's upstream gradient is multiplied by its
  *                 importance weight (needs infer_logits; weight_hi must be finite,
@@ -421,7 +422,7 @@ int dvp_monitor(const dvp_monitor_args *args);
  *
  * Limit: the workspace the arguments need (dvp_workspace_bytes with the
  * panel_rows this entry uses: pass panel_rows = 128 to that query when you pass 0
- * here, since 0 means up to 4096 there; roughly (2 H + 6 panel_rows) V +
+ * here, since 0 means 4096 or more there; roughly (2 H + 6 panel_rows) V +
  * 2 H panel_rows bytes) must fit in
  * DVP_STATIC_WORKSPACE_BYTES, e.g. H = 1024, V = 8192, any T up to a few
  * thousand.  Larger problems return DVP_ERR_WORKSPACE and launch nothing.
