@@ -393,7 +393,8 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     for (int c0 = 0; c0 < rows; c0 += panel::kIdChunk) {
       const int n = rows - c0 < panel::kIdChunk ? rows - c0 : panel::kIdChunk;
       const void *ids_c = static_cast<const char *>(p.ids) + (long long)c0 * id_bytes;
-      (void)launch_after(panel::add_sampled_hidden_kernel, (unsigned)n, 256, 0, s, ids_c, p.id_is_i32, a_coef + c0, n,
+      (void)launch_after(panel::add_sampled_hidden_kernel, (unsigned)((n + panel::kSampledWarps - 1) / panel::kSampledWarps),
+                         panel::kSampledWarps * 32, panel::kSampledSmem, s, ids_c, p.id_is_i32, a_coef + c0, n,
                          hidden + (r0 + c0) * a->ld_hidden, a->ld_hidden, a->d_w, a->ld_dw, H);
     }
     if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;

@@ -258,43 +258,108 @@ __global__ void __launch_bounds__(256) sum_ranges_kernel(const float *part, long
 }
 
 // d_w[a, :] += sum over the tokens t of the chunk (at most 4096) with a_t = a, in token order, of q_t hidden[t, :].
-// One block per token; the block of the first token with an id does all tokens with that id.  Each block looks
-// for its id among the others' itself: 134 MB of int64 ids (67 of int32) out of L2 for 4096 tokens.  (Sorting the ids took one block
-// 35 to 41 us first.)
+// One warp per token; the warp of the first token with an id does all tokens with that id, and nobody else adds to that
+// row.  A block's eight warps look for theirs among the chunk's ids in shared memory, four to a load; loads go out in
+// batches, those of d_w's row among them (reductions in memory instead, 767 x 1,448 x 10,474: 165 us a call, 160 this way).
+// With a block a token, which read all ids itself, element by element, the kernel was 15 us of 200 (512 x 1,024 x 32,000), 46
+// of 190 (767 x 1,448 x 10,474) and 110 of 1,690 (8,192 x 1,024 x 20,011); it is 8, 16 and 53.  (Sorting the ids first: 35
+// to 41 us by itself.  In the epilogue of d_w's contraction: 27 us more a call than this, 512 x 1,024 x 32,000.)
 constexpr int kIdChunk = 4096;
-__global__ void __launch_bounds__(256) add_sampled_hidden_kernel(const void *ids, int id_is_i32, const float *a_coef,
-                                                                 int n, const __nv_bfloat16 *hidden,
-                                                                 long long ld_hidden, float *d_w, long long ld_dw,
-                                                                 int H) {
-  __shared__ uint32_t same[kIdChunk / 32];  // bit j: token j has this block's id
-  __shared__ int any;
-  const int i = blockIdx.x;
+constexpr int kSampledWarps = 8;
+constexpr size_t kSampledSmem = (size_t)kIdChunk * 4 + kSampledWarps * kIdChunk / 8;
+__global__ void __launch_bounds__(kSampledWarps * 32)
+add_sampled_hidden_kernel(const void *ids, int id_is_i32, const float *a_coef, int n, const __nv_bfloat16 *hidden,
+                          long long ld_hidden, float *d_w, long long ld_dw, int H) {
+  extern __shared__ __align__(16) int id_of[];  // [kIdChunk], -1: nothing to add
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t *same = reinterpret_cast<uint32_t *>(id_of + kIdChunk) + warp * (kIdChunk / 32);  // bit j: token j has our id
+  const int i = (int)blockIdx.x * kSampledWarps + warp;
   begin_after();
-  if (a_coef[i] == 0.f) return;
-  const long long a = load_id(ids, id_is_i32, i);
-  for (int k = threadIdx.x; k < kIdChunk / 32; k += blockDim.x) same[k] = 0;
-  if (threadIdx.x == 0) any = 0;
+  const int n4 = (n + 127) & ~127;
+  constexpr int kBlk = kSampledWarps * 32, kLoads = 8;  // all of a batch before the first is stored
+  for (int j0 = threadIdx.x; j0 < n4; j0 += kLoads * kBlk) {
+    long long of[kLoads];
+    float c[kLoads];
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int at = min(j0 + u * kBlk, n - 1);
+      of[u] = load_id(ids, id_is_i32, at);
+      c[u] = a_coef[at];
+    }
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int j = j0 + u * kBlk;
+      if (j < n4) id_of[j] = j < n && c[u] != 0.f ? (int)of[u] : -1;
+    }
+  }
+  for (int k = lane; k < kIdChunk / 32; k += 32) same[k] = 0;
   __syncthreads();
-  bool earlier = false;
-  for (int j = threadIdx.x; j < n; j += blockDim.x)
-    if (j != i && load_id(ids, id_is_i32, j) == a && a_coef[j] != 0.f) {
-      if (j < i) {
-        earlier = true;
-      } else {
-        atomicOr(&same[j >> 5], 1u << (j & 31));
-        any = 1;
+  const int a = i < n ? id_of[i] : -1;
+  if (a < 0) return;
+  bool earlier = false, later = false;
+  for (int j = lane * 4; j < n4; j += 128) {
+    const int4 v = *reinterpret_cast<const int4 *>(id_of + j);
+    const uint32_t bits = (v.x == a ? 1u : 0u) | (v.y == a ? 2u : 0u) | (v.z == a ? 4u : 0u) | (v.w == a ? 8u : 0u);
+    if (bits) {
+      if (j < i && bits & ((1u << min(4, i - j)) - 1u)) earlier = true;
+      if (j + 3 > i && bits & ~((2u << max(0, i - j)) - (j <= i ? 1u : 2u))) {
+        later = true;
+        atomicOr(&same[j >> 5], bits << (j & 31));
       }
     }
-  if (__syncthreads_or(earlier)) return;
-  float *out = d_w + a * ld_dw;
-  for (int h = threadIdx.x; h < H; h += blockDim.x) {
-    float acc = a_coef[i] * __bfloat162float(hidden[(long long)i * ld_hidden + h]);
-    if (any)
-      for (int k = i >> 5; k < (n + 31) / 32; ++k)
-        for (uint32_t m = same[k]; m; m &= m - 1) {
-          const int t = k * 32 + __ffs(m) - 1;
-          acc = fmaf(a_coef[t], __bfloat162float(hidden[(long long)t * ld_hidden + h]), acc);
-        }
+  }
+  if (__any_sync(0xffffffffu, earlier)) return;
+  later = __any_sync(0xffffffffu, later);
+  __syncwarp();
+  const float q = a_coef[i];
+  float *out = d_w + (long long)a * ld_dw;
+  const __nv_bfloat16 *own = hidden + (long long)i * ld_hidden;
+  // f(t): for the later tokens with this id, in order
+  auto others = [&](auto f) {
+    for (int k = i >> 5; k < (n + 31) / 32; ++k)
+      for (uint32_t m = same[k]; m; m &= m - 1) {
+        const int t = k * 32 + __ffs(m) - 1;
+        if (t > i) f(t);
+      }
+  };
+  constexpr int kAhead = 3;  // pieces of 8 columns in flight
+  for (int h0 = lane * 8; h0 + 8 <= H; h0 += kAhead * 256) {  // strides are multiples of 8 elements
+    uint4 raw[kAhead];
+    float was[kAhead][8];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int h = h0 + u * 256;
+      if (h + 8 > H) break;
+      raw[u] = *reinterpret_cast<const uint4 *>(own + h);
+      asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                   : "=f"(was[u][0]), "=f"(was[u][1]), "=f"(was[u][2]), "=f"(was[u][3]), "=f"(was[u][4]), "=f"(was[u][5]),
+                     "=f"(was[u][6]), "=f"(was[u][7])
+                   : "l"(out + h));
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int h = h0 + u * 256;
+      if (h + 8 > H) break;
+      float x[8], acc[8];
+      Storage<__nv_bfloat16>::unpack(raw[u], x);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[j] = q * x[j];
+      if (later)
+        others([&](int t) {
+          const float c = a_coef[t];
+          Storage<__nv_bfloat16>::unpack(*reinterpret_cast<const uint4 *>(hidden + (long long)t * ld_hidden + h), x);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[j] = fmaf(c, x[j], acc[j]);
+        });
+      asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(out + h), "f"(was[u][0] + acc[0]),
+                   "f"(was[u][1] + acc[1]), "f"(was[u][2] + acc[2]), "f"(was[u][3] + acc[3]), "f"(was[u][4] + acc[4]),
+                   "f"(was[u][5] + acc[5]), "f"(was[u][6] + acc[6]), "f"(was[u][7] + acc[7])
+                   : "memory");
+    }
+  }
+  for (int h = (H & ~7) + lane; h < H; h += 32) {
+    float acc = q * __bfloat162float(own[h]);
+    if (later) others([&](int t) { acc = fmaf(a_coef[t], __bfloat162float(hidden[(long long)t * ld_hidden + h]), acc); });
     out[h] += acc;
   }
 }
