@@ -1,0 +1,73 @@
+"""Paths of the fused entry that depend on sizes and alignment: inference rows off the 32-byte grid, the panel's rows with
+one or two partial sums a thread, the default panel and the workspace that it fits."""
+import pytest
+import torch
+
+from paper_2512_23087_b200 import binding, inputs
+
+import parity
+import test_fused_gpu as fused
+
+pytestmark = pytest.mark.gpu
+DEV = fused.DEV
+W = inputs.WORKLOADS["c4_fused_lmhead"]
+
+
+# few rows are taken in pieces of 4 bytes, more in pieces of 16; rows of less than a piece, of one, and of several strips of
+# 512 elements with an end of their own
+@pytest.mark.parametrize("pad,offset", [(0, 1), (1, 0), (3, 5), (8, 8)])
+@pytest.mark.parametrize("T,V", [(24, 3), (24, 5), (24, 1025), (24, 9001), (600, 9), (600, 517), (600, 4099)])
+@pytest.mark.parametrize("checks", [False, True], ids=["", "bounds"])
+def test_inference_rows_that_start_anywhere(T, V, pad, offset, checks):
+    b = inputs.make_fused(W, seed=V, device=DEV, T=T, H=64, V=V)
+    b.ids[0], b.ids[1] = -1, V
+    ld = V + pad
+    buf = torch.full((offset + T * ld + 64,), 3.0e4, dtype=torch.bfloat16, device=DEV)
+    infer = buf[offset:offset + T * ld].view(T, ld)[:, :V]
+    infer.copy_(4 * b.infer)   # some of the tokens below the threshold
+    for rho in (1e-2, 0.0):
+        def run():
+            r = binding.dvp_fused_lmhead_forward_backward(b.hidden, b.w_vocab, b.ids, rho, b.upstream, infer_logits=infer)
+            torch.cuda.synchronize()
+            return r
+        if checks:
+            with binding.bounds_checking_library():
+                r = run()
+                assert binding.dvp_debug_bounds_status() == 0, "an index was out of range"
+        else:
+            r = run()
+        ids = b.ids.clone()
+        ids[1] = -1   # the oracle's name for a row without a token
+        want = parity.run_oracle(infer.contiguous(), None, ids, rho)
+        parity.check_side(r.infer, want.train, infer, V, "infer", {})
+        assert r.flags[0].item() & binding.DVP_FLAG_NO_ID and r.flags[1].item() & binding.DVP_FLAG_BAD_ID
+
+
+@pytest.mark.parametrize("T,H,V", [(591, 64, 4099), (592, 64, 4099), (600, 64, 4096), (700, 64, 1003), (600, 64, 7)])
+def test_panel_rows(T, H, V):
+    batch, res, want, rerun = fused._run_fused(T, H, V, 1e-2, seed=T + V)
+    fused._check_fused(batch, 1e-2, res, want, V, rerun=rerun)
+
+
+def test_default_panel_and_its_workspace():
+    """A small vocabulary has panels of more than 4096 tokens by default; a workspace for 4096 is still enough."""
+    T, H, V = 4300, 64, 1000
+    b = inputs.make_fused(W, seed=1, device=DEV, T=T, H=H, V=V)
+
+    def call(**kw):
+        r = binding.dvp_fused_lmhead_forward_backward(b.hidden, b.w_vocab, b.ids, 1e-3, b.upstream, infer_logits=b.infer, **kw)
+        torch.cuda.synchronize()
+        assert r.workspace[:4].view(torch.int32).item() == 0
+        return r
+    one, two = call(), call(panel_rows=4096)
+    assert one.workspace.numel() > two.workspace.numel()
+    small = call(workspace=torch.empty_like(two.workspace))
+    assert torch.equal(small.d_w, two.d_w) and torch.equal(small.d_hidden, two.d_hidden)
+    for n in ("lse", "logp_mp", "count", "log_cov"):
+        assert torch.equal(getattr(one.train, n), getattr(two.train, n)), n
+    # one sum of 4300 products instead of two: a rounding for every 16 of them
+    for x, y in ((one.d_w, two.d_w), (one.d_hidden, two.d_hidden)):
+        assert ((x - y).norm(dim=1) <= 1e-5 * y.norm(dim=1).max()).all()
+    with pytest.raises(binding.DvpError) as e:
+        call(workspace=torch.empty(two.workspace.numel() - 256, dtype=torch.uint8, device=DEV))
+    assert e.value.status == binding.DVP_ERR_WORKSPACE
