@@ -35,7 +35,7 @@ METRIC = "pruned_logprob_fwd_bwd_tokens_per_s"
 UNIT = "tokens/s"
 FALLBACK_HBM_GBS = 6650.0
 
-# DRAM bytes per call of the row kernel, two launches (dram__bytes_read.sum + dram__bytes_write.sum
+# DRAM bytes per call of the row kernel, both policies' launches (dram__bytes_read.sum + dram__bytes_write.sum
 # of one ncu capture of a dvp_forward call on T rows of the workload), keyed by (workload, rho); valid only for
 # the kernel sources whose digest is recorded with it, scaled by rows to the full batch.
 NCU_TRAFFIC = {
@@ -43,6 +43,12 @@ NCU_TRAFFIC = {
     ("c2_bf16_fwdbwd", 1e-3): {"digest": "31a815c921717097", "T": 2048, "bytes": 1.310682e9 + 0.564589e9},
     ("c3_f32_heavy", 1e-4): {"digest": "31a815c921717097", "T": 1024, "bytes": 2.147990e9 + 1.013474e9},
 }
+
+
+def _row_launches(w) -> int:
+    """Kernels of a dvp_forward call on a full batch: one a policy; for 2-byte logits with a gradient a third for the
+    log-ratios."""
+    return 3 if w.backward and w.dtype != "f32" else 2
 
 
 def _kernel_digest(names=("dvp_common.cuh", "dvp_rows_impl.cuh")) -> str:
@@ -277,7 +283,7 @@ def run_ours(args):
     ms = ev0.elapsed_time(ev1)
     ms_first = ev0.elapsed_time(ev_first) / n_first
     clocks = sampler.stop()
-    launches = 2 * args.steps      # two kernels per dvp_forward call: inference rows, training rows
+    launches = _row_launches(w) * args.steps
 
     # the workload's other threshold, timed the same way and reported beside the headline
     other = None
@@ -298,7 +304,7 @@ def run_ours(args):
         ev3.record(stream)
         barrier()
         other = {"rho": rho2, "ms_per_step": ev2.elapsed_time(ev3) / args.steps}
-        launches += 2 * args.steps
+        launches += _row_launches(w) * args.steps
 
     # ---- end to end: host buffers in, per-token results out, copies inside the timed region
     slab = min(T, 2048)
@@ -467,7 +473,7 @@ def rows_extra(name, steps, dev, peak, peak_kind, no_cpu_baseline):
         ev1.record(stream)
         torch.cuda.synchronize()
         sec = ev0.elapsed_time(ev1) * 1e-3 / steps
-        launches += 2 * steps
+        launches += _row_launches(w) * steps
         out["thresholds"].append({"rho": rho, "ms_per_step": sec * 1e3, "value": T / sec, "unit": UNIT,
                                   "achieved_gbs": alg_bytes / sec / 1e9, "frac": alg_bytes / sec / 1e9 / peak,
                                   "peak_kind": f"of {peak_kind}", "frac_of_nominal_8TBs": alg_bytes / sec / 1e9 / 8000.0})

@@ -248,6 +248,7 @@ def load_library() -> ctypes.CDLL:
             fn = lib[name]   # a function object of its own, with its own argtypes
             fn.argtypes, fn.restype = [ctypes.c_char_p], ctypes.c_int
             lib.packed[name] = fn
+        lib.forward_at = ctypes.cast(lib.dvp_forward, ctypes.c_void_p).value
         _lib = lib
     return _lib
 
@@ -381,7 +382,17 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
     call lie over one storage (at most eighty bytes a token): keeping one keeps
     that storage, and ``torch.save`` of one writes all of it unless it is cloned.
     """
-    packed = load_library().packed
+    lib = load_library()
+    mode = (DVP_MODE_FINITE_MASK if mask_value is not None else 0) | \
+        (DVP_MODE_THRESHOLD_IN_LOGITS_DTYPE if threshold_in_logits_dtype else 0)
+    if out is None and not want_mask:   # all of it in one native call
+        res = _host.forward(lib.forward_at, train_logits, ids, float(rho), infer_logits, upstream, grad_train, grad_dtype,
+                            None if stream is None else stream.cuda_stream, launch_hint & _UINT32, mode,
+                            0.0 if mask_value is None else mask_value, int(weight_kind) & _UINT32, weight_lo, weight_hi)
+        if type(res) is int:
+            raise DvpError(res, "dvp_forward")
+        return res
+    packed = lib.packed
     _check_matrix("train_logits", train_logits)
     T, V = train_logits.shape
     dtype = train_logits.dtype
@@ -418,8 +429,6 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
         grad_code, grad_ld = _DTYPES[grad_train.dtype], grad_train.stride(0)
     else:
         grad_train = None
-    mode = (DVP_MODE_FINITE_MASK if mask_value is not None else 0) | \
-        (DVP_MODE_THRESHOLD_IN_LOGITS_DTYPE if threshold_in_logits_dtype else 0)
     st = packed["dvp_forward"](_FORWARD_PACK.pack(
         _FORWARD_PACK.size, _DTYPES[dtype], grad_code, _id_dtype(ids), T, V, train_logits.stride(0),
         infer_logits.stride(0) if has_infer else 0, grad_ld, float(rho), train_logits.data_ptr(),

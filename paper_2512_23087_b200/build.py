@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import glob
 import os
+import shutil
 import subprocess
 import sys
 from concurrent.futures import ThreadPoolExecutor
@@ -61,17 +62,21 @@ def build_host(force: bool = False) -> str:
     """The Python helper ``_host`` (g++ against this interpreter's and torch's headers)."""
     src = os.path.join(CSRC, "host_outputs.cpp")
     target = host_target()
-    if not force and _host_is_for(target) and os.path.getmtime(HOST) >= os.path.getmtime(src):
+    if not force and _host_is_for(target) and os.path.getmtime(HOST) >= max(
+            os.path.getmtime(f) for f in (src, os.path.join(ROOT, "include", "dvp.h"))):
         return HOST
     import sysconfig
     import torch
     base = os.path.join(os.path.dirname(torch.__file__))
+    nvcc = shutil.which(_nvcc()) or "/usr/local/cuda/bin/nvcc"   # its headers
     tmp = HOST + f".{os.getpid()}.tmp"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", src, "-o", tmp,
            f'-DDVP_HOST_TARGET="{target}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-           "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(base, "include"),
+           "-I", os.path.join(ROOT, "include"), "-isystem", sysconfig.get_paths()["include"],
+           "-isystem", os.path.join(base, "include"),
            "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
-           "-L", os.path.join(base, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10"]
+           "-isystem", os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include"),
+           "-L", os.path.join(base, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("g++ failed: " + " ".join(cmd) + "\n" + r.stdout + r.stderr)

@@ -1255,10 +1255,10 @@ dvp_row_kernel(const __grid_constant__ RowParams p, const long long t0, const in
                              (bad_id ? DVP_FLAG_BAD_ID : 0));
     }
     if (p.log_ratio && !second_half)
-      p.log_ratio[t] = any_side && p.order == kOrderApart     ? (st.member ? 1.f : 0.f)
-                       : a < 0                                ? __int_as_float(0x7fc00000)
-                       : any_side && p.side == kSideInfer     ? log_ratio_from(p.mode, li > kNegInf, li, own)
-                                                              : log_ratio_from(p.mode, st.member, own, li);
+      p.log_ratio[t] = any_side && p.order == kOrderApart ? (st.member ? 1.f : 0.f)
+                       : a < 0                            ? __int_as_float(0x7fc00000)
+                       : any_side && p.side == kSideInfer ? log_ratio_from(p.mode, li > kNegInf, li, own)
+                                                          : log_ratio_from(p.mode, st.member, own, li);
   }
   if (out.mask)
     write_mask_row<TIn>(v.row, v.V, st.tau, out.mask + t * ((p.V + 31) / 32), grp.part, parts);
@@ -1544,11 +1544,11 @@ static inline bool grad_over_its_infer_row(const RowParams &p) {
 
 // Both policies' rows, in one launch, two or three; the second may begin while the first ends.
 //
-// One launch for calls that fill half of the chip at most, bound by the chain of their phases and by
-// what a launch costs on the host (2 of 17 us).  Device time of 64 x 4,096 float32, forward / with the gradient, two
-// launches and one: 6.5 / 8.5 and 5.8 / 7.9 us; 8 x 151,936 bfloat16 10.5 / 12.6 and 9.3 / 12.1; weighted 148 x 2,312 float32 10.1 and
-// 7.8.  Above, clusters wait for free places: 1,100 x 2,500 bfloat16 10.1 / 12.8 and 12.5 / 17.4, 32 x 151,936 (clusters
-// of 16) 13.7 / 17.6 and 16.6 / 22.1.
+// One launch for calls that fill half of the chip at most, bound by the chain of their phases and by what a launch costs on
+// the host (2 of 17 us).  Device time of 64 x 4,096 float32, forward / with the gradient, two launches and one: 6.5 / 8.5
+// and 5.8 / 7.9 us; 8 x 151,936 bfloat16 10.5 / 12.6 and 9.3 / 12.1; weighted 148 x 2,312 float32 10.1 and 7.8.  Above,
+// clusters wait for free places: 1,100 x 2,500 bfloat16 10.1 / 12.8 and 12.5 / 17.4, 32 x 151,936 (clusters of 16) 13.7 /
+// 17.6 and 16.6 / 22.1.
 // Otherwise the rows with a gradient come first: the chip's last wave then has the short rows.  While all rows fit the chip
 // at once the inference rows wait for the training rows at their end; in larger batches they would hold their places
 // idle, so that neither launch waits for the other and a third one forms the log-ratios and flags (the inference rows'

@@ -45,6 +45,62 @@ def test_out_of_memory_keeps_its_type():
     assert binding._host.outputs(torch.empty(1, device="cuda:0"), 5, 3, 0)[2] == 32
 
 
+def test_forward_refuses_what_it_is_not_made_for():
+    """Before anything is launched, with the types of error that Python code gives."""
+    x, ids = torch.zeros(3, 5), torch.zeros(3, dtype=torch.int64)
+    for error, call in ((ValueError, lambda: binding.dvp_forward(x, ids, 0.1)),
+                        (ValueError, lambda: binding.dvp_forward(x[0], ids, 0.1)),
+                        (TypeError, lambda: binding.dvp_forward(None, ids, 0.1)),
+                        (TypeError, lambda: binding.dvp_forward(x, ids, 0.1, launch_hint=2.0)),
+                        (ValueError, lambda: binding.dvp_forward(x, ids, "a"))):
+        with pytest.raises(error):
+            call()
+    with pytest.raises(TypeError):
+        binding._host.forward(1, 2)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("infer", [False, True])
+def test_forward_gives_what_the_packed_call_gives(infer, weighted):
+    """A call that also wants the masks goes through Python; all else must be the same, refusals too."""
+    if weighted and not infer:
+        return
+    g = torch.Generator(device="cuda:0").manual_seed(1)
+    z = torch.randn(7, 1003, generator=g, device="cuda:0") * 4
+    zi = z + 0.1 * torch.randn(7, 1003, generator=g, device="cuda:0") if infer else None
+    ids = torch.randint(0, 1003, (7,), generator=g, device="cuda:0", dtype=torch.int32)
+    up = torch.randn(7, generator=g, device="cuda:0")
+    kw = dict(infer_logits=zi, upstream=up, grad_dtype=torch.bfloat16, mask_value=-50.0)
+    if weighted:
+        kw.update(weight_kind=binding.DVP_WEIGHT_TRUNCATE, weight_hi=1.01)
+    stream = torch.cuda.Stream()
+    a, b = binding.dvp_forward(z, ids, 1e-2, **kw), binding.dvp_forward(z, ids, 1e-2, want_mask=True, **kw)
+    torch.cuda.synchronize()
+    c = binding.dvp_forward(z, ids, 1e-2, stream=stream, grad_train=torch.empty_like(a.grad_train), **{**kw, "grad_dtype": None})
+    torch.cuda.synchronize()
+    assert set(vars(a)) == set(vars(b)) and (a.infer is None) == (not infer) and a.train.mask is None
+    for r in (a, c):
+        for n in vars(b):
+            x, y = getattr(r, n), getattr(b, n)
+            if n in ("train", "infer") and y is not None:
+                assert list(vars(x)) == list(vars(y))
+                assert all(torch.equal(getattr(x, m), getattr(y, m)) for m in vars(y) if m != "mask"), n
+            elif y is None:
+                assert x is None
+            else:
+                assert x.dtype == y.dtype and x.shape == y.shape and torch.equal(x, y), n
+    for error, bad in ((ValueError, dict(infer_logits=z[:, :5])), (TypeError, dict(upstream=up.double())),
+                       (binding.DvpError, dict(weight_kind=binding.DVP_WEIGHT_RATIO, infer_logits=None)),
+                       (KeyError, dict(grad_train=torch.empty(7, 1003, device="cuda:0", dtype=torch.float64)))):
+        with pytest.raises(error):
+            binding.dvp_forward(z, ids, 1e-2, **{**kw, **bad})
+    with pytest.raises(TypeError):
+        binding.dvp_forward(z, ids.float(), 1e-2)
+    with pytest.raises(KeyError):
+        binding.dvp_forward(z.double(), ids, 1e-2)
+
+
 def test_helper_is_rebuilt_for_another_torch(monkeypatch, tmp_path):
     """A helper built against another torch (or interpreter) lays tensors over the wrong layout: it is neither kept by the
     build nor used by the binding."""
