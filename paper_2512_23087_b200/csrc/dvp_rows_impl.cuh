@@ -1254,17 +1254,19 @@ dvp_row_kernel(const __grid_constant__ RowParams p, const long long t0, const in
       p.flags[t] = (uint8_t)((st.member ? member : 0) | before | (has_id ? 0 : DVP_FLAG_NO_ID) |
                              (bad_id ? DVP_FLAG_BAD_ID : 0));
     }
-    if (p.log_ratio && !second_half)
+    if (p.log_ratio && !second_half) {
+      const bool swapped = any_side && p.side == kSideInfer;  // li is ln pi^mp_train(a) then, or -inf: no member
+      const float ratio = log_ratio_from(p.mode, swapped ? li > kNegInf : st.member, swapped ? li : own, swapped ? own : li);
       p.log_ratio[t] = any_side && p.order == kOrderApart ? (st.member ? 1.f : 0.f)
                        : a < 0                            ? __int_as_float(0x7fc00000)
-                       : any_side && p.side == kSideInfer ? log_ratio_from(p.mode, li > kNegInf, li, own)
-                                                          : log_ratio_from(p.mode, st.member, own, li);
+                                                          : ratio;
+    }
+    // whoever waits for this launch waits for the one before too
+    if (any_side && p.order == kOrderApart && (blockIdx.x | (parts - 1)) == gridDim.x - 1)
+      asm volatile("griddepcontrol.wait;" ::: "memory");
   }
   if (out.mask)
     write_mask_row<TIn>(v.row, v.V, st.tau, out.mask + t * ((p.V + 31) / 32), grp.part, parts);
-  // whoever waits for this launch waits for the one before too
-  if (any_side && p.order == kOrderApart && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
   // no block may leave while another one can still read its exchange slots
   if (both || (parts > 1 && !(kGrad != Grad::kNone && weighted))) {
     __syncwarp();
