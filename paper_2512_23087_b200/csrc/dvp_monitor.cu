@@ -299,7 +299,6 @@ dvp_monitor_kernel(const MonitorParams p, const int log_parts) {
 #pragma unroll
       for (int i = 0; i < 10; ++i) left[i] = v[i];
     }
-    __syncwarp();
     cluster_arrive();
     cluster_wait();
     if (part == 0 && tid == 0) {
@@ -311,7 +310,6 @@ dvp_monitor_kernel(const MonitorParams p, const int log_parts) {
         rb = combine(rb, {v[5], v[6], v[7], v[8], v[9]});
       }
     }
-    __syncwarp();
     cluster_arrive();  // no block leaves before its sums are read
     cluster_wait();
   }

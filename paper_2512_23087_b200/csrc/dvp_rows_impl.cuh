@@ -489,10 +489,14 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
+// The aligned forms want a whole warp at the same instruction, which a branch before them (one thread writing a slot) does
+// not leave behind by itself: both bring the warp together first.
 __device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ uint32_t cluster_addr(const void *local, uint32_t rank) {
@@ -515,7 +519,6 @@ struct RowGroup {
   __device__ __forceinline__ float max(float m) const {
     if (parts == 1) return m;
     if (threadIdx.x == 0) slots[0] = m;
-    __syncwarp();
     cluster_arrive();
     cluster_wait();
     float hi = kNegInf;
@@ -530,7 +533,6 @@ struct RowGroup {
       slots[2] = safe.s;
       slots[3] = __int_as_float(safe.n);
     }
-    __syncwarp();
     cluster_arrive();
     cluster_wait();
     all = 0.f;
@@ -1268,10 +1270,8 @@ dvp_row_kernel(const __grid_constant__ RowParams p, const long long t0, const in
   if (out.mask)
     write_mask_row<TIn>(v.row, v.V, st.tau, out.mask + t * ((p.V + 31) / 32), grp.part, parts);
   // no block may leave while another one can still read its exchange slots
-  if (both || (parts > 1 && !(kGrad != Grad::kNone && weighted))) {
-    __syncwarp();
+  if (both || (parts > 1 && !(kGrad != Grad::kNone && weighted)))
     cluster_wait();
-  }
 }
 
 // ---- scalar kernel: any row length --------------------------------------------
