@@ -1,5 +1,6 @@
-"""The aligned cluster barriers are undefined where a warp is not together, as after a branch that one thread takes: every one
-of them stands directly behind a __syncwarp() or another such barrier, whatever code calls it."""
+"""Aligned instructions are undefined where a warp is not together, as after a branch that some of its threads take: every
+cluster barrier and every read of tensor memory stands directly behind a __syncwarp() or another such instruction, whatever
+code calls it."""
 import glob
 import os
 import re
@@ -12,13 +13,20 @@ def _statements(path):
     return [" ".join(s.split()) for s in re.split(r";(?=\s*\n)|[{}]", text)]
 
 
-def test_warps_are_together_at_cluster_barriers():
+ALIGNED = ("barrier.cluster", "tcgen05.ld.sync", "tcgen05.wait::ld.sync")
+
+
+def _aligned(statement):
+    return any(name in statement for name in ALIGNED)
+
+
+def test_warps_are_together_at_aligned_instructions():
     found = 0
     for path in sorted(glob.glob(os.path.join(ROOT, "paper_2512_23087_b200", "csrc", "*.cu*"))):
         before = ""
         for s in _statements(path):
-            if "barrier.cluster" in s:
+            if _aligned(s):
                 found += 1
-                assert before == "__syncwarp()" or "barrier.cluster" in before, f"{os.path.basename(path)}: {s}"
+                assert before == "__syncwarp()" or _aligned(before), f"{os.path.basename(path)}: {s}"
             before = s
-    assert found >= 4
+    assert found >= 6
