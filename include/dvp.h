@@ -271,8 +271,9 @@ int dvp_backward(const dvp_backward_args *args);
  *                 Its first 32-bit word is a status: 0 after a run in which
  *                 every tensor-core kernel finished, non-zero if one gave up
  *                 waiting (results are then invalid).
- *   panel_rows    0 = library default (4096, or more where 6 V panel_rows bytes are
- *                 at most 1 GiB and the workspace has room); otherwise a multiple of 128
+ *   panel_rows    0 = library default (4096, or more where the buffers of a panel,
+ *                 (6 V + 2 H) panel_rows bytes and a little, stay within 1 GiB and the
+ *                 workspace has room); otherwise a multiple of 128
  *   weight_kind   DVP_WEIGHT_NONE, DVP_WEIGHT_TRUNCATE or DVP_WEIGHT_MASK, as in
  *                 dvp_forward: each token's upstream gradient is multiplied by its
  *                 importance weight (needs infer_logits; weight_hi must be finite,

@@ -132,15 +132,18 @@ struct FusedLayout {
   long long max_pieces;
 };
 
-// The default panel: 4096 tokens, or with a small vocabulary as many as keep its logits and gradients within 1 GiB.  Every
-// panel after the first adds to all of d_w (H = 2,864, V = 12,179: 98 us for 631 tokens, of which the products are 26).
+// The default panel: 4096 tokens, or as many as keep everything that it is made of within 1 GiB.  Every panel after the
+// first adds to all of d_w (H = 2,864, V = 12,179: 98 us for 631 tokens, of which the products are 26).
 constexpr long long kPanelRows = 4096, kPanelBytes = 1LL << 30;
 
 bool fused_layout(const dvp_fused_args *a, FusedLayout *L, bool small = false) {
   if (a->T < 0 || a->H < 1 || a->V < 1) return false;
+  L->Vp = (a->V + 15) / 16 * 16;
+  L->max_pieces = (a->V + gemm::kBN - 1) / gemm::kBN;  // one per tile column of the logits contraction
   long long panel = a->panel_rows;
   if (panel == 0) {
-    long long most = kPanelBytes / (6 * a->V) / 128 * 128;
+    // logits and gradients, hidden rows, row maxima, three factors: what is taken by the panel's tokens below
+    long long most = kPanelBytes / (6 * L->Vp + 2 * a->H + 4 * L->max_pieces + 12) / 128 * 128;
     if (most < kPanelRows || small) most = kPanelRows;
     panel = (a->T + 127) / 128 * 128;
     if (panel > most) panel = most;
@@ -148,7 +151,6 @@ bool fused_layout(const dvp_fused_args *a, FusedLayout *L, bool small = false) {
   }
   if (panel % 128 != 0 || panel < 128) return false;
   L->panel = panel;
-  L->Vp = (a->V + 15) / 16 * 16;
   L->Tp = (a->T + 7) / 8 * 8;
   if (L->Tp == 0) L->Tp = 8;
   size_t o = 0;
@@ -166,7 +168,6 @@ bool fused_layout(const dvp_fused_args *a, FusedLayout *L, bool small = false) {
   L->off_hs = take((size_t)a->H * panel * 2);  // the panel's hidden rows, scaled, transposed, float16
   L->off_z = take((size_t)panel * L->Vp * 4);
   L->off_g = take((size_t)panel * L->Vp * 2);
-  L->max_pieces = (a->V + gemm::kBN - 1) / gemm::kBN;  // one per tile column of the logits contraction
   L->off_rmax = take((size_t)panel * L->max_pieces * 4);
   L->off_rowscale = take((size_t)panel * 4);
   L->off_hidscale = take((size_t)panel * 4);

@@ -118,6 +118,18 @@ def test_argument_errors_are_reported_before_any_launch(lib):
     assert lib.dvp_sequence_aggregate(ctypes.byref(sa)) == b.DVP_OK                # no sequences: no-op
 
 
+@pytest.mark.parametrize("T,H,V", [(200000, 4096, 1000), (200000, 4096, 1), (80000, 4096, 2000), (9000, 512, 20011), (5000, 64, 1000)])
+def test_default_panel_is_bounded(lib, T, H, V):
+    """Whatever the sizes, the default panel's buffers (logits, gradients, hidden rows) take at most 1 GiB, or 4096 tokens'."""
+    from paper_2512_23087_b200 import binding as b
+
+    def need(panel):
+        a = b.FusedArgs()
+        a.struct_size, a.T, a.H, a.V, a.panel_rows = ctypes.sizeof(b.FusedArgs), T, H, V, panel
+        return b.dvp_workspace_bytes(b.DVP_ENTRY_FUSED_LMHEAD, a)
+    assert need(4096) <= need(0) <= max(need(4096), need(128) + 2 ** 30)
+
+
 def test_missing_library_fails_loudly(tmp_path, monkeypatch):
     from paper_2512_23087_b200 import binding
     monkeypatch.setattr(binding, "_lib", None)
