@@ -388,7 +388,7 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     // contiguous, as the transposed (MN-major) A operand of the contraction; it needs nothing of sum_ranges_kernel
     e = gemm::launch_gemm_tn(p16, L.Vp, hs16, L.panel, a->d_w, a->ld_dw, V, H, rows, false, 1.f / 32.f,
                              &sc->inv_scale, panel_index > 0 || a->accumulate_dw != 0, &sc->status, sms,
-                             s, false, true, 1, nullptr, 0, nullptr, 0, gemm::Order::kEarly);
+                             s, false, true, 1, nullptr, 0, nullptr, 0, gemm::Order::kEarly, gemm::kChainK);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
     // ... + q_t hidden_t into row a_t of d_w: tokens that share a row are added in token order
     for (int c0 = 0; c0 < rows; c0 += panel::kIdChunk) {

@@ -34,6 +34,14 @@ constexpr uint32_t kTmemCols = 512;
 constexpr size_t kSmemBytes = 1024 /*alignment slack*/ + (size_t)kStages * kStageBytes + 256;
 constexpr uint32_t kSpinLimit = 1u << 22;
 
+// The tensor core cuts off what does not fit its float32 accumulator, so that terms of one sign lose more the more of them
+// one sum takes: relative error of a product of positive numbers 2.35e-5 with K = 4,096, 4.8e-5 with 8,192, 9.6e-5 with
+// 16,384.  A launch that asks for it (`chain_k`) makes a tile's K several such sums, one accumulator after the other, and
+// adds each to C while the next is formed: the error of as many launches, without their fills and drains.  (Two sums
+// kept, added on their way out and stored once: 4 % more time for a call of 4,727 x 2,864 x 12,179 than with one sum, because
+// nothing overlaps the stores then; this way 1,249 and 1,256 us, one sum 1,222 and 1,273.)
+constexpr int kChainK = 4096;
+
 enum { kErrNone = 0, kErrProducerWait = 11, kErrMmaWaitFull = 12, kErrMmaWaitTmem = 13,
        kErrEpilogueWait = 14 };
 
@@ -53,6 +61,8 @@ struct Params {
                            // accumulated into); otherwise K range i goes to C + i * range_stride (elements)
   int early;               // pair kernel: see begin_after
   const float *row_scale;  // optional (pair kernel): row `row` of the product is multiplied by row_scale[row]
+  int chain;               // pair kernel: slices of K that are added up in the tensor core (kChainK), and how many such
+  uint32_t chains;         // sums, each added to C, a unit has
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -496,6 +506,10 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   // work units: every tile once per K range; unit u is tile u % n_tiles of range u / n_tiles
   const int n_units = n_tiles * p.split_k;
   const int k_per = (k_slices + p.split_k - 1) / p.split_k;
+  // a pair's accumulators in turn hold the sums of its units, of each one p.chains; its i-th sum belongs to unit
+  // unit_of(i) and takes the slices from first_slice(i) on
+  const auto unit_of = [&](uint32_t i) { return pair + (int)(i / p.chains) * n_pairs; };
+  const auto first_slice = [&](uint32_t i) { return unit_of(i) / n_tiles * k_per + (int)(i % p.chains) * p.chain; };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages2; ++s) {
@@ -560,10 +574,10 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                              ((uint32_t)(kPairBM >> 4) << 24) | (p.a_mn_major ? (1u << 15) : 0u);
       // bytes between two K = 16 steps of A: 32 inside a K-major row, 16 K-rows of an MN-major box
       const uint32_t a_step_bytes = p.a_mn_major ? 16u * 128u : (uint32_t)(kUmmaK * 2);
-      uint32_t it = 0, local_tile = 0;
-      for (int unit = pair; unit < n_units && !*abort_flag; unit += n_pairs, ++local_tile) {
-        const int k_lo = (unit / n_tiles) * k_per, k_hi = min(k_slices, k_lo + k_per);
-        const uint32_t buf = local_tile & 1, use = local_tile >> 1;
+      uint32_t it = 0;
+      for (uint32_t i = 0; unit_of(i) < n_units && !*abort_flag; ++i) {
+        const int k_lo = first_slice(i), k_hi = min(k_slices, k_lo + p.chain);
+        const uint32_t buf = i & 1, use = i >> 1;
         if (use > 0 && !mbar_wait(smem_u32(&sh->tmem_empty[buf]), (use - 1) & 1, abort_flag)) {
           if (!*abort_flag) { *abort_flag = 1; atomicExch(p.status, kErrMmaWaitTmem); }
           break;
@@ -599,12 +613,11 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const int quarter = warp & 3;
     const bool exchange = k_per <= kExchangeSlices;
     const float alpha_all = p.alpha * (p.alpha_dev ? *p.alpha_dev : 1.f);
-    uint32_t local_tile = 0;
-    for (int unit = pair; unit < n_units; unit += n_pairs, ++local_tile) {
-      const int tile = unit % n_tiles;
+    for (uint32_t i = 0; unit_of(i) < n_units; ++i) {
+      const int unit = unit_of(i), tile = unit % n_tiles;
       const int tm = m_fastest ? tile % tiles_m : tile / tiles_n;
       const int tn = m_fastest ? tile / tiles_m : tile % tiles_n;
-      const uint32_t buf = local_tile & 1, use = local_tile >> 1;
+      const uint32_t buf = i & 1, use = i >> 1;
       // the whole warp goes on or none of it: reading tensor memory and the exchange need every lane
       if (!__all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_u32(&sh->tmem_full[buf]), use & 1, abort_flag))) {
         if (!*abort_flag) { *abort_flag = 1; atomicExch(p.status, kErrEpilogueWait); }
@@ -633,7 +646,7 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           }
         }
         if (col < p.N) {
-          if (p.accumulate || add_ranges)
+          if (p.accumulate || add_ranges || i % p.chains > 0)  // after the thread's own stores of the unit's first sum
             store_columns<Out::kAdd>(crow + col, p.ldc, lane, p.M - (row - lane), r, alpha, p.N - col, exchange);
           else
             store_columns<Out::kStore>(crow + col, p.ldc, lane, p.M - (row - lane), r, alpha, p.N - col, exchange);
@@ -747,7 +760,7 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
                                   cudaStream_t stream, bool single_block_tiles = false,
                                   bool a_mn_major = false, int split_k = 1, float *row_max = nullptr,
                                   long long row_max_ld = 0, const float *row_scale = nullptr,
-                                  long long range_stride = 0, Order order = Order::kAlone) {
+                                  long long range_stride = 0, Order order = Order::kAlone, int chain_k = 0) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   if (lda % 8 || ldb % 8 || ldc % 8 || (uintptr_t)A % 16 || (uintptr_t)B % 16 || (uintptr_t)C % 32)
     return cudaErrorInvalidValue;
@@ -762,8 +775,13 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
   // per-tile row maxima are those of the stored values: only where a tile is stored once, whole
   if (row_max && (single_block_tiles || split_k > 1 || accumulate)) return cudaErrorInvalidValue;
   if (row_scale && single_block_tiles) return cudaErrorInvalidValue;
+  const int k_per = ((K + kBK - 1) / kBK + split_k - 1) / split_k;
+  // sums of at most chain_k, about one size: none is so short that the one before is still being stored when it ends
+  const int most = chain_k > 0 && split_k == 1 ? chain_k / kBK : k_per, n_chains = (k_per + most - 1) / most;
+  const int chain = (k_per + n_chains - 1) / n_chains, chains = (k_per + chain - 1) / chain;
+  if (row_max && chains > 1) return cudaErrorInvalidValue;
   Params p{C, ldc, M, N, K, alpha, alpha_dev, accumulate ? 1 : 0, status, a_mn_major ? 1 : 0, split_k,
-           row_max, row_max_ld, range_stride, order == Order::kEarly ? 1 : 0, row_scale};
+           row_max, row_max_ld, range_stride, order == Order::kEarly ? 1 : 0, row_scale, chain, (uint32_t)chains};
   if (split_k > 1 && !accumulate && range_stride == 0) {
     const cudaError_t z = cudaMemset2DAsync(C, (size_t)ldc * 4, 0, (size_t)N * 4, (size_t)M, stream);
     if (z != cudaSuccess) return z;

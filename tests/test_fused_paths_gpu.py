@@ -71,3 +71,29 @@ def test_default_panel_and_its_workspace():
     with pytest.raises(binding.DvpError) as e:
         call(workspace=torch.empty(two.workspace.numel() - 256, dtype=torch.uint8, device=DEV))
     assert e.value.status == binding.DVP_ERR_WORKSPACE
+
+
+# two sums of 34 slices, the last one of 12 tokens; two full ones; three; several panels of two
+@pytest.mark.parametrize("T,panel", [(4300, 0), (8192, 0), (9000, 0), (20000, 8192)])
+def test_long_sums_of_d_w(T, panel):
+    """Terms of one sign, where an accumulator of the tensor core loses the more the more of them it takes: the default's
+    error is that of panels of 4096."""
+    H, V = 64, 1000
+    b = inputs.make_fused(W, seed=T, device=DEV, T=T, H=H, V=V)
+    b.hidden.copy_(b.hidden.abs()), b.upstream.copy_(b.upstream.abs() + 0.5), b.ids.zero_()
+    z = b.hidden.double() @ b.w_vocab.double().t()
+    want = -(torch.softmax(z, 1) * b.upstream.double()[:, None]).t() @ b.hidden.double()   # but for row 0
+
+    def call(rows):
+        r = binding.dvp_fused_lmhead_forward_backward(b.hidden, b.w_vocab, b.ids, 0.0, b.upstream, panel_rows=rows)
+        torch.cuda.synchronize()
+        assert r.workspace[:4].view(torch.int32).item() == 0
+        return r.d_w[1:]
+    got, short = call(panel), call(4096)
+    error, least = ((x.double() - want[1:]).norm().item() for x in (got, short))
+    assert least <= 3e-5 * want[1:].norm().item()
+    # n terms of about one size lose n^2 / 2 units: no sum is longer than 4096, and none than the others, so that theirs lose
+    # no more than panels of 4096; 2 % for what is left of the terms' sizes
+    assert error <= least * 1.02
+    if T == 8192:
+        assert torch.equal(got, short)
