@@ -1530,7 +1530,7 @@ static cudaError_t launch_rows_blk(const RowParams &p, long long t0, long long n
                                    size_t smem, cudaStream_t s) {
   switch (threads) {
     case 64:
-      if constexpr (kTogether) return cudaErrorNotSupported;  // rows of less than 128 granules
+      if constexpr (kTogether) return cudaErrorInvalidValue;  // not made: launch_rows_both does not ask for it
       return launch_rows_vec<TIn, TGrad, 64, kGrad, false>(p, t0, n, log_parts, smem, s);
     case 128: return launch_rows_vec<TIn, TGrad, 128, kGrad, kTogether>(p, t0, n, log_parts, smem, s);
     case 256: return launch_rows_vec<TIn, TGrad, 256, kGrad, kTogether>(p, t0, n, log_parts, smem, s);
@@ -1577,12 +1577,13 @@ static cudaError_t launch_rows_both(const RowParams &p_in, bool loose, int log_p
            : loose ? launch_rows_blk<TIn, TGrad, Grad::kLoose, kTogether>(p, t0, n, log_parts, threads, smem, s)
                    : launch_rows_blk<TIn, TGrad, Grad::kGranules, kTogether>(p, t0, n, log_parts, threads, smem, s);
   };
-  if (p_in.infer && (p_in.T << (log_parts + 1)) * threads <= 74 * 1024 &&
+  if (p_in.infer && threads > 64 && (p_in.T << (log_parts + 1)) * threads <= 74 * 1024 &&  // 64: less than 128 granules
       (!over_infer || grad_over_its_infer_row<TIn, TGrad>(p_in))) {
     RowParams p = p_in;
     const cudaError_t e = launch(p, 0, p.T, std::true_type{});
-    if (e == cudaSuccess) return e;
-    (void)cudaGetLastError();  // very short rows, or a cluster of 16 blocks that the device does not take: two launches
+    // a cluster of 16 blocks is more than every device (or part of one) takes: two launches then
+    if (log_parts < 3 || (e != cudaErrorInvalidClusterSize && e != cudaErrorLaunchOutOfResources)) return e;
+    (void)cudaGetLastError();
   }
   const long long per_launch = 0x7fffffffLL >> log_parts;  // a grid holds this many rows
   const bool pays = sizeof(TIn) == 2 || (p_in.T << (log_parts + 1)) * threads <= 16 * 148 * 1024LL;

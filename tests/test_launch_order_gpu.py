@@ -1,6 +1,8 @@
 """Launches of a call may begin before their predecessor ends, and the fused entry's work beside one another.  Inputs that the
 stream has not written yet when the call is made, calls that share a workspace, and captured calls must give bit for
 bit what a call on finished inputs gives."""
+import ctypes
+
 import pytest
 import torch
 
@@ -98,3 +100,19 @@ def test_captured_calls():
         graph.replay()
         torch.cuda.synchronize()
         _same(rows, rw), _same(fused, fw)
+
+
+@pytest.mark.parametrize("V", [100, 2000, 20000])
+def test_an_error_of_the_caller_is_left_alone(V):
+    """A call that succeeds says nothing about errors that the caller has yet to read, and clears none."""
+    b = inputs.make_rows(W["c2_bf16_fwdbwd"], seed=1, device=DEV, T=4, V=V)
+    _rows_call(b, False)
+    torch.cuda.synchronize()
+    runtime = ctypes.CDLL("libcudart.so.12")   # the one that torch and the library have loaded
+    assert runtime.cudaGetLastError() == 0
+    invalid_device = runtime.cudaSetDevice(1000)
+    assert invalid_device != 0 and runtime.cudaPeekAtLastError() == invalid_device
+    _rows_call(b, False)
+    assert runtime.cudaGetLastError() == invalid_device
+    assert runtime.cudaGetLastError() == 0
+    torch.cuda.synchronize()
