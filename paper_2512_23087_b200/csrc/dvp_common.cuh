@@ -524,6 +524,12 @@ __device__ __forceinline__ float log_ratio_from(int mode, bool in_train, float l
   return (mode & DVP_MODE_FINITE_MASK) ? lt - li : log_ratio_of(in_train, li > kNegInf, lt, li);
 }
 
+// Membership of the training row where the inference row is swept after it: the bit that it left in its flags; without flags
+// from ln pi^mp(a), -inf outside V_S (NaN, of a row that is not finite, is no sign of a pruned token).
+__device__ __forceinline__ bool in_train_by(const uint8_t *flags, uint8_t bits, float lt) {
+  return flags ? (bits & DVP_FLAG_IN_TRAIN) != 0 : lt != kNegInf;
+}
+
 __device__ __forceinline__ float load_li(const RowParams &p, long long t) {
   if (!p.li) return 0.f;
   const uint16_t *h = reinterpret_cast<const uint16_t *>(p.li + t * p.li_stride);

@@ -74,8 +74,9 @@ __global__ void __launch_bounds__(256) dvp_ratio_kernel(const RowParams p, const
   const long long t = t0 + i, id = p.ids ? load_id(p.ids, p.id_is_i32, t) : -1;
   const bool valid = id >= 0 && id < p.V, in_infer = p.log_ratio[t] != 0.f;
   const float lt = p.out_t.logp_mp[t], li = p.out_i.logp_mp[t];
-  p.log_ratio[t] = valid ? log_ratio_from(p.mode, lt > kNegInf, lt, li) : __int_as_float(0x7fc00000);
-  if (p.flags && in_infer) p.flags[t] |= DVP_FLAG_IN_INFER;
+  const uint8_t bits = p.flags ? p.flags[t] : 0;
+  p.log_ratio[t] = valid ? log_ratio_from(p.mode, in_train_by(p.flags, bits, lt), lt, li) : __int_as_float(0x7fc00000);
+  if (p.flags && in_infer) p.flags[t] = bits | DVP_FLAG_IN_INFER;
 }
 
 cudaError_t launch_ratio_kernel(const RowParams &p, long long t0, long long n, cudaStream_t s) {

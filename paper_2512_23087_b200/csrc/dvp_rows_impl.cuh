@@ -1249,16 +1249,18 @@ dvp_row_kernel(const __grid_constant__ RowParams p, const long long t0, const in
     st.lse = lse_from_logsum({st.m, (float)st.sum_c, st.sum_s});
     const float own = finish_side(out, t, st, has_id, bad_id);
     if (p.order == kOrderFirst) store_li(p, t, own);
+    uint8_t before = 0;  // the other policy's membership
     if (p.flags && !second_half) {
       const uint8_t theirs = any_side && p.side == kSideInfer ? DVP_FLAG_IN_TRAIN : DVP_FLAG_IN_INFER;
-      const uint8_t before = p.order == kOrderSecond ? p.flags[t] & theirs : both && slots[5] != 0.f ? theirs : 0;
+      before = p.order == kOrderSecond ? p.flags[t] & theirs : both && slots[5] != 0.f ? theirs : 0;
       const uint8_t member = any_side && p.side == kSideInfer ? DVP_FLAG_IN_INFER : DVP_FLAG_IN_TRAIN;
       p.flags[t] = (uint8_t)((st.member ? member : 0) | before | (has_id ? 0 : DVP_FLAG_NO_ID) |
                              (bad_id ? DVP_FLAG_BAD_ID : 0));
     }
     if (p.log_ratio && !second_half) {
-      const bool swapped = any_side && p.side == kSideInfer;  // li is ln pi^mp_train(a) then, or -inf: no member
-      const float ratio = log_ratio_from(p.mode, swapped ? li > kNegInf : st.member, swapped ? li : own, swapped ? own : li);
+      const bool swapped = any_side && p.side == kSideInfer;  // li is ln pi^mp_train(a) then
+      const float ratio = log_ratio_from(p.mode, swapped ? in_train_by(p.flags, before, li) : st.member,
+                                         swapped ? li : own, swapped ? own : li);
       p.log_ratio[t] = any_side && p.order == kOrderApart ? (st.member ? 1.f : 0.f)
                        : a < 0                            ? __int_as_float(0x7fc00000)
                                                           : ratio;

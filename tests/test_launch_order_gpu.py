@@ -2,6 +2,7 @@
 stream has not written yet when the call is made, calls that share a workspace, and captured calls must give bit for
 bit what a call on finished inputs gives."""
 import ctypes
+import dataclasses
 
 import pytest
 import torch
@@ -116,3 +117,30 @@ def test_an_error_of_the_caller_is_left_alone(V):
     assert runtime.cudaGetLastError() == invalid_device
     assert runtime.cudaGetLastError() == 0
     torch.cuda.synchronize()
+
+
+# one launch; the training rows first and the inference rows waiting for them; three launches
+@pytest.mark.parametrize("T", [40, 250, 400])
+def test_log_ratio_of_odd_rows_in_every_order(T):
+    """Rows that are not finite have no meaning, but a token that the flags call a member is not given the ratio of a pruned
+    one, whichever launch forms it: with the gradient as without it."""
+    V = 20000
+    b = inputs.make_rows(dataclasses.replace(W["c2_bf16_fwdbwd"], dtype="f16"), seed=4, device=DEV, T=T, V=V)
+    a = b.ids[:6].long()
+    inf = float("inf")
+    b.train[0, a[0]] = inf                        # overflowed logits of sampled tokens
+    b.infer[1, a[1]] = inf
+    b.train[2, a[2]] = b.infer[2, a[2]] = inf
+    b.train[3, a[3]] = b.infer[3, a[3]] = -inf    # with rho = 0 every token is safe
+    b.train[4] = -inf
+    b.train[5, a[5]] = -inf
+    for rho in (1e-3, 0.0):
+        with_grad = binding.dvp_forward(b.train, b.ids, rho, infer_logits=b.infer, upstream=b.upstream)
+        without = binding.dvp_forward(b.train, b.ids, rho, infer_logits=b.infer)
+        torch.cuda.synchronize()
+        assert torch.equal(with_grad.flags, without.flags)
+        x, y = with_grad.log_ratio, without.log_ratio
+        odd = ~torch.isfinite(y)
+        assert torch.equal(odd, ~torch.isfinite(x)) and odd[:6].sum() >= 4
+        assert torch.equal(torch.nan_to_num(x[odd], nan=9e9), torch.nan_to_num(y[odd], nan=9e9))
+        assert ((x - y)[~odd].abs() <= 1e-5).all()   # sums over other partial sums
