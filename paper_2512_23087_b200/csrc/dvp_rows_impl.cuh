@@ -1580,7 +1580,7 @@ static cudaError_t launch_rows_both(const RowParams &p_in, bool loose, int log_p
                    : launch_rows_blk<TIn, TGrad, Grad::kGranules, kTogether>(p, t0, n, log_parts, threads, smem, s);
   };
   if (p_in.infer && threads > 64 && (p_in.T << (log_parts + 1)) * threads <= 74 * 1024 &&  // 64: less than 128 granules
-      (!over_infer || grad_over_its_infer_row<TIn, TGrad>(p_in))) {
+      (!over_infer || (grad_over_its_infer_row<TIn, TGrad>(p_in) && !p_in.out_i.mask))) {  // masks are written last
     RowParams p = p_in;
     const cudaError_t e = launch(p, 0, p.T, std::true_type{});
     // a cluster of 16 blocks is more than every device (or part of one) takes: two launches then

@@ -144,3 +144,15 @@ def test_log_ratio_of_odd_rows_in_every_order(T):
         assert torch.equal(odd, ~torch.isfinite(x)) and odd[:6].sum() >= 4
         assert torch.equal(torch.nan_to_num(x[odd], nan=9e9), torch.nan_to_num(y[odd], nan=9e9))
         assert ((x - y)[~odd].abs() <= 1e-5).all()   # sums over other partial sums
+
+
+@pytest.mark.parametrize("T", [4, 40, 250, 400])
+def test_masks_of_the_inference_rows_before_the_gradient_takes_their_place(T):
+    b = inputs.make_rows(W["c2_bf16_fwdbwd"], seed=5, device=DEV, T=T, V=20000)
+    want = binding.dvp_forward(b.train, b.ids, 1e-3, infer_logits=b.infer, upstream=b.upstream, want_mask=True)
+    torch.cuda.synchronize()
+    got = binding.dvp_forward(b.train, b.ids, 1e-3, infer_logits=b.infer, upstream=b.upstream, grad_train=b.infer,
+                              want_mask=True)
+    torch.cuda.synchronize()
+    assert torch.equal(got.infer.mask, want.infer.mask) and torch.equal(got.train.mask, want.train.mask)
+    assert torch.equal(got.infer.count, want.infer.count) and torch.equal(got.flags, want.flags)
