@@ -893,8 +893,8 @@ __host__ __device__ constexpr int grad_align() {
 }
 
 // 2^{(z - m) l} as 2^{z l - c} 2^{c - m l}, the second factor in the coefficient: one instruction less, and one rounding
-// more, which entries of 16 bits do not show (float32 entries of 333 x 50,021 logits: relative error 5.9e-8 with it,
-// 5.0e-8 without).
+// more (float32 entries of 333 x 50,021 logits: relative error 5.9e-8 with it, 5.0e-8 without): the row kernel does so for
+// entries of 16 bits, which show it as one in some thousands rounded the other way.  The stand-alone backward does not.
 template <typename TIn, typename TGrad>
 constexpr bool kFoldedGrad = sizeof(TIn) == 2 && sizeof(TGrad) == 2;
 
@@ -903,20 +903,21 @@ template <typename TIn, typename TGrad>
 constexpr int kGradWords = Granule<TIn>::kElems * (int)sizeof(TGrad) / 4;
 
 // Gradient entries coef 2^{(z - m) l} of a whole granule (m2: -m twice, coef2: coef twice), zeros below the threshold.
-// 16-bit logits and entries: coef 2^{z l - m2}, one instruction less for two of them (see kFoldedGrad).
-template <typename TIn, typename TGrad>
+// kFold: coef 2^{z l - m2}, one instruction less for two of them (see kFoldedGrad).
+template <typename TIn, typename TGrad, bool kFold>
 __device__ __forceinline__ void grad_words(const Granule<TIn> &gr, float tau, typename SweepOps<TIn>::Tau tau_p,
                                            uint64_t m2, uint64_t coef2, uint32_t (&w)[kGradWords<TIn, TGrad>]) {
   constexpr int kElems = Granule<TIn>::kElems;
+  constexpr bool by_bits = sizeof(TIn) == 2 && sizeof(TGrad) == 2;  // two entries' comparisons are one
   const uint64_t l2 = pack2(kLog2e, kLog2e);
   float x[kElems];
   gr.get(x);
 #pragma unroll
   for (int j = 0; j < kElems; j += 2) {
     float lo, hi;
-    unpack2(kFoldedGrad<TIn, TGrad> ? fma2(pack2(x[j], x[j + 1]), l2, m2) : mul2(add2(pack2(x[j], x[j + 1]), m2), l2), lo, hi);
+    unpack2(kFold ? fma2(pack2(x[j], x[j + 1]), l2, m2) : mul2(add2(pack2(x[j], x[j + 1]), m2), l2), lo, hi);
     unpack2(mul2(pack2(ex2(lo), ex2(hi)), coef2), lo, hi);
-    if constexpr (!kFoldedGrad<TIn, TGrad>) {
+    if constexpr (!by_bits) {
       lo = x[j] >= tau ? lo : 0.f;
       hi = x[j + 1] >= tau ? hi : 0.f;
     }
@@ -930,15 +931,15 @@ __device__ __forceinline__ void grad_words(const Granule<TIn> &gr, float tau, ty
       const __half2 h = __floats2half2_rn(lo, hi);
       w[j / 2] = *reinterpret_cast<const uint32_t *>(&h);
     }
-    if constexpr (kFoldedGrad<TIn, TGrad>) w[j / 2] &= SweepOps<TIn>::reach(gr.w[j / 2], tau_p);
+    if constexpr (by_bits) w[j / 2] &= SweepOps<TIn>::reach(gr.w[j / 2], tau_p);
   }
 }
-template <typename TIn, typename TGrad>
+template <typename TIn, typename TGrad, bool kFold>
 __device__ __forceinline__ void grad_granule(const Granule<TIn> &gr, TGrad *dst, float tau,
                                              typename SweepOps<TIn>::Tau tau_p, uint64_t m2, uint64_t coef2) {
   constexpr int kWords = kGradWords<TIn, TGrad>;
   uint32_t w[kWords];
-  grad_words<TIn, TGrad>(gr, tau, tau_p, m2, coef2, w);
+  grad_words<TIn, TGrad, kFold>(gr, tau, tau_p, m2, coef2, w);
   if constexpr (kWords == 4) {
     st_stream16(dst, make_uint4(w[0], w[1], w[2], w[3]));
   } else {
@@ -1091,7 +1092,7 @@ __device__ __forceinline__ void row_grad(const RowView<TIn> &v, TGrad *grow_all,
   // one granule; the sampled token's entry replaces the one that its granule's store left
   auto emit = [&](const Granule<TIn> &gr, int g) {
     if (!DVP_IN((long long)g * kElems + kElems - 1, V, DVP_OOB_GLOBAL)) return;
-    grad_granule<TIn, TGrad>(gr, grow + (size_t)g * kElems, tau, tau_p, m2, cf2);
+    grad_granule<TIn, TGrad, kFoldedGrad<TIn, TGrad>>(gr, grow + (size_t)g * kElems, tau, tau_p, m2, cf2);
     if (g == g_here) grow_all[a_here] = Storage<TGrad>::narrow(g_a);
   };
   int step = 0;
@@ -1427,12 +1428,7 @@ __global__ void __launch_bounds__(512, 2) dvp_backward_kernel(const __grid_const
     const float out = live && x >= tau ? coef * ex2((x - m) * kLog2e) : 0.f;
     grow[k_extra] = Storage<TGrad>::narrow(k_extra == a ? out_a : out);
   }
-  float mc = m, cf = coef;
-  if constexpr (kFoldedGrad<TIn, TGrad>) {
-    mc = m * kLog2e;
-    cf = coef * ex2(-fmaf(m, kLog2e, -mc));
-  }
-  const uint64_t m2 = pack2(-mc, -mc), cf2 = pack2(cf, cf);
+  const uint64_t m2 = pack2(-m, -m), cf2 = pack2(coef, coef);
   const typename SweepOps<TIn>::Tau tau_p = SweepOps<TIn>::threshold(tau);
   const int g_a = a >= 0 ? v.granule_of(a) : -1;
   TGrad *gbase = grow + (v.base - row);
@@ -1448,12 +1444,12 @@ __global__ void __launch_bounds__(512, 2) dvp_backward_kernel(const __grid_const
         uint32_t w[kWords];
 #pragma unroll
         for (int i = 0; i < kWords; ++i) w[i] = 0;
-        if (hot) grad_words<TIn, TGrad>(gr[u], tau, tau_p, m2, cf2, w);
+        if (hot) grad_words<TIn, TGrad, false>(gr[u], tau, tau_p, m2, cf2, w);
         store_shifted(w, any, dst - lane * kElems, n, shift_smem + (tid >> 5) * kShiftWords);
         __syncwarp();  // the sampled token's entry replaces what a lane of the warp stored there
       } else if (lane < n) {
         if (any)
-          grad_granule<TIn, TGrad>(gr[u], dst, tau, tau_p, m2, cf2);
+          grad_granule<TIn, TGrad, false>(gr[u], dst, tau, tau_p, m2, cf2);
         else
           store_zero_granule<TGrad, kElems>(dst);
       }

@@ -89,6 +89,21 @@ def test_backward_rows_that_start_anywhere(dtype, grad_dtype, T, V, pad, offset,
         assert (buf[outside] == 7.0).all(), "written outside the gradient's rows"
 
 
+@pytest.mark.parametrize("grad_pad", [0, 1])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("T,V", [(64, 50021), (2000, 4096)])
+def test_backward_entries_have_one_arithmetic(T, V, dtype, grad_pad):
+    """Entries of 16 bits are those of float32, rounded: forming them costs no digit."""
+    w = dataclasses.replace(W["c2_bf16_fwdbwd"], dtype="bf16" if dtype == torch.bfloat16 else "f16")
+    b = inputs.make_rows(w, seed=V, device=DEV, T=T, V=V)
+    saved = binding.dvp_forward(b.train, b.ids, 0.0, infer_logits=b.infer)
+    exact = binding.dvp_backward(b.train, b.ids, 0.0, b.upstream, saved, grad_dtype=torch.float32)
+    buf = torch.empty(T, V + grad_pad, dtype=dtype, device=DEV)
+    got = binding.dvp_backward(b.train, b.ids, 0.0, b.upstream, saved, grad_train=buf[:, :V])
+    torch.cuda.synchronize()
+    assert torch.equal(got, exact.to(dtype))
+
+
 @pytest.mark.parametrize("cluster", [2, 4])
 @pytest.mark.parametrize("V,grad_pad", [(151935, 0), (70001, 1)])
 def test_clusters_share_rows_that_start_anywhere(V, grad_pad, cluster):
