@@ -406,8 +406,7 @@ def dvp_forward(train_logits: torch.Tensor, ids: torch.Tensor, rho: float, *,
         train_at, infer_at = _addresses(res.train), _addresses(res.infer) if has_infer else _NO_SIDE
     else:
         sides, rest, flags = _token_outputs(train_logits, T, 2 if has_infer else 1, has_infer + weighted)
-        if want_mask:
-            sides = [_with_mask(side, train_logits, T, V) for side in sides]
+        sides = [_with_mask(side, train_logits, T, V) for side in sides]   # without masks the call above was made
         res = SimpleNamespace(train=sides[0][0], infer=sides[1][0] if has_infer else None,
                               log_ratio=rest[0] if has_infer else None,
                               flags=flags, grad_train=None)

@@ -1677,7 +1677,10 @@ static cudaError_t launch_rows_cs(const RowParams &p, int threads, int n_steps, 
 // While all rows fit the chip at once, more threads a row are faster (100 x 20,000 bfloat16: 17.5 at 256
 // against 21.5 at 128 and 29.7 at 64); so they are while the rows that come first do, and a thread has four granules (300 x
 // 32,000 bfloat16 with the gradient 26.7 -> 22.6; 1,000 x 20,000, which do not fit, 37.1 / 43.2), 2-byte rows up to a few
-// more than fit (600 x 32,000 42.5 -> 35.4; 300 x 27,652 float32 28.3 / 28.9).
+// more than fit (593 to 608 bfloat16 rows, 128 threads / 256: V = 16,640 29.5 / 27.5 to 30.4 / 29.2, 20,000 31.2 / 30.0 to
+// 31.5 / 31.1, 26,000 38.7 / 34.8 to 38.4 / 34.8, 32,000 45.2 / 36.9 to 46.8 / 38.0; 1,185 to 1,216 rows, 64 / 128: V = 8,320
+// 32.3 / 27.7, 10,000 33.5 / 30.7, 13,000 41.6 / 35.6, 16,000 47.7 / 36.5; 300 x 27,652 float32 28.3 / 28.9.  The two do not
+// meet there yet: 640 rows of 20,000 32.5 / 32.3, of 32,000 47.6 / 39.8).
 //
 // Then more blocks a row, V = 151,936 bfloat16, 1 / 2 / 4 / 8 blocks: T = 16 forward 36 / 28 / 21 / 19; T = 128 with the
 // gradient 57 / 47 / 41.  Blocks that share a row need at least a step and a half of it each (V = 20,000: 13 / 15), without

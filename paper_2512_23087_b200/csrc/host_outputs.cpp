@@ -61,8 +61,8 @@ PyObject *outputs(PyObject *, PyObject *const *args, Py_ssize_t n_args) {
 
 // ---- dvp_forward ------------------------------------------------------------------------------------------------------
 // What binding.dvp_forward does beside the library's call, for results that it makes itself.  In Python its checks, packing
-// and namespaces took half of a small call: 64 x 4,096 float32 with the gradient 20.7 -> 12.9 us, 16 x 151,936 bfloat16
-// forward 17.3 -> 14.6 (then the device's).
+// and namespaces took half of a small call: 64 x 4,096 float32 with the gradient 20.7 -> 12.3 us, 16 x 151,936 bfloat16
+// forward 17.3 -> 14.3 (then the device's).
 
 // The error that Python code gets for what it passes; thrown inside HANDLE_TH_ERRORS blocks.
 [[noreturn]] void refuse(PyObject *type, const char *format, const char *name = "") {

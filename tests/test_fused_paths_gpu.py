@@ -65,7 +65,7 @@ def test_default_panel_and_its_workspace():
     assert torch.equal(small.d_w, two.d_w) and torch.equal(small.d_hidden, two.d_hidden)
     for n in ("lse", "logp_mp", "count", "log_cov"):
         assert torch.equal(getattr(one.train, n), getattr(two.train, n)), n
-    # one sum of 4300 products instead of two: a rounding for every 16 of them
+    # two sums of 2176 and 2124 products instead of 4096 and 204: a rounding for every 16 of them
     for x, y in ((one.d_w, two.d_w), (one.d_hidden, two.d_hidden)):
         assert ((x - y).norm(dim=1) <= 1e-5 * y.norm(dim=1).max()).all()
     with pytest.raises(binding.DvpError) as e:

@@ -47,7 +47,8 @@ FUSED = ("hidden", "w_vocab", "infer", "ids", "upstream")
 
 
 @pytest.mark.parametrize("weighted", [False, True])
-@pytest.mark.parametrize("T,V", [(6, 151936), (900, 20000), (50, 3001)])
+# both policies' rows in one launch; three launches (with weights two); two launches that fit the chip; one launch
+@pytest.mark.parametrize("T,V", [(6, 151936), (900, 20000), (250, 20000), (50, 3001)])
 def test_rows_behind_a_long_kernel(T, V, weighted):
     first, second = (inputs.make_rows(W["c2_bf16_fwdbwd"], seed=s, device=DEV, T=T, V=V) for s in (1, 2))
     want = _rows_call(second, weighted)
@@ -80,22 +81,24 @@ def test_fused_calls_share_a_workspace(T, H, V):
         _same(g, w)
 
 
-def test_captured_calls():
-    a, b = (inputs.make_rows(W["c2_bf16_fwdbwd"], seed=s, device=DEV, T=40, V=20000) for s in (1, 2))
+# both policies' rows in one launch, in two (with and without the training rows first), and in three
+@pytest.mark.parametrize("T,weighted", [(40, True), (40, False), (250, True), (250, False), (400, False)])
+def test_captured_calls(T, weighted):
+    a, b = (inputs.make_rows(W["c2_bf16_fwdbwd"], seed=s, device=DEV, T=T, V=20000) for s in (1, 2))
     fa, fb = (inputs.make_fused(W["c4_fused_lmhead"], seed=s, device=DEV, T=140, H=128, V=4000) for s in (1, 2))
     wants = []
     for x, f in ((a, fa), (b, fb)):
-        wants.append((_rows_call(x, True), _fused_call(f)[0]))
+        wants.append((_rows_call(x, weighted), _fused_call(f)[0]))
         torch.cuda.synchronize()
-    x, f = (inputs.make_rows(W["c2_bf16_fwdbwd"], seed=3, device=DEV, T=40, V=20000),
+    x, f = (inputs.make_rows(W["c2_bf16_fwdbwd"], seed=3, device=DEV, T=T, V=20000),
             inputs.make_fused(W["c4_fused_lmhead"], seed=3, device=DEV, T=140, H=128, V=4000))
     stream = torch.cuda.Stream()
     with torch.cuda.stream(stream):   # once outside the capture
-        _rows_call(x, True), _fused_call(f)
+        _rows_call(x, weighted), _fused_call(f)
     torch.cuda.synchronize()
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph, stream=stream):
-        rows, (fused, keep) = _rows_call(x, True), _fused_call(f)
+        rows, (fused, keep) = _rows_call(x, weighted), _fused_call(f)
     for (rw, fw), (xr, xf) in zip(wants, ((a, fa), (b, fb))):
         _refill(x, xr, ROWS), _refill(f, xf, FUSED)
         graph.replay()

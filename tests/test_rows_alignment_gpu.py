@@ -5,9 +5,11 @@ themselves, must all be taken exactly once, and nothing outside the rows may be 
 import contextlib
 import dataclasses
 
+import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2512_23087_b200 import binding, inputs
 
 import parity
@@ -87,6 +89,44 @@ def test_backward_rows_that_start_anywhere(dtype, grad_dtype, T, V, pad, offset,
         outside = torch.ones_like(buf, dtype=torch.bool)
         outside[grad_offset:grad_offset + T * ld].view(T, ld)[:, :V] = False
         assert (buf[outside] == 7.0).all(), "written outside the gradient's rows"
+
+
+# the same with a finite mask (pruned sampled tokens have a gradient too), and with the entry of the sampled token formed from
+# lse_safe
+@pytest.mark.parametrize("pad,offset,grad_pad,grad_offset", [(3, 5, 3, 5), (1, 8, 0, 3)])
+@pytest.mark.parametrize("T,V", [(13, 47), (600, 4097), (3, 50021)])
+@pytest.mark.parametrize("dtype,grad_dtype", [("bf16", torch.bfloat16), ("f16", torch.float32), ("f32", torch.float32)])
+@pytest.mark.parametrize("how", ["finite mask", "no comp"])
+def test_backward_options_at_any_alignment(dtype, grad_dtype, T, V, pad, offset, grad_pad, grad_offset, how):
+    w = dataclasses.replace(W["c0_small_f32"], dtype=dtype, head_boost=5.0)
+    b = inputs.make_rows(w, seed=V + pad, device=DEV, T=T, V=V)
+    b.ids[::4] = b.train[::4].float().argmin(1)   # pruned tokens
+    b = dataclasses.replace(b, train=_place(b.train, V + pad, offset))
+    kw = {"mask_value": -50.0} if how == "finite mask" else {}
+    rho, ld = 1e-2, V + grad_pad
+    buf = torch.full((grad_offset + T * ld + 64,), 7.0, dtype=grad_dtype, device=DEV)
+    grad = buf[grad_offset:grad_offset + T * ld].view(T, ld)[:, :V]
+    saved = binding.dvp_forward(b.train, b.ids, rho, infer_logits=b.infer, **kw)
+    binding.dvp_backward(b.train, b.ids, rho, b.upstream, saved, grad_train=grad, use_comp=how != "no comp", **kw)
+    torch.cuda.synchronize()
+    ids, up = b.ids.cpu().numpy(), b.upstream.cpu().numpy().astype(np.float64)
+    if how == "finite mask":
+        want = oracle.dvp_rows_listing(b.train.cpu().double().numpy(), ids, rho, -50.0, dtype=parity.ORACLE_DTYPE[b.train.dtype],
+                                       upstream=up, threshold_in_storage_type=False)[1]
+        got = grad
+    else:
+        want = parity.run_oracle(b.train, b.infer, b.ids, rho, b.upstream).grad
+        # 1 - exp(z_a - lse_safe): one float32 rounding of lse_safe and the stored value's own
+        at = torch.arange(T, device=DEV)
+        own, at_own = grad[at, b.ids].cpu().double().numpy(), want[np.arange(T), ids]
+        bound = 2e-6 * np.abs(up) * (1 + saved.train.lse_safe.abs().cpu().double().numpy())
+        assert (np.abs(own - at_own) <= bound + parity.UNIT_ROUNDOFF[grad_dtype] * np.abs(at_own)).all()
+        got = grad.clone()
+        got[at, b.ids], want[np.arange(T), ids] = 0.0, 0.0
+    parity.check_grad(got, want, {})
+    outside = torch.ones_like(buf, dtype=torch.bool)
+    outside[grad_offset:grad_offset + T * ld].view(T, ld)[:, :V] = False
+    assert (buf[outside] == 7.0).all(), "written outside the gradient's rows"
 
 
 @pytest.mark.parametrize("grad_pad", [0, 1])
