@@ -39,7 +39,7 @@ constexpr uint32_t kSpinLimit = 1u << 22;
 // 16,384.  A launch that asks for it (`chain_k`) makes a tile's K several such sums, one accumulator after the other, and
 // adds each to C while the next is formed: the error of as many launches, without their fills and drains.  (Two sums
 // kept, added on their way out and stored once: 4 % more time for a call of 4,727 x 2,864 x 12,179 than with one sum, because
-// nothing overlaps the stores then; this way 1,249 and 1,256 us, one sum 1,222 and 1,273.)
+// nothing overlaps the stores then.  This way, and with one sum: 1,253 and 1,244 us, 8,192 x 1,024 x 20,011 1,493 and 1,471.)
 constexpr int kChainK = 4096;
 
 enum { kErrNone = 0, kErrProducerWait = 11, kErrMmaWaitFull = 12, kErrMmaWaitTmem = 13,
@@ -62,7 +62,7 @@ struct Params {
   int early;               // pair kernel: see begin_after
   const float *row_scale;  // optional (pair kernel): row `row` of the product is multiplied by row_scale[row]
   int chain;               // pair kernel: slices of K that are added up in the tensor core (kChainK), and how many such
-  uint32_t chains;         // sums, each added to C, a unit has
+  int chains;              // sums, each added to C, a unit has
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -488,6 +488,9 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
       : "memory");
 }
 
+// kChains: units of several sums (kChainK).  Products of one sum a unit, the others, have a kernel without that: short ones are
+// bound by what a tile costs beside its slices (512 x 1,024 x 32,000: 205.7 us a call, 208.1 with one kernel for all).
+template <bool kChains>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                     const Params p, const uint32_t fmt) {
@@ -506,10 +509,12 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   // work units: every tile once per K range; unit u is tile u % n_tiles of range u / n_tiles
   const int n_units = n_tiles * p.split_k;
   const int k_per = (k_slices + p.split_k - 1) / p.split_k;
-  // a pair's accumulators in turn hold the sums of its units, of each one p.chains; its i-th sum belongs to unit
-  // unit_of(i) and takes the slices from first_slice(i) on
-  const auto unit_of = [&](uint32_t i) { return pair + (int)(i / p.chains) * n_pairs; };
-  const auto first_slice = [&](uint32_t i) { return unit_of(i) / n_tiles * k_per + (int)(i % p.chains) * p.chain; };
+  // a pair's accumulators in turn hold the sums of its units, of each one p.chains: from one sum to the next
+  const auto next_sum = [&](int &unit, int &sum) {
+    if (kChains && ++sum < p.chains) return;
+    sum = 0;
+    unit += n_pairs;
+  };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages2; ++s) {
@@ -574,10 +579,11 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
                              ((uint32_t)(kPairBM >> 4) << 24) | (p.a_mn_major ? (1u << 15) : 0u);
       // bytes between two K = 16 steps of A: 32 inside a K-major row, 16 K-rows of an MN-major box
       const uint32_t a_step_bytes = p.a_mn_major ? 16u * 128u : (uint32_t)(kUmmaK * 2);
-      uint32_t it = 0;
-      for (uint32_t i = 0; unit_of(i) < n_units && !*abort_flag; ++i) {
-        const int k_lo = first_slice(i), k_hi = min(k_slices, k_lo + p.chain);
-        const uint32_t buf = i & 1, use = i >> 1;
+      uint32_t it = 0, n_sums = 0;
+      for (int unit = pair, sum = 0; unit < n_units && !*abort_flag; next_sum(unit, sum), ++n_sums) {
+        const int k_lo = (unit / n_tiles) * k_per + (kChains ? sum * p.chain : 0);
+        const int k_hi = min(k_slices, k_lo + (kChains ? p.chain : k_per));
+        const uint32_t buf = n_sums & 1, use = n_sums >> 1;
         if (use > 0 && !mbar_wait(smem_u32(&sh->tmem_empty[buf]), (use - 1) & 1, abort_flag)) {
           if (!*abort_flag) { *abort_flag = 1; atomicExch(p.status, kErrMmaWaitTmem); }
           break;
@@ -613,11 +619,12 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     const int quarter = warp & 3;
     const bool exchange = k_per <= kExchangeSlices;
     const float alpha_all = p.alpha * (p.alpha_dev ? *p.alpha_dev : 1.f);
-    for (uint32_t i = 0; unit_of(i) < n_units; ++i) {
-      const int unit = unit_of(i), tile = unit % n_tiles;
+    uint32_t n_sums = 0;
+    for (int unit = pair, sum = 0; unit < n_units; next_sum(unit, sum), ++n_sums) {
+      const int tile = unit % n_tiles;
       const int tm = m_fastest ? tile % tiles_m : tile / tiles_n;
       const int tn = m_fastest ? tile / tiles_m : tile % tiles_n;
-      const uint32_t buf = i & 1, use = i >> 1;
+      const uint32_t buf = n_sums & 1, use = n_sums >> 1;
       // the whole warp goes on or none of it: reading tensor memory and the exchange need every lane
       if (!__all_sync(0xffffffffu, !*abort_flag && mbar_wait(smem_u32(&sh->tmem_full[buf]), use & 1, abort_flag))) {
         if (!*abort_flag) { *abort_flag = 1; atomicExch(p.status, kErrEpilogueWait); }
@@ -646,7 +653,7 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           }
         }
         if (col < p.N) {
-          if (p.accumulate || add_ranges || i % p.chains > 0)  // after the thread's own stores of the unit's first sum
+          if (p.accumulate || add_ranges || (kChains && sum > 0))  // after the thread's own stores of the unit's first sum
             store_columns<Out::kAdd>(crow + col, p.ldc, lane, p.M - (row - lane), r, alpha, p.N - col, exchange);
           else
             store_columns<Out::kStore>(crow + col, p.ldc, lane, p.M - (row - lane), r, alpha, p.N - col, exchange);
@@ -781,7 +788,7 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
   const int chain = (k_per + n_chains - 1) / n_chains, chains = (k_per + chain - 1) / chain;
   if (row_max && chains > 1) return cudaErrorInvalidValue;
   Params p{C, ldc, M, N, K, alpha, alpha_dev, accumulate ? 1 : 0, status, a_mn_major ? 1 : 0, split_k,
-           row_max, row_max_ld, range_stride, order == Order::kEarly ? 1 : 0, row_scale, chain, (uint32_t)chains};
+           row_max, row_max_ld, range_stride, order == Order::kEarly ? 1 : 0, row_scale, chain, chains};
   if (split_k > 1 && !accumulate && range_stride == 0) {
     const cudaError_t z = cudaMemset2DAsync(C, (size_t)ldc * 4, 0, (size_t)N * 4, (size_t)M, stream);
     if (z != cudaSuccess) return z;
@@ -792,8 +799,8 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
     const bool ok_a = a_mn_major ? make_map(&map_a, A, K, M, lda, 64, is_bf16)
                                  : make_map(&map_a, A, M, K, lda, kBM, is_bf16);
     if (!ok_a || !make_map(&map_b, B, N, K, ldb, kBN / 2, is_bf16)) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(gemm_tn_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmemBytes2);
+    auto kernel = chains > 1 ? gemm_tn_pair_kernel<true> : gemm_tn_pair_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes2);
     if (e != cudaSuccess) return e;
     const int tiles = ((M + kPairBM - 1) / kPairBM) * ((N + kBN - 1) / kBN) * split_k;
     int pairs = sm_count / 2;
@@ -812,7 +819,7 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = order != Order::kAlone ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, gemm_tn_pair_kernel, map_a, map_b, p, is_bf16 ? 1u : 0u);
+    return cudaLaunchKernelEx(&cfg, kernel, map_a, map_b, p, is_bf16 ? 1u : 0u);
   }
   if (!make_map(&map_a, A, M, K, lda, kBM, is_bf16) || !make_map(&map_b, B, N, K, ldb, kBN, is_bf16))
     return cudaErrorInvalidValue;
