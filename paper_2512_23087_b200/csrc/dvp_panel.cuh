@@ -261,9 +261,10 @@ __global__ void __launch_bounds__(256) sum_ranges_kernel(const float *part, long
 // One warp per token; the warp of the first token with an id does all tokens with that id, and nobody else adds to that
 // row.  A block's eight warps look for theirs among the chunk's ids in shared memory, four to a load; loads go out in
 // batches, those of d_w's row among them (reductions in memory instead, 767 x 1,448 x 10,474: 165 us a call, 160 this way).
-// With a block a token, which read all ids itself, element by element, the kernel was 15 us of 200 (512 x 1,024 x 32,000), 46
-// of 190 (767 x 1,448 x 10,474) and 110 of 1,690 (8,192 x 1,024 x 20,011); it is 8, 16 and 53.  (Sorting the ids first: 35
-// to 41 us by itself.  In the epilogue of d_w's contraction: 27 us more a call than this, 512 x 1,024 x 32,000.)
+// With a block a token, which read all ids itself, element by element, the kernel by itself took 15 us (512 x 1,024 x 32,000),
+// 46 (767 x 1,448 x 10,474) and 110 (8,192 x 1,024 x 20,011); it takes 8, 16 and 53, of which calls show a part: 206.4 -> 204.9,
+// 163.5 -> 160.0 and 1,509 -> 1,477 us.  (Sorting the ids first: 35 to 41 us by itself.  In the epilogue of d_w's contraction:
+// 27 us more a call than this, 512 x 1,024 x 32,000.)
 constexpr int kIdChunk = 4096;
 constexpr int kSampledWarps = 8;
 constexpr size_t kSampledSmem = (size_t)kIdChunk * 4 + kSampledWarps * kIdChunk / 8;
