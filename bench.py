@@ -39,9 +39,9 @@ FALLBACK_HBM_GBS = 6650.0
 # of one ncu capture of a dvp_forward call on T rows of the workload), keyed by (workload, rho); valid only for
 # the kernel sources whose digest is recorded with it, scaled by rows to the full batch.
 NCU_TRAFFIC = {
-    ("c2_bf16_fwdbwd", 1e-4): {"digest": "628a37170921915c", "T": 2048, "bytes": 1.495492e9 + 0.571276e9},
-    ("c2_bf16_fwdbwd", 1e-3): {"digest": "628a37170921915c", "T": 2048, "bytes": 1.310987e9 + 0.564870e9},
-    ("c3_f32_heavy", 1e-4): {"digest": "628a37170921915c", "T": 1024, "bytes": 2.147980e9 + 1.013277e9},
+    ("c2_bf16_fwdbwd", 1e-4): {"digest": "8eedbfd9bab495b3", "T": 2048, "bytes": 1.495593e9 + 0.571945e9},
+    ("c2_bf16_fwdbwd", 1e-3): {"digest": "8eedbfd9bab495b3", "T": 2048, "bytes": 1.311073e9 + 0.564525e9},
+    ("c3_f32_heavy", 1e-4): {"digest": "8eedbfd9bab495b3", "T": 1024, "bytes": 2.148011e9 + 1.013293e9},
 }
 
 
