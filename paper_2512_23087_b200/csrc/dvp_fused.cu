@@ -85,6 +85,47 @@ static void launch_transpose(const TIn *in, long long ld_in, TOut *out, long lon
                      s, in, ld_in, out, ld_out, R, C, vec_ok, row_scale);
 }
 
+// out[r, c] = float16(in[r, c]), in pieces of 8 elements, `per_row` of them in each of `rows` rows; kHalfPieces of them a
+// block, four a thread.  Short blocks with 32 registers a thread: three of them fit on an SM beside the first contraction's
+// block, and what is left when that ends spreads over the whole chip (two blocks an SM that share all pieces: 88 us for
+// 32,000 x 1,024, which 148 x 8 threads an SM copy in 22).
+constexpr int kHalfPieces = 1024;
+__global__ void __launch_bounds__(256, 8)
+to_half_kernel(const __nv_bfloat16 *in, long long ld_in, __half *out, long long ld_out, int rows, int per_row) {
+  begin_after(true);
+  const long long first = (long long)blockIdx.x * kHalfPieces + threadIdx.x;
+  const int r0 = (int)(first / per_row), c0 = (int)(first - (long long)r0 * per_row);
+  const int dr = 256 / per_row, dc = 256 - dr * per_row;
+  constexpr int kLoads = kHalfPieces / 256;
+  // f(step, row, piece of the row)
+  const auto each = [&](auto f) {
+    int r = r0, c = c0;
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      if (r < rows) f(u, r, c);
+      r += dr;
+      c += dc;
+      if (c >= per_row) {
+        c -= per_row;
+        ++r;
+      }
+    }
+  };
+  uint4 raw[kLoads];
+  each([&](int u, int r, int c) { raw[u] = *reinterpret_cast<const uint4 *>(in + r * ld_in + c * 8); });
+  each([&](int u, int r, int c) {
+    const uint32_t b[4] = {raw[u].x, raw[u].y, raw[u].z, raw[u].w};
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const __half2 h = __floats2half2_rn(__uint_as_float(b[k] << 16), __uint_as_float(b[k] & 0xffff0000u));
+      w[k] = *reinterpret_cast<const uint32_t *>(&h);
+    }
+    *reinterpret_cast<uint4 *>(out + r * ld_out + c * 8) = make_uint4(w[0], w[1], w[2], w[3]);
+  });
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) end_after(true);  // the others leave their place to the next blocks
+}
+
 struct FusedScalars {
   int status;       // non-zero when a tensor-core kernel gave up waiting
   float scale;      // power of two applied to the gradient panel
@@ -267,7 +308,7 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
   float *lpi = a->infer.logp_mp ? a->infer.logp_mp : reinterpret_cast<float *>(ws + L.off_lpi);
   uint8_t *fli = reinterpret_cast<uint8_t *>(ws + L.off_fli);
   uint8_t *flt = a->flags ? a->flags : reinterpret_cast<uint8_t *>(ws + L.off_flt);
-  __half *wt16 = reinterpret_cast<__half *>(ws + L.off_wt);   // [H, Vp]: W^T
+  __half *w16 = reinterpret_cast<__half *>(ws + L.off_wt);    // W in float16: [V, H] as it lies, or [H, Vp]
   __half *hs16 = reinterpret_cast<__half *>(ws + L.off_hs);   // [H, panel]: the panel's hidden rows, scaled, transposed
   float *z = reinterpret_cast<float *>(ws + L.off_z);         // [panel, Vp] logits
   __half *p16 = reinterpret_cast<__half *>(ws + L.off_g);     // [panel, Vp] P = 2^14 e^{z - m} on the safe set
@@ -302,6 +343,10 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     p.bounds_status = bounds_status_word();
     return two_sweeps::launch(p, s);
   };
+  // W as d_hidden's contraction reads it: as it lies, [V, H], the transposed (MN-major) B operand; transposed where H is not a
+  // multiple of 8, the unit of TMA's strides.
+  const bool w_lies = H % 8 == 0;
+  const long long ld_w16 = w_lies ? H : L.Vp;
   int panel_index = 0;
   for (long long r0 = 0; r0 < a->T; r0 += L.panel, ++panel_index) {
     const int rows = (int)((a->T - r0 < L.panel) ? a->T - r0 : L.panel);
@@ -318,7 +363,11 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
       // rows take the log-ratio and the importance weight from them) and W^T.  512 x 1,024 x 32,000: 210 us a call
       // with both in front of the contraction, 206 with the rows there, 199 with neither.
       if (a->infer_logits && infer_rows() != cudaSuccess) return DVP_ERR_CUDA;
-      launch_transpose<__nv_bfloat16, __half>(w, a->ld_w, wt16, L.Vp, V, H, s);
+      if (w_lies)
+        (void)launch_after(to_half_kernel, (unsigned)(((long long)V * (H / 8) + kHalfPieces - 1) / kHalfPieces), 256, 0, s, w,
+                           a->ld_w, w16, ld_w16, V, H / 8);
+      else
+        launch_transpose<__nv_bfloat16, __half>(w, a->ld_w, w16, ld_w16, V, H, s);
       if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
     }
     // rows of the panel, one sweep: statistics, and the gradient panel up to a factor per row
@@ -370,12 +419,12 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     const int room = (int)(L.panel * L.Vp / ((long long)rows * Hp) < 32 ? L.panel * L.Vp / ((long long)rows * Hp) : 32);
     const int ranges = gemm::choose_ranges(dh_tiles, V, sms / 2, room > 1 ? room : 1, (double)rows * Hp * 4);
     float *dh = a->d_hidden + r0 * a->ld_dh;
-    e = ranges > 1 ? gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, z, Hp, rows, H, V, false, 1.f, nullptr, false,
+    e = ranges > 1 ? gemm::launch_gemm_tn(p16, L.Vp, w16, ld_w16, z, Hp, rows, H, V, false, 1.f, nullptr, false,
                                           &sc->status, sms, s, false, false, ranges, nullptr, 0, nullptr, rows * Hp,
-                                          gemm::Order::kAfter)
-                   : gemm::launch_gemm_tn(p16, L.Vp, wt16, L.Vp, dh, a->ld_dh, rows, H, V, false, 1.f, nullptr, false,
+                                          gemm::Order::kAfter, 0, w_lies)
+                   : gemm::launch_gemm_tn(p16, L.Vp, w16, ld_w16, dh, a->ld_dh, rows, H, V, false, 1.f, nullptr, false,
                                           &sc->status, sms, s, false, false, 1, nullptr, 0, row_scale, 0,
-                                          gemm::Order::kAfter);
+                                          gemm::Order::kAfter, 0, w_lies);
     // beside it: the panel's hidden rows times their factor (and 2^14 * scale / 512), transposed, in float16
     launch_transpose<__nv_bfloat16, __half>(hidden + r0 * a->ld_hidden, a->ld_hidden, hs16, L.panel, rows, H, s,
                                             hid_scale);

@@ -54,6 +54,7 @@ struct Params {
   int accumulate;          // C += instead of C =
   int *status;             // device word, set non-zero when a wait gives up
   int a_mn_major;          // A is stored transposed, [K, M] with M contiguous (pair kernel only)
+  int b_mn_major;          // the same for B, [K, N]
   int split_k;             // pair kernel: each tile's K range is cut into this many units (see range_stride)
   float *row_max;          // optional (pair kernel, no split, no accumulation): row_max[row * row_max_ld + tn]
   long long row_max_ld;    // = the maximum of row `row` of C over the columns of tile column tn
@@ -564,14 +565,17 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           if (rank == 0) mbar_expect_tx(bar_local, 2 * kStageBytes2);
           const uint32_t bar = map_to_rank(bar_local, 0);
           const uint32_t dst = base + s * kStageBytes2;
-          if (p.a_mn_major) {  // two boxes of 64 K-rows x 64 rows of A
-            const int m0 = tm * kPairBM + (int)rank * kBM;
-            tma_load_2d_pair(dst, &map_a, bar, m0, ks * kBK);
-            tma_load_2d_pair(dst + kBytesA / 2, &map_a, bar, m0 + 64, ks * kBK);
-          } else {
-            tma_load_2d_pair(dst, &map_a, bar, ks * kBK, tm * kPairBM + (int)rank * kBM);
-          }
-          tma_load_2d_pair(dst + kBytesA, &map_b, bar, ks * kBK, tn * kBN + (int)rank * (kBN / 2));
+          // 128 rows of A or B: one box of 128 x 64 K, or two of 64 K-rows x 64
+          const auto load = [&](uint32_t to, const CUtensorMap *map, int mn_major, int row0) {
+            if (mn_major) {
+              tma_load_2d_pair(to, map, bar, row0, ks * kBK);
+              tma_load_2d_pair(to + kBytesA / 2, map, bar, row0 + 64, ks * kBK);
+            } else {
+              tma_load_2d_pair(to, map, bar, ks * kBK, row0);
+            }
+          };
+          load(dst, &map_a, p.a_mn_major, tm * kPairBM + (int)rank * kBM);
+          load(dst + kBytesA, &map_b, p.b_mn_major, tn * kBN + (int)rank * (kBN / 2));
         }
       }
     }
@@ -579,9 +583,11 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
     // ---------------- MMA issuer (leader block only)
     if (lane == 0 && rank == 0) {
       const uint32_t idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(kBN >> 3) << 17) |
-                             ((uint32_t)(kPairBM >> 4) << 24) | (p.a_mn_major ? (1u << 15) : 0u);
-      // bytes between two K = 16 steps of A: 32 inside a K-major row, 16 K-rows of an MN-major box
-      const uint32_t a_step_bytes = p.a_mn_major ? 16u * 128u : (uint32_t)(kUmmaK * 2);
+                             ((uint32_t)(kPairBM >> 4) << 24) | (p.a_mn_major ? (1u << 15) : 0u) |
+                             (p.b_mn_major ? (1u << 16) : 0u);
+      // between two K = 16 steps of an operand: 32 bytes inside a K-major row, 16 K-rows of an MN-major box
+      const uint64_t a_step = (p.a_mn_major ? 16u * 128u : (uint32_t)(kUmmaK * 2)) >> 4;
+      const uint64_t b_step = (p.b_mn_major ? 16u * 128u : (uint32_t)(kUmmaK * 2)) >> 4;
       uint32_t it = 0, n_sums = 0;
       for (int unit = pair, sum = 0; unit < n_units && !*abort_flag; next_sum(unit, sum), ++n_sums) {
         const int k_lo = (unit / n_tiles) * k_per + (kChains ? sum * p.chain : 0);
@@ -604,13 +610,10 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
           tc_fence_after();
           const uint32_t a_addr = base + s * kStageBytes2, b_addr = a_addr + kBytesA;
           const uint64_t adesc = p.a_mn_major ? smem_desc_sw128_mn(a_addr) : smem_desc_sw128(a_addr);
-          const uint64_t bdesc = smem_desc_sw128(b_addr);
+          const uint64_t bdesc = p.b_mn_major ? smem_desc_sw128_mn(b_addr) : smem_desc_sw128(b_addr);
 #pragma unroll
-          for (int k = 0; k < kBK / kUmmaK; ++k) {
-            const uint64_t step = (uint64_t)((k * kUmmaK * 2) >> 4);
-            const uint64_t a_step = (uint64_t)((k * a_step_bytes) >> 4);
-            umma_pair(tmem_d, adesc + a_step, bdesc + step, idesc, (ks > k_lo || k > 0) ? 1u : 0u);
-          }
+          for (int k = 0; k < kBK / kUmmaK; ++k)
+            umma_pair(tmem_d, adesc + k * a_step, bdesc + k * b_step, idesc, (ks > k_lo || k > 0) ? 1u : 0u);
           umma_commit_pair(smem_u32(&sh->empty[s]));
         }
         if (!ok) break;
@@ -770,11 +773,12 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
                                   cudaStream_t stream, bool single_block_tiles = false,
                                   bool a_mn_major = false, int split_k = 1, float *row_max = nullptr,
                                   long long row_max_ld = 0, const float *row_scale = nullptr,
-                                  long long range_stride = 0, Order order = Order::kAlone, int chain_k = 0) {
+                                  long long range_stride = 0, Order order = Order::kAlone, int chain_k = 0,
+                                  bool b_mn_major = false) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   if (lda % 8 || ldb % 8 || ldc % 8 || (uintptr_t)A % 16 || (uintptr_t)B % 16 || (uintptr_t)C % 32)
     return cudaErrorInvalidValue;
-  if (a_mn_major && single_block_tiles) return cudaErrorInvalidValue;
+  if ((a_mn_major || b_mn_major) && single_block_tiles) return cudaErrorInvalidValue;
   // every K range of a split needs work
   if (single_block_tiles || split_k < 1 || (K + kBK - 1) / kBK < 2 * split_k) split_k = 1;
   if (range_stride != 0) {
@@ -790,7 +794,7 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
   const int most = chain_k > 0 && split_k == 1 ? chain_k / kBK : k_per, n_chains = (k_per + most - 1) / most;
   const int chain = (k_per + n_chains - 1) / n_chains, chains = (k_per + chain - 1) / chain;
   if (row_max && chains > 1) return cudaErrorInvalidValue;
-  Params p{C, ldc, M, N, K, alpha, alpha_dev, accumulate ? 1 : 0, status, a_mn_major ? 1 : 0, split_k,
+  Params p{C, ldc, M, N, K, alpha, alpha_dev, accumulate ? 1 : 0, status, a_mn_major ? 1 : 0, b_mn_major ? 1 : 0, split_k,
            row_max, row_max_ld, range_stride, order == Order::kEarly ? 1 : 0, row_scale, chain, chains};
   if (split_k > 1 && !accumulate && range_stride == 0) {
     const cudaError_t z = cudaMemset2DAsync(C, (size_t)ldc * 4, 0, (size_t)N * 4, (size_t)M, stream);
@@ -798,10 +802,12 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
   }
   CUtensorMap map_a, map_b;
   if (!single_block_tiles) {
-    // pairs of blocks on 256 x 256 tiles; a transposed A is [K, M]: its "rows" are K, boxes of 64 x 64
+    // pairs of blocks on 256 x 256 tiles; a transposed A is [K, M]: its "rows" are K, boxes of 64 x 64; so is a transposed B
     const bool ok_a = a_mn_major ? make_map(&map_a, A, K, M, lda, 64, is_bf16)
                                  : make_map(&map_a, A, M, K, lda, kBM, is_bf16);
-    if (!ok_a || !make_map(&map_b, B, N, K, ldb, kBN / 2, is_bf16)) return cudaErrorInvalidValue;
+    const bool ok_b = b_mn_major ? make_map(&map_b, B, K, N, ldb, 64, is_bf16)
+                                 : make_map(&map_b, B, N, K, ldb, kBN / 2, is_bf16);
+    if (!ok_a || !ok_b) return cudaErrorInvalidValue;
     auto kernel = chains > 1 ? gemm_tn_pair_kernel<true> : gemm_tn_pair_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes2);
     if (e != cudaSuccess) return e;
@@ -813,15 +819,19 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = kSmemBytes2;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[3];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_after
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    // all of the SM's shared memory: with the next smaller share, which this block fits alone, no other kernel's blocks have
+    // room beside it (767 x 1,448 x 10,474: 141.6 us a call, 128.9 this way; 512 x 1,024 x 32,000 182.4 / 177.6)
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+    attr[2].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_after
+    attr[2].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = order != Order::kAlone ? 2 : 1;
+    cfg.numAttrs = order != Order::kAlone ? 3 : 2;
     return cudaLaunchKernelEx(&cfg, kernel, map_a, map_b, p, is_bf16 ? 1u : 0u);
   }
   if (!make_map(&map_a, A, M, K, lda, kBM, is_bf16) || !make_map(&map_b, B, N, K, ldb, kBN, is_bf16))
