@@ -22,7 +22,6 @@
 #include "dvp_common.cuh"
 #include "dvp_gemm.cuh"
 #include "dvp_panel.cuh"
-#include "dvp_rows_two_sweeps.cuh"
 
 namespace dvp {
 
@@ -217,6 +216,15 @@ bool fused_layout(const dvp_fused_args *a, FusedLayout *L, bool small = false) {
   return true;
 }
 
+template <typename Kernel>
+cudaError_t launch_both(Kernel kernel, size_t smem, const panel::PanelParams &pp, const RowParams &infer, cudaStream_t s) {
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_after(kernel, (unsigned)(infer.T + pp.row.T), panel::kSums / 2, smem, s, pp, infer);
+}
+
 dvp_side_out offset_side(const dvp_side_out &o, long long r0, long long words) {
   dvp_side_out r = o;
   if (r.max) r.max += r0;
@@ -327,9 +335,10 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
   if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
 
   const double log_rho = a->rho > 0.0 ? std::log(a->rho) : -HUGE_VAL;
-  // the inference rows: an ordinary forward-only row pass over the stored logits
-  auto infer_rows = [&]() -> cudaError_t {
-    RowParams p{};
+  // the inference rows: a forward-only row pass over the stored logits
+  RowParams infer{};
+  if (a->infer_logits) {
+    RowParams &p = infer;
     p.train = a->infer_logits;
     p.ids = a->ids;
     p.T = a->T;
@@ -341,8 +350,11 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     p.out_t.logp_mp = lpi;
     p.flags = fli;
     p.bounds_status = bounds_status_word();
-    return two_sweeps::launch(p, s);
-  };
+  }
+  const two_sweeps::Shape infer_shape = a->infer_logits ? two_sweeps::shape_of(infer) : two_sweeps::Shape{};
+  // ... in one launch with the panel's rows (dvp_both_rows_kernel), where four blocks of both fit an SM
+  const bool both = a->infer_logits && !weighted && a->T <= L.panel && infer_shape.smem <= 55 * 1024 &&
+                    (infer_shape.threads == panel::kSums / 2 || infer_shape.threads == 0);
   // W as d_hidden's contraction reads it: as it lies, [V, H], the transposed (MN-major) B operand; transposed where H is not a
   // multiple of 8, the unit of TMA's strides.
   const bool w_lies = H % 8 == 0;
@@ -362,7 +374,7 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
       // Beside the first contraction, in the room that its blocks leave on an SM: the inference rows (the panel's
       // rows take the log-ratio and the importance weight from them) and W^T.  512 x 1,024 x 32,000: 210 us a call
       // with both in front of the contraction, 206 with the rows there, 199 with neither.
-      if (a->infer_logits && infer_rows() != cudaSuccess) return DVP_ERR_CUDA;
+      if (a->infer_logits && !both && two_sweeps::launch(infer, s) != cudaSuccess) return DVP_ERR_CUDA;
       if (w_lies)
         (void)launch_after(to_half_kernel, (unsigned)(((long long)V * (H / 8) + kHalfPieces - 1) / kHalfPieces), 256, 0, s, w,
                            a->ld_w, w16, ld_w16, V, H / 8);
@@ -385,7 +397,10 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     p.out_t.logp_mp = lpt + r0;
     p.flags = flt + r0;
     p.bounds_status = bounds_status_word();
-    if (a->infer_logits) {
+    panel::MeetParams meet{};
+    if (both) {
+      meet = {lpt, lpi, flt, fli, a->log_ratio};
+    } else if (a->infer_logits) {
       pp.logp_mp_i = lpi + r0;
       pp.flags_i = fli + r0;
       p.log_ratio = a->log_ratio ? a->log_ratio + r0 : nullptr;
@@ -408,7 +423,10 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     // Few rows: as many threads a row as it has sums.  More than fill the chip: half of them, so that one row's reductions
     // and results pass beside the sweeps of three others.  us a call with the first form / the second: 163 x 416 x 45,277
     // 138 / 146, 767 x 1,448 x 10,474 172 / 170, 4,727 x 2,864 x 12,179 1,274 / 1,224, 3,891 x 2,752 x 58,933 4,220 / 3,997.
-    const cudaError_t pe = rows < 4 * 148
+    const cudaError_t pe = both && infer_shape.threads
+                               ? launch_both(panel::dvp_both_rows_kernel<false>, infer_shape.smem, pp, infer, s)
+                           : both ? launch_both(panel::dvp_both_rows_kernel<true>, infer_shape.smem, pp, infer, s)
+                           : rows < 4 * 148
                                ? launch_after(panel::dvp_panel_kernel<1, 4>, (unsigned)rows, panel::kSums, 0, s, pp)
                                : launch_after(panel::dvp_panel_kernel<2, 1>, (unsigned)rows, panel::kSums / 2, 0, s, pp);
     if (pe != cudaSuccess) return DVP_ERR_CUDA;
@@ -431,7 +449,7 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     if (e == cudaSuccess)
       e = launch_after(panel::sum_ranges_kernel, (unsigned)(((H + 1023) / 1024) * (long long)rows), 256, 0, s,
                        ranges > 1 ? z : dh, rows * Hp, ranges > 1 ? Hp : a->ld_dh, ranges,
-                       ranges > 1 ? row_scale : nullptr, dh, a->ld_dh, w, a->ld_w, p.ids, p.id_is_i32, a_coef, H);
+                       ranges > 1 ? row_scale : nullptr, dh, a->ld_dh, w, a->ld_w, p.ids, p.id_is_i32, a_coef, H, meet);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
     // d_w (+)= P^T x (scaled hidden rows) * 512 / (2^14 scale): P is read as it lies, [rows, V] with V
     // contiguous, as the transposed (MN-major) A operand of the contraction; it needs nothing of sum_ranges_kernel

@@ -15,6 +15,7 @@
 #pragma once
 
 #include "dvp_rows_impl.cuh"
+#include "dvp_rows_two_sweeps.cuh"
 
 namespace dvp {
 namespace panel {
@@ -90,12 +91,9 @@ __device__ __forceinline__ void absorb_panel(const Granule<float> &gr, int g, in
 // threads a block has.  Every set has kAhead granules in flight, the first of them while the row's maximum is found.
 constexpr int kSums = 512;
 template <int kSets, int kAhead>
-__global__ void __launch_bounds__(kSums / kSets, 2 * kSets) dvp_panel_kernel(const PanelParams pp) {
-  __shared__ float scratch[96];
+__device__ __forceinline__ void panel_row(const PanelParams &pp, const long long t, float *scratch) {
   const RowParams &p = pp.row;
   constexpr int kElems = 8, kThreads = kSums / kSets;
-  begin_after();
-  const long long t = blockIdx.x;
   DVP_BOUNDS_BEGIN(p.bounds_status);
   DVP_BOUNDS_SET(n_gran, (p.V + kElems - 1) / kElems);
   DVP_BOUNDS_SET(V, p.V);
@@ -216,17 +214,63 @@ __global__ void __launch_bounds__(kSums / kSets, 2 * kSets) dvp_panel_kernel(con
     }
   }
 }
+template <int kSets, int kAhead>
+__global__ void __launch_bounds__(kSums / kSets, 2 * kSets) dvp_panel_kernel(const PanelParams pp) {
+  __shared__ float scratch[96];
+  begin_after();
+  panel_row<kSets, kAhead>(pp, blockIdx.x, scratch);
+}
+
+// The inference rows and the panel's in one launch, for calls of one panel whose panel rows need nothing of the others: the
+// inference rows come first, in the places that the logits contraction's last, partly filled wave leaves, and the panel's
+// rows follow without a wave that ends between them.  sum_ranges_kernel forms the log-ratios.  kPieces: inference rows off
+// the 32-byte grid.  us a call, two launches / one: 512 x 1,024 x 32,000 187 / 177.5, 767 x 1,448 x 10,474 145 / 136, 163 x 416 x
+// 45,277 132 / 114, 3,000 x 512 x 16,000 310 / 305, 6,000 x 512 x 16,001 670 / 622.  (Four granules a thread in flight in the
+// panel's rows instead of two: 2 % more time.)
+template <bool kPieces>
+__global__ void __launch_bounds__(kSums / 2, 4) dvp_both_rows_kernel(const __grid_constant__ PanelParams pp,
+                                                                     const __grid_constant__ RowParams infer) {
+  extern __shared__ __align__(16) float smem[];
+  const long long b = blockIdx.x;
+  if (b < infer.T) {
+    begin_after(true);
+    if constexpr (kPieces)
+      two_sweeps::row_of_pieces<2>(infer, b, smem);
+    else
+      two_sweeps::row_of_granules<kSums / 2>(infer, b, smem);
+  } else {
+    begin_after();
+    panel_row<2, 1>(pp, b - infer.T, smem);
+  }
+}
 
 // d_hidden[t, :] = c_t sum_i part_i[t, :] + q_t W[a_t, :], the ranges in order: diag(c) P W from its K ranges and
 // the 1[k = a] term, in fp32.  One range: `part` may be d_hidden itself (c_t applied already: scale null).
+// `meet`: the two policies' rows meet here (dvp_both_rows_kernel): flags and log-ratios.
+struct MeetParams {
+  const float *logp_mp_t, *logp_mp_i;
+  uint8_t *flags;
+  const uint8_t *flags_i;
+  float *log_ratio;  // or null
+};
 __global__ void __launch_bounds__(256) sum_ranges_kernel(const float *part, long long range_stride, long long ld_part,
                                                          int ranges, const float *scale, float *d_hidden,
                                                          long long ld_dh, const __nv_bfloat16 *w, long long ld_w,
-                                                         const void *ids, int id_is_i32, const float *a_coef, int H) {
+                                                         const void *ids, int id_is_i32, const float *a_coef, int H,
+                                                         const MeetParams meet) {
   begin_after();
   const unsigned per_row = (unsigned)(H + 1023) / 1024;
   const long long t = blockIdx.x / per_row;
   const int h = (int)((blockIdx.x % per_row) * 1024 + threadIdx.x * 4);
+  if (meet.flags_i && h == 0) {
+    const uint8_t f = meet.flags[t];
+    const bool in_t = f & DVP_FLAG_IN_TRAIN, in_i = meet.flags_i[t] & DVP_FLAG_IN_TRAIN;
+    meet.flags[t] = (uint8_t)(f | (in_i ? DVP_FLAG_IN_INFER : 0));
+    if (meet.log_ratio)
+      meet.log_ratio[t] = f & (DVP_FLAG_NO_ID | DVP_FLAG_BAD_ID)
+                              ? __int_as_float(0x7fc00000)
+                              : log_ratio_of(in_t, in_i, meet.logp_mp_t[t], meet.logp_mp_i[t]);
+  }
   if (h >= H) return;
   const float q = a_coef[t], c = scale ? scale[t] : 1.f;
   const __nv_bfloat16 *wa = q != 0.f ? w + load_id(ids, id_is_i32, t) * ld_w + h : nullptr;

@@ -62,14 +62,12 @@ __device__ __forceinline__ void masked_sum(const Granule<T> &gr, int g, int a, f
   }
 }
 
+// Row t, by a block of kBlk threads.
 template <int kBlk>
-__global__ void __launch_bounds__(kBlk, 1024 / kBlk) dvp_two_sweeps_kernel(const __grid_constant__ RowParams p) {
-  extern __shared__ __align__(16) float smem[];
+__device__ __forceinline__ void row_of_granules(const RowParams &p, const long long t, float *smem) {
   float *scratch = smem;                                             // 96 floats
   uint16_t *hot_smem = reinterpret_cast<uint16_t *>(smem + 96);      // kHotCap per warp
   uint32_t *bound = reinterpret_cast<uint32_t *>(smem + 96 + (kBlk / 32) * kHotCap / 2);
-  begin_after(true);  // needs nothing of the fused entry's earlier launches
-  const long long t = blockIdx.x;
   const long long id = p.ids ? load_id(p.ids, p.id_is_i32, t) : -1;
   const bool has_id = id >= 0, bad_id = id >= p.V;
   const int a = (has_id && !bad_id) ? (int)id : -1;
@@ -166,7 +164,13 @@ __global__ void __launch_bounds__(kBlk, 1024 / kBlk) dvp_two_sweeps_kernel(const
                              (bad_id ? DVP_FLAG_BAD_ID : 0));
   }
   if (p.out_t.mask) write_mask_row<T>(row, V, st.tau, p.out_t.mask + t * ((p.V + 31) / 32), 0, 1);
-  if (blockIdx.x == gridDim.x - 1 && tid == 0) end_after(true);  // the others leave their place to the next blocks
+}
+template <int kBlk>
+__global__ void __launch_bounds__(kBlk, 1024 / kBlk) dvp_two_sweeps_kernel(const __grid_constant__ RowParams p) {
+  extern __shared__ __align__(16) float smem[];
+  begin_after(true);  // needs nothing of the fused entry's earlier launches
+  row_of_granules<kBlk>(p, blockIdx.x, smem);
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) end_after(true);  // the others leave their place to the next blocks
 }
 
 // ---- rows at any alignment ---------------------------------------------------------
@@ -238,13 +242,12 @@ struct Pieces {
 };
 
 // Pieces of 16 bytes; of 4, with four times the threads, for few rows (163 x 45,277: 30 us, 47 with 64 threads a row).
+constexpr int kPieceSmem = 2 * kSums + 64;  // floats
 template <int kOwn>
-__global__ void __launch_bounds__(kSums / kOwn) dvp_piece_rows_kernel(const __grid_constant__ RowParams p) {
+__device__ __forceinline__ void row_of_pieces(const RowParams &p, const long long t, float *smem) {
   constexpr int kPieceBlk = kSums / kOwn;
   using Words = typename Pieces<kOwn>::Words;
-  __shared__ float part_m[kSums], part_s[kSums], scratch[64];
-  begin_after(true);  // needs nothing of the fused entry's earlier launches
-  const long long t = blockIdx.x;
+  float *part_m = smem, *part_s = smem + kSums, *scratch = smem + 2 * kSums;
   const long long id = p.ids ? load_id(p.ids, p.id_is_i32, t) : -1;
   const bool has_id = id >= 0, bad_id = id >= p.V;
   const int a = (has_id && !bad_id) ? (int)id : -1;
@@ -364,7 +367,13 @@ __global__ void __launch_bounds__(kSums / kOwn) dvp_piece_rows_kernel(const __gr
                              (bad_id ? DVP_FLAG_BAD_ID : 0));
   }
   if (p.out_t.mask) write_mask_row<T>(row, V, st.tau, p.out_t.mask + t * ((p.V + 31) / 32), 0, 1);
-  if (blockIdx.x == gridDim.x - 1 && tid == 0) end_after(true);  // the others leave their place to the next blocks
+}
+template <int kOwn>
+__global__ void __launch_bounds__(kSums / kOwn) dvp_piece_rows_kernel(const __grid_constant__ RowParams p) {
+  __shared__ float smem[kPieceSmem];
+  begin_after(true);  // needs nothing of the fused entry's earlier launches
+  row_of_pieces<kOwn>(p, blockIdx.x, smem);
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) end_after(true);  // the others leave their place to the next blocks
 }
 
 template <int kBlk>
@@ -377,20 +386,30 @@ static cudaError_t launch_blk(const RowParams &p, size_t smem, cudaStream_t s) {
   return launch_after(k, (unsigned)p.T, kBlk, smem, s, p);
 }
 
-static inline cudaError_t launch(const RowParams &p, cudaStream_t s) {
+// How a call's rows are swept: in granules by blocks of `threads`, with `smem` bytes; 0: in pieces.
+struct Shape {
+  int threads;
+  size_t smem;
+};
+static inline Shape shape_of(const RowParams &p) {
   const long long n_gran = (p.V + kElems - 1) / kElems;
   int threads = 256;  // fewer for short rows, so that threads are not idle
   while (threads > 64 && threads >= n_gran) threads /= 2;
   const long long steps = (n_gran + 2 * threads - 1) / (2 * threads);
   const size_t smem = ((size_t)96 + (threads / 32) * kHotCap / 2 + (size_t)steps * threads) * 4;
-  if (!aligned32(p.train, p.ld_train, sizeof(T)) || steps * 64 > 65536 || smem > 200 * 1024) {
-    return p.T < 4 * 148 ? launch_after(dvp_piece_rows_kernel<2>, (unsigned)p.T, kSums / 2, 0, s, p)
-                         : launch_after(dvp_piece_rows_kernel<8>, (unsigned)p.T, kSums / 8, 0, s, p);
-  }
-  switch (threads) {
-    case 64: return launch_blk<64>(p, smem, s);
-    case 128: return launch_blk<128>(p, smem, s);
-    default: return launch_blk<256>(p, smem, s);
+  if (!aligned32(p.train, p.ld_train, sizeof(T)) || steps * 64 > 65536 || smem > 200 * 1024) return {0, kPieceSmem * 4};
+  return {threads, smem};
+}
+
+static inline cudaError_t launch(const RowParams &p, cudaStream_t s) {
+  const Shape sh = shape_of(p);
+  switch (sh.threads) {
+    case 0:
+      return p.T < 4 * 148 ? launch_after(dvp_piece_rows_kernel<2>, (unsigned)p.T, kSums / 2, 0, s, p)
+                           : launch_after(dvp_piece_rows_kernel<8>, (unsigned)p.T, kSums / 8, 0, s, p);
+    case 64: return launch_blk<64>(p, sh.smem, s);
+    case 128: return launch_blk<128>(p, sh.smem, s);
+    default: return launch_blk<256>(p, sh.smem, s);
   }
 }
 
