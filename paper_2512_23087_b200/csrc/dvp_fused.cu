@@ -85,17 +85,17 @@ static void launch_transpose(const TIn *in, long long ld_in, TOut *out, long lon
 }
 
 // out[r, c] = float16(in[r, c]), in pieces of 8 elements, `per_row` of them in each of `rows` rows; kHalfPieces of them a
-// block, four a thread.  Short blocks with 32 registers a thread: three of them fit on an SM beside the first contraction's
-// block, and what is left when that ends spreads over the whole chip (two blocks an SM that share all pieces: 88 us for
-// 32,000 x 1,024, which 148 x 8 threads an SM copy in 22).
-constexpr int kHalfPieces = 1024;
-__global__ void __launch_bounds__(256, 8)
+// block, four a thread.  Beside the first contraction's block an SM has room for one block without shared memory, and for 768
+// threads of 32 registers.  Short blocks: what is left when the contraction ends spreads over the whole chip (two blocks of
+// 256 threads an SM that share all pieces: 88 us for 32,000 x 1,024, which the chip by itself copies in 22).
+constexpr int kHalfBlk = 768, kHalfPieces = 4 * kHalfBlk;
+__global__ void __launch_bounds__(1024, 2)
 to_half_kernel(const __nv_bfloat16 *in, long long ld_in, __half *out, long long ld_out, int rows, int per_row) {
   begin_after(true);
   const long long first = (long long)blockIdx.x * kHalfPieces + threadIdx.x;
   const int r0 = (int)(first / per_row), c0 = (int)(first - (long long)r0 * per_row);
-  const int dr = 256 / per_row, dc = 256 - dr * per_row;
-  constexpr int kLoads = kHalfPieces / 256;
+  const int dr = kHalfBlk / per_row, dc = kHalfBlk - dr * per_row;
+  constexpr int kLoads = kHalfPieces / kHalfBlk;
   // f(step, row, piece of the row)
   const auto each = [&](auto f) {
     int r = r0, c = c0;
@@ -376,7 +376,7 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
       // with both in front of the contraction, 206 with the rows there, 199 with neither.
       if (a->infer_logits && !both && two_sweeps::launch(infer, s) != cudaSuccess) return DVP_ERR_CUDA;
       if (w_lies)
-        (void)launch_after(to_half_kernel, (unsigned)(((long long)V * (H / 8) + kHalfPieces - 1) / kHalfPieces), 256, 0, s, w,
+        (void)launch_after(to_half_kernel, (unsigned)(((long long)V * (H / 8) + kHalfPieces - 1) / kHalfPieces), kHalfBlk, 0, s, w,
                            a->ld_w, w16, ld_w16, V, H / 8);
       else
         launch_transpose<__nv_bfloat16, __half>(w, a->ld_w, w16, ld_w16, V, H, s);

@@ -819,19 +819,17 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.dynamicSmemBytes = kSmemBytes2;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[3];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-    // all of the SM's shared memory: with the next smaller share, which this block fits alone, no other kernel's blocks have
-    // room beside it (767 x 1,448 x 10,474: 141.6 us a call, 128.9 this way; 512 x 1,024 x 32,000 182.4 / 177.6)
-    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-    attr[1].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
-    attr[2].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_after
-    attr[2].val.programmaticStreamSerializationAllowed = 1;
+    // No preferred carve-out: with all of an SM's shared memory asked for, so that other kernels' blocks fit beside this one's, a
+    // cluster of a launch that overlaps the one before was not begun, once in some 10,000 calls, though nothing else ran any more.
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_after
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = order != Order::kAlone ? 3 : 2;
+    cfg.numAttrs = order != Order::kAlone ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, map_a, map_b, p, is_bf16 ? 1u : 0u);
   }
   if (!make_map(&map_a, A, M, K, lda, kBM, is_bf16) || !make_map(&map_b, B, N, K, ldb, kBN, is_bf16))
