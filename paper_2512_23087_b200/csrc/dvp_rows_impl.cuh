@@ -1467,6 +1467,7 @@ __global__ void __launch_bounds__(512, 2) dvp_backward_kernel(const __grid_const
 
 
 }  // namespace dvp
+#include "dvp_rows_held.cuh"
 #include "dvp_rows_resident.cuh"
 #include "dvp_rows_store.cuh"
 namespace dvp {
@@ -1742,6 +1743,19 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
   const bool weighted = p.weight_kind != DVP_WEIGHT_NONE;
   const bool store_kernel = sizeof(TIn) == 2 && (stage_hint == 3 || stage_hint == 4);
   int log_parts = 0;
+  if (threads == 0 && cluster == 0 && !store_kernel) {
+    const bool over_infer = grad_over<TIn, TGrad>(p, p.infer, p.ld_infer);
+    held::Shape sh;
+    if (held::shape_of(p.T, p.infer != nullptr, p.grad != nullptr, n_gran_row, &sh) &&
+        (!over_infer || (grad_over_its_infer_row<TIn, TGrad>(p) && !p.out_i.mask))) {  // masks are written last
+      const cudaError_t e = !p.grad ? held::launch<TIn, TIn, Grad::kNone>(p, sh.threads, sh.log_parts, s)
+                            : loose ? held::launch<TIn, TGrad, Grad::kLoose>(p, sh.threads, sh.log_parts, s)
+                                    : held::launch<TIn, TGrad, Grad::kGranules>(p, sh.threads, sh.log_parts, s);
+      // a cluster of 16 blocks is more than every device (or part of one) takes
+      if (sh.log_parts < 3 || (e != cudaErrorInvalidClusterSize && e != cudaErrorLaunchOutOfResources)) return e;
+      (void)cudaGetLastError();
+    }
+  }
   if (threads == 0 && cluster == 0 && !store_kernel) {
     const RowShape sh = choose_shape(p.T * (p.infer ? 2 : 1), p.T * (p.infer && !p.grad ? 2 : 1), n_gran_row,
                                      sizeof(TIn) == 4 ? 512 : 256, p.grad != nullptr);
