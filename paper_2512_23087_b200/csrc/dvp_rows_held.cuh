@@ -2,7 +2,7 @@
 //
 // A call whose rows fit the chip's registers at once is bound by the chain of its phases, not by bytes or instructions.
 // The row kernel's chain is long: a guess of the maximum, exchanges while the row streams, a list of what has to be read
-// again, the second reading, the sums.  Here a thread loads its granules once, up to four; the maximum passes between
+// again, the second reading, the sums.  Here a thread loads its granules once, up to five; the maximum passes between
 // warps in one exchange, the sums under the threshold that it gives in a second one, and the gradient is formed from what
 // the registers hold.  Where a row has several blocks, warps write their results into the shared memory of all of them, so
 // that an exchange is one barrier and the reads behind it are local.  The blocks of a token's two rows are one cluster:
@@ -13,7 +13,7 @@
 namespace dvp {
 namespace held {
 
-constexpr int kGran = 4, kMaxBlk = 512, kMaxWarps = kMaxBlk / 32, kMaxBlocks = 16;
+constexpr int kMaxBlk = 512, kMaxWarps = kMaxBlk / 32, kMaxBlocks = 16;
 
 __device__ __forceinline__ void st_cluster(float *local, uint32_t rank, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(local, rank)), "f"(v) : "memory");
@@ -85,7 +85,8 @@ __device__ __forceinline__ float max_from(const Group &grp, const Slots &slots, 
   return key_value(__reduce_max_sync(0xffffffffu, order_key(m)));
 }
 
-template <typename TIn, typename TGrad, Grad kGrad>
+// kGran: granules of a row that a thread holds.
+template <typename TIn, typename TGrad, Grad kGrad, int kGran>
 __global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_constant__ RowParams p, const int log_parts) {
   using Ops = SweepOps<TIn>;
   constexpr int kElems = Granule<TIn>::kElems;
@@ -287,42 +288,50 @@ __global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_c
 }
 
 struct Shape {
-  int threads, log_parts;
+  int threads, log_parts, gran;
 };
 // Is the call one for this kernel, and with how many threads and blocks a row?  Every row's granules have to fit the chip at
-// once, 1,024 threads of four on an SM; while it has room, more threads a row are faster.  Clusters are begun one after the
-// other, so that many of them cost more than they save: up to 512 tokens, 256 without a gradient; and those of several blocks
-// a row take whole SMs of one part of the chip, of which some are left over: up to three quarters of the threads.
+// once, 1,024 threads on an SM with four of them, or with five where four are not enough (a few per cent slower where they
+// are: 148 x 32,000 with the gradient 12.7 / 13.5 us a call); while it has room, more threads a row are faster.  Clusters are
+// begun one after the other, so that many of them cost more than they save: up to 512 tokens, 256 without a gradient; and
+// those of several blocks a row take whole SMs of one part of the chip, of which some are left over: up to three quarters of
+// the threads.
 // Device us, the row kernel / this one (a graph of 20 calls): with the gradient 64 x 4,096 float32 7.5 / 5.8, 300 x 8,000 float16
 // 11.1 / 8.6, 400 x 2,100 bfloat16 10.0 / 7.5, 148 x 32,000 15.4 / 11.4, 24 x 100,000 14.1 / 11.8, 8 x 262,144 13.3 / 11.8, 512 x 4,000
 // 10.4 / 8.9, weighted 148 x 2,312 float32 7.4 / 6.0;  forward 4 x 20,000 5.7 / 5.3, 256 x 4,000 5.3 / 5.2, 148 x 32,000 11.5 / 8.3,
-// 12 x 151,936 10.7 / 8.8; one policy 64 x 30,000 7.9 / 5.6.  Beyond: with the gradient 1,000 x 2,048 11.3 / 12.6, 72 x 50,000 (two
-// blocks) 16.2 / 16.5; forward 600 x 4,000 7.5 / 9.9, 72 x 50,000 11.9 / 13.2, 16 x 151,936 12.1 / 12.4; one policy 500 x 4,000 4.4 / 4.6.
+// 12 x 151,936 10.7 / 8.8; one policy 64 x 30,000 7.9 / 5.6.  Five granules: 16 x 151,936 12.2 / 9.0 and with the gradient 15.7 /
+// 13.2, 140 x 40,000 13.0 / 9.1 and 17.7 / 13.3, 250 x 20,000 10.8 / 9.4 and 14.7 / 13.2.  Beyond: with the gradient 1,000 x 2,048 11.3 /
+// 12.6, 72 x 50,000 (two blocks a row) 16.2 / 16.5; forward 600 x 4,000 7.5 / 9.9, 72 x 50,000 11.9 / 13.2, 16 x 151,936 in eight
+// blocks of four granules 12.1 / 12.4; one policy 500 x 4,000 4.4 / 4.6.
 static inline bool shape_of(long long T, bool both, bool grad, long long n_gran, Shape *s) {
   constexpr long long kChip = 148 * 1024, kMost = 8 * kMaxBlk;
   const long long rows = both ? 2 * T : T;
-  long long per_row = 64;  // threads
-  while (per_row < kMost && per_row * kGran < n_gran) per_row *= 2;
-  if (per_row * kGran < n_gran || rows > kChip || T > (grad ? 512 : 256)) return false;
-  if (rows * per_row > (per_row > kMaxBlk ? kChip / 4 * 3 : kChip)) return false;
-  while (per_row < kMost && 4 * rows * per_row <= kChip && per_row <= n_gran) per_row *= 2;
-  s->threads = (int)(per_row < kMaxBlk ? per_row : kMaxBlk);
-  s->log_parts = 0;
-  while ((long long)s->threads << s->log_parts < per_row) ++s->log_parts;
-  return true;
+  if (T > (grad ? 512 : 256)) return false;
+  for (int gran = 4; gran <= 5; ++gran) {
+    long long per_row = 64;  // threads
+    while (per_row < kMost && per_row * gran < n_gran) per_row *= 2;
+    if (per_row * gran < n_gran || rows * per_row > (per_row > kMaxBlk ? kChip / 4 * 3 : kChip)) continue;
+    while (per_row < kMost && 4 * rows * per_row <= kChip && per_row <= n_gran) per_row *= 2;
+    s->threads = (int)(per_row < kMaxBlk ? per_row : kMaxBlk);
+    s->log_parts = 0;
+    while ((long long)s->threads << s->log_parts < per_row) ++s->log_parts;
+    s->gran = gran;
+    return true;
+  }
+  return false;
 }
 
 template <typename TIn, typename TGrad, Grad kGrad>
-static cudaError_t launch(const RowParams &p, int threads, int log_parts, cudaStream_t s) {
-  auto k = dvp_row_kernel_held<TIn, TGrad, kGrad>;
-  const int log_cluster = log_parts + (p.infer ? 1 : 0);
+static cudaError_t launch(const RowParams &p, const Shape &sh, cudaStream_t s) {
+  auto k = sh.gran == 4 ? dvp_row_kernel_held<TIn, TGrad, kGrad, 4> : dvp_row_kernel_held<TIn, TGrad, kGrad, 5>;
+  const int log_cluster = sh.log_parts + (p.infer ? 1 : 0);
   if (log_cluster > 3) {
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(p.T << log_cluster), 1, 1);
-  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.blockDim = dim3((unsigned)sh.threads, 1, 1);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -331,7 +340,7 @@ static cudaError_t launch(const RowParams &p, int threads, int log_parts, cudaSt
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = log_cluster > 0 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k, p, log_parts);
+  return cudaLaunchKernelEx(&cfg, k, p, sh.log_parts);
 }
 
 }  // namespace held

@@ -1748,9 +1748,9 @@ static cudaError_t launch_rows(const RowParams &p, uint32_t hint, cudaStream_t s
     held::Shape sh;
     if (held::shape_of(p.T, p.infer != nullptr, p.grad != nullptr, n_gran_row, &sh) &&
         (!over_infer || (grad_over_its_infer_row<TIn, TGrad>(p) && !p.out_i.mask))) {  // masks are written last
-      const cudaError_t e = !p.grad ? held::launch<TIn, TIn, Grad::kNone>(p, sh.threads, sh.log_parts, s)
-                            : loose ? held::launch<TIn, TGrad, Grad::kLoose>(p, sh.threads, sh.log_parts, s)
-                                    : held::launch<TIn, TGrad, Grad::kGranules>(p, sh.threads, sh.log_parts, s);
+      const cudaError_t e = !p.grad ? held::launch<TIn, TIn, Grad::kNone>(p, sh, s)
+                            : loose ? held::launch<TIn, TGrad, Grad::kLoose>(p, sh, s)
+                                    : held::launch<TIn, TGrad, Grad::kGranules>(p, sh, s);
       // a cluster of 16 blocks is more than every device (or part of one) takes
       if (sh.log_parts < 3 || (e != cudaErrorInvalidClusterSize && e != cudaErrorLaunchOutOfResources)) return e;
       (void)cudaGetLastError();

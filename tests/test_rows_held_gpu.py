@@ -33,7 +33,9 @@ def _call(b, rho, **kw):
 # longest row of eight blocks and one beyond it; 512 tokens and one more
 SIZES = [("bf16", 3, 1), ("f16", 5, 15), ("f32", 2, 9), ("bf16", 7, 4096), ("bf16", 7, 4097 + 15), ("f16", 4, 32768),
          ("bf16", 4, 32769), ("f32", 4, 16384), ("f32", 3, 16393), ("bf16", 1, 262144), ("bf16", 2, 262145), ("f32", 2, 100003),
-         ("bf16", 512, 515), ("bf16", 513, 515), ("f32", 500, 1001)]
+         ("bf16", 512, 515), ("bf16", 513, 515), ("f32", 500, 1001),
+         # five granules a thread: two blocks of them, one block full and one granule beyond it, where the chip is full
+         ("bf16", 16, 151936), ("f32", 148, 20480), ("f32", 148, 20488), ("f16", 148, 40960), ("bf16", 1, 327680)]
 
 
 @pytest.mark.parametrize("checks", [False, True], ids=["", "bounds"])
