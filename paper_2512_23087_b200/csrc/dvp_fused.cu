@@ -84,15 +84,58 @@ static void launch_transpose(const TIn *in, long long ld_in, TOut *out, long lon
                      s, in, ld_in, out, ld_out, R, C, vec_ok, row_scale);
 }
 
+struct FusedScalars {
+  int status;       // non-zero when a tensor-core kernel gave up waiting
+  float scale;      // power of two applied to the gradient panel
+  float inv_scale;  // its inverse
+};
+
+// scale = 2^(14 - x) with max|g| < 2^x, so that |scale * G| < 2^14.
+// `factor` bounds what the kernel multiplies into the upstream gradients (an importance weight).
+__device__ __forceinline__ void grad_scale(const float *upstream, long long T, float factor, FusedScalars *out) {
+  __shared__ float red[32];
+  float m = 0.f;
+  for (long long t = threadIdx.x; t < T; t += blockDim.x) {
+    const float v = fabsf(upstream[t]);
+    if (v < __int_as_float(0x7f800000)) m = fmaxf(m, v);
+  }
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
+    m *= factor;
+    int x = 0;
+    if (m > 0.f) frexpf(m, &x);
+    int e = 14 - x;
+    e = e > 60 ? 60 : (e < -60 ? -60 : e);
+    out->scale = ldexpf(1.f, e);
+    out->inv_scale = ldexpf(1.f, -e);
+  }
+}
+__global__ void grad_scale_kernel(const float *upstream, long long T, float factor, FusedScalars *out) {
+  begin_after(true);
+  grad_scale(upstream, T, factor, out);
+  if (threadIdx.x == 0) end_after(true);
+}
+
 // out[r, c] = float16(in[r, c]), in pieces of 8 elements, `per_row` of them in each of `rows` rows; kHalfPieces of them a
 // block, four a thread.  Beside the first contraction's block an SM has room for one block without shared memory, and for 768
 // threads of 32 registers.  Short blocks: what is left when the contraction ends spreads over the whole chip (two blocks of
 // 256 threads an SM that share all pieces: 88 us for 32,000 x 1,024, which the chip by itself copies in 22).
+//
+// The first block finds the scale of the upstream gradients.  (By a launch of its own in front of the contraction: 64 x 512 x
+// 8,000 46.7 us a call, 45.0 this way, 1,200 x 1,024 x 16,000 200.8 / 198.6.)
 constexpr int kHalfBlk = 768, kHalfPieces = 4 * kHalfBlk;
 __global__ void __launch_bounds__(1024, 2)
-to_half_kernel(const __nv_bfloat16 *in, long long ld_in, __half *out, long long ld_out, int rows, int per_row) {
+to_half_kernel(const __nv_bfloat16 *in, long long ld_in, __half *out, long long ld_out, int rows, int per_row,
+               const float *upstream, long long T, float factor, FusedScalars *scalars) {
   begin_after(true);
-  const long long first = (long long)blockIdx.x * kHalfPieces + threadIdx.x;
+  if (blockIdx.x == 0) {
+    grad_scale(upstream, T, factor, scalars);
+    return;
+  }
+  const long long first = (blockIdx.x - 1LL) * kHalfPieces + threadIdx.x;
   const int r0 = (int)(first / per_row), c0 = (int)(first - (long long)r0 * per_row);
   const int dr = kHalfBlk / per_row, dc = kHalfBlk - dr * per_row;
   constexpr int kLoads = kHalfPieces / kHalfBlk;
@@ -123,42 +166,6 @@ to_half_kernel(const __nv_bfloat16 *in, long long ld_in, __half *out, long long 
     *reinterpret_cast<uint4 *>(out + r * ld_out + c * 8) = make_uint4(w[0], w[1], w[2], w[3]);
   });
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) end_after(true);  // the others leave their place to the next blocks
-}
-
-struct FusedScalars {
-  int status;       // non-zero when a tensor-core kernel gave up waiting
-  float scale;      // power of two applied to the gradient panel
-  float inv_scale;  // its inverse
-};
-
-// scale = 2^(14 - x) with max|g| < 2^x, so that |scale * G| < 2^14.
-// `factor` bounds what the kernel multiplies into the upstream gradients (an importance weight).
-__global__ void grad_scale_kernel(const float *upstream, long long T, float factor, FusedScalars *out) {
-  __shared__ float red[32];
-  float m = 0.f;
-  // the first contraction, early, may begin: its status word is clear (512 x 1,024 x 32,000: 196.8 -> 194.7 us a call)
-  if (threadIdx.x == 0) {
-    out->status = 0;
-    __threadfence();
-    begin_after(true);
-  }
-  for (long long t = threadIdx.x; t < T; t += blockDim.x) {
-    const float v = fabsf(upstream[t]);
-    if (v < __int_as_float(0x7f800000)) m = fmaxf(m, v);
-  }
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
-    m *= factor;
-    int x = 0;
-    if (m > 0.f) frexpf(m, &x);
-    int e = 14 - x;
-    e = e > 60 ? 60 : (e < -60 ? -60 : e);
-    out->scale = ldexpf(1.f, e);
-    out->inv_scale = ldexpf(1.f, -e);
-  }
 }
 
 namespace {
@@ -331,8 +338,7 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
   const long long mask_words = (a->V + 31) / 32;
 
   const bool weighted = a->weight_kind != DVP_WEIGHT_NONE;
-  grad_scale_kernel<<<1, 1024, 0, s>>>(a->upstream, a->T, weighted ? fmaxf(1.f, a->weight_hi) : 1.f, sc);
-  if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
+  const float factor = weighted ? fmaxf(1.f, a->weight_hi) : 1.f;
 
   const double log_rho = a->rho > 0.0 ? std::log(a->rho) : -HUGE_VAL;
   // the inference rows: a forward-only row pass over the stored logits
@@ -364,22 +370,25 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
     const int rows = (int)((a->T - r0 < L.panel) ? a->T - r0 : L.panel);
     // logits of the panel: z = hidden[r0 : r0 + rows] x W^T (bf16 operands, fp32 accumulate)
     // its epilogue also leaves each row's maximum, one piece per tile column: the panel's row pass
-    // then knows the threshold before it reads the panel.  Early: from the second panel on the launch before it is
+    // then knows the threshold before it reads the panel.  Early from the second panel on: the launch before it is
     // the last of d_w's, when nobody reads z or the maxima any more
     cudaError_t e = gemm::launch_gemm_tn(hidden + r0 * a->ld_hidden, a->ld_hidden, w, a->ld_w, z, L.Vp,
                                          rows, V, H, true, 1.f, nullptr, false, &sc->status, sms, s, false,
-                                         false, 1, rmax, L.max_pieces, nullptr, 0, gemm::Order::kEarly);
+                                         false, 1, rmax, L.max_pieces, nullptr, 0,
+                                         panel_index == 0 ? gemm::Order::kFirst : gemm::Order::kEarly);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
     if (panel_index == 0) {
       // Beside the first contraction, in the room that its blocks leave on an SM: the inference rows (the panel's
       // rows take the log-ratio and the importance weight from them) and W^T.  512 x 1,024 x 32,000: 210 us a call
       // with both in front of the contraction, 206 with the rows there, 199 with neither.
       if (a->infer_logits && !both && two_sweeps::launch(infer, s) != cudaSuccess) return DVP_ERR_CUDA;
-      if (w_lies)
-        (void)launch_after(to_half_kernel, (unsigned)(((long long)V * (H / 8) + kHalfPieces - 1) / kHalfPieces), kHalfBlk, 0, s, w,
-                           a->ld_w, w16, ld_w16, V, H / 8);
-      else
+      if (w_lies) {
+        (void)launch_after(to_half_kernel, (unsigned)(((long long)V * (H / 8) + kHalfPieces - 1) / kHalfPieces + 1), kHalfBlk, 0,
+                           s, w, a->ld_w, w16, ld_w16, V, H / 8, a->upstream, a->T, factor, sc);
+      } else {
+        (void)launch_after(grad_scale_kernel, 1, 1024, 0, s, a->upstream, a->T, factor, sc);
         launch_transpose<__nv_bfloat16, __half>(w, a->ld_w, w16, ld_w16, V, H, s);
+      }
       if (cudaGetLastError() != cudaSuccess) return DVP_ERR_CUDA;
     }
     // rows of the panel, one sweep: statistics, and the gradient panel up to a factor per row

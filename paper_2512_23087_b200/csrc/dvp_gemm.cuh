@@ -53,6 +53,7 @@ struct Params {
   const float *alpha_dev;  // optional device scalar multiplied into alpha
   int accumulate;          // C += instead of C =
   int *status;             // device word, set non-zero when a wait gives up
+  int clear_status;        // the word is cleared first (pair kernel); a wait gives up after seconds
   int a_mn_major;          // A is stored transposed, [K, M] with M contiguous (pair kernel only)
   int b_mn_major;          // the same for B, [K, N]
   int split_k;             // pair kernel: each tile's K range is cut into this many units (see range_stride)
@@ -543,6 +544,7 @@ gemm_tn_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_cons
   cluster_barrier();  // barriers of both blocks are initialised before anyone signals them
   tc_fence_after();
   begin_after(p.early != 0);
+  if (p.clear_status && blockIdx.x == 0 && threadIdx.x == 0) *p.status = 0;
   const uint32_t tmem_base = sh->tmem_base;
   volatile int *abort_flag = &sh->abort_flag;
 
@@ -760,9 +762,9 @@ inline int choose_ranges(long long tiles, int K, int pairs, int most, double out
   return best;
 }
 
-// How the launch follows the one before: in the ordinary way; overlapping its end (launch_after); the same without
-// needing its results.
-enum class Order { kAlone, kAfter, kEarly };
+// How the launch follows the one before: in the ordinary way; in the ordinary way as the first of a call's, which the next
+// may overlap and which clears the status word; overlapping its end (launch_after); the same without needing its results.
+enum class Order { kAlone, kFirst, kAfter, kEarly };
 
 // C[M,N] (+)= alpha * A[M,K] * B[N,K]^T.  lda, ldb multiples of 8; ldc of 8; bases 16-byte
 // (A, B) and 32-byte (C) aligned.  Returns a CUDA error code; cudaErrorInvalidValue for
@@ -794,8 +796,10 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
   const int most = chain_k > 0 && split_k == 1 ? chain_k / kBK : k_per, n_chains = (k_per + most - 1) / most;
   const int chain = (k_per + n_chains - 1) / n_chains, chains = (k_per + chain - 1) / chain;
   if (row_max && chains > 1) return cudaErrorInvalidValue;
-  Params p{C, ldc, M, N, K, alpha, alpha_dev, accumulate ? 1 : 0, status, a_mn_major ? 1 : 0, b_mn_major ? 1 : 0, split_k,
-           row_max, row_max_ld, range_stride, order == Order::kEarly ? 1 : 0, row_scale, chain, chains};
+  const bool overlaps = order == Order::kAfter || order == Order::kEarly;
+  const int early = order == Order::kEarly || order == Order::kFirst ? 1 : 0, clear = order == Order::kFirst ? 1 : 0;
+  Params p{C, ldc, M, N, K, alpha, alpha_dev, accumulate ? 1 : 0, status, clear, a_mn_major ? 1 : 0, b_mn_major ? 1 : 0, split_k,
+           row_max, row_max_ld, range_stride, early, row_scale, chain, chains};
   if (split_k > 1 && !accumulate && range_stride == 0) {
     const cudaError_t z = cudaMemset2DAsync(C, (size_t)ldc * 4, 0, (size_t)N * 4, (size_t)M, stream);
     if (z != cudaSuccess) return z;
@@ -829,7 +833,7 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_after
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = order != Order::kAlone ? 2 : 1;
+    cfg.numAttrs = overlaps ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, map_a, map_b, p, is_bf16 ? 1u : 0u);
   }
   if (!make_map(&map_a, A, M, K, lda, kBM, is_bf16) || !make_map(&map_b, B, N, K, ldb, kBN, is_bf16))

@@ -164,14 +164,16 @@ __global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_c
       }
       float x[kElems], e[kElems];
       g.get(x);
+      uint64_t of_granule = 0;  // added up by themselves first: see Sweep1::absorb
 #pragma unroll
       for (int j = 0; j < kElems; j += 2) {
         unpack2(fma2(pack2(x[j], x[j + 1]), l2, c2), e[j], e[j + 1]);
         e[j] = ex2(e[j]);
         e[j + 1] = ex2(e[j + 1]);
-        sum = add2(sum, pack2(e[j], e[j + 1]));
+        of_granule = add2(of_granule, pack2(e[j], e[j + 1]));
         Ops::masked(g, j / 2, x[j], x[j + 1], e[j], e[j + 1], tau_p, safe, cnt);
       }
+      sum = add2(sum, of_granule);
     }
   }
   int n = Ops::count(cnt);
