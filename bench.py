@@ -39,9 +39,9 @@ FALLBACK_HBM_GBS = 6650.0
 # of one ncu capture of a dvp_forward call on T rows of the workload), keyed by (workload, rho); valid only for
 # the kernel sources whose digest is recorded with it, scaled by rows to the full batch.
 NCU_TRAFFIC = {
-    ("c2_bf16_fwdbwd", 1e-4): {"digest": "8eedbfd9bab495b3", "T": 2048, "bytes": 1.495593e9 + 0.571945e9},
-    ("c2_bf16_fwdbwd", 1e-3): {"digest": "8eedbfd9bab495b3", "T": 2048, "bytes": 1.311073e9 + 0.564525e9},
-    ("c3_f32_heavy", 1e-4): {"digest": "8eedbfd9bab495b3", "T": 1024, "bytes": 2.148011e9 + 1.013293e9},
+    ("c2_bf16_fwdbwd", 1e-4): {"digest": "fbf171d1213483e9", "T": 2048, "bytes": 1.495955e9 + 0.571765e9},
+    ("c2_bf16_fwdbwd", 1e-3): {"digest": "fbf171d1213483e9", "T": 2048, "bytes": 1.311043e9 + 0.565727e9},
+    ("c3_f32_heavy", 1e-4): {"digest": "fbf171d1213483e9", "T": 1024, "bytes": 2.148007e9 + 1.015726e9},
 }
 
 
@@ -547,7 +547,8 @@ def fused_measure(args, rank, world, dev):
     clocks = sampler.stop()
     status = int(res.workspace[:4].view(torch.int32).item())
     n_panels = (T + (args.panel_rows or min(4096, (T + 127) // 128 * 128)) - 1) // (args.panel_rows or min(4096, (T + 127) // 128 * 128))
-    launches = args.steps * (3 + 7 * n_panels)
+    # seven a panel, the conversion of W, and with several panels the inference rows by themselves
+    launches = args.steps * ((1 if n_panels == 1 else 2) + 7 * n_panels)
     safe_total = float(res.train.count.double().sum().item())
 
     # end to end: operands from pinned host memory, per-token results back

@@ -14,7 +14,7 @@
 // contraction's epilogue and, times a power of two chosen from max |upstream|, the
 // hidden rows as they are converted to float16 for the d_w contraction; the inverse
 // power of two is applied in that contraction's epilogue.  tcgen05 kind::f16 needs
-// both operands of one type, so W^T is converted to a float16 copy once per call
+// both operands of one type, so W is converted to a float16 copy once per call
 // (exact for bfloat16 values in float16's normal range).
 #include <cmath>
 #include <mutex>
@@ -378,9 +378,8 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
                                          panel_index == 0 ? gemm::Order::kFirst : gemm::Order::kEarly);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
     if (panel_index == 0) {
-      // Beside the first contraction, in the room that its blocks leave on an SM: the inference rows (the panel's
-      // rows take the log-ratio and the importance weight from them) and W^T.  512 x 1,024 x 32,000: 210 us a call
-      // with both in front of the contraction, 206 with the rows there, 199 with neither.
+      // Beside the first contraction, in the room that its blocks leave on an SM: the inference rows, where they have a
+      // launch of their own (the panel's rows take the log-ratio and the importance weight from them), and W.
       if (a->infer_logits && !both && two_sweeps::launch(infer, s) != cudaSuccess) return DVP_ERR_CUDA;
       if (w_lies) {
         (void)launch_after(to_half_kernel, (unsigned)(((long long)V * (H / 8) + kHalfPieces - 1) / kHalfPieces + 1), kHalfBlk, 0,

@@ -199,10 +199,10 @@ __device__ __forceinline__ void tc_fence_after() {
 //
 // `exchange`: four neighbouring lanes exchange their rows' 32-byte pieces first, so that a store instruction of the
 // warp fills 8 whole lines instead of a piece of 32 of them.  With the pieces as they lie a 32,000 x 1,024 C leaves
-// the chip at 2.9 TB/s (zeroing it runs at 6.3), which bounds products with a short K; the exchange goes through the
-// shared-memory path that the MMAs read their operands by, which long ones are bound by.  us without / with it, K = 64,
-// 256, 512, 1,024, 2,048: 45.9 / 38.8, 49.4 / 41.2, 53.6 / 49.5, 67.3 / 69.2, 110 / 116; twice the epilogue
-// warps: no change.
+// the chip at 3.4 TB/s (5.5 in whole lines, with nothing else to do), which bounds products with a short K; the exchange
+// goes through the shared-memory path that the MMAs read their operands by, which long ones are bound by.  us without /
+// with it, K = 64, 256, 512, 640, 768, 1,024, 2,048: 39.2 / 31.1, 41.5 / 34.8, 46.3 / 42.9, 50.9 / 49.4, 55.9 / 55.6, 63.6 / 67.5,
+// 111 / 114.  Rows of 256 bytes by way of shared memory: K = 512 42.4.
 constexpr int kExchangeSlices = 8;  // up to this many slices of K in a unit
 enum class Out { kStore, kAdd };
 // c_own: where the thread's own row (`lane` of the warp's rows) begins; rows: how many of the warp's rows C has.

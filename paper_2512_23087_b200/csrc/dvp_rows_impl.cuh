@@ -1162,7 +1162,7 @@ enum class Grad { kNone, kGranules, kLoose };
 // last rows of the first are still swept (launch_rows_both says which is first and how the two meet).
 //
 // Small calls are one launch, a token's two rows in one cluster (kTogether): ln pi^mp_infer(a) and the membership pass
-// through shared memory.
+// through shared memory.  Smaller ones, whose rows the chip's registers hold, do not come here (dvp_rows_held.cuh).
 //
 // kBehind: the inference rows where the training rows come first.  Kernels of their own, because what they do at a row's
 // end costs short rows in the kernel that sweeps rows without a gradient in every other order.  us, forward, with it there /
@@ -1552,7 +1552,7 @@ static inline bool grad_over_its_infer_row(const RowParams &p) {
 // Both policies' rows, in one launch, two or three; the second may begin while the first ends.
 //
 // One launch for calls that fill half of the chip at most, bound by the chain of their phases and by what a launch costs on
-// the host (2 of 17 us).  Device time of 64 x 4,096 float32, forward / with the gradient, two launches and one: 6.5 / 8.5
+// the host (2 of 17 us); the sizes below are now those of dvp_rows_held.cuh.  Device time of 64 x 4,096 float32, forward / with the gradient, two launches and one: 6.5 / 8.5
 // and 5.8 / 7.9 us; 8 x 151,936 bfloat16 10.5 / 12.6 and 9.3 / 12.1; weighted 148 x 2,312 float32 10.1 and 7.8.  Above,
 // clusters wait for free places: 1,100 x 2,500 bfloat16 10.1 / 12.8 and 12.5 / 17.4, 32 x 151,936 (clusters of 16) 13.7 /
 // 17.6 and 16.6 / 22.1.
