@@ -97,7 +97,11 @@ __global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_c
   const Group grp{parts << both, log_parts, 31 - __clz(n_thr >> 5)};
   const int rank = grp.blocks > 1 ? (int)cluster_rank() : 0, part = rank & (parts - 1), r0 = rank - part;
   const bool second = rank >= parts;  // the inference row's half
-  if (grp.blocks > 1) cluster_arrive();  // blocks write to one another's shared memory once all have begun
+  // Blocks write to one another's shared memory once all have begun.  Where a row has one block and the gradient takes the
+  // inference row's place, they meet when both rows have been read instead, which no other barrier in front of the gradient
+  // says there: the blocks of a longer row meet across the cluster for their maximum, weights wait for the inference row.
+  const bool over_infer = kGrad != Grad::kNone && log_parts == 0 && p.grad == p.infer;
+  if (grp.blocks > 1 && !over_infer) cluster_arrive();
   const long long t = blockIdx.x >> (log_parts + both);
   const long long id = p.ids ? load_id(p.ids, p.id_is_i32, t) : -1;
   const TIn *train = reinterpret_cast<const TIn *>(p.train) + t * p.ld_train;
@@ -125,13 +129,17 @@ __global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_c
     if (u * n_thr < v.n_full) m = fmaxf(m, gr[u].max());
   m = key_value(__reduce_max_sync(0xffffffffu, order_key(m)));
   const int own_slot = rank * kMaxWarps + warp;
-  if (grp.blocks > 1) cluster_wait();  // all blocks have begun
+  if (grp.blocks > 1 && !over_infer) cluster_wait();  // all blocks have begun
   if (log_parts > 0) {
     if (lane < parts) st_cluster(&slots.max[own_slot], r0 + lane, m);
   } else if (lane == 0) {
     slots.max[own_slot] = m;
   }
   grp.meet();
+  if (over_infer) {  // the maximum is one of all that the block's threads hold
+    cluster_arrive();
+    cluster_wait();
+  }
   m = max_from(grp, slots, r0);
 
   // ---- the sums, without the sampled token
@@ -208,6 +216,7 @@ __global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_c
 
   const SideStats st = stats_from<TIn>(grp, slots, r0, m, p, has_a, z_a);
   const bool weighted = p.weight_kind != DVP_WEIGHT_NONE;
+  const float upstream = kGrad != Grad::kNone && !second ? p.upstream[t] : 0.f;
   if (both) {
     if (second && part == 0 && tid < parts) {
       st_cluster(&slots.li, tid, logp_mp_of(st));
@@ -222,7 +231,7 @@ __global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_c
   // ---- the gradient (row_grad's arithmetic)
   if constexpr (kGrad != Grad::kNone) {
     if (!second) {
-      float g = p.upstream[t];
+      float g = upstream;
       if (weighted && both) {  // weights need inference rows
         cluster_wait();
         const float w = has_a ? token_weight(ratio_of(), p.weight_kind, p.weight_lo, p.weight_hi) : __int_as_float(0x7fc00000);

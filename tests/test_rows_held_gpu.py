@@ -96,11 +96,28 @@ def test_rows_that_are_not_ordinary(dtype, mask_value):
             assert ((x - y).abs() <= unit * y.abs() + 2e-6).all(), n
 
 
-def test_place_of_the_inference_rows():
-    """The gradient over the inference rows, which are read before."""
-    b = _batch("bf16", 6, 30000)
-    want = _call(b, 1e-3, launch_hint=0).grad_train.clone()
-    infer = b.infer.clone()
-    res = binding.dvp_forward(b.train, b.ids, 1e-3, infer_logits=infer, upstream=b.upstream, grad_train=infer)
-    torch.cuda.synchronize()
-    assert torch.equal(res.grad_train, want)
+# four blocks a row; one, of 512 threads, 128, 512, 256 and 64
+@pytest.mark.parametrize("dtype,T,V", [("bf16", 6, 30000), ("bf16", 148, 32000), ("f16", 300, 8000), ("f32", 148, 16000),
+                                       ("bf16", 148, 5003), ("f32", 500, 1001)])
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("one_matrix", [False, True])
+def test_place_of_the_inference_rows(dtype, T, V, weighted, one_matrix):
+    """The gradient over the inference rows, which are read before: every result is that of a call with a gradient of its
+    own.  The inference rows come from memory, the training rows from L2 where they are others."""
+    b = _batch(dtype, T, V)
+    if one_matrix:
+        b.infer.copy_(b.train)
+    kw = dict(weight_kind=binding.DVP_WEIGHT_TRUNCATE, weight_hi=1.01) if weighted else {}
+    want = _call(b, 1e-3, **kw)
+    infer, other = b.infer.clone(), torch.empty(1 << 26, device=DEV)
+    for _ in range(3):
+        infer.copy_(b.infer)
+        other.zero_()   # twice L2
+        train = infer if one_matrix else b.train.copy_(b.train.clone())
+        got = binding.dvp_forward(train, b.ids, 1e-3, infer_logits=infer, upstream=b.upstream, grad_train=infer, **kw)
+        torch.cuda.synchronize()
+        assert torch.equal(got.grad_train, want.grad_train) and torch.equal(got.flags, want.flags)
+        pairs = [(n, getattr(getattr(got, s), n), getattr(getattr(want, s), n)) for s in ("train", "infer") for n in SIDE]
+        pairs += [("log_ratio", got.log_ratio, want.log_ratio)] + ([("weight", got.weight, want.weight)] if weighted else [])
+        for n, x, y in pairs:
+            assert torch.equal(x.view(torch.int32), y.view(torch.int32)), n
