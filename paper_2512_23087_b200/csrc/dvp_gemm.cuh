@@ -828,8 +828,12 @@ inline cudaError_t launch_gemm_tn(const void *A, long long lda, const void *B, l
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-    // No preferred carve-out: with all of an SM's shared memory asked for, so that other kernels' blocks fit beside this one's, a
-    // cluster of a launch that overlaps the one before was not begun, once in some 10,000 calls, though nothing else ran any more.
+    // No preferred carve-out: with all of an SM's shared memory asked for (34 KB beside this block for blocks of other kernels,
+    // 1,792 bytes without), calls hung, once in some 10,000: one cluster of a launch that overlaps the one before did not get
+    // past its allocation of tensor memory and its first barrier, while all other blocks that were counted had ended.  Why is
+    // not known: the waits before that point (for places, for tensor memory, of the cluster) are the chip's and have no limit, and
+    // no kernel that they could wait for was left.  The launches overlap all the same, without the attribute; not overlapping
+    // them costs 4 to 7 % of small calls (512 x 1,024 x 32,000 170.5 / 178.0 us, 163 x 416 x 45,277 113.7 / 122.0).
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_after
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
