@@ -90,10 +90,16 @@ struct FusedScalars {
   float inv_scale;  // its inverse
 };
 
+// What a block beside a pair contraction's may take of shared memory: an SM that holds the latter alone is set to 196 KB, of which
+// every block takes 1 KB more than it asks for.  grad_scale's scratch is all that to_half_kernel has.
+constexpr size_t kBesidePair = 196 * 1024 - (gemm::kSmemBytes2 + 1024) - 1024;
+constexpr int kScaleFloats = 32;
+static_assert(kScaleFloats * sizeof(float) <= kBesidePair, "to_half_kernel's blocks fit beside the first contraction's");
+
 // scale = 2^(14 - x) with max|g| < 2^x, so that |scale * G| < 2^14.
 // `factor` bounds what the kernel multiplies into the upstream gradients (an importance weight).
 __device__ __forceinline__ void grad_scale(const float *upstream, long long T, float factor, FusedScalars *out) {
-  __shared__ float red[32];
+  __shared__ float red[kScaleFloats];
   float m = 0.f;
   for (long long t = threadIdx.x; t < T; t += blockDim.x) {
     const float v = fabsf(upstream[t]);
@@ -120,8 +126,8 @@ __global__ void grad_scale_kernel(const float *upstream, long long T, float fact
 }
 
 // out[r, c] = float16(in[r, c]), in pieces of 8 elements, `per_row` of them in each of `rows` rows; kHalfPieces of them a
-// block, four a thread.  Beside the first contraction's block an SM has room for one block without shared memory, and for 768
-// threads of 32 registers.  Short blocks: what is left when the contraction ends spreads over the whole chip (two blocks of
+// block, four a thread.  Beside the first contraction's block an SM has room for one block with kBesidePair bytes of shared
+// memory, and for 768 threads of 32 registers.  Short blocks: what is left when the contraction ends spreads over the whole chip (two blocks of
 // 256 threads an SM that share all pieces: 88 us for 32,000 x 1,024, which the chip by itself copies in 22).
 //
 // The first block finds the scale of the upstream gradients.  (By a launch of its own in front of the contraction: 64 x 512 x
@@ -378,8 +384,9 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
                                          panel_index == 0 ? gemm::Order::kFirst : gemm::Order::kEarly);
     if (e != cudaSuccess) return e == cudaErrorInvalidValue ? DVP_ERR_UNSUPPORTED : DVP_ERR_CUDA;
     if (panel_index == 0) {
-      // Beside the first contraction, in the room that its blocks leave on an SM: the inference rows, where they have a
-      // launch of their own (the panel's rows take the log-ratio and the importance weight from them), and W.
+      // While the first contraction runs: the inference rows, where they have a launch of their own (the panel's rows take
+      // the log-ratio and the importance weight from them), on SMs that it does not use or has left, since their blocks
+      // take more shared memory than kBesidePair; behind them W, whose blocks lie beside the contraction's.
       if (a->infer_logits && !both && two_sweeps::launch(infer, s) != cudaSuccess) return DVP_ERR_CUDA;
       if (w_lies) {
         (void)launch_after(to_half_kernel, (unsigned)(((long long)V * (H / 8) + kHalfPieces - 1) / kHalfPieces + 1), kHalfBlk, 0,
@@ -451,7 +458,7 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
                    : gemm::launch_gemm_tn(p16, L.Vp, w16, ld_w16, dh, a->ld_dh, rows, H, V, false, 1.f, nullptr, false,
                                           &sc->status, sms, s, false, false, 1, nullptr, 0, row_scale, 0,
                                           gemm::Order::kAfter, 0, w_lies);
-    // beside it: the panel's hidden rows times their factor (and 2^14 * scale / 512), transposed, in float16
+    // while it runs, on SMs that it does not use or has left: the panel's hidden rows times their factor (and 2^14 * scale / 512), transposed, in float16
     launch_transpose<__nv_bfloat16, __half>(hidden + r0 * a->ld_hidden, a->ld_hidden, hs16, L.panel, rows, H, s,
                                             hid_scale);
     if (e == cudaSuccess)
