@@ -470,7 +470,9 @@ int dvp_static_workspace_status(uint32_t *status_out);
  *             stride lda (not with bit 1): the tensor cores read it as it lies;
  *             bit 3: every output tile is computed as two halves of the k range
  *             that are added into C with atomics (for few tiles and a long k;
- *             with two addends the sum does not depend on their order)
+ *             with two addends the sum does not depend on their order);
+ *             bit 4: `b` points to B transposed, [k, n] with n contiguous and row
+ *             stride ldb (not with bit 1), read as it lies too
  *   status    device int32, written non-zero if a kernel gave up waiting
  * Errors: DVP_ERR_INVALID_ARG (null pointers, negative sizes),
  * DVP_ERR_UNSUPPORTED (dtype, alignment), DVP_ERR_CUDA.

@@ -279,7 +279,8 @@ int dvp_gemm_tn(const void *a, int64_t lda, const void *b, int64_t ldb, float *c
       dvp::gemm::launch_gemm_tn(a, lda, b, ldb, c, ldc, (int)m, (int)n, (int)k, dtype == DVP_BF16, alpha,
                                 nullptr, (accumulate & 1) != 0, status, sms,
                                 static_cast<cudaStream_t>(stream), (accumulate & 2) != 0, (accumulate & 4) != 0,
-                                (accumulate & 8) ? 2 : 1);
+                                (accumulate & 8) ? 2 : 1, nullptr, 0, nullptr, 0, dvp::gemm::Order::kAlone, 0,
+                                (accumulate & 16) != 0);
   if (e == cudaErrorInvalidValue) return DVP_ERR_UNSUPPORTED;
   return e == cudaSuccess ? DVP_OK : DVP_ERR_CUDA;
 }
@@ -458,7 +459,8 @@ int dvp_fused_lmhead_forward_backward(const dvp_fused_args *a) {
                    : gemm::launch_gemm_tn(p16, L.Vp, w16, ld_w16, dh, a->ld_dh, rows, H, V, false, 1.f, nullptr, false,
                                           &sc->status, sms, s, false, false, 1, nullptr, 0, row_scale, 0,
                                           gemm::Order::kAfter, 0, w_lies);
-    // while it runs, on SMs that it does not use or has left: the panel's hidden rows times their factor (and 2^14 * scale / 512), transposed, in float16
+    // while it runs, on SMs that it does not use or has left: the panel's hidden rows times their factor (and
+    // 2^14 * scale / 512), transposed, in float16
     launch_transpose<__nv_bfloat16, __half>(hidden + r0 * a->ld_hidden, a->ld_hidden, hs16, L.panel, rows, H, s,
                                             hid_scale);
     if (e == cudaSuccess)

@@ -85,6 +85,34 @@ def test_gemm_tn_transposed_a_operand(dtype, m, n, k):
         binding.dvp_gemm_tn(at, b, a_transposed=True, single_block_tiles=True)
 
 
+# one tile; columns that end inside a box, inside a block's half and inside the pair's tile; a k that ends inside a slice
+@pytest.mark.parametrize("a_too", [False, True])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("m,n,k", [(256, 256, 64), (8, 8, 8), (304, 72, 200), (520, 136, 1032), (776, 1000, 4099), (264, 4104, 512)])
+def test_gemm_tn_transposed_b_operand(dtype, m, n, k, a_too):
+    """B given as [k, n] with n contiguous (this is how d_hidden = G W takes W as it lies), alone and with A the same."""
+    g = torch.Generator(device=DEV).manual_seed(m * 5 + n * 3 + k)
+    a = torch.randn(k, m + 8, generator=g, device=DEV).to(dtype)[:, :m]
+    bt = torch.randn(k, n + 8, generator=g, device=DEV).to(dtype)[:, :n]      # padded row stride
+    if not a_too:
+        kp = (k + 7) // 8 * 8
+        rows = torch.full((m, kp), 9.0, dtype=dtype, device=DEV)
+        rows[:, :k] = a.t()
+        a = rows[:, :k]
+    ref = (a.double().t() if a_too else a.double()) @ bt.double()
+    kw = dict(a_transposed=a_too, b_transposed=True)
+    tol = (2.0 ** -24 * (k / 16) + 1e-6) * ref.abs().max().item()   # as above
+    for more in ({}, dict(split_k=True)):
+        out, status = binding.dvp_gemm_tn(a, bt, alpha=0.5, **kw, **more)
+        out2, status2 = binding.dvp_gemm_tn(a, bt, alpha=0.25, out=out.clone(), accumulate=True, **kw, **more)
+        torch.cuda.synchronize()
+        assert status.item() == 0 and status2.item() == 0
+        assert (out.double() - 0.5 * ref).abs().max().item() <= tol
+        assert (out2.double() - 0.75 * ref).abs().max().item() <= 2 * tol
+    with pytest.raises(binding.DvpError):          # only the paired kernel reads a transposed B
+        binding.dvp_gemm_tn(a, bt, single_block_tiles=True, **kw)
+
+
 @pytest.mark.parametrize("m,n,k,transposed", [(256, 256, 8192, False), (1000, 776, 4104, False), (512, 264, 20000, True),
                                               (300, 520, 200, False), (128, 256, 64, False)])
 def test_gemm_tn_split_k(m, n, k, transposed):
