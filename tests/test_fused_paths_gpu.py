@@ -1,5 +1,8 @@
 """Paths of the fused entry that depend on sizes and alignment: inference rows off the 32-byte grid, the panel's rows with
 one or two partial sums a thread, the default panel and the workspace that it fits."""
+import ctypes
+import dataclasses
+
 import pytest
 import torch
 
@@ -47,6 +50,38 @@ def test_inference_rows_that_start_anywhere(T, V, pad, offset, checks):
 def test_panel_rows(T, H, V):
     batch, res, want, rerun = fused._run_fused(T, H, V, 1e-2, seed=T + V)
     fused._check_fused(batch, 1e-2, res, want, V, rerun=rerun)
+
+
+# several K ranges for d_hidden; several panels; a whole number of tiles
+@pytest.mark.parametrize("T,H,V,panel", [(200, 100, 3000, 0), (300, 33, 2051, 128), (64, 260, 4096, 0)])
+def test_hidden_sizes_that_are_no_multiple_of_8(T, H, V, panel):
+    """W is transposed for d_hidden then.  The strides are multiples of 8, and what lies between the rows is neither read nor
+    written."""
+    rho, ld = 1e-2, (H + 7) // 8 * 8
+    b = inputs.make_fused(W, seed=V, device=DEV, T=T, H=H, V=V)
+
+    def padded(rows, fill, like=None):
+        m = torch.full((rows, ld), fill, dtype=torch.float32 if like is None else like.dtype, device=DEV)
+        if like is not None:
+            m[:, :H] = like
+        return m
+    hidden, w = padded(T, 3.0e4, b.hidden), padded(V, 3.0e4, b.w_vocab)
+    b = dataclasses.replace(b, hidden=hidden[:, :H], w_vocab=w[:, :H])
+
+    def rerun(upstream):
+        d_hidden, d_w = padded(T, 7.0), padded(V, 7.0)
+        a, res = binding._fused_args(b.hidden, b.w_vocab, b.ids, rho, upstream, b.infer, d_w[:, :H], False, panel, None, True)
+        res.d_hidden, a.d_hidden, a.ld_dh = d_hidden[:, :H], d_hidden.data_ptr(), ld
+        workspace = torch.empty(binding.dvp_workspace_bytes(binding.DVP_ENTRY_FUSED_LMHEAD, a), dtype=torch.uint8, device=DEV)
+        a.workspace, a.workspace_bytes = workspace.data_ptr(), workspace.numel()
+        assert binding.load_library().dvp_fused_lmhead_forward_backward(ctypes.byref(a)) == binding.DVP_OK
+        torch.cuda.synchronize()
+        assert workspace[:4].view(torch.int32).item() == 0
+        assert (d_hidden[:, H:] == 7).all() and (d_w[:, H:] == 7).all()
+        return res
+    res = rerun(b.upstream)
+    want, _ = fused._oracle_with_the_devices_set(b, rho, res)
+    fused._check_fused(b, rho, res, want, V, rerun=rerun)
 
 
 def test_default_panel_and_its_workspace():

@@ -53,9 +53,11 @@ def test_edges(dtype, T, V, checks):
             parity.check_forward(res, b, rho, V, True)
 
 
-@pytest.mark.parametrize("dtype,T,V,parts", [("bf16", 9, 30001, 1), ("f16", 5, 50021, 2), ("f32", 3, 60000, 4)])
+# one, two, four and eight blocks a row
+@pytest.mark.parametrize("dtype,T,V", [("bf16", 148, 30001), ("f32", 300, 2003), ("f16", 50, 50021), ("f32", 50, 20003),
+                                       ("bf16", 9, 30001), ("bf16", 25, 100001), ("f16", 5, 50021), ("f32", 3, 60000)])
 @pytest.mark.parametrize("pad", [0, 3, 16])
-def test_weights_and_gradient_rows_that_lie_differently(dtype, T, V, parts, pad):
+def test_weights_and_gradient_rows_that_lie_differently(dtype, T, V, pad):
     b = _batch(dtype, T, V, ld=V + 5)
     grad = torch.full((T, V + pad), 7.0, dtype=b.train.dtype, device=DEV)
     weight = (oracle.WEIGHT_TRUNCATE, 0.0, 1.01)
@@ -94,6 +96,30 @@ def test_rows_that_are_not_ordinary(dtype, mask_value):
             x, y = (torch.nan_to_num(v, nan=0.0, posinf=1.0, neginf=-1.0) for v in (x, y))
             unit = {"f32": 1e-6, "bf16": 2.0 ** -7, "f16": 2.0 ** -10}[dtype] if n == "gradient" else 1e-6
             assert ((x - y).abs() <= unit * y.abs() + 2e-6).all(), n
+
+
+# eight blocks a row (two-byte logits); five granules a thread; float32; rows of less than a block's threads
+@pytest.mark.parametrize("dtype,V", [("bf16", 151936), ("bf16", 327680), ("f16", 50021), ("f32", 163840), ("f32", 30001),
+                                     ("bf16", 2051)])
+def test_full_sum_keeps_small_terms(dtype, V):
+    """One token at 0 and all others at -17, where e^-17 = 0.69 * 2^-24 is lost when it is added to 1 by itself.  The sum that
+    holds the 1 is rounded by half a unit, 2^-24, with each of the at most 8 pairs of its granule, 5 granules, the other half
+    of the pair, the row's end, 5 exchanges in the warp, 4 slots a lane, 5 exchanges of those, the sampled token, and a few
+    times in the logarithm."""
+    train = torch.full((6, V), -17.0, dtype=inputs.torch_dtype(dtype), device=DEV)
+    for t, k in enumerate((3, 40, 700, 1023, 2047, 2050)):
+        train[t, k] = 0.0
+    ids = torch.tensor([3, V - 1, 5, 1023, -1, 2050], device=DEV)
+    bound = (8 + 5 + 1 + 1 + 5 + 4 + 5 + 1 + 4) * 2.0 ** -24
+    z = train.double()
+    lse = torch.logsumexp(z, 1)
+    logp = z.gather(1, ids.clamp(min=0)[:, None])[:, 0] - lse
+    one, two = (binding.dvp_forward(train, ids, 1e-3, **kw) for kw in ({}, dict(infer_logits=train.clone())))
+    torch.cuda.synchronize()
+    for side in (one.train, two.train, two.infer):
+        assert (side.lse.double() - lse).abs().max().item() <= bound
+        assert (side.log_cov.double() + lse).abs().max().item() <= bound   # the safe set is the one token: ln Z = -lse
+        assert ((side.logp.double() - logp).abs() <= bound + 2.0 ** -24 * logp.abs())[ids >= 0].all()
 
 
 # four blocks a row; one, of 512 threads, 128, 512, 256 and 64

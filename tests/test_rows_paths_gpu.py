@@ -109,7 +109,9 @@ def test_outputs_left_out(kept, V, weighted):
 
 @pytest.mark.parametrize("T,V,dtype", [(1, 5003, "bf16"), (148, 5003, "bf16"), (149, 5003, "bf16"), (592, 5003, "bf16"),
                                        (1300, 5003, "bf16"), (5, 151936, "bf16"), (37, 151936, "f16"), (74, 4096, "f32"),
-                                       (75, 4096, "f32"), (9, 262143, "f32")])
+                                       (75, 4096, "f32"), (9, 262143, "f32"),
+                                       # rows longer than registers hold, in one launch and in two
+                                       (18, 330001, "bf16"), (19, 330001, "bf16"), (9, 170001, "f32"), (10, 170001, "f32")])
 def test_launches_of_a_call(T, V, dtype):
     """Both policies' rows in one launch, in two with either first, and in three, on both sides of the rules' lines.  Without
     some of the outputs, or with the gradient over the inference rows, the order is another one and the results the same."""
@@ -137,6 +139,16 @@ def test_launches_of_a_call(T, V, dtype):
         assert all(torch.equal(y, getattr(full, n)) for y in (getattr(again, n), getattr(placed, n), x)), n
     for n in ("lse", "logp_mp", "log_cov", "count"):
         assert all(torch.equal(getattr(r.infer, n), getattr(full.infer, n)) for r in (again, placed)), n
+
+
+# the last call in one launch and the first in two; the last whose rows are held in registers and the next
+@pytest.mark.parametrize("T", [296, 297, 256, 257])
+@pytest.mark.parametrize("dtype,V", [("bf16", 3001), ("f16", 2048), ("f32", 1500)])
+def test_launches_without_a_gradient(T, dtype, V):
+    b = inputs.make_rows(dataclasses.replace(W["c2_bf16_fwdbwd"], dtype=dtype), seed=T, device=DEV, T=T, V=V)
+    res = binding.dvp_forward(b.train, b.ids, 1e-3, infer_logits=b.infer, want_mask=True)
+    torch.cuda.synchronize()
+    parity.check_forward(res, b, 1e-3, V, False)
 
 
 @pytest.mark.parametrize("dtype,V,hint", [("bf16", 151936, 64), ("bf16", 151936, 256), ("bf16", 151936, 256 | (2 << 24)),
