@@ -39,9 +39,9 @@ FALLBACK_HBM_GBS = 6650.0
 # of one ncu capture of a dvp_forward call on T rows of the workload), keyed by (workload, rho); valid only for
 # the kernel sources whose digest is recorded with it, scaled by rows to the full batch.
 NCU_TRAFFIC = {
-    ("c2_bf16_fwdbwd", 1e-4): {"digest": "fbf171d1213483e9", "T": 2048, "bytes": 1.495955e9 + 0.571765e9},
-    ("c2_bf16_fwdbwd", 1e-3): {"digest": "fbf171d1213483e9", "T": 2048, "bytes": 1.311043e9 + 0.565727e9},
-    ("c3_f32_heavy", 1e-4): {"digest": "fbf171d1213483e9", "T": 1024, "bytes": 2.148007e9 + 1.015726e9},
+    ("c2_bf16_fwdbwd", 1e-4): {"digest": "82850c4fa03b6a92", "T": 2048, "bytes": 1.495955e9 + 0.571765e9},
+    ("c2_bf16_fwdbwd", 1e-3): {"digest": "82850c4fa03b6a92", "T": 2048, "bytes": 1.311043e9 + 0.565727e9},
+    ("c3_f32_heavy", 1e-4): {"digest": "82850c4fa03b6a92", "T": 1024, "bytes": 2.148007e9 + 1.015726e9},
 }
 
 
@@ -64,9 +64,9 @@ def _kernel_digest(names=("dvp_common.cuh", "dvp_rows_impl.cuh")) -> str:
 # panels of 4096 rows): the first panel's three and a later panel's three (whose d_w contraction also reads
 # the d_w it adds to).  Valid for the sources whose digest is recorded; a step of P panels is taken as the
 # first panel's launches plus P - 1 times the later panel's.
-NCU_TRAFFIC_FUSED = {"digest": "5d40d86b109ab9fb", "H": 4096, "V": 151936, "panel": 4096,
-                     "first": (4.615540e9 + 2.485369e9) + (13.608092e9 + 0.127318e9) + (5.593785e9 + 2.459819e9),
-                     "later": (4.840493e9 + 2.484551e9) + (12.678872e9 + 0.127140e9) + (8.013996e9 + 2.456163e9)}
+NCU_TRAFFIC_FUSED = {"digest": "db57252215816db0", "H": 4096, "V": 151936, "panel": 4096,
+                     "first": (3.018167e9 + 2.480462e9) + (11.236731e9 + 0.123671e9) + (3.646053e9 + 2.459666e9),
+                     "later": (3.338261e9 + 2.479805e9) + (11.140675e9 + 0.123398e9) + (5.728769e9 + 2.454251e9)}
 FUSED_SOURCES = ("dvp_gemm.cuh", "dvp_fused.cu", "dvp_panel.cuh")
 
 

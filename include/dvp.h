@@ -140,7 +140,7 @@ typedef struct {
  *   grad_train    device [T, ld_grad] of grad_dtype: g_t (1[k=a] - pi^mp(k))
  *                 on V_S, 0 off it, the whole row 0 when a is not in V_S;
  *                 rounded to nearest-even in grad_dtype.  With the default
- *                 kernel it may take the place of train_logits or
+ *                 kernels it may take the place of train_logits or
  *                 infer_logits (the same type, base and stride) when no
  *                 `mask` is asked for; other overlaps with the logits are
  *                 not allowed.  With weights and none of infer.logp_mp,
@@ -154,14 +154,18 @@ typedef struct {
  *                 grad_train; weight_lo <= weight_hi, both >= 0, not NaN
  *   weight_out    device [T] float32 or NULL: the weight each token used (NaN
  *                 for a row without a valid sampled id)
- *   launch_hint   0 = library default; otherwise threads per block (a multiple
+ *   launch_hint   0 = library default: calls of up to 512 tokens (256 without a gradient)
+ *                 whose rows the registers of the chip hold at once are one launch of a
+ *                 kernel that reads every row once and keeps it there, all others go to
+ *                 the row kernel below; otherwise threads per block (a multiple
  *                 of 32, at most 512) in the low 16 bits, a kernel choice in the
  *                 next 8 bits, and the number of blocks that share one row (0, 1, 2,
  *                 4 or 8; a thread-block cluster) in the top 8 bits.  Kernel choice:
- *                 0 or 2 the default kernel (64, 128, 256 or 512 threads, the largest
+ *                 0 or 2 the row kernel (64, 128, 256 or 512 threads, the largest
  *                 not above the hint, 64 for a hint of 32; one sweep with the masked sum under a guess of
  *                 the maximum, then revisits of the 32-byte pieces of the row that can
- *                 hold safe tokens); 3 or 4 (2-byte
+ *                 hold safe tokens), where threads or blocks are given for small calls
+ *                 too; 3 or 4 (2-byte
  *                 logits, at most 256 threads, no cluster) the kernel that keeps
  *                 the candidates of the safe set in shared memory while the row
  *                 streams and reads nothing twice, with 3 or 4 blocks per SM;
@@ -169,7 +173,7 @@ typedef struct {
  *                 in shared memory (rows of up to 480 KB whose byte length is a
  *                 multiple of 16).  Choices 3, 4 and 0x11 need every row of every
  *                 matrix on a 32-byte boundary.  Rows a chosen kernel cannot take run the
- *                 default one.  Tuning only: the safe set and counts do not
+ *                 row kernel.  Tuning only: the safe set and counts do not
  *                 depend on it.
  *                 TEST ONLY: 0x1e in the second byte is a self-test of the 0x11
  *                 kernel's wait limit, not an operating mode: its first block
@@ -177,7 +181,7 @@ typedef struct {
  *                 a second, the launch ends by itself with undefined outputs and
  *                 dvp_row_wait_status reports code 1 or 2
  *
- * The default kernel takes any row stride and any base that is aligned to its element
+ * The default kernels take any row stride and any base that is aligned to its element
  * type at full width: rows are cut at their own 32-byte boundaries.  Needs no workspace.
  * Errors: DVP_ERR_INVALID_ARG for NULL required
  * pointers, T < 0, V < 1, ld < V, rho outside [0,1] or NaN, upstream without

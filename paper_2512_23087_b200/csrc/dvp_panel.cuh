@@ -224,8 +224,8 @@ __global__ void __launch_bounds__(kSums / kSets, 2 * kSets) dvp_panel_kernel(con
 // The inference rows and the panel's in one launch, for calls of one panel whose panel rows need nothing of the others: the
 // inference rows come first, in the places that the logits contraction's last, partly filled wave leaves, and the panel's
 // rows follow without a wave that ends between them.  sum_ranges_kernel forms the log-ratios.  kPieces: inference rows off
-// the 32-byte grid.  us a call, two launches / one: 512 x 1,024 x 32,000 187 / 177.5, 767 x 1,448 x 10,474 145 / 136, 163 x 416 x
-// 45,277 132 / 114, 3,000 x 512 x 16,000 310 / 305, 6,000 x 512 x 16,001 670 / 622.  (Four granules a thread in flight in the
+// the 32-byte grid.  us a call, two launches / one: 512 x 1,024 x 32,000 184.7 / 169.6, 767 x 1,448 x 10,474 154.7 / 140.4, 163 x
+// 416 x 45,277 132.1 / 113.6, 1,200 x 1,024 x 16,000 204.3 / 195.4, 3,000 x 512 x 16,000 304 / 295, 6,000 x 512 x 16,001 640 / 626.  (Four granules a thread in flight in the
 // panel's rows instead of two: 2 % more time.)
 template <bool kPieces>
 __global__ void __launch_bounds__(kSums / 2, 4) dvp_both_rows_kernel(const __grid_constant__ PanelParams pp,
@@ -320,8 +320,9 @@ add_sampled_hidden_kernel(const void *ids, int id_is_i32, const float *a_coef, i
   uint32_t *same = reinterpret_cast<uint32_t *>(id_of + kIdChunk) + warp * (kIdChunk / 32);  // bit j: token j has our id
   const int i = (int)blockIdx.x * kSampledWarps + warp;
   // Which token adds what needs only the ids and the panel's coefficients, which were complete before d_w's contraction
-  // began: it is found while that ends.  d_w itself is waited for.  (512 x 1,024 x 32,000 173 -> 167 us a call, 767 x 1,448 x
-  // 10,474 141 -> 139.5.)
+  // began: it is found while that ends.  d_w itself is waited for.  (us a call with the wait in front / here: 163 x 416 x 45,277
+  // 115.0 / 113.6, 1,200 x 1,024 x 16,000 197.0 / 195.4, 3,000 x 512 x 16,000 301 / 295; 512 x 1,024 x 32,000 173 / 170 and 767 x
+  // 1,448 x 10,474 140.4 / 140.4, no more than processes differ.)
   const int n4 = (n + 127) & ~127;
   constexpr int kBlk = kSampledWarps * 32, kLoads = 8;  // all of a batch before the first is stored
   for (int j0 = threadIdx.x; j0 < n4; j0 += kLoads * kBlk) {

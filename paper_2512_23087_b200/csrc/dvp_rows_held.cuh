@@ -307,11 +307,11 @@ struct Shape {
 // begun one after the other, so that many of them cost more than they save: up to 512 tokens, 256 without a gradient; and
 // those of several blocks a row take whole SMs of one part of the chip, of which some are left over: up to three quarters of
 // the threads.
-// Device us, the row kernel / this one (a graph of 20 calls): with the gradient 64 x 4,096 float32 7.5 / 5.8, 300 x 8,000 float16
-// 11.1 / 8.6, 400 x 2,100 bfloat16 10.0 / 7.5, 148 x 32,000 15.4 / 11.4, 24 x 100,000 14.1 / 11.8, 8 x 262,144 13.3 / 11.8, 512 x 4,000
-// 10.4 / 8.9, weighted 148 x 2,312 float32 7.4 / 6.0;  forward 4 x 20,000 5.7 / 5.3, 256 x 4,000 5.3 / 5.2, 148 x 32,000 11.5 / 8.3,
-// 12 x 151,936 10.7 / 8.8; one policy 64 x 30,000 7.9 / 5.6.  Five granules: 16 x 151,936 12.2 / 9.0 and with the gradient 15.7 /
-// 13.2, 140 x 40,000 13.0 / 9.1 and 17.7 / 13.3, 250 x 20,000 10.8 / 9.4 and 14.7 / 13.2.  Beyond: with the gradient 1,000 x 2,048 11.3 /
+// Device us, the row kernel / this one (a graph of 20 calls): with the gradient 64 x 4,096 float32 7.3 / 5.7, 300 x 8,000 float16
+// 11.0 / 8.7, 400 x 2,100 bfloat16 10.1 / 7.5, 148 x 32,000 15.4 / 11.3, 24 x 100,000 13.9 / 11.4, 8 x 262,144 13.2 / 11.8, 512 x 4,000
+// 10.5 / 8.8, weighted 148 x 2,312 float32 7.5 / 6.1;  forward 4 x 20,000 5.7 / 5.3, 256 x 4,000 5.3 / 5.3, 148 x 32,000 11.2 / 8.4,
+// 12 x 151,936 11.3 / 8.8; one policy 64 x 30,000 7.8 / 5.5.  Five granules: 16 x 151,936 12.4 / 9.2 and with the gradient 15.8 /
+// 12.9, 140 x 40,000 13.0 / 9.2 and 17.8 / 13.4, 250 x 20,000 10.9 / 9.4 and 14.8 / 13.3.  Beyond: with the gradient 1,000 x 2,048 11.3 /
 // 12.6, 72 x 50,000 (two blocks a row) 16.2 / 16.5; forward 600 x 4,000 7.5 / 9.9, 72 x 50,000 11.9 / 13.2, 16 x 151,936 in eight
 // blocks of four granules 12.1 / 12.4; one policy 500 x 4,000 4.4 / 4.6.
 static inline bool shape_of(long long T, bool both, bool grad, long long n_gran, Shape *s) {

@@ -1552,10 +1552,13 @@ static inline bool grad_over_its_infer_row(const RowParams &p) {
 // Both policies' rows, in one launch, two or three; the second may begin while the first ends.
 //
 // One launch for calls that fill half of the chip at most, bound by the chain of their phases and by what a launch costs on
-// the host (2 of 17 us); the sizes below are now those of dvp_rows_held.cuh.  Device time of 64 x 4,096 float32, forward / with the gradient, two launches and one: 6.5 / 8.5
-// and 5.8 / 7.9 us; 8 x 151,936 bfloat16 10.5 / 12.6 and 9.3 / 12.1; weighted 148 x 2,312 float32 10.1 and 7.8.  Above,
-// clusters wait for free places: 1,100 x 2,500 bfloat16 10.1 / 12.8 and 12.5 / 17.4, 32 x 151,936 (clusters of 16) 13.7 /
-// 17.6 and 16.6 / 22.1.
+// the host.  Most of them go to dvp_rows_held.cuh; left are 257 to 296 short rows without a gradient, and rows that are too
+// long for registers.  Device us, two launches / one (a graph of 20 calls): forward 280 x 3,000 bfloat16 6.0 / 5.2, 296 x 3,001
+// 6.3 / 5.5, 296 x 1,500 float32 6.0 / 5.3, 260 x 2,048 float16 5.2 / 5.2; with the gradient 4 x 400,000 bfloat16 15.0 / 13.5.  Long
+// rows near the line, clusters of 16 blocks, lose by it: 18 x 330,001 bfloat16 20.9 / 21.8 with the gradient, 16.1 / 16.0
+// without, 9 x 170,001 float32 13.9 / 16.3 and 11.5 / 12.3, 4 x 262,144 float32 13.6 / 13.9 and 11.5 / 11.0.  Above the line
+// clusters wait for free places: forward 400 x 3,000 bfloat16 6.5 / 6.8, 560 x 3,000 7.3 / 7.9, 24 x 330,001 19.0 / 20.2; with the
+// gradient 19 x 330,001 19.2 / 20.5, 24 x 330,001 22.8 / 27.1, 12 x 170,001 float32 15.3 / 16.9, 18 x 170,001 19.8 / 26.0.
 // Otherwise the rows with a gradient come first: the chip's last wave then has the short rows.  While all rows fit the chip
 // at once the inference rows wait for the training rows at their end; in larger batches they would hold their places
 // idle, so that neither launch waits for the other and a third one forms the log-ratios and flags (the inference rows'
