@@ -85,22 +85,25 @@ __device__ __forceinline__ float max_from(const Group &grp, const Slots &slots, 
   return key_value(__reduce_max_sync(0xffffffffu, order_key(m)));
 }
 
-// kGran: granules of a row that a thread holds.
+// kGran: granules of a row that a thread holds.  `shape`: log2 of the blocks of a row, and kOverInfer where a row has one block
+// and the gradient takes the inference rows' place.  (As a flag of the launch: the pointers compared here instead, and the
+// shift by an unmasked argument, cost 0.3 us: 64 x 4,096 float32 with the gradient 5.9 / 5.4 us, 148 x 16,000 9.6 / 9.4.)
+constexpr int kOverInfer = 16;
 template <typename TIn, typename TGrad, Grad kGrad, int kGran>
-__global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_constant__ RowParams p, const int log_parts) {
+__global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_constant__ RowParams p, const int shape) {
   using Ops = SweepOps<TIn>;
   constexpr int kElems = Granule<TIn>::kElems;
   __shared__ Slots slots;
   __shared__ __align__(16) uint32_t shift_smem[kGrad == Grad::kLoose ? kMaxWarps * kShiftWords : 1];
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, n_thr = (int)blockDim.x;
-  const int both = p.infer ? 1 : 0, parts = 1 << log_parts;
+  const int log_parts = shape & (kOverInfer - 1), both = p.infer ? 1 : 0, parts = 1 << log_parts;
   const Group grp{parts << both, log_parts, 31 - __clz(n_thr >> 5)};
   const int rank = grp.blocks > 1 ? (int)cluster_rank() : 0, part = rank & (parts - 1), r0 = rank - part;
   const bool second = rank >= parts;  // the inference row's half
   // Blocks write to one another's shared memory once all have begun.  Where a row has one block and the gradient takes the
   // inference row's place, they meet when both rows have been read instead, which no other barrier in front of the gradient
   // says there: the blocks of a longer row meet across the cluster for their maximum, weights wait for the inference row.
-  const bool over_infer = kGrad != Grad::kNone && log_parts == 0 && p.grad == p.infer;
+  const bool over_infer = kGrad != Grad::kNone && (shape & kOverInfer);
   if (grp.blocks > 1 && !over_infer) cluster_arrive();
   const long long t = blockIdx.x >> (log_parts + both);
   const long long id = p.ids ? load_id(p.ids, p.id_is_i32, t) : -1;
@@ -216,7 +219,6 @@ __global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_c
 
   const SideStats st = stats_from<TIn>(grp, slots, r0, m, p, has_a, z_a);
   const bool weighted = p.weight_kind != DVP_WEIGHT_NONE;
-  const float upstream = kGrad != Grad::kNone && !second ? p.upstream[t] : 0.f;
   if (both) {
     if (second && part == 0 && tid < parts) {
       st_cluster(&slots.li, tid, logp_mp_of(st));
@@ -231,7 +233,7 @@ __global__ void __launch_bounds__(kMaxBlk, 2) dvp_row_kernel_held(const __grid_c
   // ---- the gradient (row_grad's arithmetic)
   if constexpr (kGrad != Grad::kNone) {
     if (!second) {
-      float g = upstream;
+      float g = p.upstream[t];
       if (weighted && both) {  // weights need inference rows
         cluster_wait();
         const float w = has_a ? token_weight(ratio_of(), p.weight_kind, p.weight_lo, p.weight_hi) : __int_as_float(0x7fc00000);
@@ -351,7 +353,8 @@ static cudaError_t launch(const RowParams &p, const Shape &sh, cudaStream_t s) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = log_cluster > 0 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, k, p, sh.log_parts);
+  const bool over_infer = kGrad != Grad::kNone && sh.log_parts == 0 && p.grad == p.infer;
+  return cudaLaunchKernelEx(&cfg, k, p, sh.log_parts | (over_infer ? kOverInfer : 0));
 }
 
 }  // namespace held
