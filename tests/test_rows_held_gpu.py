@@ -53,6 +53,21 @@ def test_edges(dtype, T, V, checks):
             parity.check_forward(res, b, rho, V, True)
 
 
+# one block a row with three granules a thread, with two, and the next rows, which have several without a gradient or with one
+@pytest.mark.parametrize("dtype,T,V", [("bf16", 6, 24576), ("bf16", 6, 24577), ("f16", 40, 8209), ("f32", 6, 12288), ("f32", 6, 12289),
+                                       ("bf16", 6, 16384), ("bf16", 6, 16385), ("f32", 40, 8192), ("f32", 6, 8193)])
+def test_one_policy(dtype, T, V):
+    b = _batch(dtype, T, V)
+    for rho in (1e-4, 0.0):
+        res = binding.dvp_forward(b.train, b.ids, rho, upstream=b.upstream)
+        alone = binding.dvp_forward(b.train, b.ids, rho)
+        torch.cuda.synchronize()
+        want = parity.run_oracle(b.train, None, b.ids, rho, upstream=b.upstream)
+        for r in (res, alone):
+            parity.check_side(r.train, want.train, b.train, V, "train", {})
+        parity.check_grad(res.grad_train, want.grad, {})
+
+
 # one, two, four and eight blocks a row
 @pytest.mark.parametrize("dtype,T,V", [("bf16", 148, 30001), ("f32", 300, 2003), ("f16", 50, 50021), ("f32", 50, 20003),
                                        ("bf16", 9, 30001), ("bf16", 25, 100001), ("f16", 5, 50021), ("f32", 3, 60000)])
