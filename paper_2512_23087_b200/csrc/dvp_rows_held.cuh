@@ -308,18 +308,18 @@ struct Shape {
 // are: 148 x 32,000 with the gradient 12.7 / 13.5 us a call); while it has room, more threads a row are faster.  Clusters are
 // begun one after the other, so that many of them cost more than they save: up to 512 tokens, 256 without a gradient; and
 // those of several blocks a row take whole SMs of one part of the chip, of which some are left over: up to three quarters of
-// the threads.  A row of one policy needs no cluster while one block holds it with three granules a thread.  Device us, the row
-// kernel / two or four blocks / one, 30 x 8,200 bfloat16 4.15 / 5.09 / 4.18, 30 x 16,000 4.56 / 4.98 / 4.52, 30 x 24,000 5.77 / 5.09 /
-// 5.00, 1 x 7,000 float32 4.46 / 4.60 / 4.15, 30 x 12,001 4.98 / 4.98 / 4.57.  With the gradient two: 12 x 8,200 bfloat16 6.0 / 6.0 /
-// 5.3, 30 x 16,000 7.3 / 6.2 / 6.0, 30 x 20,001 8.9 / 6.2 / 6.8.
-// Device us, the row kernel / this one (a graph of 20 calls): with the gradient 64 x 4,096 float32 7.3 / 5.7, 300 x 8,000 float16
-// 11.0 / 8.7, 400 x 2,100 bfloat16 10.1 / 7.5, 148 x 32,000 15.4 / 11.3, 24 x 100,000 13.9 / 11.4, 8 x 262,144 13.2 / 11.8, 512 x 4,000
-// 10.5 / 8.8, weighted 148 x 2,312 float32 7.5 / 6.1;  forward 4 x 20,000 5.7 / 5.3, 256 x 4,000 5.3 / 5.3, 148 x 32,000 11.2 / 8.4,
-// 12 x 151,936 11.3 / 8.8; one policy 64 x 30,000 7.8 / 5.5.  Five granules: 16 x 151,936 12.4 / 9.2 and with the gradient 15.8 /
-// 12.9, 140 x 40,000 13.0 / 9.2 and 17.8 / 13.4, 250 x 20,000 10.9 / 9.4 and 14.8 / 13.3.  Beyond: with the gradient 1,000 x 2,048 11.3 /
+// the threads.  A row of one policy needs no cluster while one block holds it with three granules a thread.  Device
+// us, the row kernel / two or four blocks / one: 30 x 8,200 bfloat16 4.1 / 5.1 / 4.1, 30 x 16,000 4.6 / 5.0 / 4.3, 30 x 24,000 5.9 /
+// 5.1 / 4.7, 1 x 7,000 float32 4.2 / 4.6 / 3.7, 30 x 12,001 4.9 / 5.0 / 4.4.  With the gradient two: 12 x 8,200 bfloat16 6.0 / 6.0 / 4.9,
+// 30 x 16,000 7.4 / 6.2 / 5.9, 30 x 20,001 8.8 / 6.0 / 6.8.
+// Device us, the row kernel / this one (a graph of 20 calls): with the gradient 64 x 4,096 float32 7.4 / 5.2, 300 x 8,000 float16
+// 10.9 / 8.1, 400 x 2,100 bfloat16 10.1 / 7.4, 148 x 32,000 15.4 / 11.2, 24 x 100,000 13.9 / 11.8, 8 x 262,144 12.9 / 11.7, 512 x 4,000
+// 10.5 / 8.6, weighted 148 x 2,312 float32 7.5 / 5.7;  forward 4 x 20,000 5.7 / 5.3, 256 x 4,000 5.4 / 5.4, 148 x 32,000 11.2 / 8.3,
+// 12 x 151,936 11.3 / 8.6; one policy 64 x 30,000 7.9 / 5.3.  Five granules: 16 x 151,936 12.2 / 9.6 and with the gradient 15.5 /
+// 13.2, 140 x 40,000 13.1 / 8.9 and 17.8 / 13.4, 250 x 20,000 10.9 / 9.2 and 14.8 / 13.2.  Beyond: with the gradient 1,000 x 2,048 11.3 /
 // 12.6, 72 x 50,000 (two blocks a row) 16.2 / 16.5; forward 600 x 4,000 7.5 / 9.9, 72 x 50,000 11.9 / 13.2, 16 x 151,936 in eight
-// blocks of four granules 12.1 / 12.4; one policy 500 x 4,000 4.4 / 4.6.  Slower inside it by 2 to 4 %: forward 240 and 256 tokens of
-// 12,500 to 16,384 bfloat16 logits (256 x 16,000 8.4 / 8.7; 17,000 11.3 / 9.4, 220 x 16,000 7.9 / 7.6).
+// blocks of four granules 12.1 / 12.4; one policy 500 x 4,000 4.4 / 4.6.  Inside, where the chip is full, as fast: forward 256 x 16,000
+// bfloat16 8.4 / 8.4, 240 x 12,500 8.2 / 8.3; slower 256 x 2,100 5.4 / 5.6.
 static inline bool shape_of(long long T, bool both, bool grad, long long n_gran, Shape *s) {
   constexpr long long kChip = 148 * 1024, kMost = 8 * kMaxBlk;
   const long long rows = both ? 2 * T : T;
